@@ -48,7 +48,7 @@ struct __align__(16) ColMeta {
   uint8_t flags;    // F_PROVEN | F_FINAL | F_NEWPIV
   uint8_t cleared;  // zeroed by clearing (Lemma 1)
   uint8_t low_seen; // the id was the low of some column at the start of some pass
-  uint8_t spare;
+  uint8_t spare;    // rows in its delta: added to it, but not in its list yet
 };
 static_assert(sizeof(ColMeta) == 16, "one 16-byte record per column");
 
@@ -61,7 +61,7 @@ __device__ __forceinline__ ColMeta load_meta(const ColMeta* p) {
   m.flags = (uint8_t)(v.w & 0xff);
   m.cleared = (uint8_t)((v.w >> 8) & 0xff);
   m.low_seen = (uint8_t)((v.w >> 16) & 0xff);
-  m.spare = 0;
+  m.spare = (uint8_t)((v.w >> 24) & 0xff);
   return m;
 }
 
@@ -95,12 +95,21 @@ struct ReduceState {
   int32_t** nxt_ptr = nullptr; // per active slot: new location
   int32_t* nxt_len = nullptr;
   int32_t* owner = nullptr;    // per row id: proven pivot with that low, -1
-  int32_t* tab = nullptr;      // two tables per row id: left-most column with that low (pass p: p & 1)
+  unsigned long long* tab = nullptr;  // per row id: left-most column with that low
+  int32_t* dirty = nullptr;    // segments whose first_unp became paired: search state, flags, list
   int32_t* first_unp = nullptr;// per segment: first row id not known to be paired
   void* tiles = nullptr;       // scan scratch
   void* look = nullptr;        // look-back states of the survivor scan
   void* dlist = nullptr;       // deferred column updates
   void* src_e = nullptr;       // per active slot: source candidate of Phase II
+  int32_t* lows = nullptr;     // [lows_rows][m] per pass (ring) and slot: the low at its start
+  int32_t lows_rows = 0;
+  int32_t* due = nullptr;      // per slot: the pass whose additions visit its column next
+  void* prec = nullptr;        // per row: its proven pivot's rows (int4)
+  int32_t* delta = nullptr;    // per id: rows added to the column that are not in its list yet
+  uint8_t* kind = nullptr;     // per slot: what k_merge does with its column
+  int32_t* newpos = nullptr;   // per slot: its place after a compacting pass, -1
+  int32_t* work = nullptr;     // slots of the columns that k_merge takes in this pass
   uint32_t* unp_bits = nullptr;  // Corollary 10 predictions: unpaired-row bitmap
   int32_t* unp_words = nullptr;  // and its per-word prefix counts
   int32_t* pred = nullptr;       // per id: predicted lowstar, -1
@@ -114,12 +123,16 @@ struct ReduceState {
   void* hstate = nullptr;      // pinned host mirror of it
   int64_t* pass_stats = nullptr;  // device [stats_rows][PH_PS_N]
   int32_t stats_rows = 0;
-  ColStore arena[2];           // pass p writes its survivors into arena[p & 1]
+  ColStore arena[2];           // survivors; compacting passes change from one to the other
+  struct Retired {
+    int32_t* p;
+    int32_t until;             // holds columns up to this (compacting) pass
+  };
+  std::vector<Retired> retired;  // arena buffers outgrown between two compacting passes
   std::vector<ColStore> pivots;  // chunks holding proven columns
-  // the pass loop: one pass as the body of a conditional while node, per variant of the
-  // additions kernel (+1 bit-packed columns, +2 one chunk per warp, +4 jobs merged by lanes;
-  // 8, 9: 8-slot warp chunks with merge pieces, without and with bit-packed columns)
-  static constexpr int kAddVariants = 10;
+  // the pass loop: one pass as the body of a conditional while node, per variant of its additions
+  // (add_variant)
+  static constexpr int kAddVariants = 14;
   cudaGraph_t graph[kAddVariants] = {};
   cudaGraphExec_t graph_exec[kAddVariants] = {};
   int32_t passes = 0;
@@ -189,6 +202,9 @@ struct ph_ctx {
   int32_t* p_dim = nullptr;
   int64_t *e_idx = nullptr, *e_d2 = nullptr;
   int32_t* e_dim = nullptr;
+
+  // a column of the boundary matrix has at most three rows
+  bool three_rows() const { return col_off == nullptr && max_dim <= 2; }
 
   void* dalloc(size_t bytes);
   void dfree(void* p);

@@ -42,6 +42,7 @@
 // from a host loop or as the body of a graph's conditional while node. Each kernel may start
 // while its predecessor drains (programmatic dependent launch) and waits for it first.
 #include <algorithm>
+#include <utility>
 
 #include "ph_internal.cuh"
 
@@ -51,6 +52,7 @@ namespace ph {
 enum : int32_t { ST_RUN = 0, ST_DONE = 1, ST_CAPPED = 2, ST_HOST = 3, ST_FAULT = 4,
                  ST_TIMEOUT = 5, ST_SWITCH = 6 };
 constexpr int kSpinLimit = 1 << 22;  // iterations of a look-back wait before it gives up
+constexpr int kBarrierLimit = 1 << 24;  // ... of a grid barrier's (a second or so)
 
 struct DevState {
   int32_t* act;   // active ids, ascending
@@ -58,8 +60,7 @@ struct DevState {
   int32_t* alen;   // per slot of act: its column's stored length (ColMeta::len)
   int32_t* alen2;  // the same for act2
   int64_t n_act;
-  int32_t* arena[2];  // pass p writes its survivors into arena[p & 1]
-  int32_t* tab[2];    // pass p reads its left-most-column table tab[p & 1], builds tab[(p+1) & 1]
+  int32_t* arena[2];  // survivors are written into arena[arena_cur]
   int64_t arena_cap[2];
   int32_t* piv_base;  // current chunk of the pivot store
   int64_t piv_cap;
@@ -82,6 +83,10 @@ struct DevState {
   alignas(128) unsigned int queue;             // next chunk for k_add
   alignas(128) unsigned int tile_queue;        // next tile for k_phase1
   alignas(128) int32_t n_deferred;             // entries of dlist
+  alignas(128) unsigned int n_work;            // entries of work
+  alignas(128) unsigned int n_dirty;           // entries of dirty
+  alignas(128) unsigned int bar_count;         // grid barriers of k_loop: blocks arrived, and
+  alignas(128) unsigned int bar_gen;           // barriers done
   alignas(128) int32_t fault;                  // a bounded wait ran out
   int32_t debug_fault;  // the first failed bounds check of the debug build (PH_DCHECK), 0 if none
   // bit-packed columns: the passes after the first one that saw a target that may reach its
@@ -101,11 +106,23 @@ struct DevState {
   // switches once per reduction (ST_SWITCH)
   int32_t lane_on;
   int64_t lane_words;
-  // ... and once merge pieces are on and fewer than narrow_below columns are active, warp
-  // chunks of 8 slots, so that the short late passes spread over more warps (ST_SWITCH, once)
+  // ... and once merge pieces are on and fewer than narrow_below columns are active, rounds of
+  // 8 columns per warp, so that the short late passes spread over more warps (ST_SWITCH, once)
+  unsigned int loop_blocks;  // blocks of the loop kernel still at work
+  int64_t loop_below;  // the loop kernel takes over from the graph at this many columns (-1: never)
   int32_t narrow_on;
   int64_t narrow_below;
-  int32_t chunk_slots;  // slots per chunk of this pass's additions kernel (8, 32 or 128)
+  int32_t chunk_slots;  // slots per chunk of this pass's k_add (8, 32, 64 or 128)
+  // Look-ahead (see look_ahead): a column visited by the additions of pass p may run up to
+  // `ahead` passes at once, but never past the pass `horizon`, where every column is up to date
+  // again, the active list is compacted and the columns move to the other arena
+  int32_t ahead;       // 1: every pass's additions are k_add's, all columns, as in Algorithm 2
+  int64_t ahead_above; // ... from the first horizon with fewer columns than this
+  int32_t horizon;
+  int32_t compact;    // this pass compacts the active list (its columns are all up to date)
+  int32_t arena_cur;  // the arena this pass writes into
+  int32_t drain;      // past the time bound: no more look-ahead, stop at the horizon
+  int32_t leave;      // the last pass of look-ahead
 };
 
 struct RArgs {
@@ -116,7 +133,11 @@ struct RArgs {
   int32_t** nxt_ptr;
   int32_t* nxt_len;
   int32_t* owner;
-  int32_t* first_unp;
+  unsigned long long* tab;  // per row: the left-most column with that low (tab_key_of)
+  int32_t* first_unp;       // per segment: its first row not known to be paired
+  int32_t* next_unp;        // ... while it is searched for (INT32_MAX otherwise)
+  int32_t* dirty;           // segments whose first_unp became paired in this pass,
+  int32_t* dirty_on;        // and per segment whether it is among them
   const int32_t* seg;
   int64_t rows_end;
   int nseg;           // (cloud, dim) segments
@@ -125,8 +146,19 @@ struct RArgs {
   int cor10;
   unsigned long long* tile_st;  // per Phase I tile: look-back state of its aggregate / prefix
   unsigned long long* look;  // per Phase II chunk: look-back state of the survivor count
-  int32_t* dlist;     // active slots whose column update waits for k_commit
+  int32_t* dlist;     // columns whose update (nxt_ptr, nxt_len) waits for k_commit
+  int32_t* newpos;    // per active slot, in a pass that compacts: its place in the next list, -1
   int32_t* src_e;     // per active slot: the colliding column's left-most column, -1 if none
+  // look-ahead: lows[(q & ring) * m + e] is the low of slot e's column at the start of pass q,
+  // for the passes up to due[e], the pass whose additions visit the column next
+  int32_t* lows;
+  int32_t* due;
+  int64_t lows_stride;
+  int32_t ring;       // rows of `lows` less one (a power of two less one)
+  int4* prec;         // per row: its proven pivot's other rows (rec_of)
+  int32_t* delta;     // per id: rows added to the column that are not in its list yet
+  uint8_t* kind;      // per slot, and
+  int32_t* work;      // the slots, of the columns that k_visit leaves to k_merge
   // bit-packed columns: a job's result is a bitmap over its row segment when the sum of the two
   // row counts exceeds the threshold, max(the stored bitmap's words, t0) with t0 = dense_mode
   // when > 0, else 32 (dense_mode < 0: never), or when either column is already a bitmap
@@ -161,9 +193,20 @@ struct PV {
   int dense_on;
   int64_t arena_next_cap;  // words of arena_next and of the pivot store's chunk (bounds checks)
   int64_t piv_cap;
-  int32_t* tab;       // per row: the left-most active column with that low (or its pivot)
-  int32_t* tab_next;  // the same for the next pass, built during this one
+  unsigned long long tab_key;  // tab_key_of the next pass, whose table is built during this one
+  int32_t compact;
+  int32_t limit;      // the last pass a column visited now may run ahead to
+  int32_t ahead;      // passes a visit may run ahead; 1: every pass visits every column
+  int32_t whole;      // ... and the lists must be whole there (the pass cap, or the time bound)
 };
+
+// The left-most-column table holds, per row, a column below the pass it was entered for, counted
+// down: an atomicMin lets later passes' entries replace earlier ones, and the left-most
+// column win within a pass, so the table is never reset. A proven pivot is the left-most column of
+// its low for good: its entry has no pass and wins for ever.
+__device__ __forceinline__ unsigned long long tab_key_of(int32_t pass) {
+  return (unsigned long long)(0x7fffffff - pass) << 32;
+}
 
 __device__ __forceinline__ PV pass_view(const DevState* ds) {
   PV v;
@@ -174,13 +217,17 @@ __device__ __forceinline__ PV pass_view(const DevState* ds) {
   v.n_act = ds->n_act;
   v.do_adds = ds->pass < ds->max_passes;
   v.stats = ds->stats ? ds->stats + (int64_t)ds->pass * PH_PS_N : nullptr;
-  v.arena_next = ds->arena[ds->pass & 1];
+  v.arena_next = ds->arena[ds->arena_cur];
   v.piv_base = ds->piv_base;
   v.dense_on = ds->dense_on;
-  v.arena_next_cap = ds->arena_cap[ds->pass & 1];
+  v.arena_next_cap = ds->arena_cap[ds->arena_cur];
   v.piv_cap = ds->piv_cap;
-  v.tab = ds->tab[ds->pass & 1];
-  v.tab_next = ds->tab[(ds->pass + 1) & 1];
+  v.tab_key = tab_key_of(ds->pass + 1);
+  v.compact = ds->compact;
+  v.ahead = ds->ahead;
+  v.limit = ds->drain || ds->leave ? ds->pass + 1
+                      : min(min(ds->pass + ds->ahead, ds->horizon), ds->max_passes);
+  v.whole = ds->drain || v.limit == ds->max_passes;
   return v;
 }
 
@@ -216,63 +263,113 @@ __device__ __forceinline__ bool last_block(unsigned int* done, unsigned int part
 }
 
 // ------------------------------------------------------------------------------------------
-// The row state pass q reads, from the pivots, flags and beta as they stand when the pass before
-// it ends (k_commit; at set-up for the first pass): the reset, to the proven pivots (owner), of
-// the table that pass q's additions fill for pass q + 1; the first row of each (cloud, dim)
-// segment that is not known to be paired (Corollary 10; two copies alternate between passes);
-// and the unpaired bitmap (pair predictions). Every block of the grid takes part; the grid's last
-// block then finishes it with rows_of_pass_last.
-__device__ void rows_of_pass(const RArgs& a, int32_t q) {
-  int32_t* tab_reset = a.ds->tab[(q + 1) & 1];
-  int32_t* fu = a.first_unp + (int64_t)(q & 1) * a.nseg;
+// The row state of the next pass, from the pivots, flags and beta as they stand: at set-up the
+// first row of each (cloud, dim) segment that is not known to be paired (Corollary 10; later
+// passes move it on in next_unpaired), and for every pass the unpaired bitmap (pair predictions).
+// Every block of the grid takes part; the last block then finishes it with rows_of_pass_last.
+__device__ __forceinline__ bool is_unpaired(const RArgs& a, int64_t x) {
+  return !((a.meta[x].flags & F_PROVEN) || a.beta[x] >= 0 || a.owner[x] >= 0);
+}
+template <bool kFirst>
+__device__ void rows_of_pass(const RArgs& a, unsigned blocks) {
   // warp-uniform loop: each iteration a warp covers 32 consecutive rows, one bitmap word
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  const int64_t stride = (int64_t)blocks * blockDim.x;
   for (int64_t x0 = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); x0 < a.rows_end;
        x0 += stride) {
     const int64_t x = x0 + (threadIdx.x & 31);
-    bool unpaired = false;
-    if (x < a.rows_end) {
-      int32_t o = a.owner[x];
-      tab_reset[x] = o < 0 ? INT32_MAX : o;
-      unpaired = !((a.meta[x].flags & F_PROVEN) || a.beta[x] >= 0 || o >= 0);
-    }
+    const bool unpaired = x < a.rows_end && is_unpaired(a, x);
     const unsigned w = __ballot_sync(0xffffffffu, unpaired);
-    if (unpaired) {  // one atomic per segment present among the warp's unpaired rows: its first
+    if (kFirst && unpaired) {  // one atomic per segment among the warp's unpaired rows: its first
       const int32_t sg = a.seg[x];
       const unsigned same = __match_any_sync(w, sg);
-      if ((threadIdx.x & 31) == __ffs(same) - 1) atomicMin(&fu[sg], (int32_t)x);
+      if ((threadIdx.x & 31) == __ffs(same) - 1) atomicMin(&a.first_unp[sg], (int32_t)x);
     }
     if (a.predict && (threadIdx.x & 31) == 0) a.unp_bits[x0 >> 5] = w;
   }
 }
 
-// by the last block: the bitmap's prefix counts per word, and the first-unpaired copy of pass
-// q + 1 cleared for the atomics at the end of pass q
-__device__ void rows_of_pass_last(const RArgs& a, int32_t q) {
-  if (a.predict) {
-    __shared__ int64_t sh[kWarps + 1];
-    const int64_t nwords = (a.rows_end + 31) / 32;
-    int64_t carry = 0;
-    for (int64_t base = 0; base < nwords; base += kThreads) {
-      const int64_t w = base + threadIdx.x;
-      const int64_t c = w < nwords ? __popc(__ldcg(a.unp_bits + w)) : 0;
-      int64_t tot;
-      const int64_t ex = block_excl_sum<int64_t>(c, sh, tot);
-      if (w < nwords) a.unp_words[w] = (int32_t)(carry + ex);
-      carry += tot;
-    }
-    if (threadIdx.x == 0) a.unp_words[nwords] = (int32_t)carry;
+// by the last block: the bitmap's prefix counts per word
+__device__ void rows_of_pass_last(const RArgs& a) {
+  if (!a.predict) return;
+  __shared__ int64_t sh[kWarps + 1];
+  const int64_t nwords = (a.rows_end + 31) / 32;
+  int64_t carry = 0;
+  for (int64_t base = 0; base < nwords; base += kThreads) {
+    const int64_t w = base + threadIdx.x;
+    const int64_t c = w < nwords ? __popc(__ldcg(a.unp_bits + w)) : 0;
+    int64_t tot;
+    const int64_t ex = block_excl_sum<int64_t>(c, sh, tot);
+    if (w < nwords) a.unp_words[w] = (int32_t)(carry + ex);
+    carry += tot;
   }
-  int32_t* fu_next = a.first_unp + (int64_t)((q + 1) & 1) * a.nseg;
-  for (int i = threadIdx.x; i < a.nseg; i += blockDim.x) fu_next[i] = INT32_MAX;
+  if (threadIdx.x == 0) a.unp_words[nwords] = (int32_t)carry;
+}
+
+// The segments whose first unpaired row became paired in this pass get their next one. Rows stay
+// paired, so the search starts at the old one; it ends some rows on as a rule, but far away after
+// the first pass, or when the row that held up a long run of paired ones is paired at last.
+// A few segments are searched by all blocks together, in strides that end once a lower row is
+// found, and next_unpaired_last, by the last block, takes over the result; many (of a batch, or
+// by a single block) by one block each.
+constexpr unsigned kSearchTogether = 4;
+__device__ __forceinline__ void next_unpaired(const RArgs& a, unsigned blocks) {
+  const unsigned nd = a.ds->n_dirty;
+  if (nd == 0) return;
+  if (nd <= kSearchTogether && blocks > 1) {
+    for (unsigned i = 0; i < nd; i++) {
+      const int32_t s = a.dirty[i];
+      const int64_t end = a.seg_start[s + 1];
+      int64_t x0 = (int64_t)a.first_unp[s] + blockIdx.x * blockDim.x + (threadIdx.x & ~31);
+      for (; x0 < end && x0 < *(volatile int32_t*)&a.next_unp[s];
+           x0 += (int64_t)blocks * blockDim.x) {  // by whole warps
+        const int64_t x = x0 + (threadIdx.x & 31);
+        const unsigned w = __ballot_sync(0xffffffffu, x < end && is_unpaired(a, x));
+        if (w) {
+          if ((threadIdx.x & 31) == __ffs(w) - 1) atomicMin(&a.next_unp[s], (int32_t)x);
+          break;
+        }
+      }
+    }
+    return;
+  }
+  __shared__ int32_t s_first;
+  for (unsigned i = blockIdx.x; i < nd; i += blocks) {
+    const int32_t s = a.dirty[i];
+    const int64_t end = a.seg_start[s + 1];
+    int32_t first = INT32_MAX;
+    for (int64_t x0 = a.first_unp[s]; x0 < end && first == INT32_MAX; x0 += blockDim.x) {
+      if (threadIdx.x == 0) s_first = INT32_MAX;
+      __syncthreads();
+      const int64_t x = x0 + threadIdx.x;
+      const unsigned w = __ballot_sync(0xffffffffu, x < end && is_unpaired(a, x));
+      if (w && (threadIdx.x & 31) == __ffs(w) - 1) atomicMin(&s_first, (int32_t)x);
+      __syncthreads();
+      first = s_first;
+      __syncthreads();
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      a.first_unp[s] = first;
+      a.dirty_on[s] = 0;
+    }
+  }
+}
+__device__ __forceinline__ void next_unpaired_last(const RArgs& a, unsigned blocks) {
+  const unsigned nd = a.ds->n_dirty;
+  if (nd > kSearchTogether || blocks == 1) return;
+  for (unsigned i = threadIdx.x; i < nd; i += blockDim.x) {
+    const int32_t s = a.dirty[i];
+    a.first_unp[s] = *(volatile int32_t*)&a.next_unp[s];
+    a.next_unp[s] = INT32_MAX;
+    a.dirty_on[s] = 0;
+  }
 }
 
 // set-up: the first pass's row state
 __global__ void k_rows_first(RArgs a) {
-  const int32_t q = a.ds->pass;
-  rows_of_pass(a, q);
+  rows_of_pass<true>(a, gridDim.x);
   if (last_block(&a.ds->blocks_done, gridDim.x)) {
-    rows_of_pass_last(a, q);
+    rows_of_pass_last(a);
     if (threadIdx.x == 0) a.ds->blocks_done = 0;
   }
 }
@@ -324,7 +421,8 @@ __global__ void k_tab(RArgs a) {
 #pragma unroll
     for (int k = 0; k < kTI; k++) {
       if (l[k] >= 0 && PH_DCHECK(&a.ds->debug_fault, l[k] < a.rows_end, 1)) {
-        if (v.tab[l[k]] > j[k]) atomicMin(&v.tab[l[k]], j[k]);
+        const unsigned long long key = tab_key_of(a.ds->pass) | (unsigned)j[k];
+        if (a.tab[l[k]] > key) atomicMin(&a.tab[l[k]], key);
         if (!a.meta[l[k]].low_seen) a.meta[l[k]].low_seen = 1;  // for the essential estimate
       }
     }
@@ -402,6 +500,60 @@ __device__ __forceinline__ bool goes_dense(const RArgs& a, int32_t j, int64_t n)
 
 
 // ------------------------------------------------------------------------------------------
+// look-ahead
+// ------------------------------------------------------------------------------------------
+// Nearly every addition's source is a proven pivot (95-99 % on Vietoris-Rips complexes), and
+// nearly every pivot is an unreduced column of d + 1 rows. A proven pivot is the left-most
+// column of its low for good and never changes, so as long as a column's low belongs to one, its
+// next additions depend on nothing else: the additions kernel runs them for several passes in
+// one visit (look_ahead) and stores the low of each pass. The passes in between read the stored
+// lows (k_phase1: Phase I, Corollary 10) and leave the column alone. Only the low of a column is
+// ever seen by other columns while it collides with a pivot, so every pass decides as if the
+// columns had been added one pass at a time. A column is visited again when its stored lows end
+// (due[e]), at the latest at the horizon, where all are up to date: then the active list is
+// compacted, its slots fixed until the next horizon (a slot whose column left holds dead_slot).
+constexpr int kAheadMax = 8;  // passes per visit (a power of two: rows of stored lows)
+// What visits add to a column gathers in a block of its own (its delta) until it is merged into
+// the column's list: up to kOld rows are kept from visit to visit, and a visit adds up to R rows
+// per pass: R = 2, the rows of a triangle's boundary beside its low. (Look-ahead is for complexes
+// whose columns have at most three rows; with R = 3, for tetrahedra, it lost: 8 Gaussian
+// dimensions, 120 points, 0.9 M simplices, 1.8 -> 2.8 ms.)
+constexpr int kSourceRows = 2;
+constexpr int kOld = 8;
+constexpr int64_t kAheadFrom = 3000000;   // columns from which look-ahead pays, and
+constexpr int64_t kAheadAbove = 500000;   // down to which it goes on
+constexpr int kLonger = 12;  // the longest source inside a visit: kRecRows + this many rows
+constexpr int kDeltaRows = kOld + kSourceRows * kAheadMax;
+
+// The rows of a row's proven pivot, one 16-byte record: x is its length (0: no pivot yet), y, z
+// and w its rows below the low, then INT32_MAX (length <= kRecRows), or y and z the address of its rows. A
+// bit-packed pivot's record holds kRecLong alone.
+constexpr int32_t kRecRows = 4;
+constexpr int32_t kRecLong = INT32_MAX;
+
+__device__ __forceinline__ int32_t dead_slot(int32_t j) { return -2 - j; }
+__device__ __forceinline__ int32_t slot_id(int32_t a) { return a >= 0 ? a : -2 - a; }
+
+__device__ __forceinline__ int4 rec_of(const int32_t* rows, int32_t len) {
+  int4 r = make_int4(len, INT32_MAX, INT32_MAX, INT32_MAX);
+  if (len < 0) {
+    r.x = kRecLong;
+  } else if (len <= kRecRows) {
+    if (len > 1) r.y = rows[0];
+    if (len > 2) r.z = rows[1];
+    if (len > 3) r.w = rows[2];
+  } else {
+    r.y = (int32_t)(unsigned)((unsigned long long)rows & 0xffffffffu);
+    r.z = (int32_t)(unsigned)((unsigned long long)rows >> 32);
+  }
+  return r;
+}
+__device__ __forceinline__ const int32_t* rec_rows(const int4& r) {
+  return reinterpret_cast<const int32_t*>((unsigned long long)(unsigned)r.y |
+                                          ((unsigned long long)(unsigned)r.z << 32));
+}
+
+// ------------------------------------------------------------------------------------------
 // Phase I scan
 // ------------------------------------------------------------------------------------------
 // exclusive block scan with carry-in; returns the exclusive prefix, sets the running total
@@ -433,12 +585,67 @@ __device__ __forceinline__ SegMax block_scan_segmax(SegMax v, SegMax carry, SegM
 }
 
 
+constexpr unsigned long long kLookAgg = 1ull << 38, kLookIncl = 2ull << 38;
+constexpr unsigned long long kLookFlags = 3ull << 38, kLookVal = (1ull << 38) - 1;
+
+// Decoupled look-back over the tiles before `chunk`: the number of places kept by all earlier
+// tiles. A tile publishes its own count (an aggregate state), then its inclusive prefix. Each
+// state word holds its value, so no fence is needed; states carry the pass number and never
+// need resetting within one reduction. Tiles are claimed in order from the work queue, so every
+// predecessor belongs to a running or finished block. A wait that runs past its bound records a
+// fault (reported as an error) and counts as zero.
+__device__ __forceinline__ unsigned long long look_tag(int32_t pass) {
+  return (unsigned long long)(pass & 0xffffff) << 40;
+}
+
+__device__ __forceinline__ void look_publish(const RArgs& a, int32_t pass, int64_t chunk,
+                                             int64_t agg) {
+  atomicExch(a.look + chunk,
+             look_tag(pass) | (chunk == 0 ? kLookIncl : kLookAgg) | (unsigned long long)agg);
+}
+
+// by one full warp; returns the exclusive prefix of `chunk` and publishes its inclusive one
+__device__ __forceinline__ int64_t look_back(const RArgs& a, int32_t pass, int64_t chunk,
+                                             int64_t agg) {
+  if (chunk == 0) return 0;
+  const int lane = lane_id();
+  const unsigned long long tag = look_tag(pass);
+  const unsigned long long* st = a.look;
+  int64_t prefix = 0;
+  bool fault = false;
+  for (int64_t p = chunk - 1;; p -= 32) {
+    const int64_t q = p - lane;
+    unsigned long long w = tag | kLookIncl;  // before chunk 0: nothing
+    if (q >= 0) {
+      for (int it = 0;; it++) {
+        w = *(const volatile unsigned long long*)(st + q);
+        if ((w >> 40) == (tag >> 40) && (w & kLookFlags)) break;
+        if (it > kSpinLimit) {
+          fault = true;
+          w = tag | kLookIncl;
+          break;
+        }
+        __nanosleep(32);
+      }
+    }
+    const bool incl = (w & kLookFlags) == kLookIncl;
+    const unsigned im = __ballot_sync(0xffffffffu, incl);
+    const int stop = im ? __ffs(im) - 1 : 32;  // nearest inclusive state
+    const int64_t val = lane <= stop ? (int64_t)(w & kLookVal) : 0;
+    prefix += __shfl_sync(0xffffffffu, warp_incl_sum(val), 31);
+    if (im || p < 32) break;
+  }
+  if (lane == 0) atomicExch(a.look + chunk, tag | kLookIncl | (unsigned long long)(prefix + agg));
+  if (__any_sync(0xffffffffu, fault) && lane == 0) a.ds->fault = 1;
+  return prefix;
+}
+
 // the space this pass's Phase II can need (arena, pivot store) against what the host provided;
 // no column has changed yet, and the marks made depend only on the pass's starting state, so a
 // pass stopped here continues at Phase II once the host has grown the buffers
 __device__ __forceinline__ void check_capacity(DevState* ds) {
   int reason = 0;
-  if (ds->bound_words > (unsigned long long)ds->arena_cap[ds->pass & 1]) reason |= 1;
+  if (ds->arena_used + ds->bound_words > (unsigned long long)ds->arena_cap[ds->arena_cur]) reason |= 1;
   if (ds->bound_piv + ds->piv_used > (unsigned long long)ds->piv_cap) reason |= 2;
   if (reason) {
     ds->host_reason = reason;
@@ -526,29 +733,32 @@ __device__ __forceinline__ SegMax tile_look_back(const RArgs& a, int32_t pass, i
   return acc;
 }
 
-__global__ void __launch_bounds__(kThreads, 4) k_phase1(RArgs a) {
+// A pass that compacts also gives every slot whose column may survive its place in the next active
+// list (newpos), by a second look-back over the tiles: a column that left all the same (proven
+// by its P_j, or cleared) leaves a dead place there.
+template <bool kLookAhead>
+__device__ __forceinline__ void phase1_pass(const RArgs& a, unsigned parts) {
   __shared__ SegMax sh[kWarps + 1];
   __shared__ int64_t shs[kWarps + 1];
   __shared__ int64_t s_tile;
   __shared__ SegMax s_pre;
+  __shared__ int s_keep[kWarps + 1];
+  __shared__ int64_t s_place;
   constexpr int kFI = kFItems;
-  pdl_wait();
-  pdl_trigger();
+  if (blockIdx.x >= parts) return;
   DevState* ds = a.ds;
-  if (ds->status != ST_RUN) return;
   const PV v = pass_view(ds);
   const int32_t pass = ds->pass;
-  const int32_t* fu = a.first_unp + (int64_t)(pass & 1) * a.nseg;  // this pass's copy
+  const int32_t* fu = a.first_unp;
+  const int32_t* lows = a.lows + (int64_t)(pass & a.ring) * a.lows_stride;
+  constexpr int32_t ahead = kLookAhead ? kAheadMax : 1;
+  const int32_t visit_rows = ahead > 1 ? kDeltaRows : 0;  // rows a visit may add to a column
   const int64_t ntiles = (v.n_act + kFTile - 1) / kFTile;
-  // no more blocks take part than there are tiles (the others leave at once: a short pass's
-  // grid is mostly idle); block 0 always does (the last block checks capacity)
-  const unsigned parts = (unsigned)std::max<int64_t>(1, std::min<int64_t>(gridDim.x, ntiles));
-  if (blockIdx.x >= parts) return;
   int64_t bw = 0, bp = 0;
   int64_t n_zero = 0, n_piv = 0, n_c10 = 0, n_pred = 0, n_empty = 0;
   bool want = false;  // a target whose addition may reach its dimension's bit-packing threshold
   bool fault = false;
-  for (;;) {
+  for (;;) {  // (a tile is claimed only when its work begins: later tiles wait for its state)
     if (threadIdx.x == 0) s_tile = atomicAdd(&ds->tile_queue, 1u);
     __syncthreads();
     const int64_t t = s_tile;
@@ -558,27 +768,39 @@ __global__ void __launch_bounds__(kThreads, 4) k_phase1(RArgs a) {
     // the top dimension (ids from t_b on), the smallest of the others below it
     int32_t t_b = 0, t_hi = INT32_MAX, t_lo = INT32_MAX;
     if (a.dense_floor != INT32_MAX) {
-      const int32_t j0 = v.act[tile0];
-      const int32_t j1 = v.act[min(tile0 + kFTile, v.n_act) - 1];
+      const int32_t j0 = slot_id(v.act[tile0]);
+      const int32_t j1 = slot_id(v.act[min(tile0 + kFTile, v.n_act) - 1]);
       t_b = dim_start_of(a, j1);
       t_hi = dense_min_of(a, j1);
       t_lo = dense_min_between(a, j0, t_b - 1);
     }
     const int64_t e0 = tile0 + (int64_t)threadIdx.x * kFI;
+    // a column ahead of this pass (its additions run up to a later one) collides with a pivot
+    // here; of it only the stored low matters
+    constexpr int32_t kAhead = -2;  // in place of its source
     int32_t j[kFI], l[kFI], sg[kFI], n[kFI], b[kFI], s[kFI];
 #pragma unroll
-    for (int i = 0; i < kFI; i++) j[i] = e0 + i < v.n_act ? v.act[e0 + i] : -1;
+    for (int i = 0; i < kFI; i++) {
+      j[i] = e0 + i < v.n_act ? v.act[e0 + i] : INT32_MIN;
+      s[i] = l[i] = -1;
+      if (ahead > 1 && e0 + i < v.n_act) {
+        if (a.due[e0 + i] > pass) s[i] = kAhead;
+        l[i] = lows[e0 + i];
+      }
+    }
 #pragma unroll
     for (int i = 0; i < kFI; i++) {
-      l[i] = j[i] >= 0 ? a.low[j[i]] : -1;
-      sg[i] = j[i] >= 0 ? seg_of(a, j[i]) : INT32_MAX;
-      n[i] = j[i] >= 0 ? v.alen[e0 + i] : 0;
+      // (a slot whose column left keeps its segment, so the scan's runs stay whole)
+      sg[i] = j[i] != INT32_MIN ? seg_of(a, slot_id(j[i])) : INT32_MAX;
+      if (j[i] < 0) j[i] = l[i] = -1;
+      else if (ahead == 1) l[i] = a.low[j[i]];
+      n[i] = j[i] >= 0 && s[i] != kAhead ? v.alen[e0 + i] : 0;
       b[i] = j[i] >= 0 ? a.beta[j[i]] : -1;
     }
 #pragma unroll
     for (int i = 0; i < kFI; i++) {
       if (!PH_DCHECK(&ds->debug_fault, l[i] < a.rows_end, 2)) l[i] = -1, j[i] = -1;
-      s[i] = l[i] >= 0 ? v.tab[l[i]] : -1;
+      if (s[i] != kAhead) s[i] = l[i] >= 0 ? (int32_t)(unsigned)a.tab[l[i]] : -1;
     }
     // Phase I values (the low of a colliding column, in its (cloud, dim) segment) and the space
     // bounds: a column's reservation is its stored words (its rows, or its bitmap with the
@@ -588,11 +810,11 @@ __global__ void __launch_bounds__(kThreads, 4) k_phase1(RArgs a) {
     for (int i = 0; i < kFI; i++) {
       const bool collide = l[i] >= 0 && s[i] != j[i];
       bw += stored_words(n[i]);
-      if (collide) {
+      if (collide && s[i] != kAhead) {
         const int32_t ns = stored_words(a.meta[s[i]].len);
-        bw += ns;
+        bw += max(ns, visit_rows);
         want |= n[i] + ns > (j[i] >= t_b ? t_hi : t_lo);
-      } else if (l[i] >= 0) {
+      } else if (l[i] >= 0 && !collide) {
         bp += stored_words(n[i]);
       }
       x[i] = SegMax{sg[i], collide ? l[i] : -1};
@@ -612,18 +834,40 @@ __global__ void __launch_bounds__(kThreads, 4) k_phase1(RArgs a) {
     // pass that marks them; the new-pivot mark goes with them), so marks are stored without a
     // load. Only a left-most column whose low is not its beta needs P_j: the others are marked
     // while warp 0 looks back, the rest after the tile's prefix is known.
+    auto dirty = [&](int32_t seg) {
+      if (atomicExch(&a.dirty_on[seg], 1) == 0) a.dirty[atomicAdd(&ds->n_dirty, 1u)] = seg;
+    };
     auto pivot = [&](int i) {
+      if (ahead > 1) {
+        const ColMeta mj = load_meta(a.meta + j[i]);
+        a.prec[l[i]] = rec_of(mj.ptr, mj.len);
+      }
       a.meta[j[i]].flags = F_PROVEN | F_NEWPIV;
       a.owner[l[i]] = j[i];
-      atomicMin(&v.tab_next[l[i]], j[i]);  // its row's pivot from the next pass on
+      a.tab[l[i]] = (unsigned)j[i];  // its row's left-most column from now on (as it is now)
+      // a paired row: its segment's first unpaired one?
+      if (l[i] == fu[sg[i] - a.nc]) dirty(sg[i] - a.nc);
+      if (j[i] == fu[sg[i]]) dirty(sg[i]);
       a.meta[l[i]].cleared = 1;  // clearing (Lemma 1): column l is positive and paired with j
       n_piv++;
     };
-    auto unproven = [&](int i) {
+    // a zeroed column: one ahead of the pass leaves its slot at once (it is nobody's source); one
+    // that is up to date in the additions kernel, where others may be reading it
+    auto zero = [&](int i) {
+      a.meta[j[i]].flags = F_FINAL;
+      if (s[i] == kAhead) {
+        a.meta[j[i]].len = 0;
+        a.low[j[i]] = -1;
+        v.act[e0 + i] = dead_slot(j[i]);
+      }
+    };
+    auto unproven = [&](int i) {  // true: zeroed
       if (a.cor10 && b[i] < 0 && l[i] < fu[sg[i] - a.nc]) {
-        a.meta[j[i]].flags = F_FINAL;  // Corollary 10, zero case
+        zero(i);  // Corollary 10, zero case
         n_c10++;
-      } else if (a.predict && b[i] >= 0 && a.pred[j[i]] < 0) {
+        return true;
+      }
+      if (a.predict && b[i] >= 0 && a.pred[j[i]] < 0) {
         const int32_t pi = predicted_low(a, b[i], l[i]);
         if (pi >= 0) {
           a.pred[j[i]] = pi;
@@ -632,25 +876,51 @@ __global__ void __launch_bounds__(kThreads, 4) k_phase1(RArgs a) {
           n_empty++;
         }
       }
+      return false;
     };
     unsigned waits = 0;  // items whose mark needs P_j
+    unsigned keeps = 0;  // items whose column may stay active
 #pragma unroll
     for (int i = 0; i < kFI; i++) {
-      if (j[i] < 0) continue;
-      a.src_e[e0 + i] = s[i] != j[i] ? s[i] : -1;  // Phase II reads it in list order
+      if (j[i] < 0) {
+        if (e0 + i < v.n_act) a.src_e[e0 + i] = -1;
+        continue;
+      }
+      if (s[i] != kAhead)
+        a.src_e[e0 + i] = s[i] != j[i] ? s[i] : -1;  // Phase II reads it in list order
       (void)PH_DCHECK(&ds->debug_fault, a.meta[j[i]].flags == 0, 7);
       if (l[i] < 0) {
-        a.meta[j[i]].flags = F_FINAL;
+        zero(i);
         n_zero++;
       } else if (s[i] != j[i]) {
-        unproven(i);
+        if (!unproven(i)) keeps |= 1u << i;
       } else if (l[i] == b[i]) {
         pivot(i);
       } else {
         waits |= 1u << i;
+        keeps |= 1u << i;
+      }
+    }
+    int place = 0;  // of this thread's first kept item among the tile's
+    if (v.compact && ahead > 1) {
+      int kept;
+      place = block_excl_sum<int>(__popc(keeps), s_keep, kept);
+      if (threadIdx.x < 32) {
+        if (threadIdx.x == 0) look_publish(a, pass, t, kept);
+        const int64_t before = look_back(a, pass, t, kept);
+        if (threadIdx.x == 0) s_place = before;
       }
     }
     __syncthreads();
+    if (v.compact && ahead > 1) {
+#pragma unroll
+      for (int i = 0; i < kFI; i++) {
+        if (j[i] < 0) continue;
+        const bool kept = (keeps >> i) & 1u;
+        a.newpos[e0 + i] =
+            kept ? (int32_t)(s_place + place + __popc(keeps & ((1u << i) - 1u))) : -1;
+      }
+    }
     if (waits) {
       SegMax run = threadIdx.x == 0 ? s_pre : segmax_combine(s_pre, pre_t);
 #pragma unroll
@@ -679,6 +949,24 @@ __global__ void __launch_bounds__(kThreads, 4) k_phase1(RArgs a) {
     atomicAdd(&ds->bound_words, (unsigned long long)tw);
     atomicAdd(&ds->bound_piv, (unsigned long long)tp);
   }
+}
+
+// no more blocks take part in Phase I than there are tiles (the others leave at once: a short
+// pass's grid is mostly idle); block 0 always does
+__device__ __forceinline__ unsigned phase1_parts(const DevState* ds, unsigned blocks) {
+  const int64_t ntiles = (ds->n_act + kFTile - 1) / kFTile;
+  return (unsigned)std::max<int64_t>(1, std::min<int64_t>(blocks, ntiles));
+}
+
+template <bool kLookAhead>
+__global__ void __launch_bounds__(kThreads, 4) k_phase1(RArgs a) {
+  pdl_wait();
+  pdl_trigger();
+  DevState* ds = a.ds;
+  if (ds->status != ST_RUN) return;
+  const unsigned parts = phase1_parts(ds, gridDim.x);
+  if (blockIdx.x >= parts) return;
+  phase1_pass<kLookAhead>(a, parts);
   // the last of the taking-part blocks checks the space this pass's Phase II needs
   if (last_block(&ds->blocks_done, parts)) {
     if (threadIdx.x == 0) {
@@ -769,15 +1057,15 @@ __global__ void k_set_apply(RArgs a) {
 // T's header and returns its row count; its largest row goes to low, its stored words to words.
 __device__ __noinline__ int32_t dense_job_warp(const RArgs& a, int32_t j, const int32_t* A,
                                               int na, bool dense_a, const int32_t* B, int nb,
-                                              bool dense_b, int32_t* T, int32_t& low,
-                                              int32_t& words) {
+                                              bool dense_b, int32_t* T, int64_t room,
+                                              int32_t& low, int32_t& words) {
   const int lane = lane_id();
   int64_t base;
   int32_t W;
   row_segment(a, j, base, W);
 #ifdef PH_DEBUG
-  // the bitmap fits the slot reserved for the job (na + nb stored words)
-  if (!PH_DCHECK(&a.ds->debug_fault, W + kDenseHead <= na + nb, 6)) {
+  // the bitmap fits the slot reserved for the job (room words)
+  if (!PH_DCHECK(&a.ds->debug_fault, W + kDenseHead <= room, 6)) {
     low = -1;
     words = 0;
     return 0;
@@ -847,6 +1135,7 @@ __device__ __forceinline__ Job job_of(const RArgs& a, const PV& v, int64_t e) {
   // every load is issued up front: the column and its source candidate are known from the
   // active list and k_phase1's per-slot source, so no load waits on another's result
   const int32_t j = v.act[e];
+  if (j < 0) return jb;  // (a place that look-ahead left empty)
   const int32_t se = a.src_e[e];  // -1: no collision; <= -2: a target whose set waits
   const int32_t s = se >= 0 ? se : -1;
   const ColMeta mj = load_meta(a.meta + j);  // one 16-byte load per column
@@ -889,12 +1178,250 @@ __device__ __forceinline__ Job job_of(const RArgs& a, const PV& v, int64_t e) {
 }
 
 // ------------------------------------------------------------------------------------------
+// look_ahead: the additions of several passes on one column, by one lane
+// ------------------------------------------------------------------------------------------
+// The rows added to a column that are not in its list yet, one per place in any order (every index
+// is static): what earlier visits left in the first kOld places, and the rows of this visit's
+// sources, R places per pass. A place holds a row negated, or kEmpty. Rows above the column's low
+// are spent, and a row may be there several times: the low only falls, so the next low is the
+// largest row below it that is there an odd number of times, and nothing has to be taken out on
+// the way.
+constexpr int32_t kEmpty = -INT32_MAX;
+struct Delta {
+  int32_t c[kDeltaRows];
+};
+
+// odd ^= how many of x[I..] equal l, one instruction per value (the predicate chain stays inside)
+__device__ __forceinline__ bool odd_of4(bool odd, int32_t l, int32_t x0, int32_t x1, int32_t x2,
+                                        int32_t x3) {
+  int32_t r;
+  asm("{\n.reg .pred p;\n"
+      "setp.ne.s32 p, %1, 0;\n"
+      "setp.eq.xor.s32 p, %3, %2, p;\n"
+      "setp.eq.xor.s32 p, %4, %2, p;\n"
+      "setp.eq.xor.s32 p, %5, %2, p;\n"
+      "setp.eq.xor.s32 p, %6, %2, p;\n"
+      "selp.s32 %0, 1, 0, p;\n}"
+      : "=r"(r)
+      : "r"((int32_t)odd), "r"(l), "r"(x0), "r"(x1), "r"(x2), "r"(x3));
+  return r != 0;
+}
+
+// the next low of a column of which low l was added to: the first kOld places if `old`, N places
+// after them, and the column's own rows A[0 .. na), whose end is shortened (top is its last
+// row, or -1)
+template <int N>
+__device__ __forceinline__ int32_t next_low(const Delta& d, bool old, const int32_t* A, int& na,
+                                            int32_t& top, int32_t l) {
+  for (;;) {
+    if (top == l) {
+      na--;
+      top = na > 0 ? A[na - 1] : -1;
+    }
+    // the largest row below l, as the smallest unsigned distance from l - 1 (one add-min per
+    // place): spent rows and empty places wrap around, and -1 (top at the least) is the farthest
+    const int32_t lim = l - 1;
+    unsigned best = (unsigned)(lim - top);
+    if (old) {
+#pragma unroll
+      for (int i = 0; i < kOld; i++) best = __viaddmin_u32((unsigned)d.c[i], (unsigned)lim, best);
+    }
+#pragma unroll
+    for (int i = kOld; i < kOld + N; i++)
+      best = __viaddmin_u32((unsigned)d.c[i], (unsigned)lim, best);
+    l = lim - (int32_t)best;
+    if (l < 0) return -1;
+    bool odd = top == l;
+    if (old) {
+#pragma unroll
+      for (int i = 0; i < kOld; i += 4)
+        odd = odd_of4(odd, -l, d.c[i], d.c[i + 1], d.c[i + 2], d.c[i + 3]);
+    }
+#pragma unroll
+    for (int i = kOld; i < kOld + N; i += 4)
+      odd = odd_of4(odd, -l, d.c[i], i + 1 < kOld + N ? d.c[i + 1] : kEmpty,
+                    i + 2 < kOld + N ? d.c[i + 2] : kEmpty, i + 3 < kOld + N ? d.c[i + 3] : kEmpty);
+    if (odd) return l;
+  }
+}
+
+// Batcher's odd-even merge sort of N values (any N) as a list of exchanges known at compile time
+template <int N>
+struct SortNet {
+  int n = 0;
+  int lo[N * N] = {}, hi[N * N] = {};
+  constexpr SortNet() {
+    for (int p = 1; p < N; p *= 2)
+      for (int k = p; k >= 1; k /= 2)
+        for (int j = k % p; j + k < N; j += 2 * k)
+          for (int i = 0; i < k && i + j + k < N; i++)
+            if ((i + j) / (2 * p) == (i + j + k) / (2 * p)) {
+              lo[n] = i + j;
+              hi[n] = i + j + k;
+              n++;
+            }
+  }
+};
+template <int N>
+constexpr SortNet<N> kSortNet{};
+template <int N, size_t... I>
+__device__ __forceinline__ void sort_asc(int32_t (&c)[N], std::index_sequence<I...>) {
+  const auto exchange = [&](int32_t& x, int32_t& y) {
+    const int32_t m = min(x, y);
+    y = max(x, y);
+    x = m;
+  };
+  (exchange(c[std::integral_constant<int, kSortNet<N>.lo[I]>::value],
+            c[std::integral_constant<int, kSortNet<N>.hi[I]>::value]),
+   ...);
+}
+// sorts the values, smallest first
+template <int N>
+__device__ __forceinline__ void sort_asc(int32_t (&c)[N]) {
+  sort_asc(c, std::make_index_sequence<(size_t)kSortNet<N>.n>{});
+}
+
+
+// one column's visit, before and after
+struct Visit {
+  Delta d;             // (after tidy: the rows left, ascending, then INT32_MAX)
+  int k;               // rows in d
+  const int32_t* A;    // its list
+  int na;
+  const int32_t* B;    // its first source's rows (nb of them) if that has no short record
+  int nb;
+  int4 rec;            // that source's record
+  int32_t low;
+  int32_t due;         // the pass whose additions visit the column next
+  bool gone;           // done for: zeroed in pass due - 1 at the latest, its rows needed no more
+  bool settle;         // its list has to be whole for the next visit
+};
+
+// Runs the additions of passes pass .. v.limit - 1 on the column of each lane that is on (low
+// w.low) as far as their sources are known: the first source is given, a later one must be a
+// proven pivot (its record in prec, complete after k_phase1's marks). A source of at most R rows
+// beside its low takes this pass's places; one longer source per visit fills places from the
+// far end, which leaves fewer passes. pos: the slot whose stored lows the run writes. A run ends
+// early before another low, and when the column is done for: its low is -1 (k_phase1 of that
+// pass makes it final), or lies below fu, the first unpaired row (Corollary 10 zeroes it in that
+// pass: the row has a pivot, so the column collides, and fu never falls); that pass itself takes it
+// off the list. Returns whether any lane used the places of earlier visits.
+__device__ __forceinline__ bool look_ahead(const RArgs& a, const PV& v, int32_t pass, bool on,
+                                           int32_t fu, int64_t pos, Visit& w) {
+  constexpr int R = kSourceRows, N = R * kAheadMax;
+  const int32_t* A = w.A;
+  const int32_t* S = w.B;  // the rows of a longer source
+  int32_t l = w.low;
+  int na = on ? w.na : 0;
+  int32_t top = na > 0 ? A[na - 1] : -1;
+  int4 q = w.rec;
+  const bool visited = on;
+  const bool old = __any_sync(0xffffffffu, on && w.k > 0);
+  int n_low = 0;
+  int most = kAheadMax;  // passes the places suffice for
+  bool longer = on && (q.x == 0 || q.x > R + 1);  // this pass's source is a longer one
+  bool any_longer = false, in_rec = false;
+  int n = longer ? w.nb - 1 : 0;
+  auto next = [&](int t) {  // pass + t + 1 starts with low l; is its source known?
+    a.lows[(int64_t)((pass + t + 1) & a.ring) * a.lows_stride + pos] = l;
+    n_low = t + 1;
+    w.gone = l < 0;
+    on = false;
+    if (l >= 0 && PH_DCHECK(&a.ds->debug_fault, l < a.rows_end && na >= 0, 8)) {
+      q = a.prec[l];
+      w.gone = q.x > 0 && l < fu;
+      w.settle = q.x == 0 || q.x > N + 1;
+      on = q.x > 0 && !w.gone && t + 1 < most && pass + t + 1 < v.limit;
+      longer = on && q.x > R + 1;
+      if (longer) {  // one per visit, of as many rows as leave this pass its place
+        n = q.x - 1;
+        on = longer = most == kAheadMax && q.x <= kRecRows + kLonger && n <= N - R * (t + 1);
+        in_rec = q.x <= kRecRows;
+        S = in_rec ? nullptr : rec_rows(q);
+      }
+    }
+  };
+  // (one copy of the code for all passes: unrolled, it would not stay in the instruction caches)
+#pragma unroll 1
+  for (int t = 0; t < kAheadMax && __any_sync(0xffffffffu, on); t++) {
+    const bool put = on && !longer;
+    const int32_t y = -q.y, z = -q.z;
+#pragma unroll
+    for (int i = 0; i < kAheadMax; i++) {
+      if (t == i && put) {
+        w.d.c[kOld + R * i] = y;
+        w.d.c[kOld + R * i + 1] = z;
+      }
+    }
+    if (__any_sync(0xffffffffu, longer)) {
+      any_longer = true;
+#pragma unroll
+      for (int i = 0; i < N; i++) {
+        if (i >= 4 && i % 4 == 0 && !__any_sync(0xffffffffu, longer && i < n)) break;
+        if (longer && i < n)
+          w.d.c[kOld + N - 1 - i] = -(i < 3 && in_rec ? (i == 0 ? q.y : i == 1 ? q.z : q.w) : S[i]);
+      }
+      if (longer) {
+        most = max((N - n) / R, t + 1);
+        longer = false;
+      }
+    }
+    if (on) {
+      if (!any_longer && t < kAheadMax / 2) l = next_low<N / 2>(w.d, old, A, na, top, l);
+      else l = next_low<N>(w.d, old, A, na, top, l);
+      next(t);
+    }
+  }
+  if (visited) {
+    w.low = l;
+    w.due = pass + n_low + (w.gone ? 1 : 0);
+    w.na = w.gone ? 0 : na;
+  }
+  return old;
+}
+
+// the rows of a visited column's delta that are left, in order from place FROM on (the places
+// before it are empty); a row that is there twice cancels
+template <int FROM>
+__device__ __forceinline__ void tidy(Visit& w, bool on) {
+  constexpr int N = kDeltaRows - FROM;
+  int32_t c[N];
+#pragma unroll
+  for (int i = 0; i < N; i++) {
+    const int32_t x = -w.d.c[FROM + i];
+    c[i] = on && x <= w.low ? x : INT32_MAX;
+  }
+#pragma unroll 1
+  for (int round = 0; round < 2; round++) {
+    sort_asc(c);
+    if (round == 1) break;
+    bool twice = false;
+#pragma unroll
+    for (int i = 0; i + 1 < N; i++) {
+      if (c[i] != INT32_MAX && c[i] == c[i + 1]) {
+        c[i] = c[i + 1] = INT32_MAX;
+        twice = true;
+      }
+    }
+    if (!__any_sync(0xffffffffu, twice)) break;
+  }
+  w.k = 0;
+#pragma unroll
+  for (int i = 0; i < N; i++) {
+    w.k += c[i] != INT32_MAX ? 1 : 0;
+    w.d.c[i] = c[i];
+  }
+#pragma unroll
+  for (int i = N; i < kDeltaRows; i++) w.d.c[i] = INT32_MAX;
+}
+
+// ------------------------------------------------------------------------------------------
 // column arithmetic over F2: symmetric difference of two ascending row lists
 // ------------------------------------------------------------------------------------------
 // merge-path split on diagonal d with ties taken from A first; an equal pair A[x-1] == B[y]
 // is kept on the same side of the split so that cancellations never straddle two lanes
-__device__ __forceinline__ void merge_split(const int32_t* __restrict__ A, int na,
-                                            const int32_t* __restrict__ B, int nb, int d, int& x,
+__device__ __forceinline__ void merge_split(const int32_t* A, int na,
+                                            const int32_t* B, int nb, int d, int& x,
                                             int& y) {
   int lo = d > nb ? d - nb : 0, hi = d < na ? d : na;
   while (lo < hi) {
@@ -908,9 +1435,8 @@ __device__ __forceinline__ void merge_split(const int32_t* __restrict__ A, int n
 
 // warp-cooperative symmetric difference straight from global memory (used for merges too long
 // to stage in shared memory); every lane returns the output length and the last row written
-__device__ __forceinline__ int warp_symdiff(const int32_t* __restrict__ A, int na,
-                                            const int32_t* __restrict__ B, int nb,
-                                            int32_t* __restrict__ dst, int32_t& last) {
+__device__ __forceinline__ int warp_symdiff(const int32_t* A, int na, const int32_t* B, int nb,
+                                            int32_t* dst, int32_t& last) {
   constexpr int K = 4;
   const int lane = lane_id();
   const int N = na + nb;
@@ -971,6 +1497,7 @@ __device__ __forceinline__ int warp_symdiff(const int32_t* __restrict__ A, int n
 // sentinel (at most KM + 1 words, KM <= 16).
 constexpr int kStage = 1024;
 constexpr int kStageSlack = 32;
+constexpr int kScan = 64;  // slots a warp looks through at a time for due ones
 struct __align__(16) WarpStage {
   int32_t in[kStage + kStageSlack];
   int32_t* jout[32];  // output slot of the job (its reserved words in the next arena)
@@ -982,7 +1509,6 @@ struct __align__(16) WarpStage {
   int32_t jcnt[32];   // output rows of the job so far
   int32_t jlow[32];   // largest output row (new low), -1 if none
 };
-// Phase II blocks: 128 threads, so a block's barriers wait on 4 warps rather than 8
 constexpr int kAddThreads = 128;
 constexpr int kAddWarps = kAddThreads / 32;
 constexpr size_t kAddSmem = sizeof(WarpStage) * kAddWarps;
@@ -1035,14 +1561,13 @@ __device__ __forceinline__ int lane_symdiff(const int32_t* __restrict__ sA, int 
 // equal rows -- one from each column -- end up adjacent and cancel. Returns the output length
 // and the last (largest) row written, -1 if none.
 template <int S>
-__device__ __forceinline__ int reg_symdiff(const int32_t* __restrict__ A, int na,
-                                           const int32_t* __restrict__ B, int nb,
-                                           int32_t* __restrict__ dst, int32_t& last) {
+__device__ __forceinline__ int reg_symdiff(const int32_t* A, int na, const int32_t* B, int nb,
+                                           int32_t* dst, int32_t& last) {
   int32_t c[2 * S];
 #pragma unroll
-  for (int i = 0; i < S; i++) c[i] = i < na ? __ldg(A + i) : INT32_MAX;
+  for (int i = 0; i < S; i++) c[i] = i < na ? A[i] : INT32_MAX;
 #pragma unroll
-  for (int i = 0; i < S; i++) c[2 * S - 1 - i] = i < nb ? __ldg(B + i) : INT32_MAX;
+  for (int i = 0; i < S; i++) c[2 * S - 1 - i] = i < nb ? B[i] : INT32_MAX;
 #pragma unroll
   for (int st = S; st >= 1; st >>= 1) {
 #pragma unroll
@@ -1066,62 +1591,6 @@ __device__ __forceinline__ int reg_symdiff(const int32_t* __restrict__ A, int na
     }
   }
   return k;
-}
-
-constexpr unsigned long long kLookAgg = 1ull << 38, kLookIncl = 2ull << 38;
-constexpr unsigned long long kLookFlags = 3ull << 38, kLookVal = (1ull << 38) - 1;
-
-// Decoupled look-back over the chunks before `chunk`: the number of survivors in all earlier
-// chunks. A chunk publishes its own count (an aggregate state) as soon as its block scan is
-// done and looks back only after its merges, when its predecessors have mostly finished and
-// published inclusive prefixes. Each state word holds its value, so no fence is needed; states
-// carry the pass number and never need resetting within one reduction. Chunks are claimed in
-// order from the work queue, so every predecessor belongs to a running or finished block. A
-// wait that runs past its bound records a fault (reported as an error) and counts as zero.
-__device__ __forceinline__ unsigned long long look_tag(int32_t pass) {
-  return (unsigned long long)(pass & 0xffffff) << 40;
-}
-
-__device__ __forceinline__ void look_publish(const RArgs& a, int32_t pass, int64_t chunk,
-                                             int64_t agg) {
-  atomicExch(a.look + chunk,
-             look_tag(pass) | (chunk == 0 ? kLookIncl : kLookAgg) | (unsigned long long)agg);
-}
-
-// by one full warp; returns the exclusive prefix of `chunk` and publishes its inclusive one
-__device__ __forceinline__ int64_t look_back(const RArgs& a, int32_t pass, int64_t chunk,
-                                             int64_t agg) {
-  if (chunk == 0) return 0;
-  const int lane = lane_id();
-  const unsigned long long tag = look_tag(pass);
-  const unsigned long long* st = a.look;
-  int64_t prefix = 0;
-  bool fault = false;
-  for (int64_t p = chunk - 1;; p -= 32) {
-    const int64_t q = p - lane;
-    unsigned long long w = tag | kLookIncl;  // before chunk 0: nothing
-    if (q >= 0) {
-      for (int it = 0;; it++) {
-        w = *(const volatile unsigned long long*)(st + q);
-        if ((w >> 40) == (tag >> 40) && (w & kLookFlags)) break;
-        if (it > kSpinLimit) {
-          fault = true;
-          w = tag | kLookIncl;
-          break;
-        }
-        __nanosleep(32);
-      }
-    }
-    const bool incl = (w & kLookFlags) == kLookIncl;
-    const unsigned im = __ballot_sync(0xffffffffu, incl);
-    const int stop = im ? __ffs(im) - 1 : 32;  // nearest inclusive state
-    const int64_t val = lane <= stop ? (int64_t)(w & kLookVal) : 0;
-    prefix += __shfl_sync(0xffffffffu, warp_incl_sum(val), 31);
-    if (im || p < 32) break;
-  }
-  if (lane == 0) atomicExch(a.look + chunk, tag | kLookIncl | (unsigned long long)(prefix + agg));
-  if (__any_sync(0xffffffffu, fault) && lane == 0) a.ds->fault = 1;
-  return prefix;
 }
 
 // waits for all of this thread's asynchronous copies (cp_async16)
@@ -1310,8 +1779,228 @@ __device__ __forceinline__ int lane_merge_job(const int32_t* __restrict__ in, in
 template <bool kNewLow>
 __device__ __forceinline__ void next_tab(const RArgs& a, const PV& v, int32_t l, int32_t j) {
   if (l < 0 || !PH_DCHECK(&a.ds->debug_fault, l < a.rows_end, 1)) return;
-  if (v.tab_next[l] > j) atomicMin(&v.tab_next[l], j);
+  const unsigned long long key = v.tab_key | (unsigned)j;
+  if (a.tab[l] > key) atomicMin(&a.tab[l], key);
   if (kNewLow && !a.meta[l].low_seen) a.meta[l].low_seen = 1;
+}
+
+enum : int {
+  kCntTargets, kCntActive, kCntCleared, kCntAdds, kCntXors, kCntCopied, kCntPacked, kNumCnt
+};
+
+__device__ __forceinline__ int64_t warp_sum64(int64_t v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// Merges by one warp: per lane the column A (rows, or a bit-packed column if dense_a) and the
+// source B (likewise, dense_b; null: the column moves) into the lane's slot of the arena (null: no
+// job), whose words suffice for all rows. Short columns are merged in registers (one thread per
+// job); longer ones are staged in shared memory and merged, each job by its own lane (short
+// jobs) or by a merge path over the batch's jobs cut into pieces of km positions (8 unless
+// ph_opts.merge_items says otherwise); merges longer than the staging bound run from global
+// memory; bit-packed jobs run one at a time by the whole warp. kSlots: lanes with jobs. Returns how
+// the lane's job was done (4: bit-packed); o_ptr, o_len, low: the result's place, length and low.
+template <bool kDense, int kSlots, bool kLane>
+__device__ __forceinline__ int merge_rows(const RArgs& a, const PV& v, WarpStage& S, int32_t j,
+                                          int32_t* slot, const int32_t* A, int na, bool dense_a,
+                                          const int32_t* B, int nb, bool dense_b, int32_t*& o_ptr,
+                                          int& o_len, int32_t& low) {
+  const int lane = lane_id();
+  const int N = slot != nullptr ? na + nb : 0;
+  o_ptr = slot;
+  o_len = 0;
+  low = -1;
+  // short merges: one thread per job, in registers
+  // (cls 1: register merge, 3: staged or from global memory). The register path pays off when
+  // most of the warp takes it; a few short jobs among long ones would keep the rest of the warp
+  // waiting, so they join the staged path instead. One network size serves the whole warp.
+  const int need = max(na, nb);
+  // cls 4: bit-packed (the column is, or the source is, or the sum exceeds the threshold)
+  const bool dense_job =
+      kDense && N > 0 && (dense_a || (B != nullptr && (dense_b || (v.dense_on && goes_dense(a, j, N)))));
+  // the register network for jobs of up to kRegMax rows per column; the piece kernels keep it
+  // small (8), their registers go to the merge pieces
+  constexpr int kRegMax = kLane ? 16 : 8;
+  int cls = N == 0 ? 0 : (dense_job ? 4 : (need <= kRegMax ? 1 : 3));
+  constexpr int kRegMinJobs = 12 * kSlots / 32;  // of the warp's slots
+  if (__popc(__ballot_sync(0xffffffffu, cls == 1)) < kRegMinJobs && cls == 1) cls = 3;
+  const unsigned wneed = __reduce_max_sync(0xffffffffu, cls == 1 ? (unsigned)need : 0u);
+  if (cls == 1) {
+    int32_t last;
+    int len;
+    if constexpr (kRegMax == 16) {
+      len = wneed <= 4   ? reg_symdiff<4>(A, na, B, nb, slot, last)
+            : wneed <= 8 ? reg_symdiff<8>(A, na, B, nb, slot, last)
+                         : reg_symdiff<16>(A, na, B, nb, slot, last);
+    } else {
+      len = wneed <= 4 ? reg_symdiff<4>(A, na, B, nb, slot, last)
+                       : reg_symdiff<8>(A, na, B, nb, slot, last);
+    }
+    o_ptr = slot;
+    o_len = len;
+    low = last;
+  }
+  const unsigned smask = __ballot_sync(0xffffffffu, cls == 3);
+  if (smask) {
+    // longer merges: staged in shared memory, merge path over the concatenated jobs. Each list
+    // takes a 16-byte aligned span (its misalignment, its rows, a sentinel, rounded up to 4 words)
+    const int ra = (int)(((uintptr_t)A >> 2) & 3u);
+    const int rb = B ? (int)(((uintptr_t)B >> 2) & 3u) : 0;
+    const int span_a = (ra + na + 1 + 3) & ~3;
+    const int span_b = (rb + nb + 1 + 3) & ~3;
+    const bool staged = cls == 3 && N <= a.staged_max && span_a + span_b <= kStage;
+    const bool big = cls == 3 && !staged;
+    const unsigned stmask = __ballot_sync(0xffffffffu, staged);
+    const int ord = __popc(stmask & ((1u << lane) - 1u));  // ordinal among the staged jobs
+    const int words = staged ? span_a + span_b : 0;
+    const int w_ex = warp_incl_sum(words) - words;
+    const int km = a.force_km > 0 ? a.force_km : 8;
+    const int npc = staged ? (N + km - 1) / km : 0;  // merge pieces of the job
+    const int p_first = warp_incl_sum(npc) - npc;
+    if (staged) {
+      S.jout[ord] = slot;
+      S.na[ord] = na;
+      S.nb[ord] = nb;
+      S.pc[ord] = p_first;
+      S.jcnt[ord] = 0;
+      S.jlow[ord] = -1;
+    }
+    __syncwarp();
+    unsigned rest = stmask;
+    while (rest) {
+      // batch: the staged jobs from lane c on whose spans fit together
+      const int c = __ffs(rest) - 1;
+      const int w0 = __shfl_sync(0xffffffffu, w_ex, c);
+      const bool mine = staged && lane >= c && w_ex + words - w0 <= kStage;
+      const unsigned bmask = __ballot_sync(0xffffffffu, mine);
+      rest &= ~bmask;
+      const int o0 = __popc(stmask & ((1u << c) - 1u));
+      const int base = w_ex - w0;  // this job's spans in `in`
+      if (mine) {
+        S.ia[ord] = base + ra;
+        S.ib[ord] = base + span_a + rb;
+      }
+      // stage: 16-byte chunks from the lists' aligned starts (the column stores carry slack
+      // after their last column for the rounding); jobs of 16+ chunks by the whole warp,
+      // shorter ones by their lane; all copies of the batch are in flight together
+      const int ch_a = span_a >> 2;
+      const int ch_n = ch_a + (B ? span_b >> 2 : 0);
+      const int32_t* ga = A - ra;
+      const int32_t* gb = B ? B - rb : nullptr;
+      unsigned lmask = __ballot_sync(0xffffffffu, mine && ch_n >= 16);
+      while (lmask) {
+        const int src = __ffs(lmask) - 1;
+        lmask &= lmask - 1;
+        const int32_t* wa = (const int32_t*)__shfl_sync(0xffffffffu, (unsigned long long)ga, src);
+        const int32_t* wb = (const int32_t*)__shfl_sync(0xffffffffu, (unsigned long long)gb, src);
+        const int wca = __shfl_sync(0xffffffffu, ch_a, src);
+        const int wcn = __shfl_sync(0xffffffffu, ch_n, src);
+        int32_t* d = S.in + __shfl_sync(0xffffffffu, base, src);
+        for (int q = lane; q < wcn; q += 32)
+          cp_async16(d + 4 * q, q < wca ? wa + 4 * q : wb + 4 * (q - wca));
+      }
+      if (mine && ch_n < 16) {
+        int32_t* d = S.in + base;
+        for (int q = 0; q < ch_n; q++) cp_async16(d + 4 * q, q < ch_a ? ga + 4 * q : gb + 4 * (q - ch_a));
+      }
+      cp_async_wait_all();
+      __syncwarp();
+      if (mine) {  // the sentinels go after the copies, which may have covered their words
+        S.in[base + ra + na] = INT32_MAX;
+        S.in[base + span_a + rb + nb] = INT32_MAX;
+      }
+      __syncwarp();
+      if constexpr (kLane) {  // each job by its own lane
+        if (mine) {
+          int32_t lastv;
+          const int len = lane_merge_job(S.in, base + ra, base + span_a + rb, N, slot, &lastv);
+          S.jcnt[ord] = len;
+          S.jlow[ord] = lastv;
+        }
+      } else {  // pieces of every job spread over the lanes
+        const int P0 = __shfl_sync(0xffffffffu, p_first, c);
+        const int P1 = P0 + (int)__reduce_add_sync(0xffffffffu, mine ? (unsigned)npc : 0u);
+        switch (km) {
+          case 8: staged_rounds<8>(S, P0, P1, o0, mine, p_first, km); break;
+          default: staged_rounds<0>(S, P0, P1, o0, mine, p_first, km); break;
+        }
+      }
+      __syncwarp();
+    }
+    if (staged) {
+      o_ptr = slot;
+      o_len = S.jcnt[ord];
+      low = S.jlow[ord];
+    }
+    // merges too long to stage: straight from global memory into their slot
+    unsigned bmask = __ballot_sync(0xffffffffu, big);
+    while (bmask) {
+      const int src = __ffs(bmask) - 1;
+      bmask &= bmask - 1;
+      const int32_t* wA = (const int32_t*)__shfl_sync(0xffffffffu, (unsigned long long)A, src);
+      const int32_t* wB = (const int32_t*)__shfl_sync(0xffffffffu, (unsigned long long)B, src);
+      const int wna = __shfl_sync(0xffffffffu, na, src);
+      const int wnb = __shfl_sync(0xffffffffu, nb, src);
+      int32_t* wd = (int32_t*)__shfl_sync(0xffffffffu, (unsigned long long)slot, src);
+      int len;
+      int32_t last = -1;
+      if (wB) {
+        len = warp_symdiff(wA, wna, wB, wnb, wd, last);
+      } else {
+        for (int q = lane; q < wna; q += 32) wd[q] = wA[q];
+        len = wna;
+      }
+      if (lane == src) {
+        low = last;
+        o_ptr = wd;
+        o_len = len;
+      }
+    }
+  }
+  // ---- bit-packed columns, one job at a time by the whole warp
+  unsigned dnmask = kDense ? __ballot_sync(0xffffffffu, cls == 4) : 0u;
+  while (dnmask) {
+    const int src = __ffs(dnmask) - 1;
+    dnmask &= dnmask - 1;
+    const int32_t* wA = (const int32_t*)__shfl_sync(0xffffffffu, (unsigned long long)A, src);
+    const int32_t* wB = (const int32_t*)__shfl_sync(0xffffffffu, (unsigned long long)B, src);
+    const int wna = __shfl_sync(0xffffffffu, na, src);
+    int32_t* wd = (int32_t*)__shfl_sync(0xffffffffu, (unsigned long long)slot, src);
+    const bool wdense_a = __shfl_sync(0xffffffffu, (int)dense_a, src) != 0;
+    if (wB == nullptr) {  // a bit-packed column with nothing to add moves as it is
+      for (int q = lane; q < wna; q += 32) wd[q] = wA[q];
+      if (lane == src) {
+        o_ptr = wd;
+        o_len = dense_len(wna);
+      }
+      continue;
+    }
+    int32_t dlow, words;
+    const int32_t rows = dense_job_warp(a, __shfl_sync(0xffffffffu, j, src), wA, wna, wdense_a,
+                                        wB, __shfl_sync(0xffffffffu, nb, src),
+                                        __shfl_sync(0xffffffffu, (int)dense_b, src) != 0, wd,
+                                        wna + __shfl_sync(0xffffffffu, nb, src), dlow, words);
+    if (lane == src) {
+      o_ptr = wd;
+      o_len = rows ? dense_len(words) : 0;  // a zero column stores nothing
+      low = dlow;
+    }
+  }
+  return cls;
+}
+
+// by thread 0, after the block's rounds: its counters into the pass's
+__device__ __forceinline__ void flush_counters(const RArgs& a, const PV& v,
+                                               const unsigned long long* s_cnt) {
+  if (s_cnt[kCntTargets]) atomicAdd(&a.ds->totals[1], s_cnt[kCntTargets]);
+  if (v.stats) {
+    const int idx[kNumCnt] = {PH_PS_TARGETS, PH_PS_ACTIVE, PH_PS_CLEARED,
+                              PH_PS_ADDS,    PH_PS_XORS,   PH_PS_COPIED, PH_PS_PACKED};
+    for (int i = 0; i < kNumCnt; i++)
+      if (s_cnt[i]) atomicAdd((unsigned long long*)&v.stats[idx[i]], s_cnt[i]);
+  }
 }
 
 // Phase II for one chunk of the active list (128 slots of a block, or 32 of a warp). Survivors
@@ -1324,16 +2013,6 @@ __device__ __forceinline__ void next_tab(const RArgs& a, const PV& v, int32_t l,
 // bound run from global memory; bit-packed jobs run one at a time by the whole warp. Targets
 // and zeroed columns are updated in place (no other job reads them this pass); new pivots and
 // left-most survivors, which other jobs may be reading as sources, are updated by k_commit.
-enum : int {
-  kCntTargets, kCntActive, kCntCleared, kCntAdds, kCntXors, kCntCopied, kCntPacked, kNumCnt
-};
-
-__device__ __forceinline__ int64_t warp_sum64(int64_t v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
 // kSlots > 0: the chunk is kSlots (32 or 8) slots of one warp, lanes kSlots.. without a job
 // (warp scan, no block barrier); kSlots = 0: kBT slots of the whole block of kBT threads
 template <bool kDense, int kSlots, bool kLane, int kBT>
@@ -1428,193 +2107,21 @@ __device__ __forceinline__ void add_chunk(const RArgs& a, const PV& v, int64_t c
   }
 
   // ---- survivors: every job writes into its own reserved slot of the next arena
-  int32_t* slot = jb.surv ? v.arena_next + off : nullptr;
-  const int N = jb.surv ? na + nb : 0;
-  // short merges: one thread per job, in registers
-  // (cls 1: register merge, 3: staged or from global memory). The register path pays off when
-  // most of the warp takes it; a few short jobs among long ones would keep the rest of the warp
-  // waiting, so they join the staged path instead. One network size serves the whole warp.
-  const int need = max(na, nb);
-  // cls 4: bit-packed (the column is, or the source is, or the sum exceeds the threshold)
-  const bool dense_job =
-      kDense && jb.surv &&
-      (jb.dense_a || (B != nullptr && (jb.dense_b || goes_dense(a, jb.j, N))));
-  // the register network for jobs of up to kRegMax rows per column; the piece kernels keep it
-  // small (8), their registers go to the merge pieces
-  constexpr int kRegMax = kLane ? 16 : 8;
-  int cls = !jb.surv ? 0 : (dense_job ? 4 : (need <= kRegMax ? 1 : 3));
-  constexpr int kRegMinJobs = kWarp ? 12 * kSlots / 32 : 12;  // of the warp's slots
-  if (__popc(__ballot_sync(0xffffffffu, cls == 1)) < kRegMinJobs && cls == 1) cls = 3;
-  const unsigned wneed = __reduce_max_sync(0xffffffffu, cls == 1 ? (unsigned)need : 0u);
-  if (cls == 1) {
-    int32_t last;
-    int len;
-    if constexpr (kRegMax == 16) {
-      len = wneed <= 4   ? reg_symdiff<4>(A, na, B, nb, slot, last)
-            : wneed <= 8 ? reg_symdiff<8>(A, na, B, nb, slot, last)
-                         : reg_symdiff<16>(A, na, B, nb, slot, last);
-    } else {
-      len = wneed <= 4 ? reg_symdiff<4>(A, na, B, nb, slot, last)
-                       : reg_symdiff<8>(A, na, B, nb, slot, last);
-    }
-    o_ptr = slot;
-    o_len = len;
-    if (B) {
-      a.low[jb.j] = last;
-      next_tab<true>(a, v, last, jb.j);
-    }
-  }
-  const unsigned smask = __ballot_sync(0xffffffffu, cls == 3);
-  if (smask) {
-    // longer merges: staged in shared memory, merge path over the concatenated jobs. Each list
-    // takes a 16-byte aligned span (its misalignment, its rows, a sentinel, rounded up to 4 words)
-    const int ra = (int)(((uintptr_t)A >> 2) & 3u);
-    const int rb = B ? (int)(((uintptr_t)B >> 2) & 3u) : 0;
-    const int span_a = (ra + na + 1 + 3) & ~3;
-    const int span_b = (rb + nb + 1 + 3) & ~3;
-    const bool staged = cls == 3 && N <= a.staged_max && span_a + span_b <= kStage;
-    const bool big = cls == 3 && !staged;
-    const unsigned stmask = __ballot_sync(0xffffffffu, staged);
-    const int ord = __popc(stmask & ((1u << lane) - 1u));  // ordinal among the staged jobs
-    const int words = staged ? span_a + span_b : 0;
-    const int w_ex = warp_incl_sum(words) - words;
-    const int km = a.force_km > 0 ? a.force_km : 8;
-    const int npc = staged ? (N + km - 1) / km : 0;  // merge pieces of the job
-    const int p_first = warp_incl_sum(npc) - npc;
-    if (staged) {
-      S.jout[ord] = slot;
-      S.na[ord] = na;
-      S.nb[ord] = nb;
-      S.pc[ord] = p_first;
-      S.jcnt[ord] = 0;
-      S.jlow[ord] = -1;
-    }
-    __syncwarp();
-    unsigned rest = stmask;
-    while (rest) {
-      // batch: the staged jobs from lane c on whose spans fit together
-      const int c = __ffs(rest) - 1;
-      const int w0 = __shfl_sync(0xffffffffu, w_ex, c);
-      const bool mine = staged && lane >= c && w_ex + words - w0 <= kStage;
-      const unsigned bmask = __ballot_sync(0xffffffffu, mine);
-      rest &= ~bmask;
-      const int o0 = __popc(stmask & ((1u << c) - 1u));
-      const int base = w_ex - w0;  // this job's spans in `in`
-      if (mine) {
-        S.ia[ord] = base + ra;
-        S.ib[ord] = base + span_a + rb;
-      }
-      // stage: 16-byte chunks from the lists' aligned starts (the column stores carry slack
-      // after their last column for the rounding); jobs of 16+ chunks by the whole warp,
-      // shorter ones by their lane; all copies of the batch are in flight together
-      const int ch_a = span_a >> 2;
-      const int ch_n = ch_a + (B ? span_b >> 2 : 0);
-      const int32_t* ga = A - ra;
-      const int32_t* gb = B ? B - rb : nullptr;
-      unsigned lmask = __ballot_sync(0xffffffffu, mine && ch_n >= 16);
-      while (lmask) {
-        const int src = __ffs(lmask) - 1;
-        lmask &= lmask - 1;
-        const int32_t* wa = (const int32_t*)__shfl_sync(0xffffffffu, (unsigned long long)ga, src);
-        const int32_t* wb = (const int32_t*)__shfl_sync(0xffffffffu, (unsigned long long)gb, src);
-        const int wca = __shfl_sync(0xffffffffu, ch_a, src);
-        const int wcn = __shfl_sync(0xffffffffu, ch_n, src);
-        int32_t* d = S.in + __shfl_sync(0xffffffffu, base, src);
-        for (int q = lane; q < wcn; q += 32)
-          cp_async16(d + 4 * q, q < wca ? wa + 4 * q : wb + 4 * (q - wca));
-      }
-      if (mine && ch_n < 16) {
-        int32_t* d = S.in + base;
-        for (int q = 0; q < ch_n; q++) cp_async16(d + 4 * q, q < ch_a ? ga + 4 * q : gb + 4 * (q - ch_a));
-      }
-      cp_async_wait_all();
-      __syncwarp();
-      if (mine) {  // the sentinels go after the copies, which may have covered their words
-        S.in[base + ra + na] = INT32_MAX;
-        S.in[base + span_a + rb + nb] = INT32_MAX;
-      }
-      __syncwarp();
-      if constexpr (kLane) {  // each job by its own lane
-        if (mine) {
-          int32_t lastv;
-          const int len = lane_merge_job(S.in, base + ra, base + span_a + rb, N, slot, &lastv);
-          S.jcnt[ord] = len;
-          S.jlow[ord] = lastv;
-        }
-      } else {  // pieces of every job spread over the lanes
-        const int P0 = __shfl_sync(0xffffffffu, p_first, c);
-        const int P1 = P0 + (int)__reduce_add_sync(0xffffffffu, mine ? (unsigned)npc : 0u);
-        switch (km) {
-          case 8: staged_rounds<8>(S, P0, P1, o0, mine, p_first, km); break;
-          default: staged_rounds<0>(S, P0, P1, o0, mine, p_first, km); break;
-        }
-      }
-      __syncwarp();
-    }
-    if (staged) {
-      o_ptr = slot;
-      o_len = S.jcnt[ord];
+  int cls = 0;
+  {
+    int32_t* m_ptr;
+    int m_len;
+    int32_t low;
+    cls = merge_rows<kDense, kWarp ? kSlots : 32, kLane>(
+        a, v, S, jb.j, jb.surv ? v.arena_next + off : nullptr, A, na, jb.dense_a, B, nb, jb.dense_b,
+        m_ptr, m_len, low);
+    if (jb.surv) {
+      o_ptr = m_ptr;
+      o_len = m_len;
       if (B) {
-        a.low[jb.j] = S.jlow[ord];
-        next_tab<true>(a, v, S.jlow[ord], jb.j);
+        a.low[jb.j] = low;
+        next_tab<true>(a, v, low, jb.j);
       }
-    }
-    // merges too long to stage: straight from global memory into their slot
-    unsigned bmask = __ballot_sync(0xffffffffu, big);
-    while (bmask) {
-      const int src = __ffs(bmask) - 1;
-      bmask &= bmask - 1;
-      const int32_t* wA = (const int32_t*)__shfl_sync(0xffffffffu, (unsigned long long)A, src);
-      const int32_t* wB = (const int32_t*)__shfl_sync(0xffffffffu, (unsigned long long)B, src);
-      const int wna = __shfl_sync(0xffffffffu, na, src);
-      const int wnb = __shfl_sync(0xffffffffu, nb, src);
-      int32_t* wd = (int32_t*)__shfl_sync(0xffffffffu, (unsigned long long)slot, src);
-      int len;
-      int32_t last = -1;
-      if (wB) {
-        len = warp_symdiff(wA, wna, wB, wnb, wd, last);
-      } else {
-        for (int q = lane; q < wna; q += 32) wd[q] = wA[q];
-        len = wna;
-      }
-      if (lane == src) {
-        if (B) {
-          a.low[jb.j] = last;
-          next_tab<true>(a, v, last, jb.j);
-        }
-        o_ptr = wd;
-        o_len = len;
-      }
-    }
-  }
-  // ---- bit-packed columns, one job at a time by the whole warp
-  unsigned dnmask = kDense ? __ballot_sync(0xffffffffu, cls == 4) : 0u;
-  while (dnmask) {
-    const int src = __ffs(dnmask) - 1;
-    dnmask &= dnmask - 1;
-    const int32_t* wA = (const int32_t*)__shfl_sync(0xffffffffu, (unsigned long long)A, src);
-    const int32_t* wB = (const int32_t*)__shfl_sync(0xffffffffu, (unsigned long long)B, src);
-    const int wna = __shfl_sync(0xffffffffu, na, src);
-    int32_t* wd = (int32_t*)__shfl_sync(0xffffffffu, (unsigned long long)slot, src);
-    const bool wdense_a = __shfl_sync(0xffffffffu, (int)jb.dense_a, src) != 0;
-    if (wB == nullptr) {  // a bit-packed column with nothing to add moves as it is
-      for (int q = lane; q < wna; q += 32) wd[q] = wA[q];
-      if (lane == src) {
-        o_ptr = wd;
-        o_len = dense_len(wna);
-      }
-      continue;
-    }
-    int32_t low, words;
-    const int32_t rows = dense_job_warp(a, __shfl_sync(0xffffffffu, jb.j, src), wA, wna, wdense_a,
-                                        wB, __shfl_sync(0xffffffffu, nb, src),
-                                        __shfl_sync(0xffffffffu, (int)jb.dense_b, src) != 0, wd,
-                                        low, words);
-    if (lane == src) {
-      o_ptr = wd;
-      o_len = rows ? dense_len(words) : 0;  // a zero column stores nothing
-      a.low[jb.j] = low;
-      next_tab<true>(a, v, low, jb.j);
     }
   }
   // ---- the survivors' places in the next active list
@@ -1648,16 +2155,17 @@ __device__ __forceinline__ void add_chunk(const RArgs& a, const PV& v, int64_t c
     }
   }
   const bool defer = jb.newpiv || (jb.surv && !jb.target);
-  if (defer) {
-    a.nxt_ptr[e] = o_ptr;
-    a.nxt_len[e] = o_len;
-  }
   const unsigned dmask = __ballot_sync(0xffffffffu, defer);
   if (dmask) {
     int d0 = 0;
     if (lane == __ffs(dmask) - 1) d0 = atomicAdd(&a.ds->n_deferred, __popc(dmask));
     d0 = __shfl_sync(0xffffffffu, d0, __ffs(dmask) - 1);
-    if (defer) a.dlist[d0 + __popc(dmask & ((1u << lane) - 1))] = (int32_t)e;
+    if (defer) {
+      d0 += __popc(dmask & ((1u << lane) - 1));
+      a.dlist[d0] = jb.j;
+      a.nxt_ptr[d0] = o_ptr;
+      a.nxt_len[d0] = o_len;
+    }
   }
   // ---- counters, per warp into the block's shared totals
   const int n_tgt = __popc(__ballot_sync(0xffffffffu, jb.target));
@@ -1686,41 +2194,38 @@ __device__ __forceinline__ void add_chunk(const RArgs& a, const PV& v, int64_t c
   }
 }
 
-// kDense: the pass may meet bit-packed columns or convert some; the row-list variant carries none
-// of it. kSlots: chunks of kSlots (32 or 8) slots claimed by single warps, 0: chunks of 128 slots
-// claimed by blocks. kLane: each staged job merged by its own lane (short columns), else merge
-// pieces spread over the lanes. The host picks the variant from DevState::dense_on, warp_on,
-// narrow_on and lane_on (a separate graph for each).
-template <bool kDense, int kSlots, bool kLane, int kBT = kAddThreads>
-__global__ void __launch_bounds__(kBT, 1024 / kBT) k_add(RArgs a) {
+// one pass's additions, by every block of the grid. kLoop: in the loop kernel (every block resident),
+// where chunks are dealt out in order; otherwise they are claimed in order from a work queue
+template <bool kDense, int kSlots, bool kLane, int kBT, bool kLoop>
+__device__ __forceinline__ void add_pass(const RArgs& a, WarpStage& S, unsigned blocks) {
   constexpr bool kWarp = kSlots > 0;
   __shared__ int64_t sh[kBT / 32 + 1];
   __shared__ int64_t s_chunk;
   __shared__ int64_t s_prefix[2];
   __shared__ unsigned long long s_cnt[kNumCnt];
   __shared__ PV s_v;  // per-pass values from shared memory rather than held in registers
-  extern __shared__ __align__(16) unsigned char add_smem[];
-  pdl_wait();
-  pdl_trigger();
-  if (a.ds->status != ST_RUN) return;
   if (threadIdx.x == 0) s_v = pass_view(a.ds);
   if (blockIdx.x == 0 && threadIdx.x == 0) a.ds->chunk_slots = kWarp ? kSlots : kBT;
   const PV& v = s_v;
-  WarpStage& S = reinterpret_cast<WarpStage*>(add_smem)[threadIdx.x >> 5];
   if (threadIdx.x < kNumCnt) s_cnt[threadIdx.x] = 0;
   if constexpr (kWarp) {
     __syncthreads();  // publishes s_v and the zeroed counters
     const int64_t nchunks = (v.n_act + kSlots - 1) / kSlots;
-    for (;;) {  // device work queue of kSlots-slot chunks, claimed in order by whole warps
-      unsigned int chunk = 0;
-      if (lane_id() == 0) chunk = atomicAdd(&a.ds->queue, 1u);
-      chunk = __shfl_sync(0xffffffffu, chunk, 0);
+    unsigned int next = (threadIdx.x >> 5) * blocks + blockIdx.x;
+    for (;;) {  // chunks of kSlots slots for whole warps
+      unsigned int chunk = next;
+      if (kLoop) {
+        next += blocks * (kBT / 32);
+      } else {
+        if (lane_id() == 0) chunk = atomicAdd(&a.ds->queue, 1u);
+        chunk = __shfl_sync(0xffffffffu, chunk, 0);
+      }
       if ((int64_t)chunk >= nchunks) break;
       add_chunk<kDense, kSlots, kLane, kBT>(a, v, chunk, S, sh, s_prefix, s_cnt);
     }
     __syncthreads();
   } else {
-    for (;;) {  // device work queue of 128-slot chunks, claimed in order
+    for (;;) {  // chunks of kBT slots for the whole block
       if (threadIdx.x == 0) s_chunk = atomicAdd(&a.ds->queue, 1u);
       __syncthreads();  // also publishes s_v, written by thread 0 before the loop
       const int64_t chunk = s_chunk;
@@ -1730,30 +2235,447 @@ __global__ void __launch_bounds__(kBT, 1024 / kBT) k_add(RArgs a) {
       add_chunk<kDense, 0, kLane, kBT>(a, v, chunk, S, sh, s_prefix, s_cnt);
     }
   }
-  if (threadIdx.x == 0 && s_cnt[kCntTargets]) atomicAdd(&a.ds->totals[1], s_cnt[kCntTargets]);
-  if (v.stats && threadIdx.x == 0) {
-    const int idx[kNumCnt] = {PH_PS_TARGETS, PH_PS_ACTIVE, PH_PS_CLEARED,
-                              PH_PS_ADDS,    PH_PS_XORS,   PH_PS_COPIED, PH_PS_PACKED};
-    for (int i = 0; i < kNumCnt; i++)
-      if (s_cnt[i]) atomicAdd((unsigned long long*)&v.stats[idx[i]], s_cnt[i]);
-  }
+  if (threadIdx.x == 0) flush_counters(a, v, s_cnt);
 }
 
-// |E^l| after this pass's marks (per-pass counter; only with collect_stats)
-__global__ void k_ess_count(RArgs a, int64_t m) {
-  __shared__ int64_t sh[kWarps + 1];
+// kDense: the pass may meet bit-packed columns or convert some; the row-list variant carries none
+// of it. kSlots: chunks of kSlots (32 or 8) slots claimed by single warps, 0: chunks of 128 slots
+// claimed by blocks. kLane: each staged job merged by its own lane (short columns), else merge
+// pieces spread over the lanes. The host picks the variant from DevState::dense_on, warp_on,
+// narrow_on and lane_on (a separate graph for each).
+template <bool kDense, int kSlots, bool kLane, int kBT = kAddThreads>
+__global__ void __launch_bounds__(kBT, 1024 / kBT) k_add(RArgs a) {
+  extern __shared__ __align__(16) unsigned char add_smem[];
   pdl_wait();
   pdl_trigger();
   if (a.ds->status != ST_RUN) return;
+  add_pass<kDense, kSlots, kLane, kBT, false>(
+      a, reinterpret_cast<WarpStage*>(add_smem)[threadIdx.x >> 5], gridDim.x);
+}
+
+// what k_merge does with a column
+enum : uint8_t {
+  kNothing = 0,
+  kMerge,     // its delta goes into its list
+  kAdd,       // the source whose id is in its delta's first place is added to its list
+  kMove,      // its list moves to this pass's arena
+  kMoveLate,  // ... but others may be reading it in this pass: published by k_commit
+};
+
+// Phase II with look-ahead, first half: every column that is due gets its source for this pass. A source of few
+// rows starts a visit (look_ahead), which leaves the column's list as it is, only shortened, and
+// its delta beside it; the columns whose list has to be rewritten, or whose source is too long
+// for a visit, are left to k_merge. In a pass that compacts that is every survivor: it gets its
+// place in the next active list from a decoupled look-back over the chunks. New pivots are
+// copied to the pivot store. Targets and zeroed columns are updated in place (no other job reads
+// them this pass); new pivots and left-most survivors, which other jobs may be reading as
+// sources, are updated by k_commit.
+struct VisitStage {
+  int32_t pend[32 + kScan];  // slots gathered for the next rounds
+};
+
+// by one warp. e, j: this lane's slot and its column (-1: none), which is due
+__device__ __forceinline__ void visit_round(const RArgs& a, const PV& v, int32_t e, int32_t j,
+                                            unsigned long long* s_cnt) {
+  constexpr int R = kSourceRows, kNew = R * kAheadMax;
+  const int lane = lane_id();
+  const int32_t pass = a.ds->pass;
+  // every load is issued up front: the column, its low and its source candidate are known from
+  // the active list, the stored lows and k_phase1's per-slot source, so no load waits on
+  // another's result
+  Visit w;
+  bool surv = false, newpiv = false, target = false, add = false, eager = false, dense_a = false;
+  int32_t s = -1;
+  w.low = -1;
+  w.na = w.nb = w.k = 0;
+  w.A = w.B = nullptr;
+  w.rec = make_int4(0, 0, 0, 0);
+  w.gone = w.settle = false;
+  // its place in the next active list: compacted, or where it is (a due column's low is its own)
+  int64_t pos = e;
+  if (j >= 0) {
+    w.low = a.low[j];
+    if (v.compact) pos = a.newpos[e];
+    const int32_t se = a.src_e[e];  // -1: no collision; <= -2: a target whose set waits
+    const ColMeta mj = load_meta(a.meta + j);
+    if (se >= 0) w.rec = a.prec[w.low];
+    newpiv = (mj.flags & F_NEWPIV) != 0;
+    surv = !(mj.flags & (F_PROVEN | F_FINAL)) && !mj.cleared;
+    target = surv && se != -1;
+    dense_a = mj.len < 0;
+    w.A = mj.ptr;
+    w.na = stored_words(mj.len);
+    w.k = mj.spare;
+    if (target && se >= 0 && v.do_adds) {
+      s = se;
+      if (w.rec.x > 0 && w.rec.x <= R + 1) {  // a proven pivot's record says it all
+        add = true;
+        eager = dense_a;
+      } else {
+        const ColMeta ms = load_meta(a.meta + s);
+        add = !(ms.flags & F_FINAL) && !ms.cleared && (!a.strict || (ms.flags & F_PROVEN));
+        w.B = ms.ptr;
+        w.nb = ms.len;
+        eager = add && (dense_a || ms.len < 0 || ms.len > kNew + 1);
+      }
+    }
+  }
+  w.due = pass + 1;
+  const int na0 = w.na;
+  const bool visit = add && !eager;
+  if (__any_sync(0xffffffffu, visit)) {
+    int32_t* block = a.delta + (int64_t)max(j, 0) * kDeltaRows;
+#pragma unroll
+    for (int i = 0; i < kOld; i += 4) {
+      int4 x = make_int4(INT32_MAX, INT32_MAX, INT32_MAX, INT32_MAX);
+      if (visit && i < w.k) x = *reinterpret_cast<const int4*>(block + i);
+      w.d.c[i] = -x.x;
+      w.d.c[i + 1] = i + 1 < w.k ? -x.y : kEmpty;
+      w.d.c[i + 2] = i + 2 < w.k ? -x.z : kEmpty;
+      w.d.c[i + 3] = i + 3 < w.k ? -x.w : kEmpty;
+    }
+#pragma unroll
+    for (int i = kOld; i < kDeltaRows; i++) w.d.c[i] = kEmpty;
+    const bool c10 = visit && a.cor10 && a.beta[j] < 0;
+    const int32_t fu =
+        c10 ? a.first_unp[seg_of(a, j) - a.nc] : INT32_MIN;
+    if (look_ahead(a, v, pass, visit, fu, pos, w)) tidy<0>(w, visit && !w.gone);
+    else tidy<kOld>(w, visit && !w.gone);
+    if (visit) {
+#pragma unroll
+      for (int i = 0; i < kDeltaRows; i += 4)
+        if (i < w.k)
+          *reinterpret_cast<int4*>(block + i) =
+              make_int4(w.d.c[i], w.d.c[i + 1], w.d.c[i + 2], w.d.c[i + 3]);
+    }
+  }
+
+  // what is left to k_merge: a compacting pass rewrites every list, another one those whose delta
+  // is full or that have to be whole; at the cap the lists are what the caller can read
+  int kind = kNothing;
+  if (eager) {
+    kind = kAdd;
+    a.delta[(int64_t)j * kDeltaRows] = s;
+  } else if (visit) {
+    if (!w.gone && (v.compact || w.k > kOld ||
+                    (w.k > 0 && (w.settle || v.whole))))
+      kind = kMerge;
+  } else if (surv && v.compact) {
+    kind = target ? kMove : kMoveLate;
+  }
+  if (v.compact) {
+    if (j >= 0 && pos >= 0 && PH_DCHECK(&a.ds->debug_fault, pos < v.n_act, 5)) {
+      v.act2[pos] = surv ? j : dead_slot(j);
+      v.alen2[pos] = w.na;
+      a.kind[pos] = (uint8_t)kind;
+    }
+  } else {
+    if (j >= 0 && !surv) v.act[e] = dead_slot(j);
+    if (visit) v.alen[e] = w.na;
+    const unsigned km = __ballot_sync(0xffffffffu, kind != kNothing);
+    if (km) {
+      unsigned int base = 0;
+      if (lane == 0) base = atomicAdd(&a.ds->n_work, (unsigned int)__popc(km));
+      base = __shfl_sync(0xffffffffu, base, 0);
+      if (kind) {
+        a.work[base + __popc(km & ((1u << lane) - 1))] = e;
+        a.kind[e] = (uint8_t)kind;
+      }
+    }
+  }
+
+  // ---- new pivots: their columns never change again; move them to the pivot store (a
+  // bit-packed column moves as its stored words)
+  int32_t* p_ptr = nullptr;
+  unsigned pmask = __ballot_sync(0xffffffffu, newpiv);
+  if (pmask) {  // the warp's new pivots take one run of the pivot store
+    const unsigned all = pmask;
+    const int mine = newpiv ? na0 : 0;
+    const int incl = warp_incl_sum(mine);
+    const int ptot = __shfl_sync(0xffffffffu, incl, 31);
+    unsigned long long w0 = 0;
+    int d0 = 0;
+    if (lane == 0) {
+      w0 = atomicAdd(&a.ds->piv_used, (unsigned long long)ptot);
+      d0 = atomicAdd(&a.ds->n_deferred, __popc(all));
+    }
+    w0 = __shfl_sync(0xffffffffu, w0, 0) + (unsigned long long)(incl - mine);
+    d0 = __shfl_sync(0xffffffffu, d0, 0) + __popc(all & ((1u << lane) - 1));
+#ifdef PH_DEBUG
+    // the warp's run lies in the pivot store's chunk (else the warp's copies are dropped)
+    const bool in_store = PH_DCHECK(&a.ds->debug_fault, (int64_t)(w0 + mine) <= v.piv_cap, 4);
+    if (!__all_sync(0xffffffffu, in_store)) pmask = 0;
+#endif
+    if (newpiv) {
+      p_ptr = v.piv_base + w0;
+      a.dlist[d0] = j;
+      a.nxt_ptr[d0] = p_ptr;
+      a.nxt_len[d0] = dense_a ? dense_len(na0) : na0;
+    }
+  }
+  while (pmask) {
+    const int src = __ffs(pmask) - 1;
+    pmask &= pmask - 1;
+    const int32_t* wA = (const int32_t*)__shfl_sync(0xffffffffu, (unsigned long long)w.A, src);
+    const int wna = __shfl_sync(0xffffffffu, na0, src);
+    int32_t* dst = (int32_t*)__shfl_sync(0xffffffffu, (unsigned long long)p_ptr, src);
+    for (int q = lane; q < wna; q += 32) dst[q] = wA[q];
+  }
+
+  // ---- publish: the lows of the coming passes (k_merge knows those of its additions), a visited
+  // column's shortened list and its delta, a zeroed column
+  if (surv && PH_DCHECK(&a.ds->debug_fault, pos >= 0 && pos < v.n_act, 5)) {
+    a.due[pos] = w.due;
+    if (visit) {
+      if (w.due == pass + 1) next_tab<true>(a, v, w.low, j);
+    } else if (!eager) {  // its low stays
+      a.lows[(int64_t)((pass + 1) & a.ring) * a.lows_stride + pos] = w.low;
+      next_tab<false>(a, v, w.low, j);
+    }
+  }
+  if (visit) {
+    a.low[j] = w.low;
+    a.meta[j].len = w.na;
+    a.meta[j].spare = (uint8_t)w.k;
+  } else if (j >= 0 && !surv && !newpiv) {
+    a.meta[j].flags |= F_FINAL;
+    a.low[j] = -1;
+    a.meta[j].len = 0;
+  }
+  // ---- counters, per warp into the block's shared totals
+  const int n_tgt = __popc(__ballot_sync(0xffffffffu, target));
+  if (lane == 0 && n_tgt) atomicAdd(&s_cnt[kCntTargets], (unsigned long long)n_tgt);
+}
+
+// one pass's visits, by every block of the grid
+__device__ __forceinline__ void visit_pass(const RArgs& a, VisitStage& S, unsigned blocks) {
+  __shared__ unsigned long long s_cnt[kNumCnt];
+  __shared__ PV s_v;  // per-pass values from shared memory rather than held in registers
+  if (threadIdx.x == 0) s_v = pass_view(a.ds);
+  const PV& v = s_v;
+  const int lane = lane_id();
+  const int warps = blockDim.x >> 5;
+  if (threadIdx.x < kNumCnt) s_cnt[threadIdx.x] = 0;
+  __syncthreads();  // publishes s_v and the zeroed counters
+  // A pass that compacts: every column is due, 32 slots per round. Otherwise few columns are due:
+  // every warp looks through its share of the slots and gathers the due ones for full rounds. A column ahead of the pass stays a target, unless clearing zeroes it (only below the
+  // top dimension); its last stored low enters the next pass's table when it is due then.
+  const int32_t pass = a.ds->pass;
+  const int32_t* lows_next = a.lows + (int64_t)((pass + 1) & a.ring) * a.lows_stride;
+  const int64_t warp = (int64_t)blockIdx.x * warps + (threadIdx.x >> 5);
+  int64_t i0 = warp * (v.compact ? 32 : kScan);
+  int np = 0, n_tgt = 0;
+  for (;;) {
+    int32_t e = 0, jv = -1;
+    if (v.compact) {
+      if (i0 >= v.n_act) break;
+      const int64_t x = i0 + lane;
+      i0 += (int64_t)blocks * warps * 32;
+      if (x < v.n_act) {
+        e = (int32_t)x;
+        jv = max(v.act[e], -1);
+      }
+    } else {
+      for (; np < 32 && i0 < v.n_act; i0 += (int64_t)blocks * warps * kScan) {
+        int32_t js[kScan / 32], ds[kScan / 32];
+#pragma unroll
+        for (int u = 0; u < kScan / 32; u++) {
+          const int64_t x = i0 + 32 * u + lane;
+          js[u] = x < v.n_act ? v.act[x] : -1;
+          ds[u] = x < v.n_act ? a.due[x] : 0;
+        }
+#pragma unroll
+        for (int u = 0; u < kScan / 32; u++) {
+          const int32_t x = (int32_t)(i0 + 32 * u + lane);
+          const int32_t j = js[u];
+          if (j >= 0 && ds[u] > pass) {
+            if (j < a.rows_end && a.meta[j].cleared) {
+              a.meta[j].flags |= F_FINAL;
+              a.meta[j].len = 0;
+              a.low[j] = -1;
+              v.act[x] = dead_slot(j);
+            } else {
+              n_tgt++;
+              if (ds[u] == pass + 1) next_tab<true>(a, v, lows_next[x], j);
+            }
+          }
+          const bool due = j >= 0 && ds[u] <= pass;
+          const unsigned m = __ballot_sync(0xffffffffu, due);
+          if (due) S.pend[np + __popc(m & ((1u << lane) - 1u))] = x;
+          np += __popc(m);
+        }
+        __syncwarp();
+      }
+      if (np == 0) break;
+      const int n = min(np, 32);
+      np -= n;
+      if (lane < n) {
+        e = S.pend[np + lane];
+        jv = v.act[e];
+      }
+      __syncwarp();
+    }
+    visit_round(a, v, e, jv, s_cnt);
+  }
+  if (!v.compact) {
+    const unsigned t = __reduce_add_sync(0xffffffffu, (unsigned)n_tgt);
+    if (lane == 0 && t) atomicAdd(&s_cnt[kCntTargets], (unsigned long long)t);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) flush_counters(a, v, s_cnt);
+}
+
+__global__ void __launch_bounds__(kAddThreads, 1024 / kAddThreads) k_visit(RArgs a) {
+  __shared__ VisitStage s_stage[kAddWarps];
+  pdl_wait();
+  pdl_trigger();
+  if (a.ds->status != ST_RUN) return;
+  visit_pass(a, s_stage[threadIdx.x >> 5], gridDim.x);
+}
+
+// the places of the next active list in a pass that compacts: the inclusive prefix that the last
+// chunk of k_add, or with look-ahead Phase I's last tile, published in its look-back (false: there
+// is none, an internal error)
+__device__ __forceinline__ bool survivors(const RArgs& a, const DevState* ds, int64_t n_act,
+                                          int32_t ahead, int32_t pass, int64_t& n) {
+  const int64_t per = ahead > 1 ? kFTile : ds->chunk_slots;
+  const int64_t nch = (n_act + per - 1) / per;
+  n = 0;
+  if (nch == 0) return true;
+  const unsigned long long w = *(const volatile unsigned long long*)(a.look + nch - 1);
+  if ((w >> 40) != (look_tag(pass) >> 40) || (w & kLookFlags) != kLookIncl) return false;
+  n = (int64_t)(w & kLookVal);
+  return true;
+}
+
+// Phase II with look-ahead, second half, by one warp: the lists of columns that k_visit left to it.
+// pos: this lane's slot, kind: what to do with its column. The warp's jobs take one contiguous run
+// of the arena, from one atomic.
+template <bool kDense, bool kLane>
+__device__ __forceinline__ void merge_round(const RArgs& a, const PV& v, int32_t pos, int kind,
+                                            WarpStage& S) {
+  const int lane = lane_id();
+  int32_t j = -1;
+  const int32_t* A = nullptr;
+  const int32_t* B = nullptr;
+  int na = 0, nb = 0;
+  bool dense_a = false, dense_b = false;
+  if (kind) {
+    j = (v.compact ? v.act2 : v.act)[pos];
+    const ColMeta mj = load_meta(a.meta + j);
+    A = mj.ptr;
+    na = kDense ? stored_words(mj.len) : mj.len;
+    dense_a = kDense && mj.len < 0;
+    if (kind == kMerge) {
+      B = a.delta + (int64_t)j * kDeltaRows;
+      nb = mj.spare;
+    } else if (kind == kAdd) {
+      const ColMeta ms = load_meta(a.meta + a.delta[(int64_t)j * kDeltaRows]);
+      B = ms.ptr;
+      nb = kDense ? stored_words(ms.len) : ms.len;
+      dense_b = kDense && ms.len < 0;
+    }
+  }
+  const int64_t words = kind ? na + nb : 0;
+  const int64_t wincl = warp_incl_sum(words);
+  const int64_t wtot = __shfl_sync(0xffffffffu, wincl, 31);
+  unsigned long long wbase = 0;
+  if (lane == 0 && wtot) wbase = atomicAdd(&a.ds->arena_used, (unsigned long long)wtot);
+  const int64_t off = (int64_t)__shfl_sync(0xffffffffu, wbase, 0) + wincl - words;
+#ifdef PH_DEBUG
+  // the job's slot lies in the arena this pass writes (else the job is dropped and reported)
+  if (kind && !PH_DCHECK(&a.ds->debug_fault, off >= 0 && off + words <= v.arena_next_cap, 3)) {
+    kind = kNothing;
+    j = -1;
+  }
+#endif
+  int32_t* o_ptr;  // the column's new place, length and low
+  int o_len;
+  int32_t low;
+  merge_rows<kDense, 32, kLane>(a, v, S, j, kind ? v.arena_next + off : nullptr, A, na,
+                                                dense_a, B, nb, dense_b, o_ptr, o_len, low);
+  // ---- publish
+  if (kind) {
+    (v.compact ? v.alen2 : v.alen)[pos] = o_len;
+    if (kind != kMoveLate) {
+      a.meta[j].ptr = o_ptr;
+      a.meta[j].len = o_len;
+    }
+    if (kind == kMerge) a.meta[j].spare = 0;
+    if (kind == kAdd) {
+      a.low[j] = low;
+      a.lows[(int64_t)((a.ds->pass + 1) & a.ring) * a.lows_stride + pos] = low;
+      next_tab<true>(a, v, low, j);
+    }
+  }
+  const unsigned dmask = __ballot_sync(0xffffffffu, kind == kMoveLate);
+  if (dmask) {
+    int d0 = 0;
+    if (lane == 0) d0 = atomicAdd(&a.ds->n_deferred, __popc(dmask));
+    d0 = __shfl_sync(0xffffffffu, d0, 0) + __popc(dmask & ((1u << lane) - 1));
+    if (kind == kMoveLate) {
+      a.dlist[d0] = j;
+      a.nxt_ptr[d0] = o_ptr;
+      a.nxt_len[d0] = o_len;
+    }
+  }
+}
+
+// kDense: the pass may meet bit-packed columns or convert some; the row-list variant carries none
+// of it. kSlots: columns per warp and round (32 or 8). kLane: each staged job merged by its own
+// lane (short columns), else merge pieces spread over the lanes. The host picks the variant from
+// DevState::dense_on, narrow_on and lane_on (a separate graph for each).
+template <bool kDense, bool kLane>
+__device__ __forceinline__ void merge_pass(const RArgs& a, WarpStage& S, unsigned blocks) {
+  __shared__ PV s_v;  // per-pass values from shared memory rather than held in registers
+  if (threadIdx.x == 0) s_v = pass_view(a.ds);
+  const PV& v = s_v;
+  const int lane = lane_id();
+  __syncthreads();  // publishes s_v
+  int64_t n = 0;
+  if (!v.compact) n = a.ds->n_work;
+  else if (!survivors(a, a.ds, v.n_act, v.ahead, a.ds->pass, n)) a.ds->fault = 1;
+  // full rounds, or the few columns spread over all warps
+  const int64_t warps = (int64_t)blocks * (blockDim.x >> 5);
+  const int per = (int)std::min<int64_t>(32, (n + warps - 1) / warps);
+  for (int64_t i = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * per; i < n;
+       i += warps * per) {
+    const bool mine = lane < per && i + lane < n;
+    const int32_t pos = !mine ? 0 : v.compact ? (int32_t)(i + lane) : a.work[i + lane];
+    merge_round<kDense, kLane>(a, v, pos, mine ? a.kind[pos] : kNothing, S);
+    __syncwarp();
+  }
+}
+
+template <bool kDense, bool kLane>
+__global__ void __launch_bounds__(kAddThreads, 1024 / kAddThreads) k_merge(RArgs a) {
+  extern __shared__ __align__(16) unsigned char add_smem[];
+  pdl_wait();
+  pdl_trigger();
+  if (a.ds->status != ST_RUN) return;
+  merge_pass<kDense, kLane>(a, reinterpret_cast<WarpStage*>(add_smem)[threadIdx.x >> 5],
+                                    gridDim.x);
+}
+
+// |E^l| after this pass's marks (per-pass counter; only with collect_stats)
+__device__ __forceinline__ void ess_count(const RArgs& a, int64_t m, unsigned blocks) {
+  __shared__ int64_t sh[kWarps + 1];
   int64_t n = 0;
   for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < m;
-       x += (int64_t)gridDim.x * blockDim.x)
+       x += (int64_t)blocks * blockDim.x)
     n += in_essential_estimate(load_meta(a.meta + x), a.beta[x], a.owner[x]);
   int64_t tot;
   block_excl_sum<int64_t>(n, sh, tot);
   if (threadIdx.x == 0 && tot)
     atomicAdd((unsigned long long*)&a.ds->stats[(int64_t)a.ds->pass * PH_PS_N + PH_PS_ESS_EST],
               (unsigned long long)tot);
+}
+
+__global__ void k_ess_count(RArgs a, int64_t m) {
+  pdl_wait();
+  pdl_trigger();
+  if (a.ds->status != ST_RUN) return;
+  ess_count(a, m, gridDim.x);
 }
 
 // E^l of the ids [lo, hi) (one dimension of one cloud), as bytes at their filtration index
@@ -1772,8 +2694,11 @@ __global__ void k_ess_flags(int64_t lo, int64_t hi, const ColMeta* __restrict__ 
   }
 }
 
+// where a pass runs: host-driven, in the graph's loop (which stops when another variant of the
+// additions, or the loop kernel, suits the next passes better), in the loop kernel
+enum : int { kHostLoop = 0, kInGraph = 1, kInLoop = 2 };
 // the deferred column updates: new pivots (now in the pivot store) and left-most survivors
-__device__ void end_of_pass(const RArgs& a, cudaGraphConditionalHandle cond, int in_graph);
+__device__ void end_of_pass(const RArgs& a, cudaGraphConditionalHandle cond, int mode);
 
 // the counters a pass accumulates, cleared for the next one
 __host__ __device__ inline void reset_counters(DevState* ds) {
@@ -1781,39 +2706,134 @@ __host__ __device__ inline void reset_counters(DevState* ds) {
   ds->bound_piv = 0;
   ds->queue = 0;
   ds->tile_queue = 0;
-  ds->arena_used = 0;
   ds->n_deferred = 0;
+  ds->n_work = 0;
+  ds->n_dirty = 0;
   ds->totals[0] = ds->totals[1] = 0;
 }
 
 // the deferred column updates and the next pass's row state, then (last block) the end of the
 // pass and the reset of the per-pass counters. A pass stopped for space (ST_HOST) continues at
 // Phase II on the row state it had, so neither is touched then (the host resets the counters).
-__global__ void k_commit(RArgs a, cudaGraphConditionalHandle cond, int in_graph) {
-  pdl_wait();
+__device__ __forceinline__ void commit_pass(const RArgs& a, unsigned blocks) {
   DevState* ds = a.ds;
-  const bool run = ds->status == ST_RUN;
-  const int32_t p = ds->pass;
-  const int64_t n = run ? (int64_t)ds->n_deferred : 0;
-  if (n > 0) {
-    const PV v = pass_view(ds);
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-      const int32_t e = a.dlist[i];
-      const int32_t j = v.act[e];
-      a.meta[j].ptr = a.nxt_ptr[e];
-      a.meta[j].len = a.nxt_len[e];
-      a.meta[j].flags &= (uint8_t)~F_NEWPIV;
+  const int64_t n = (int64_t)ds->n_deferred;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+       i += (int64_t)blocks * blockDim.x) {
+    const int32_t j = a.dlist[i];
+    const ColMeta mj = load_meta(a.meta + j);
+    a.meta[j].ptr = a.nxt_ptr[i];
+    a.meta[j].len = a.nxt_len[i];
+    if (mj.flags & F_NEWPIV) {  // a long pivot's record points to its rows
+      if (ds->ahead > 1 && mj.len > kRecRows) a.prec[a.low[j]] = rec_of(a.nxt_ptr[i], mj.len);
+      a.meta[j].flags = (uint8_t)(mj.flags & ~F_NEWPIV);
     }
   }
-  if (run) rows_of_pass(a, p + 1);
+  next_unpaired(a, blocks);
+  if (a.predict) rows_of_pass<false>(a, blocks);
+}
+// by the last block
+__device__ __forceinline__ void commit_last(const RArgs& a, cudaGraphConditionalHandle cond,
+                                            int mode, unsigned blocks) {
+  const bool run = a.ds->status == ST_RUN;
+  if (run) {
+    rows_of_pass_last(a);
+    next_unpaired_last(a, blocks);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    end_of_pass(a, cond, mode);
+    if (run) reset_counters(a.ds);
+  }
+}
+
+__global__ void k_commit(RArgs a, cudaGraphConditionalHandle cond, int mode) {
+  pdl_wait();
+  DevState* ds = a.ds;
+  if (ds->status == ST_RUN) commit_pass(a, gridDim.x);
   if (last_block(&ds->blocks_done, gridDim.x)) {
-    if (run) rows_of_pass_last(a, p + 1);
+    if (threadIdx.x == 0) ds->blocks_done = 0;
+    commit_last(a, cond, mode, gridDim.x);
+  }
+}
+
+// ------------------------------------------------------------------------------------------
+// the pass loop in one kernel
+// ------------------------------------------------------------------------------------------
+// On a short active list a pass's kernels take some microseconds each, whatever they do: launch,
+// first loads, last-block handshakes, drain. k_loop runs all passes in one cooperative grid
+// (every block resident, so they may wait for each other), the parts of a pass separated by
+// grid barriers.
+//
+// A grid barrier: true in every block once all have arrived and the last one to arrive has run
+// `tail`; what was written before it is visible after it. The wait is bounded: a block that gives
+// up records a fault, and returns false.
+template <typename F>
+__device__ __forceinline__ bool grid_sync(DevState* ds, unsigned blocks, F tail) {
+  __shared__ int s_last, s_ok;
+  __shared__ unsigned int s_gen;
+  __syncthreads();
+  if (blocks == 1) {
+    tail();
+    __syncthreads();
+    return true;
+  }
+  if (threadIdx.x == 0) {
+    s_gen = *(volatile unsigned int*)&ds->bar_gen;
+    s_ok = 1;
+    __threadfence();
+    s_last = atomicAdd(&ds->bar_count, 1u) == blocks - 1;
+  }
+  __syncthreads();
+  if (s_last) {
+    __threadfence();
+    tail();
+    __syncthreads();
     if (threadIdx.x == 0) {
-      ds->blocks_done = 0;
-      end_of_pass(a, cond, in_graph);
-      if (run) reset_counters(ds);
+      ds->bar_count = 0;
+      __threadfence();
+      atomicExch(&ds->bar_gen, s_gen + 1);
     }
+  } else if (threadIdx.x == 0) {
+    int it = 0;
+    while (*(volatile unsigned int*)&ds->bar_gen == s_gen) {
+      if (++it > kBarrierLimit) {
+        ds->fault = 1;
+        s_ok = 0;
+        break;
+      }
+      __nanosleep(20);
+    }
+  }
+  if (threadIdx.x == 0) __threadfence();
+  __syncthreads();
+  return s_ok != 0;
+}
+
+constexpr int kLoopBlocks = 2;  // per SM: registers for every part of a pass without spills
+__global__ void __launch_bounds__(kThreads, kLoopBlocks) k_loop(RArgs a, int64_t m) {
+  extern __shared__ __align__(16) unsigned char add_smem[];
+  WarpStage& S = reinterpret_cast<WarpStage*>(add_smem)[threadIdx.x >> 5];
+  DevState* ds = a.ds;
+  const auto nothing = [] {};
+  // a shrinking list is left to fewer blocks, at last to one, whose barriers cost next to nothing
+  for (;;) {
+    const unsigned blocks = *(volatile unsigned int*)&ds->loop_blocks;
+    if (blockIdx.x >= blocks || *(volatile int32_t*)&ds->status != ST_RUN) return;
+    phase1_pass<false>(a, phase1_parts(ds, blocks));
+    if (!grid_sync(ds, blocks, [&] {
+          if (threadIdx.x == 0) check_capacity(ds);
+        }))
+      return;
+    if (*(volatile int32_t*)&ds->status != ST_RUN) return;
+    if (ds->stats) {
+      ess_count(a, m, blocks);
+      if (!grid_sync(ds, blocks, nothing)) return;
+    }
+    add_pass<true, 32, false, kThreads, true>(a, S, blocks);
+    if (!grid_sync(ds, blocks, nothing)) return;
+    commit_pass(a, blocks);
+    if (!grid_sync(ds, blocks, [&] { commit_last(a, 0, kInLoop, blocks); })) return;
   }
 }
 
@@ -1826,67 +2846,103 @@ __device__ __forceinline__ unsigned long long global_ns() {
 
 __global__ void k_clock_start(DevState* ds) { ds->t_start = global_ns(); }
 
+// blocks of the loop kernel for an active list of n columns: one for a tile of Phase I, else one per
+// 256 columns
+__host__ __device__ inline unsigned int loop_blocks_for(int64_t n) {
+  return n <= kFTile ? 1u : (unsigned int)std::min<int64_t>((n + kThreads - 1) / kThreads, 1 << 20);
+}
+
 // end of a pass: the next active list, convergence (no target left), the pass cap, the time
 // bound, and the graph's loop condition
-__device__ void end_of_pass(const RArgs& a, cudaGraphConditionalHandle cond, int in_graph) {
+__device__ void end_of_pass(const RArgs& a, cudaGraphConditionalHandle cond, int mode) {
+  const bool in_graph = mode == kInGraph;
   DevState* ds = a.ds;
-  if (ds->status == ST_RUN && (ds->fault || ds->debug_fault)) ds->status = ST_FAULT;
-  const bool to_dense = ds->dense_want && !ds->dense_on;
+  // one thread's work, on the path of every pass: its loads are issued together
+  const int32_t fault = ds->fault, debug_fault = ds->debug_fault, p = ds->pass;
+  const int32_t dense_want = ds->dense_want, dense_on = ds->dense_on, compact = ds->compact;
+  const int32_t was_ahead = ds->ahead, was_leave = ds->leave, horizon = ds->horizon;
+  const int32_t arena_cur = ds->arena_cur, max_passes = ds->max_passes, warp_on = ds->warp_on;
+  const int32_t lane_on = ds->lane_on, narrow_on = ds->narrow_on, drain = ds->drain;
+  const int32_t stats_rows = ds->stats_rows;
+  const int64_t n_act = ds->n_act, warp_below = ds->warp_below, warp_words = ds->warp_words;
+  const int64_t lane_words = ds->lane_words, narrow_below = ds->narrow_below;
+  const int64_t ahead_above = ds->ahead_above, loop_below = ds->loop_below;
+  const unsigned long long used = ds->arena_used, targets = ds->totals[1];
+  const unsigned long long t_start = ds->t_start, t_limit = ds->t_limit;
+  int32_t* const act = ds->act;
+  int32_t* const act2 = ds->act2;
+  int32_t* const alen = ds->alen;
+  int32_t* const alen2 = ds->alen2;
+  const bool stats = ds->stats != nullptr;
+  int32_t status = ds->status;
+  int64_t n_surv = n_act;
+  if (status == ST_RUN &&
+      (fault || debug_fault || (compact && !survivors(a, ds, n_act, was_ahead, p, n_surv))))
+    status = ST_FAULT;
+  const bool to_dense = dense_want && !dense_on;
   if (to_dense) ds->dense_on = 1;
-  if (ds->status == ST_RUN) {
-    const int32_t p = ds->pass;
-    // the survivors of the pass: the inclusive prefix the last chunk published in its look-back
-    // (anything but an inclusive state of this pass is an internal error)
-    const int64_t nch = (ds->n_act + ds->chunk_slots - 1) / ds->chunk_slots;
-    int64_t n_surv = 0;
-    if (nch > 0) {
-      const unsigned long long w = *(const volatile unsigned long long*)(a.look + nch - 1);
-      if ((w >> 40) != (look_tag(p) >> 40) || (w & kLookFlags) != kLookIncl) {
-        ds->status = ST_FAULT;
-        if (in_graph) cudaGraphSetConditional(cond, 0u);
-        return;
-      }
-      n_surv = (int64_t)(w & kLookVal);
-    }
+  if (status == ST_RUN) {
     ds->n_act = n_surv;
-    int32_t* t = ds->act;
-    ds->act = ds->act2;
-    ds->act2 = t;
-    t = ds->alen;
-    ds->alen = ds->alen2;
-    ds->alen2 = t;
-    if (ds->totals[1] == 0) {
-      ds->status = ST_DONE;
+    if (compact) {
+      ds->act = act2;
+      ds->act2 = act;
+      ds->alen = alen2;
+      ds->alen2 = alen;
+    }
+    if (mode == kInLoop) ds->loop_blocks = min(ds->loop_blocks, loop_blocks_for(n_surv));
+    // the next pass: at the horizon it compacts into the other arena; before it, visited columns
+    // take new slots after the ones in use. Look-ahead ends with a compacting pass that runs no
+    // column ahead and makes every list whole
+    const bool next_compact = p + 1 >= horizon;
+    const bool to_add = was_leave != 0;
+    const int32_t ahead = to_add ? 1 : was_ahead;
+    const bool leave = next_compact && ahead > 1 && n_surv < ahead_above;
+    ds->compact = next_compact ? 1 : 0;
+    ds->ahead = ahead;
+    ds->leave = leave ? 1 : 0;
+    if (next_compact) {
+      ds->horizon = p + 1 + (leave ? 1 : ahead);
+      ds->arena_cur = arena_cur ^ 1;
+      ds->arena_used = 0;
+    }
+    if (targets == 0) {
+      status = ST_DONE;
       ds->passes = p;
-    } else if (p >= ds->max_passes) {
-      ds->status = ST_CAPPED;
+    } else if (p >= max_passes) {
+      status = ST_CAPPED;
       ds->passes = p;
     } else {
       ds->pass = p + 1;
       // ... and only once the jobs are long (mean arena words per survivor), where warps of one
       // block would otherwise wait on each other's merges
-      const bool to_warp = !ds->warp_on && ds->n_act < ds->warp_below &&
-                           ds->arena_used >= (unsigned long long)ds->warp_words * n_surv;
+      const bool to_warp = compact && !warp_on && n_surv < warp_below &&
+                           used >= (unsigned long long)warp_words * n_surv;
       if (to_warp) ds->warp_on = 1;
       // merge pieces over the lanes once the jobs are long enough to share them out
       const bool to_pieces =
-          ds->lane_on && ds->arena_used >= (unsigned long long)ds->lane_words * n_surv;
+          compact && lane_on && used >= (unsigned long long)lane_words * n_surv;
       if (to_pieces) ds->lane_on = 0;
-      // 8-slot warp chunks once the active list is short
-      const bool to_narrow =
-          ds->warp_on && !ds->lane_on && !ds->narrow_on && n_surv < ds->narrow_below;
+      // 8 columns per warp once the active list is short
+      const bool to_narrow = compact && (warp_on || to_warp) && ahead == 1 &&
+                             (!lane_on || to_pieces) && !narrow_on && n_surv < narrow_below;
       if (to_narrow) ds->narrow_on = 1;
       // the pass is complete, so a later call can resume from the next one
-      if (global_ns() - ds->t_start > ds->t_limit) ds->status = ST_TIMEOUT;
-      else if (to_dense || to_warp || to_pieces || to_narrow) ds->status = ST_SWITCH;
+      // (with columns ahead of the pass, it first runs on to where all are up to date)
+      const bool late = drain || global_ns() - t_start > t_limit;
+      if (late) ds->drain = 1;
+      if (late && next_compact) status = ST_TIMEOUT;
+      else if (mode != kInLoop && (to_dense || to_warp || to_pieces || to_narrow || to_add))
+        status = ST_SWITCH;
+      else if (in_graph && ahead == 1 && n_surv <= loop_below) status = ST_SWITCH;
       // counter rows for the next pass: its first kernel writes them before any capacity check
-      if (ds->status != ST_TIMEOUT && ds->stats && ds->pass >= ds->stats_rows) {
+      if (status != ST_TIMEOUT && stats && p + 1 >= stats_rows) {
         ds->host_reason = 4;
-        ds->status = ST_HOST;
+        status = ST_HOST;
       }
     }
   }
-  if (in_graph) cudaGraphSetConditional(cond, ds->status == ST_RUN ? 1u : 0u);
+  ds->status = status;
+  if (in_graph) cudaGraphSetConditional(cond, status == ST_RUN ? 1u : 0u);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1903,7 +2959,8 @@ struct InitLayout {
 // col_off: the columns of a loaded matrix (any length); null: d + 1 rows at a fixed stride
 __global__ void k_reduce_init(int64_t m, InitLayout L, int32_t* rows0,
                               const int64_t* __restrict__ col_off, ColMeta* meta, int32_t* low,
-                              int32_t* act, int32_t* alen, int32_t* owner, int32_t* tab0) {
+                              int32_t* act, int32_t* alen, int32_t* owner, unsigned long long* tab,
+                              int32_t* lows0, int32_t* due, int4* prec) {
   for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < m;
        x += (int64_t)gridDim.x * blockDim.x) {
     int d = 0;
@@ -1919,11 +2976,19 @@ __global__ void k_reduce_init(int64_t m, InitLayout L, int32_t* rows0,
     mx.low_seen = 0;
     mx.spare = 0;
     meta[x] = mx;
-    low[x] = n > 0 ? c[n - 1] : -1;  // largest row of the unreduced column
+    const int32_t l = n > 0 ? c[n - 1] : -1;  // largest row of the unreduced column
+    low[x] = l;
+    if (due) {
+      lows0[x] = l;
+      due[x] = 0;
+    }
+    if (x < L.dimoff[L.maxd]) {  // rows: no pivot yet
+      if (due) prec[x] = make_int4(0, INT32_MAX, INT32_MAX, INT32_MAX);
+      tab[x] = ~0ull;
+    }
     act[x] = (int32_t)x;
     alen[x] = n;
     owner[x] = -1;
-    tab0[x] = INT32_MAX;  // the first pass's table before its atomics: no pivot yet
   }
 }
 
@@ -1938,9 +3003,13 @@ static RArgs make_args(ph_ctx* ctx) {
   a.nxt_len = rs.nxt_len;
   a.owner = rs.owner;
   a.first_unp = rs.first_unp;
+  a.tab = rs.tab;
   a.seg = ctx->seg;
   a.rows_end = ctx->dimoff[ctx->max_dim];
   a.nseg = (int)ctx->seg_start.size() - 1;
+  a.next_unp = rs.dirty;
+  a.dirty_on = rs.dirty + a.nseg;
+  a.dirty = rs.dirty + 2 * a.nseg;
   a.nc = ctx->n_clouds;
   a.strict = ctx->opts.strict_phase2;
   a.cor10 = ctx->opts.use_cor10;
@@ -1948,6 +3017,15 @@ static RArgs make_args(ph_ctx* ctx) {
   a.look = static_cast<unsigned long long*>(rs.look);
   a.dlist = static_cast<int32_t*>(rs.dlist);
   a.src_e = static_cast<int32_t*>(rs.src_e);
+  a.lows = rs.lows;
+  a.due = rs.due;
+  a.lows_stride = std::max<int64_t>(ctx->m, 1);
+  a.ring = kAheadMax - 1;
+  a.prec = static_cast<int4*>(rs.prec);
+  a.delta = rs.delta;
+  a.kind = rs.kind;
+  a.newpos = rs.newpos;
+  a.work = rs.work;
   a.predict = ctx->opts.predict_pairs ? 1 : 0;
   a.unp_bits = rs.unp_bits;
   a.unp_words = rs.unp_words;
@@ -1978,13 +3056,22 @@ static RArgs make_args(ph_ctx* ctx) {
   return a;
 }
 
-// the additions kernel a pass runs: 1 = handles bit-packed columns (DevState::dense_on) + 2 = one
-// chunk per warp (DevState::warp_on) + 4 = each job merged by its own lane (DevState::lane_on);
-// 8 + 1 = bit-packed: 8-slot warp chunks with merge pieces (DevState::narrow_on)
+// the kernels of a pass's additions: k_add as 1 = handles bit-packed columns (DevState::dense_on) + 2
+// = one chunk per warp (DevState::warp_on) + 4 = each job merged by its own lane
+// (DevState::lane_on), 8 + 1 = bit-packed: 8-slot warp chunks with merge pieces
+// (DevState::narrow_on); or k_visit and k_merge (DevState::ahead > 1), 10 + 1 = bit-packed + 2 = each
+// job merged by its own lane
 static int add_variant(const DevState& h) {
+  if (h.ahead > 1) return 10 + (h.dense_on ? 1 : 0) + (h.lane_on ? 2 : 0);
   if (h.narrow_on) return 8 + (h.dense_on ? 1 : 0);
   return (h.dense_on ? 1 : 0) + (h.warp_on ? 2 : 0) + (h.lane_on ? 4 : 0);
 }
+static void (*const add_kernels[10])(RArgs) = {
+    k_add<false, 0, false, kPieceBlockThreads>, k_add<true, 0, false, kPieceBlockThreads>,
+    k_add<false, 32, false>, k_add<true, 32, false>, k_add<false, 0, true>, k_add<true, 0, true>,
+    k_add<false, 32, true>, k_add<true, 32, true>, k_add<false, 8, false>, k_add<true, 8, false>};
+static void (*const merge_kernels[4])(RArgs) = {k_merge<false, false>, k_merge<true, false>,
+                                                k_merge<false, true>, k_merge<true, true>};
 
 // grid of the persistent additions kernel: add_blocks_per_sm units of two 128-thread blocks per
 // SM, no more blocks than the largest active list (all m columns) can use
@@ -2065,25 +3152,25 @@ static void launch_pass_rest(ph_ctx* ctx, const RArgs& a, cudaGraphConditionalHa
     rs.ev.push_back(e1);
     PH_CUDA(cudaEventRecord(e0, st));
   }
-  static void (*const add_kernels[ReduceState::kAddVariants])(RArgs) = {
-      k_add<false, 0, false, kPieceBlockThreads>, k_add<true, 0, false, kPieceBlockThreads>,
-      k_add<false, 32, false>,
-      k_add<true, 32, false>,  k_add<false, 0, true>, k_add<true, 0, true>,
-      k_add<false, 32, true>,  k_add<true, 32, true>, k_add<false, 8, false>,
-      k_add<true, 8, false>};
   // (an event recorded between two kernels needs the first one complete: no early start then)
-  // block chunks with merge pieces (variants 0, 1) in smaller blocks, as many warps per SM
-  const int bt = variant <= 1 ? kPieceBlockThreads : kAddThreads;
-  launch_k(ctx, !time_add, add_kernels[variant], add_grid_of(ctx) * (kAddThreads / bt), bt,
-           sizeof(WarpStage) * (bt / 32), st, a);
+  if (variant >= 10) {
+    launch_k(ctx, !time_add, k_visit, add_grid_of(ctx), kAddThreads, 0, st, a);
+    launch_k(ctx, true, merge_kernels[variant - 10], add_grid_of(ctx), kAddThreads, kAddSmem, st, a);
+  } else {
+    // block chunks with merge pieces (variants 0, 1) in smaller blocks, as many warps per SM
+    const int bt = variant <= 1 ? kPieceBlockThreads : kAddThreads;
+    launch_k(ctx, !time_add, add_kernels[variant], add_grid_of(ctx) * (kAddThreads / bt), bt,
+             sizeof(WarpStage) * (bt / 32), st, a);
+  }
   if (time_add) PH_CUDA(cudaEventRecord(rs.ev.back(), st));
   launch_k(ctx, !time_add, k_commit, blocks(sms * 2, kThreads), kThreads, 0, st, a, cond,
-           in_graph ? 1 : 0);
+           in_graph ? kInGraph : kHostLoop);
 }
 
 static void launch_pass(ph_ctx* ctx, const RArgs& a, cudaGraphConditionalHandle cond,
                         bool in_graph, int variant, bool time_add, cudaStream_t st) {
-  launch_k(ctx, true, k_phase1, pass_blocks(ctx, ctx->num_sms * 8, kFTile), kThreads, 0, st, a);
+  launch_k(ctx, true, variant >= 10 ? k_phase1<true> : k_phase1<false>,
+           pass_blocks(ctx, ctx->num_sms * 8, kFTile), kThreads, 0, st, a);
   launch_pass_rest(ctx, a, cond, in_graph, variant, time_add, st);
 }
 
@@ -2115,18 +3202,37 @@ void reduce_init(ph_ctx* ctx) {
   rs.nxt_ptr = alloc_n<int32_t*>(ctx, m);
   rs.nxt_len = alloc_n<int32_t>(ctx, m);
   rs.owner = alloc_n<int32_t>(ctx, m);
-  rs.tab = alloc_n<int32_t>(ctx, 2 * std::max<int64_t>(m, 1));  // two alternating tables
+  rs.tab = alloc_n<unsigned long long>(ctx, ctx->dimoff[ctx->max_dim]);
   int nseg = (int)ctx->seg_start.size() - 1;
-  rs.first_unp = alloc_n<int32_t>(ctx, 2 * nseg);  // two copies, alternating between passes
-  PH_CUDA(cudaMemsetAsync(rs.first_unp, 0x7f, 2 * nseg * sizeof(int32_t), st));  // above every id
+  rs.first_unp = alloc_n<int32_t>(ctx, nseg);
+  PH_CUDA(cudaMemsetAsync(rs.first_unp, 0x7f, nseg * sizeof(int32_t), st));  // above every id
+  rs.dirty = alloc_n<int32_t>(ctx, 3 * nseg);  // next_unp, dirty_on, dirty
+  PH_CUDA(cudaMemsetAsync(rs.dirty, 0x7f, nseg * sizeof(int32_t), st));
+  PH_CUDA(cudaMemsetAsync(rs.dirty + nseg, 0, nseg * sizeof(int32_t), st));
   const int64_t ntiles = (m + kFTile - 1) / kFTile;
   rs.tiles_bytes = (ntiles + 1) * sizeof(unsigned long long);
   rs.tiles = ctx->dalloc(rs.tiles_bytes);
   PH_CUDA(cudaMemsetAsync(rs.tiles, 0, rs.tiles_bytes, st));  // no state published yet
-  const int64_t nchunks = (m + 7) / 8 + 1;  // chunks of any shape (8 slots or more)
+  const int64_t nchunks = (m + 7) / 8 + 1;  // chunks of any shape (8 slots or more), or tiles
   rs.look = alloc_n<unsigned long long>(ctx, nchunks);
   PH_CUDA(cudaMemsetAsync(rs.look, 0, nchunks * sizeof(unsigned long long), st));
   rs.dlist = alloc_n<int32_t>(ctx, m);
+  // look-ahead for long lists (per-pass counters, and sets chosen pass by pass, need every pass to
+  // take every column)
+  const int32_t ahead =
+      ctx->opts.collect_stats || ctx->opts.phase2_sets > 0 || !ctx->three_rows() || m < kAheadFrom
+          ? 1
+          : kAheadMax;
+  rs.prec = alloc_n<int4>(ctx, ahead > 1 ? ctx->dimoff[ctx->max_dim] : 1);
+  if (ahead > 1) {
+    rs.lows_rows = kAheadMax;
+    rs.lows = alloc_n<int32_t>(ctx, rs.lows_rows * m);
+    rs.due = alloc_n<int32_t>(ctx, m);
+    rs.delta = alloc_n<int32_t>(ctx, kDeltaRows * m + kColSlack);
+    rs.kind = alloc_n<uint8_t>(ctx, m);
+    rs.newpos = alloc_n<int32_t>(ctx, m);
+    rs.work = alloc_n<int32_t>(ctx, m);
+  }
   rs.src_e = alloc_n<int32_t>(ctx, m);
   if (ctx->opts.predict_pairs) {
     const int64_t rows = ctx->dimoff[ctx->max_dim];
@@ -2156,11 +3262,14 @@ void reduce_init(ph_ctx* ctx) {
   }
   k_reduce_init<<<grid_for(ctx, m, kThreads), kThreads, 0, st>>>(
       m, L, ctx->rows0, ctx->col_off, static_cast<ColMeta*>(rs.meta), ctx->low, rs.act,
-      rs.alen, rs.owner, rs.tab);
+      rs.alen, rs.owner, rs.tab, rs.lows, rs.due, static_cast<int4*>(rs.prec));
   PH_CHECK_LAUNCH();
-  // first arenas: pass 0 needs at most the boundary matrix twice over
-  // passes 0 and 1 need about the same; later passes less (they grow on demand otherwise)
-  const int64_t arena0 = ctx->opts.arena_words > 0 ? ctx->opts.arena_words : 2 * ctx->nnz + 1;
+  // first arenas: pass 0 needs at most the boundary matrix twice over, or once and a visit's
+  // rows per column; later passes need less (they grow on demand otherwise)
+  const int64_t n_cols = m - ctx->dimoff[1];
+  const int64_t arena0 = ctx->opts.arena_words > 0 ? ctx->opts.arena_words
+                         : ahead > 1               ? ctx->nnz + kDeltaRows * n_cols + 1
+                                                   : 2 * ctx->nnz + 1;
   grow_store(ctx, rs.arena[0], arena0);
   grow_store(ctx, rs.arena[1], arena0);
   ColStore c{};
@@ -2181,7 +3290,6 @@ void reduce_init(ph_ctx* ctx) {
   for (int i = 0; i < 2; i++) {
     h.arena[i] = rs.arena[i].p;
     h.arena_cap[i] = rs.arena[i].cap;
-    h.tab[i] = rs.tab + i * std::max<int64_t>(m, 1);
   }
   h.piv_base = c.p;
   h.piv_cap = c.cap;
@@ -2190,6 +3298,11 @@ void reduce_init(ph_ctx* ctx) {
   h.stats_rows = rs.stats_rows;
   h.pass = 0;
   h.status = ST_RUN;
+  h.ahead = ahead;
+  h.ahead_above = kAheadAbove;
+  h.horizon = ahead;
+  h.compact = 1;
+  h.arena_cur = 0;
   h.warp_below = ctx->opts.warp_chunks_below < 0   ? 0
                  : ctx->opts.warp_chunks_below == 0 ? (int64_t)1 << 22
                                                     : ctx->opts.warp_chunks_below;
@@ -2214,15 +3327,9 @@ void reduce_init(ph_ctx* ctx) {
     launch_k(ctx, false, k_tab, (unsigned)grid_for(ctx, m, kThreads * kTabItems), kThreads, 0, st,
              a0);
   }
-  const void* add_kernels[ReduceState::kAddVariants] = {
-      (const void*)k_add<false, 0, false, kPieceBlockThreads>,
-      (const void*)k_add<true, 0, false, kPieceBlockThreads>,
-      (const void*)k_add<false, 32, false>, (const void*)k_add<true, 32, false>,
-      (const void*)k_add<false, 0, true>,   (const void*)k_add<true, 0, true>,
-      (const void*)k_add<false, 32, true>,  (const void*)k_add<true, 32, true>,
-      (const void*)k_add<false, 8, false>,  (const void*)k_add<true, 8, false>};
-  for (const void* f : add_kernels)
-    PH_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kAddSmem));
+  for (auto f : merge_kernels)
+    PH_CUDA(cudaFuncSetAttribute((const void*)f, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)kAddSmem));
   rs.passes = 0;
   rs.init = true;
   rs.done = false;
@@ -2233,11 +3340,30 @@ void reduce_init(ph_ctx* ctx) {
 static void serve_host_request(ph_ctx* ctx, DevState& h) {
   ReduceState& rs = ctx->rs;
   cudaStream_t st = ctx->stream;
-  if (h.host_reason & 1) {  // the arena this pass writes into; its contents are dead
-    ColStore& s = rs.arena[h.pass & 1];
-    grow_store(ctx, s, (int64_t)h.bound_words);
-    h.arena[h.pass & 1] = s.p;
-    h.arena_cap[h.pass & 1] = s.cap;
+  // buffers retired between two compacting passes hold no column any more after the next one
+  if (h.compact) {
+    for (auto it = rs.retired.begin(); it != rs.retired.end();) {
+      if (it->until < h.pass) {
+        ctx->dfree(it->p);
+        it = rs.retired.erase(it);
+      } else {
+        ++it;
+      }
+    }
+  }
+  if (h.host_reason & 1) {  // the arena this pass writes into
+    ColStore& s = rs.arena[h.arena_cur];
+    if (h.compact) {  // its contents are dead
+      grow_store(ctx, s, (int64_t)h.bound_words);
+    } else {  // it holds columns until the next compacting pass: a further buffer beside it
+      ColStore c{};
+      grow_store(ctx, c, (int64_t)h.bound_words);
+      rs.retired.push_back({s.p, h.horizon});
+      s = c;
+      h.arena_used = 0;
+    }
+    h.arena[h.arena_cur] = s.p;
+    h.arena_cap[h.arena_cur] = s.cap;
   }
   if (h.host_reason & 2) {  // a new pivot chunk; the old ones stay (their columns live there)
     ColStore c{};
@@ -2263,6 +3389,19 @@ static void serve_host_request(ph_ctx* ctx, DevState& h) {
   h.host_reason = 0;
   h.status = ST_RUN;
 }
+
+// grid of the loop kernel: no more blocks than can be resident at once, or than the columns
+// can use (0: the device cannot run it)
+constexpr size_t kLoopSmem = sizeof(WarpStage) * kWarps;
+static unsigned loop_grid(ph_ctx* ctx) {
+  const void* kern = (const void*)k_loop;
+  PH_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLoopSmem));
+  int per_sm = 0;
+  PH_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, kLoopSmem));
+  const int64_t most = (int64_t)ctx->num_sms * per_sm;
+  return (unsigned)std::min<int64_t>(most, (ctx->m + kThreads - 1) / kThreads);
+}
+constexpr int64_t kLoopBelow = (int64_t)1 << 14;
 
 // the pass loop as one graph: a conditional while node around one pass, with one of the
 // additions kernel variants (see launch_pass)
@@ -2321,7 +3460,7 @@ int reduce_run(ph_ctx* ctx, int32_t max_passes) {
   // a resumed reduction continues after the pass that hit the previous cap
   PH_CUDA(cudaMemcpyAsync(&h, rs.dstate, sizeof(DevState), cudaMemcpyDeviceToHost, st));
   PH_CUDA(cudaStreamSynchronize(st));
-  if (h.status == ST_CAPPED) {
+  if (h.status == ST_CAPPED) {  // every column is up to date there
     h.pass = h.passes + 1;
     h.status = ST_RUN;
   } else if (h.status == ST_TIMEOUT) {  // stopped between two passes
@@ -2334,6 +3473,10 @@ int reduce_run(ph_ctx* ctx, int32_t max_passes) {
   // every pass proves or zeroes at least one column, so m + 1 passes always suffice
   h.max_passes = max_passes < 0 ? (int32_t)std::min<int64_t>(ctx->m + 1, INT32_MAX) : max_passes;
   h.blocks_done = 0;
+  h.bar_count = h.bar_gen = 0;
+  const unsigned loop_blocks = use_graph ? loop_grid(ctx) : 0;
+  h.loop_below = loop_blocks ? kLoopBelow : -1;
+  h.drain = 0;
   const int64_t limit_ms = ctx->opts.timeout_ms > 0 ? ctx->opts.timeout_ms : 60000;
   h.t_limit = (unsigned long long)limit_ms * 1000000ull;
   PH_CUDA(cudaMemcpyAsync(rs.dstate, &h, sizeof(DevState), cudaMemcpyHostToDevice, st));
@@ -2346,24 +3489,34 @@ int reduce_run(ph_ctx* ctx, int32_t max_passes) {
     const int32_t first_pass = h.pass;
     NvtxRange nvtx_range_(use_graph ? "pass loop (graph)" : "pass");
     bool ran_graph = false;
+    const int variant = add_variant(h);
     if (rest_only) {
       rest_only = false;
-      launch_pass_rest(ctx, a, 0, false, add_variant(h), time_add, st);
+      launch_pass_rest(ctx, a, 0, false, variant, time_add, st);
       if (time_add) rs.add_launches++;
+    } else if (use_graph && loop_blocks && h.ahead == 1 && h.n_act <= h.loop_below) {
+      h.loop_blocks = std::min(loop_blocks, loop_blocks_for(h.n_act));
+      PH_CUDA(cudaMemcpyAsync(&static_cast<DevState*>(rs.dstate)->loop_blocks, &h.loop_blocks,
+                              sizeof(h.loop_blocks), cudaMemcpyHostToDevice, st));
+      RArgs args = a;
+      int64_t m = ctx->m;
+      void* params[] = {&args, &m};
+      PH_CUDA(cudaLaunchCooperativeKernel((const void*)k_loop, dim3(h.loop_blocks), dim3(kThreads),
+                                          params, kLoopSmem, st));
+      PH_CHECK_LAUNCH();
     } else if (use_graph) {
       ran_graph = true;
-      const int variant = add_variant(h);
       if (!rs.graph_exec[variant]) build_graph(ctx, a, variant);
       PH_CUDA(cudaGraphLaunch(rs.graph_exec[variant], st));
     } else {
-      launch_pass(ctx, a, 0, false, add_variant(h), time_add, st);
+      launch_pass(ctx, a, 0, false, variant, time_add, st);
       if (time_add) rs.add_launches++;
     }
     PH_CUDA(cudaMemcpyAsync(&h, rs.dstate, sizeof(DevState), cudaMemcpyDeviceToHost, st));
     PH_CUDA(cudaStreamSynchronize(st));
     if (ran_graph) {  // kernels per executed pass of the graph's loop
       const int32_t last = (h.status == ST_DONE || h.status == ST_CAPPED) ? h.passes : h.pass;
-      const int per_pass = 3 + (ctx->opts.collect_stats ? 1 : 0);
+      const int per_pass = (variant >= 10 ? 4 : 3) + (ctx->opts.collect_stats ? 1 : 0);
       ctx->launches += per_pass * (int64_t)(last - first_pass + 1);
     }
     if (h.status == ST_RUN) continue;
@@ -2384,7 +3537,11 @@ int reduce_run(ph_ctx* ctx, int32_t max_passes) {
       // rows (reason 4): asked for between two passes, the next pass runs whole
       rest_only = (h.host_reason & 3) != 0;
       serve_host_request(ctx, h);
-      if (rest_only) reset_counters(&h);
+      if (rest_only) {
+        const unsigned int n_dirty = h.n_dirty;  // the marks' segments wait for the end of the pass
+        reset_counters(&h);
+        h.n_dirty = n_dirty;
+      }
       PH_CUDA(cudaMemcpyAsync(rs.dstate, &h, sizeof(DevState), cudaMemcpyHostToDevice, st));
       continue;
     }
@@ -2589,13 +3746,15 @@ void free_reduce_state(ph_ctx* ctx) {
   }
   for (void* p : {(void*)rs.act, (void*)rs.act2, (void*)rs.alen, (void*)rs.alen2, rs.meta,
                   (void*)rs.nxt_ptr, (void*)rs.nxt_len, (void*)rs.owner, (void*)rs.tab,
-                  (void*)rs.first_unp, rs.tiles, rs.dstate,
-                  rs.look, rs.dlist, rs.src_e, (void*)rs.unp_bits, (void*)rs.unp_words,
+                  (void*)rs.first_unp, (void*)rs.dirty, rs.tiles, rs.dstate,
+                  rs.look, rs.dlist, rs.src_e, (void*)rs.lows, (void*)rs.due, rs.prec,
+                  (void*)rs.delta, (void*)rs.kind, (void*)rs.newpos, (void*)rs.work, (void*)rs.unp_bits, (void*)rs.unp_words,
                   (void*)rs.pred, (void*)rs.set_n, (void*)rs.set_neg, (void*)rs.set_on,
                   (void*)rs.set_key,
                   (void*)rs.pass_stats})
     ctx->dfree(p);
   for (auto& a : rs.arena) ctx->dfree(a.p);
+  for (auto& r : rs.retired) ctx->dfree(r.p);
   for (auto& c : rs.pivots) ctx->dfree(c.p);
   if (rs.hstate) cudaFreeHost(rs.hstate);
   for (auto e : rs.ev) cudaEventDestroy(e);
