@@ -9,22 +9,67 @@
 // ---------------------------------------------------------------------------------------------
 // device memory of a context
 // ---------------------------------------------------------------------------------------------
+// Blocks of up to kKeepBlock bytes that a context is done with are kept for its next allocations
+// (kKeepTotal bytes in all), so that a program that builds and reduces small complexes again and
+// again does not go through its allocator some sixty times per call. All use is in the order of
+// the context's stream, so a kept block can be handed out at once. Blocks that no build since the
+// one before last has used go back, and all do when an allocation fails.
+constexpr size_t kKeepBlock = size_t(32) << 20, kKeepTotal = size_t(256) << 20;
+
+void ph_ctx::give_back(const Block& b) {
+  if (has_alloc) alloc.free(b.p, b.bytes, alloc.user, (void*)stream);
+  else cudaFreeAsync(b.p, stream);
+}
+
+void ph_ctx::drop_kept(int64_t before) {
+  size_t n = 0;
+  for (const Kept& k : kept) {
+    if (k.build < before) {
+      give_back(k.b);
+      kept_bytes -= k.b.bytes;
+    } else {
+      kept[n++] = k;
+    }
+  }
+  kept.resize(n);
+}
+
 void* ph_ctx::dalloc(size_t bytes) {
-  if (bytes == 0) bytes = 16;
+  bytes = bytes <= 256 ? 256 : (bytes + 255) & ~size_t(255);
+  // the smallest kept block that fits without much waste
+  size_t best = kept.size();
+  for (size_t i = 0; i < kept.size(); i++) {
+    const size_t n = kept[i].b.bytes;
+    if (n >= bytes && n <= 2 * bytes + 65536 && (best == kept.size() || n < kept[best].b.bytes))
+      best = i;
+  }
+  if (best < kept.size()) {
+    const Block b = kept[best].b;
+    kept_bytes -= b.bytes;
+    kept[best] = kept.back();
+    kept.pop_back();
+    blocks.push_back(b);
+    return b.p;
+  }
   void* p = nullptr;
-  if (has_alloc) {
-    p = alloc.alloc(bytes, alloc.user, (void*)stream);
-  } else if (cudaMallocAsync(&p, bytes, stream) != cudaSuccess) {
-    cudaGetLastError();
-    p = nullptr;
+  for (int attempt = 0; attempt < 2 && !p; attempt++) {
+    if (attempt > 0) {  // make room
+      if (kept.empty()) break;
+      drop_kept(INT64_MAX);
+    }
+    if (has_alloc) {
+      p = alloc.alloc(bytes, alloc.user, (void*)stream);
+    } else if (cudaMallocAsync(&p, bytes, stream) != cudaSuccess) {
+      cudaGetLastError();
+      p = nullptr;
+    }
   }
   if (!p) {
     err = "device allocation of " + std::to_string(bytes) + " bytes failed";
     throw ph::Fail{PH_ERR_ALLOC};
   }
   if (reinterpret_cast<uintptr_t>(p) % 256 != 0) {  // the kernels copy in 16-byte units
-    if (has_alloc) alloc.free(p, bytes, alloc.user, (void*)stream);
-    else cudaFreeAsync(p, stream);
+    give_back({p, bytes});
     err = "the device allocator returned memory that is not 256-byte aligned";
     throw ph::Fail{PH_ERR_ALLOC};
   }
@@ -32,25 +77,49 @@ void* ph_ctx::dalloc(size_t bytes) {
   return p;
 }
 
+void ph_ctx::keep_or_give_back(const Block& b) {
+  if (b.bytes <= kKeepBlock && kept_bytes + b.bytes <= kKeepTotal) {
+    kept.push_back({b, builds});
+    kept_bytes += b.bytes;
+  } else {
+    give_back(b);
+  }
+}
+
 void ph_ctx::dfree(void* p) {
   if (!p) return;
-  for (size_t i = 0; i < blocks.size(); i++) {
+  for (size_t i = blocks.size(); i-- > 0;) {
     if (blocks[i].p == p) {
-      if (has_alloc) alloc.free(p, blocks[i].bytes, alloc.user, (void*)stream);
-      else cudaFreeAsync(p, stream);
+      const Block b = blocks[i];
       blocks[i] = blocks.back();
       blocks.pop_back();
+      keep_or_give_back(b);
       return;
     }
   }
 }
 
+void* ph_ctx::pinned(size_t bytes) {
+  if (bytes > h_pinned_bytes) {
+    if (h_pinned) cudaFreeHost(h_pinned);
+    h_pinned = nullptr;
+    h_pinned_bytes = 0;
+    if (cudaMallocHost(&h_pinned, bytes) != cudaSuccess) {
+      cudaGetLastError();
+      h_pinned = nullptr;
+      err = "page-locked host allocation failed";
+      throw ph::Fail{PH_ERR_ALLOC};
+    }
+    h_pinned_bytes = bytes;
+  }
+  return h_pinned;
+}
+
 void ph_ctx::free_all() {
   ph::free_reduce_state(this);
-  for (auto& b : blocks) {
-    if (has_alloc) alloc.free(b.p, b.bytes, alloc.user, (void*)stream);
-    else cudaFreeAsync(b.p, stream);
-  }
+  builds++;
+  drop_kept(builds - 1);
+  for (auto& b : blocks) keep_or_give_back(b);
   blocks.clear();
   built = reduced = extracted = is_vr = false;
   // every pointer into the freed blocks must go: a stale one handed to dfree later could match
@@ -328,6 +397,10 @@ void ph_destroy(ph_ctx* ctx) {
   if (!ctx) return;
   cudaStreamSynchronize(ctx->stream);
   ctx->free_all();
+  ctx->drop_kept(INT64_MAX);
+  ph::free_graphs(ctx);
+  if (ctx->rs.hstate) cudaFreeHost(ctx->rs.hstate);
+  if (ctx->h_pinned) cudaFreeHost(ctx->h_pinned);
   cudaStreamSynchronize(ctx->stream);
   delete ctx;
 }

@@ -618,7 +618,9 @@ void build_vr(ph_ctx* ctx, const int32_t* coords, const int64_t* cloud_offsets, 
     k_pairwise<<<g, kThreads, 0, st>>>(coords, D, ct, d2, (unsigned long long*)(d_misc + 1));
     PH_CHECK_LAUNCH();
   }
-  int64_t h_misc[2];
+  // page-locked scratch: status words and per-cloud counts come back through it
+  int64_t* h_misc = static_cast<int64_t*>(
+      ctx->pinned((2 + (int64_t)kMaxVrDim * nc) * sizeof(int64_t)));
   PH_CUDA(cudaMemcpyAsync(h_misc, d_misc, 2 * sizeof(int64_t), cudaMemcpyDeviceToHost, st));
   PH_CUDA(cudaStreamSynchronize(st));
   PH_REQUIRE(h_misc[0] == 0, PH_ERR_INVALID, "coordinates must lie in [-2^24, 2^24] grid units");
@@ -656,10 +658,9 @@ void build_vr(ph_ctx* ctx, const int32_t* coords, const int64_t* cloud_offsets, 
       radix_sort_u64(ctx, kbuf, vbuf, cand[2][nc], 0, bitlen((uint64_t)nc), ktmp, vtmp);
     }
   }
-  PH_CUDA(cudaMemcpyAsync(h_cnt.data(), cnt_dim(1), nc * sizeof(int64_t), cudaMemcpyDeviceToHost,
-                          st));
+  PH_CUDA(cudaMemcpyAsync(h_misc, cnt_dim(1), nc * sizeof(int64_t), cudaMemcpyDeviceToHost, st));
   PH_CUDA(cudaStreamSynchronize(st));
-  for (int c = 0; c < nc; c++) cnts[1] += h_cnt[c];
+  for (int c = 0; c < nc; c++) cnts[1] += h_cnt[c] = h_misc[c];
   const int64_t E = cnts[1];
 
   // sizes known for dims 0, 1; ids and initial storage for those two now, higher dims after
@@ -693,8 +694,9 @@ void build_vr(ph_ctx* ctx, const int32_t* coords, const int64_t* cloud_offsets, 
     k_edge_finish<<<grid_for(ctx, E, kThreads), kThreads, 0, st>>>(
         vbuf, E, ct, flag, excl, ed2, N, eid, erank, ctx->d2tab, o, 0);
     PH_CHECK_LAUNCH();
-    PH_CUDA(cudaMemcpyAsync(&n_d2, d_nd2, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
+    PH_CUDA(cudaMemcpyAsync(h_misc, d_nd2, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
     PH_CUDA(cudaStreamSynchronize(st));
+    n_d2 = h_misc[0];
     ctx->dfree(flag);
     ctx->dfree(excl);
     ctx->dfree(ed2);
@@ -721,10 +723,10 @@ void build_vr(ph_ctx* ctx, const int32_t* coords, const int64_t* cloud_offsets, 
           ct, d_cand(k), cand[k][nc], k, erank, (uint64_t)n_d2, kbuf, vbuf, cnt_dim(d));
       PH_CHECK_LAUNCH();
       radix_sort_u64(ctx, kbuf, vbuf, cand[k][nc], 0, rbits, ktmp, vtmp);
-      PH_CUDA(cudaMemcpyAsync(h_cnt.data() + (int64_t)(d - 1) * nc, cnt_dim(d),
-                              nc * sizeof(int64_t), cudaMemcpyDeviceToHost, st));
+      PH_CUDA(cudaMemcpyAsync(h_misc, cnt_dim(d), nc * sizeof(int64_t), cudaMemcpyDeviceToHost,
+                              st));
       PH_CUDA(cudaStreamSynchronize(st));
-      for (int c = 0; c < nc; c++) Q += h_cnt[(int64_t)(d - 1) * nc + c];
+      for (int c = 0; c < nc; c++) Q += h_cnt[(int64_t)(d - 1) * nc + c] = h_misc[c];
     }
     if (Q > 0) {
       if (k == 3) {

@@ -131,10 +131,15 @@ struct ReduceState {
   std::vector<Retired> retired;  // arena buffers outgrown between two compacting passes
   std::vector<ColStore> pivots;  // chunks holding proven columns
   // the pass loop: one pass as the body of a conditional while node, per variant of its additions
-  // (add_variant)
+  // (add_variant), with the arguments it was made with; a graph outlives the reduction and runs
+  // again while another one's arguments are the same (a context that builds complexes of one
+  // size again and again)
   static constexpr int kAddVariants = 14;
-  cudaGraph_t graph[kAddVariants] = {};
-  cudaGraphExec_t graph_exec[kAddVariants] = {};
+  struct Loop {
+    cudaGraph_t graph = nullptr;
+    cudaGraphExec_t exec = nullptr;
+    std::vector<unsigned char> args;
+  };
   int32_t passes = 0;
   bool init = false;
   bool done = false;
@@ -155,6 +160,8 @@ struct ph_ctx {
   ph_opts opts{};
   ph_allocator alloc{};
   bool has_alloc = false;
+  ph::ReduceState::Loop loops[ph::ReduceState::kAddVariants];
+  int loop_blocks_per_sm = -1;  // resident blocks of the loop kernel (-1: not asked yet)
   std::string err;
   int64_t launches = 0;  // kernels launched by this context
 
@@ -162,7 +169,16 @@ struct ph_ctx {
     void* p;
     size_t bytes;
   };
-  std::vector<Block> blocks;  // every device allocation of the context
+  std::vector<Block> blocks;  // every device allocation of the context that is in use
+  struct Kept {
+    Block b;
+    int64_t build;  // the build during which it was last in use
+  };
+  std::vector<Kept> kept;  // ... and the small ones kept for the next allocations
+  size_t kept_bytes = 0;
+  int64_t builds = 0;      // filtrations built or loaded
+  void* h_pinned = nullptr;  // page-locked host scratch
+  size_t h_pinned_bytes = 0;
 
   // filtration
   bool built = false;
@@ -208,6 +224,10 @@ struct ph_ctx {
 
   void* dalloc(size_t bytes);
   void dfree(void* p);
+  void give_back(const Block& b);
+  void keep_or_give_back(const Block& b);
+  void drop_kept(int64_t before);
+  void* pinned(size_t bytes);  // at least this many bytes; a later call may move it
   void free_all();
 };
 
@@ -355,6 +375,7 @@ void reduce_init(ph_ctx* ctx);
 int reduce_run(ph_ctx* ctx, int32_t max_passes);
 void extract_all(ph_ctx* ctx);
 void free_reduce_state(ph_ctx* ctx);
+void free_graphs(ph_ctx* ctx);
 // E^l of one cloud, one byte per simplex in filtration order, into host memory (n bytes)
 void essential_estimate(ph_ctx* ctx, int32_t cloud, uint8_t* host_out, int64_t n);
 // predicted lowstar per simplex of one cloud (filtration indices, -1), into host memory

@@ -42,6 +42,7 @@
 // from a host loop or as the body of a graph's conditional while node. Each kernel may start
 // while its predecessor drains (programmatic dependent launch) and waits for it first.
 #include <algorithm>
+#include <cstring>
 #include <utility>
 
 #include "ph_internal.cuh"
@@ -2994,7 +2995,8 @@ __global__ void k_reduce_init(int64_t m, InitLayout L, int32_t* rows0,
 
 static RArgs make_args(ph_ctx* ctx) {
   ReduceState& rs = ctx->rs;
-  RArgs a{};
+  RArgs a;
+  std::memset(&a, 0, sizeof(a));  // (whole: pass_graph compares the bytes)
   a.ds = static_cast<DevState*>(rs.dstate);
   a.low = ctx->low;
   a.beta = ctx->beta;
@@ -3250,7 +3252,7 @@ void reduce_init(ph_ctx* ctx) {
     rs.set_key = alloc_n<uint64_t>(ctx, 4 * rows);
   }
   rs.dstate = ctx->dalloc(sizeof(DevState));
-  PH_CUDA(cudaMallocHost(&rs.hstate, sizeof(DevState)));
+  if (!rs.hstate) PH_CUDA(cudaMallocHost(&rs.hstate, sizeof(DevState)));  // kept by the context
   rs.h_stats.clear();
   InitLayout L{};
   L.maxd = ctx->max_dim;
@@ -3327,9 +3329,6 @@ void reduce_init(ph_ctx* ctx) {
     launch_k(ctx, false, k_tab, (unsigned)grid_for(ctx, m, kThreads * kTabItems), kThreads, 0, st,
              a0);
   }
-  for (auto f : merge_kernels)
-    PH_CUDA(cudaFuncSetAttribute((const void*)f, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)kAddSmem));
   rs.passes = 0;
   rs.init = true;
   rs.done = false;
@@ -3393,20 +3392,35 @@ static void serve_host_request(ph_ctx* ctx, DevState& h) {
 // grid of the loop kernel: no more blocks than can be resident at once, or than the columns
 // can use (0: the device cannot run it)
 constexpr size_t kLoopSmem = sizeof(WarpStage) * kWarps;
+static_assert(kAddSmem <= 48 * 1024 && kLoopSmem <= 48 * 1024, "above, kernels must opt in");
 static unsigned loop_grid(ph_ctx* ctx) {
-  const void* kern = (const void*)k_loop;
-  PH_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLoopSmem));
-  int per_sm = 0;
-  PH_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, kLoopSmem));
-  const int64_t most = (int64_t)ctx->num_sms * per_sm;
+  if (ctx->loop_blocks_per_sm < 0)  // asked once per context
+    PH_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctx->loop_blocks_per_sm, k_loop, kThreads,
+                                                          kLoopSmem));
+  const int64_t most = (int64_t)ctx->num_sms * ctx->loop_blocks_per_sm;
   return (unsigned)std::min<int64_t>(most, (ctx->m + kThreads - 1) / kThreads);
 }
 constexpr int64_t kLoopBelow = (int64_t)1 << 14;
 
 // the pass loop as one graph: a conditional while node around one pass, with one of the
 // additions kernel variants (see launch_pass)
-static void build_graph(ph_ctx* ctx, const RArgs& a, int variant) {
-  ReduceState& rs = ctx->rs;
+static void free_loop(ReduceState::Loop& l) {
+  if (l.exec) cudaGraphExecDestroy(l.exec);
+  if (l.graph) cudaGraphDestroy(l.graph);
+  l = ReduceState::Loop{};
+}
+void free_graphs(ph_ctx* ctx) {
+  for (auto& l : ctx->loops) free_loop(l);
+}
+
+static cudaGraphExec_t pass_graph(ph_ctx* ctx, const RArgs& a, int variant) {
+  // everything the graph's kernels and grids depend on besides the context's options
+  ReduceState::Loop& loop = ctx->loops[variant];
+  std::vector<unsigned char> args(sizeof(RArgs) + sizeof(int64_t));
+  std::memcpy(args.data(), &a, sizeof(RArgs));
+  std::memcpy(args.data() + sizeof(RArgs), &ctx->m, sizeof(int64_t));
+  if (loop.exec && loop.args == args) return loop.exec;
+  free_loop(loop);
   cudaGraph_t g;
   PH_CUDA(cudaGraphCreate(&g, 0));
   cudaGraphConditionalHandle cond;
@@ -3444,10 +3458,10 @@ static void build_graph(ph_ctx* ctx, const RArgs& a, int variant) {
   cudaStreamDestroy(cs);
   if (ce != cudaSuccess) cudaGraphDestroy(g);
   PH_CUDA(ce);
-  cudaGraphExec_t exec;
-  PH_CUDA(cudaGraphInstantiate(&exec, g, 0));
-  rs.graph[variant] = g;
-  rs.graph_exec[variant] = exec;
+  loop.graph = g;  // (freed with the loop, also when the next call fails)
+  PH_CUDA(cudaGraphInstantiate(&loop.exec, g, 0));
+  loop.args = std::move(args);
+  return loop.exec;
 }
 
 int reduce_run(ph_ctx* ctx, int32_t max_passes) {
@@ -3506,8 +3520,7 @@ int reduce_run(ph_ctx* ctx, int32_t max_passes) {
       PH_CHECK_LAUNCH();
     } else if (use_graph) {
       ran_graph = true;
-      if (!rs.graph_exec[variant]) build_graph(ctx, a, variant);
-      PH_CUDA(cudaGraphLaunch(rs.graph_exec[variant], st));
+      PH_CUDA(cudaGraphLaunch(pass_graph(ctx, a, variant), st));
     } else {
       launch_pass(ctx, a, 0, false, variant, time_add, st);
       if (time_add) rs.add_launches++;
@@ -3740,15 +3753,12 @@ void reduced_columns(ph_ctx* ctx, int32_t cloud, int64_t n, int64_t* colptr, int
 
 void free_reduce_state(ph_ctx* ctx) {
   ReduceState& rs = ctx->rs;
-  for (int d = 0; d < ReduceState::kAddVariants; d++) {
-    if (rs.graph_exec[d]) cudaGraphExecDestroy(rs.graph_exec[d]);
-    if (rs.graph[d]) cudaGraphDestroy(rs.graph[d]);
-  }
   for (void* p : {(void*)rs.act, (void*)rs.act2, (void*)rs.alen, (void*)rs.alen2, rs.meta,
                   (void*)rs.nxt_ptr, (void*)rs.nxt_len, (void*)rs.owner, (void*)rs.tab,
                   (void*)rs.first_unp, (void*)rs.dirty, rs.tiles, rs.dstate,
                   rs.look, rs.dlist, rs.src_e, (void*)rs.lows, (void*)rs.due, rs.prec,
-                  (void*)rs.delta, (void*)rs.kind, (void*)rs.newpos, (void*)rs.work, (void*)rs.unp_bits, (void*)rs.unp_words,
+                  (void*)rs.delta, (void*)rs.kind, (void*)rs.newpos, (void*)rs.work,
+                  (void*)rs.unp_bits, (void*)rs.unp_words,
                   (void*)rs.pred, (void*)rs.set_n, (void*)rs.set_neg, (void*)rs.set_on,
                   (void*)rs.set_key,
                   (void*)rs.pass_stats})
@@ -3756,9 +3766,10 @@ void free_reduce_state(ph_ctx* ctx) {
   for (auto& a : rs.arena) ctx->dfree(a.p);
   for (auto& r : rs.retired) ctx->dfree(r.p);
   for (auto& c : rs.pivots) ctx->dfree(c.p);
-  if (rs.hstate) cudaFreeHost(rs.hstate);
   for (auto e : rs.ev) cudaEventDestroy(e);
+  void* hstate = rs.hstate;  // (page-locked: kept by the context)
   rs = ReduceState{};
+  rs.hstate = hstate;
 }
 
 }  // namespace ph
