@@ -385,5 +385,7 @@ void reduced_columns(ph_ctx* ctx, int32_t cloud, int64_t n, int64_t* colptr, int
 // generic device helpers (ph_scan.cu)
 void excl_scan_i64(ph_ctx* ctx, const int64_t* in, int64_t* out, int64_t n, int64_t* total_dev);
 void radix_sort_u64(ph_ctx* ctx, uint64_t* keys, uint64_t* vals, int64_t n, int lo_bit,
-                    int hi_bit, uint64_t* tmp_keys, uint64_t* tmp_vals);
+                    int hi_bit, uint64_t* tmp_keys, uint64_t* tmp_vals, int32_t* fault);
+void scan_counts(ph_ctx* ctx, const int32_t* a, const int32_t* b, int64_t n, int64_t* oa,
+                 int64_t* ob, int32_t* fault);
 }  // namespace ph

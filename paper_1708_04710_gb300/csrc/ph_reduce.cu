@@ -3134,12 +3134,14 @@ static void launch_pass_rest(ph_ctx* ctx, const RArgs& a, cudaGraphConditionalHa
     uint64_t* row = rs.set_key + rows;
     k_set_tiekeys<<<grid_for(ctx, rows, kThreads), kThreads, 0, st>>>(a, ctx->gidx, key, row);
     PH_CHECK_LAUNCH();
-    radix_sort_u64(ctx, key, row, rows, 0, bits, rs.set_key + 2 * rows, rs.set_key + 3 * rows);
+    int32_t* fault = &static_cast<DevState*>(rs.dstate)->fault;
+    radix_sort_u64(ctx, key, row, rows, 0, bits, rs.set_key + 2 * rows, rs.set_key + 3 * rows,
+                   fault);
     k_set_keys<<<grid_for(ctx, rows, kThreads), kThreads, 0, st>>>(
         a, ctx->opts.phase2_priority, bits, key, row);
     PH_CHECK_LAUNCH();
     radix_sort_u64(ctx, key, row, rows, 0, ctx->opts.phase2_priority == 1 ? 2 * bits : bits,
-                   rs.set_key + 2 * rows, rs.set_key + 3 * rows);
+                   rs.set_key + 2 * rows, rs.set_key + 3 * rows, fault);
     const int64_t p = std::min<int64_t>(ctx->opts.phase2_sets, rows);
     k_set_select<<<grid_for(ctx, p, kThreads), kThreads, 0, st>>>(a, p, row);
     PH_CHECK_LAUNCH();

@@ -1,8 +1,11 @@
 // Device scans and the LSD radix sort used to order simplices by squared diameter.
 //
 // Both are tile based: a tile is kThreads * kItems consecutive elements handled by one block.
-// (1) per-tile reduction, (2) one block scans the tile aggregates, (3) per-tile scan with the
-// tile's prefix. No kernel waits on another block, so nothing here can spin.
+// excl_scan_i64: (1) per-tile reduction, (2) one block scans the tile aggregates, (3) per-tile scan
+// with the tile's prefix. The others take one kernel, whose tiles wait for earlier ones (in order,
+// with a bound).
+#include <utility>
+
 #include "ph_internal.cuh"
 
 namespace ph {
@@ -73,98 +76,282 @@ void excl_scan_i64(ph_ctx* ctx, const int64_t* in, int64_t* out, int64_t n, int6
 }
 
 // ---------------------------------------------------------------------------------------------
-// LSD radix sort of (uint64 key, uint64 value) pairs by key bits [lo_bit, hi_bit), stable.
-// 8-bit digits. Histograms are digit-major ([256][ntiles]) so that one exclusive scan over
-// them gives every tile's output offset per digit.
+// exclusive scans of one or two int32 arrays into int64 (n + 1 values each, the total last), in one
+// kernel: tiles in order from a ticket, each publishing its sum and looking back over the tiles
+// before it (decoupled look-back). state: per array one word per tile, zeroed before
 // ---------------------------------------------------------------------------------------------
-__global__ void k_radix_hist(const uint64_t* __restrict__ keys, int64_t n, int shift,
-                             int64_t ntiles, int64_t* hist) {
-  __shared__ unsigned cnt[256];
-  cnt[threadIdx.x] = 0;
-  __syncthreads();
-  int64_t base = (int64_t)blockIdx.x * kTile;
-  for (int it = 0; it < kItems; it++) {
-    int64_t i = base + it * kThreads + threadIdx.x;
-    if (i < n) atomicAdd(&cnt[(keys[i] >> shift) & 255u], 1u);
+constexpr unsigned long long kAgg = 1ull << 62, kIncl = 2ull << 62, kFlags = 3ull << 62;
+constexpr int kWaitLimit = 1 << 22;  // polls of a look-back before it gives up (and reports it)
+
+// waits for a state word's flags; 0 (and *fault set) if they never come
+__device__ __forceinline__ unsigned long long wait_state(const unsigned long long* p,
+                                                         int32_t* fault) {
+  for (int it = 0; it < kWaitLimit; it++) {
+    const unsigned long long w = *(const volatile unsigned long long*)p;
+    if (w & kFlags) return w;
+    __nanosleep(20);
   }
-  __syncthreads();
-  hist[(int64_t)threadIdx.x * ntiles + blockIdx.x] = cnt[threadIdx.x];
+  *fault = 1;
+  return kIncl;
 }
 
-__global__ void k_radix_scatter(const uint64_t* __restrict__ kin, const uint64_t* __restrict__ vin,
-                                uint64_t* __restrict__ kout, uint64_t* __restrict__ vout,
-                                int64_t n, int shift, int64_t ntiles,
-                                const int64_t* __restrict__ offs) {
+// by one warp: the sum of the tiles before t, whose own sum is agg; publishes t's states
+__device__ __forceinline__ int64_t tile_prefix(unsigned long long* st, int64_t t, int64_t agg,
+                                               int32_t* fault) {
+  const int lane = lane_id();
+  if (lane == 0) atomicExch(st + t, (t == 0 ? kIncl : kAgg) | (unsigned long long)agg);
+  if (t == 0) return 0;
+  int64_t prefix = 0;
+  for (int64_t p = t - 1;; p -= 32) {
+    const unsigned long long w = p - lane >= 0 ? wait_state(st + p - lane, fault) : kIncl;
+    const unsigned im = __ballot_sync(0xffffffffu, (w & kFlags) == kIncl);
+    const int stop = im ? __ffs(im) - 1 : 32;
+    const int64_t val = lane <= stop ? (int64_t)(w & ~kFlags) : 0;
+    prefix += __shfl_sync(0xffffffffu, warp_incl_sum(val), 31);
+    if (im) break;
+  }
+  if (lane == 0) atomicExch(st + t, kIncl | (unsigned long long)(prefix + agg));
+  return prefix;
+}
+
+__global__ void k_scan_counts(const int32_t* __restrict__ a, const int32_t* __restrict__ b, int64_t n,
+                              int64_t* oa, int64_t* ob, unsigned long long* state,
+                              int64_t ntiles, unsigned int* ticket, int32_t* fault) {
+  __shared__ int64_t sh[kWarps + 1];
+  __shared__ int64_t s_prefix[2];
+  __shared__ unsigned int s_tile;
+  if (threadIdx.x == 0) s_tile = atomicAdd(ticket, 1u);
+  __syncthreads();
+  const int64_t t = s_tile;
+  const int64_t i0 = t * kTile + threadIdx.x * kItems;
+  for (int k = 0; k < (b ? 2 : 1); k++) {
+    const int32_t* in = k ? b : a;
+    int64_t* out = k ? ob : oa;
+    int32_t x[kItems];
+    int64_t sum = 0;
+#pragma unroll
+    for (int i = 0; i < kItems; i++) {
+      x[i] = i0 + i < n ? in[i0 + i] : 0;
+      sum += x[i];
+    }
+    int64_t tot;
+    int64_t run = block_excl_sum<int64_t>(sum, sh, tot);
+    if (threadIdx.x < 32) {
+      const int64_t p = tile_prefix(state + k * ntiles, t, tot, fault);
+      if (threadIdx.x == 0) s_prefix[k] = p;
+    }
+    __syncthreads();
+    run += s_prefix[k];
+#pragma unroll
+    for (int i = 0; i < kItems; i++) {
+      if (i0 + i < n) out[i0 + i] = run;
+      run += x[i];
+      if (i0 + i == n - 1) out[n] = run;
+    }
+  }
+}
+
+// a (and b, unless null): n counts each; n >= 1. fault: set when a bounded wait ran out
+void scan_counts(ph_ctx* ctx, const int32_t* a, const int32_t* b, int64_t n, int64_t* oa,
+                 int64_t* ob, int32_t* fault) {
+  const int64_t ntiles = (n + kTile - 1) / kTile;
+  unsigned long long* state = alloc_n<unsigned long long>(ctx, 2 * ntiles + 1);
+  PH_CUDA(cudaMemsetAsync(state, 0, (2 * ntiles + 1) * sizeof(unsigned long long), ctx->stream));
+  k_scan_counts<<<(unsigned)ntiles, kThreads, 0, ctx->stream>>>(
+      a, b, n, oa, ob, state, ntiles, (unsigned int*)(state + 2 * ntiles), fault);
+  PH_CHECK_LAUNCH();
+  ctx->dfree(state);
+}
+
+// ---------------------------------------------------------------------------------------------
+// LSD radix sort of (uint64 key, uint64 value) pairs by key bits [lo_bit, hi_bit), stable.
+// 8-bit digits, one kernel per digit: a tile ranks its elements per digit value in shared memory,
+// publishes its 256 counts and looks back for those of the tiles before it, one thread per
+// digit value, and scatters. One kernel before them counts every digit over all keys. A sort of
+// one tile is a single kernel. Bound by the scattered 16-byte writes; against separate count, scan and
+// scatter kernels per digit it reads the keys once less per digit and a small sort of five digits
+// is 1 launch instead of 25 (the build of 15 points to dimension 5, seven sorts: 540 -> 330 us).
+// ---------------------------------------------------------------------------------------------
+constexpr int kMaxDigits = 8;
+
+__global__ void k_radix_count(const uint64_t* __restrict__ keys, int64_t n, int lo_bit, int digits,
+                              unsigned long long* hist) {
+  __shared__ unsigned cnt[kMaxDigits][256];
+  for (int d = 0; d < digits; d++) cnt[d][threadIdx.x] = 0;
+  __syncthreads();
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    const uint64_t k = keys[i] >> lo_bit;
+    for (int d = 0; d < digits; d++) atomicAdd(&cnt[d][(k >> (8 * d)) & 255u], 1u);
+  }
+  __syncthreads();
+  for (int d = 0; d < digits; d++)
+    if (cnt[d][threadIdx.x])
+      atomicAdd(&hist[d * 256 + threadIdx.x], (unsigned long long)cnt[d][threadIdx.x]);
+}
+
+// Ranks of a tile's elements: element i of a thread is the tile's element warp * 256 + 32 i + lane.
+// cnt[w][d] becomes the number of the tile's elements with digit d in warps before w; returns this
+// thread's digit value's (threadIdx.x) number in the tile.
+__device__ __forceinline__ unsigned tile_ranks(const unsigned (&digit)[kItems],
+                                               unsigned (&rank)[kItems],
+                                               unsigned (*cnt)[257]) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  for (int d = lane; d < 257; d += 32) cnt[w][d] = 0;
+  __syncwarp();
+#pragma unroll
+  for (int i = 0; i < kItems; i++) {
+    const unsigned peers = __match_any_sync(0xffffffffu, digit[i]);
+    const unsigned old = cnt[w][digit[i]];
+    rank[i] = old + __popc(peers & ((1u << lane) - 1u));
+    __syncwarp();
+    if (lane == __ffs(peers) - 1) cnt[w][digit[i]] = old + __popc(peers);
+    __syncwarp();
+  }
+  __syncthreads();
+  unsigned run = 0;
+#pragma unroll
+  for (int v = 0; v < kWarps; v++) {
+    const unsigned c = cnt[v][threadIdx.x];
+    cnt[v][threadIdx.x] = run;
+    run += c;
+  }
+  return run;
+}
+
+__global__ void __launch_bounds__(kThreads) k_radix_pass(
+    const uint64_t* __restrict__ kin, const uint64_t* __restrict__ vin,
+    uint64_t* __restrict__ kout, uint64_t* __restrict__ vout, int64_t n, int shift,
+    const unsigned long long* __restrict__ hist, unsigned long long* state, unsigned int* ticket,
+    int32_t* fault) {
+  __shared__ unsigned cnt[kWarps][257];
   __shared__ int64_t base[256];
-  __shared__ unsigned wcnt[kWarps][256];
-  __shared__ unsigned tot[256];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  base[tid] = offs[(int64_t)tid * ntiles + blockIdx.x];
-#pragma unroll
-  for (int w = 0; w < kWarps; w++) wcnt[w][tid] = 0;
+  __shared__ int64_t sh[kWarps + 1];
+  __shared__ unsigned int s_tile;
+  if (threadIdx.x == 0) s_tile = atomicAdd(ticket, 1u);  // tiles in order: the look-back waits
   __syncthreads();
-  const int64_t tile0 = (int64_t)blockIdx.x * kTile;
-  for (int it = 0; it < kItems; it++) {
-    int64_t i = tile0 + it * kThreads + tid;
-    bool valid = i < n;
-    uint64_t k = valid ? kin[i] : 0, v = valid ? vin[i] : 0;
-    unsigned d = valid ? (unsigned)((k >> shift) & 255u) : 256u;
-    unsigned peers = __match_any_sync(0xffffffffu, d);
-    unsigned rank = __popc(peers & ((1u << lane) - 1u));
-    if (valid && lane == __ffs(peers) - 1) wcnt[warp][d] = __popc(peers);
-    __syncthreads();
-    unsigned run = 0;
+  const int64_t t = s_tile;
+  const int64_t i0 = t * kTile + (threadIdx.x >> 5) * (32 * kItems) + (threadIdx.x & 31);
+  uint64_t k[kItems], v[kItems];
+  unsigned digit[kItems], rank[kItems];
 #pragma unroll
-    for (int w = 0; w < kWarps; w++) {
-      unsigned c = wcnt[w][tid];
-      wcnt[w][tid] = run;
-      run += c;
+  for (int i = 0; i < kItems; i++) {
+    const bool in = i0 + 32 * i < n;
+    k[i] = in ? kin[i0 + 32 * i] : 0;
+    v[i] = in ? vin[i0 + 32 * i] : 0;
+    digit[i] = in ? (unsigned)((k[i] >> shift) & 255u) : 256u;
+  }
+  const unsigned mine = tile_ranks(digit, rank, cnt);
+  int64_t tot;
+  int64_t b = block_excl_sum<int64_t>((int64_t)hist[threadIdx.x], sh, tot);
+  unsigned long long* st = state + t * 256 + threadIdx.x;
+  atomicExch(st, (t == 0 ? kIncl : kAgg) | mine);
+  if (t > 0) {
+    int64_t prefix = 0;
+    for (const unsigned long long* p = st - 256;; p -= 256) {
+      const unsigned long long w = wait_state(p, fault);
+      prefix += (int64_t)(w & ~kFlags);
+      if ((w & kFlags) == kIncl) break;
     }
-    tot[tid] = run;
-    __syncthreads();
-    if (valid) {
-      int64_t pos = base[d] + wcnt[warp][d] + rank;
-      kout[pos] = k;
-      vout[pos] = v;
-    }
-    __syncthreads();
-    base[tid] += tot[tid];
+    atomicExch(st, kIncl | (unsigned long long)(prefix + mine));
+    b += prefix;
+  }
+  base[threadIdx.x] = b;
+  __syncthreads();
 #pragma unroll
-    for (int w = 0; w < kWarps; w++) wcnt[w][tid] = 0;
-    __syncthreads();
+  for (int i = 0; i < kItems; i++) {
+    if (digit[i] == 256u) continue;
+    const int64_t pos = base[digit[i]] + cnt[threadIdx.x >> 5][digit[i]] + rank[i];
+    if (pos >= n) continue;  // (only after a wait that gave up)
+    kout[pos] = k[i];
+    vout[pos] = v[i];
   }
 }
 
+// one tile, all digits: elements stay in registers and change places in shared memory
+__global__ void __launch_bounds__(kThreads) k_radix_tile(uint64_t* keys, uint64_t* vals, int n,
+                                                         int lo_bit, int digits) {
+  __shared__ unsigned cnt[kWarps][257];
+  __shared__ int64_t sh[kWarps + 1];
+  __shared__ unsigned base[256];
+  __shared__ uint64_t xk[kTile];
+  __shared__ uint64_t xv[kTile];
+  const int i0 = (threadIdx.x >> 5) * (32 * kItems) + (threadIdx.x & 31);
+  uint64_t k[kItems], v[kItems];
+  unsigned digit[kItems], rank[kItems];
+#pragma unroll
+  for (int i = 0; i < kItems; i++) {
+    k[i] = i0 + 32 * i < n ? keys[i0 + 32 * i] : 0;
+    v[i] = i0 + 32 * i < n ? vals[i0 + 32 * i] : 0;
+  }
+  for (int p = 0; p < digits; p++) {
+#pragma unroll
+    for (int i = 0; i < kItems; i++)
+      digit[i] = i0 + 32 * i < n ? (unsigned)((k[i] >> (lo_bit + 8 * p)) & 255u) : 256u;
+    const unsigned mine = tile_ranks(digit, rank, cnt);
+    int64_t tot;
+    base[threadIdx.x] = (unsigned)block_excl_sum<int64_t>((int64_t)mine, sh, tot);
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kItems; i++) {
+      if (digit[i] == 256u) continue;
+      const unsigned pos = base[digit[i]] + cnt[threadIdx.x >> 5][digit[i]] + rank[i];
+      xk[pos] = k[i];
+      xv[pos] = v[i];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kItems; i++) {
+      if (i0 + 32 * i < n) {
+        k[i] = xk[i0 + 32 * i];
+        v[i] = xv[i0 + 32 * i];
+      }
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int i = 0; i < kItems; i++) {
+    if (i0 + 32 * i < n) {
+      keys[i0 + 32 * i] = k[i];
+      vals[i0 + 32 * i] = v[i];
+    }
+  }
+}
+
+// fault: device word, set when a bounded wait ran out (the order is then incomplete)
 void radix_sort_u64(ph_ctx* ctx, uint64_t* keys, uint64_t* vals, int64_t n, int lo_bit,
-                    int hi_bit, uint64_t* tmp_keys, uint64_t* tmp_vals) {
+                    int hi_bit, uint64_t* tmp_keys, uint64_t* tmp_vals, int32_t* fault) {
   if (n <= 1 || hi_bit <= lo_bit) return;
-  int64_t ntiles = (n + kTile - 1) / kTile;
-  int64_t nh = 256 * ntiles;
-  int64_t* hist = alloc_n<int64_t>(ctx, nh);
-  int passes = (hi_bit - lo_bit + 7) / 8;
+  cudaStream_t st = ctx->stream;
+  const int digits = (hi_bit - lo_bit + 7) / 8;
+  if (n <= kTile) {
+    k_radix_tile<<<1, kThreads, 0, st>>>(keys, vals, (int)n, lo_bit, digits);
+    PH_CHECK_LAUNCH();
+    return;
+  }
+  const int64_t ntiles = (n + kTile - 1) / kTile;
+  // per digit: its counts, its tiles' states, its ticket
+  const int64_t words = 256 * digits + 256 * ntiles * digits + digits;
+  unsigned long long* buf = alloc_n<unsigned long long>(ctx, words);
+  unsigned long long* state = buf + 256 * digits;
+  unsigned long long* ticket = state + 256 * ntiles * digits;
+  PH_CUDA(cudaMemsetAsync(buf, 0, words * sizeof(unsigned long long), st));
+  k_radix_count<<<grid_for(ctx, n, kThreads * 4), kThreads, 0, st>>>(keys, n, lo_bit, digits, buf);
+  PH_CHECK_LAUNCH();
   uint64_t *ka = keys, *va = vals, *kb = tmp_keys, *vb = tmp_vals;
-  for (int p = 0; p < passes; p++) {
-    int shift = lo_bit + 8 * p;
-    k_radix_hist<<<(unsigned)ntiles, kThreads, 0, ctx->stream>>>(ka, n, shift, ntiles, hist);
+  for (int p = 0; p < digits; p++) {
+    k_radix_pass<<<(unsigned)ntiles, kThreads, 0, st>>>(
+        ka, va, kb, vb, n, lo_bit + 8 * p, buf + 256 * p, state + 256 * ntiles * p,
+        (unsigned int*)(ticket + p), fault);
     PH_CHECK_LAUNCH();
-    excl_scan_i64(ctx, hist, hist, nh, nullptr);
-    k_radix_scatter<<<(unsigned)ntiles, kThreads, 0, ctx->stream>>>(ka, va, kb, vb, n, shift,
-                                                                   ntiles, hist);
-    PH_CHECK_LAUNCH();
-    uint64_t* t = ka;
-    ka = kb;
-    kb = t;
-    t = va;
-    va = vb;
-    vb = t;
+    std::swap(ka, kb);
+    std::swap(va, vb);
   }
   if (ka != keys) {
-    PH_CUDA(cudaMemcpyAsync(keys, ka, n * sizeof(uint64_t), cudaMemcpyDeviceToDevice,
-                            ctx->stream));
-    PH_CUDA(cudaMemcpyAsync(vals, va, n * sizeof(uint64_t), cudaMemcpyDeviceToDevice,
-                            ctx->stream));
+    PH_CUDA(cudaMemcpyAsync(keys, ka, n * sizeof(uint64_t), cudaMemcpyDeviceToDevice, st));
+    PH_CUDA(cudaMemcpyAsync(vals, va, n * sizeof(uint64_t), cudaMemcpyDeviceToDevice, st));
   }
-  ctx->dfree(hist);
+  ctx->dfree(buf);
 }
 
 }  // namespace ph
