@@ -210,10 +210,14 @@ struct ph_ctx {
 
   ph::ReduceState rs;
 
-  // extraction cache
+  // extraction: places of the pairs and essential simplices, then (for per-cloud and host
+  // requests) all of them in internal arrays
   bool extracted = false;
   std::vector<int64_t> pair_off, ess_off;  // per cloud, host
   int64_t n_pairs = 0, n_ess = 0;
+  uint8_t* is_low = nullptr;                 // per id: the low of some column
+  unsigned long long* out_before = nullptr;  // per tile: pairs and essentials before it
+  int64_t* out_delta = nullptr;              // per segment: shift to its output places, both kinds
   int64_t *p_birth = nullptr, *p_death = nullptr, *p_bd2 = nullptr, *p_dd2 = nullptr;
   int32_t* p_dim = nullptr;
   int64_t *e_idx = nullptr, *e_d2 = nullptr;
@@ -359,6 +363,41 @@ __device__ __forceinline__ SegMax warp_incl_segmax(SegMax v) {
   return v;
 }
 
+// decoupled look-back over 64-bit tile states (2 flag bits, 62 value bits), zeroed before
+constexpr unsigned long long kAgg = 1ull << 62, kIncl = 2ull << 62, kFlags = 3ull << 62;
+constexpr int kWaitLimit = 1 << 22;  // polls of a look-back before it gives up (and reports it)
+
+// waits for a state word's flags; 0 (and *fault set) if they never come
+__device__ __forceinline__ unsigned long long wait_state(const unsigned long long* p,
+                                                         int32_t* fault) {
+  for (int it = 0; it < kWaitLimit; it++) {
+    const unsigned long long w = *(const volatile unsigned long long*)p;
+    if (w & kFlags) return w;
+    __nanosleep(20);
+  }
+  *fault = 1;
+  return kIncl;
+}
+
+// by one warp: the sum of the tiles before t, whose own sum is agg; publishes t's states
+__device__ __forceinline__ int64_t tile_prefix(unsigned long long* st, int64_t t, int64_t agg,
+                                               int32_t* fault) {
+  const int lane = lane_id();
+  if (lane == 0) atomicExch(st + t, (t == 0 ? kIncl : kAgg) | (unsigned long long)agg);
+  if (t == 0) return 0;
+  int64_t prefix = 0;
+  for (int64_t p = t - 1;; p -= 32) {
+    const unsigned long long w = p - lane >= 0 ? wait_state(st + p - lane, fault) : kIncl;
+    const unsigned im = __ballot_sync(0xffffffffu, (w & kFlags) == kIncl);
+    const int stop = im ? __ffs(im) - 1 : 32;
+    const int64_t val = lane <= stop ? (int64_t)(w & ~kFlags) : 0;
+    prefix += __shfl_sync(0xffffffffu, warp_incl_sum(val), 31);
+    if (im) break;
+  }
+  if (lane == 0) atomicExch(st + t, kIncl | (unsigned long long)(prefix + agg));
+  return prefix;
+}
+
 }  // namespace ph
 
 // host entry points shared between translation units
@@ -373,7 +412,6 @@ void load_boundary(ph_ctx* ctx, int64_t m, const int32_t* dims, const int64_t* c
 void compute_beta(ph_ctx* ctx);
 void reduce_init(ph_ctx* ctx);
 int reduce_run(ph_ctx* ctx, int32_t max_passes);
-void extract_all(ph_ctx* ctx);
 void free_reduce_state(ph_ctx* ctx);
 void free_graphs(ph_ctx* ctx);
 // E^l of one cloud, one byte per simplex in filtration order, into host memory (n bytes)
@@ -384,6 +422,9 @@ void reduced_columns(ph_ctx* ctx, int32_t cloud, int64_t n, int64_t* colptr, int
                      int64_t capacity, int64_t* nnz_out);
 // generic device helpers (ph_scan.cu)
 void excl_scan_i64(ph_ctx* ctx, const int64_t* in, int64_t* out, int64_t n, int64_t* total_dev);
+constexpr int kSortTile = 8192;  // pairs that one block sorts
+void radix_sort_tiles(ph_ctx* ctx, uint64_t* keys, uint64_t* vals, const int64_t* off, int ntiles,
+                      int64_t longest, int lo_bit, int hi_bit);
 void radix_sort_u64(ph_ctx* ctx, uint64_t* keys, uint64_t* vals, int64_t n, int lo_bit,
                     int hi_bit, uint64_t* tmp_keys, uint64_t* tmp_vals, int32_t* fault);
 void scan_counts(ph_ctx* ctx, const int32_t* a, const int32_t* b, int64_t n, int64_t* oa,

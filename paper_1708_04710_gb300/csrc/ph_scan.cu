@@ -80,40 +80,6 @@ void excl_scan_i64(ph_ctx* ctx, const int64_t* in, int64_t* out, int64_t n, int6
 // kernel: tiles in order from a ticket, each publishing its sum and looking back over the tiles
 // before it (decoupled look-back). state: per array one word per tile, zeroed before
 // ---------------------------------------------------------------------------------------------
-constexpr unsigned long long kAgg = 1ull << 62, kIncl = 2ull << 62, kFlags = 3ull << 62;
-constexpr int kWaitLimit = 1 << 22;  // polls of a look-back before it gives up (and reports it)
-
-// waits for a state word's flags; 0 (and *fault set) if they never come
-__device__ __forceinline__ unsigned long long wait_state(const unsigned long long* p,
-                                                         int32_t* fault) {
-  for (int it = 0; it < kWaitLimit; it++) {
-    const unsigned long long w = *(const volatile unsigned long long*)p;
-    if (w & kFlags) return w;
-    __nanosleep(20);
-  }
-  *fault = 1;
-  return kIncl;
-}
-
-// by one warp: the sum of the tiles before t, whose own sum is agg; publishes t's states
-__device__ __forceinline__ int64_t tile_prefix(unsigned long long* st, int64_t t, int64_t agg,
-                                               int32_t* fault) {
-  const int lane = lane_id();
-  if (lane == 0) atomicExch(st + t, (t == 0 ? kIncl : kAgg) | (unsigned long long)agg);
-  if (t == 0) return 0;
-  int64_t prefix = 0;
-  for (int64_t p = t - 1;; p -= 32) {
-    const unsigned long long w = p - lane >= 0 ? wait_state(st + p - lane, fault) : kIncl;
-    const unsigned im = __ballot_sync(0xffffffffu, (w & kFlags) == kIncl);
-    const int stop = im ? __ffs(im) - 1 : 32;
-    const int64_t val = lane <= stop ? (int64_t)(w & ~kFlags) : 0;
-    prefix += __shfl_sync(0xffffffffu, warp_incl_sum(val), 31);
-    if (im) break;
-  }
-  if (lane == 0) atomicExch(st + t, kIncl | (unsigned long long)(prefix + agg));
-  return prefix;
-}
-
 __global__ void k_scan_counts(const int32_t* __restrict__ a, const int32_t* __restrict__ b, int64_t n,
                               int64_t* oa, int64_t* ob, unsigned long long* state,
                               int64_t ntiles, unsigned int* ticket, int32_t* fault) {
@@ -167,10 +133,13 @@ void scan_counts(ph_ctx* ctx, const int32_t* a, const int32_t* b, int64_t n, int
 // LSD radix sort of (uint64 key, uint64 value) pairs by key bits [lo_bit, hi_bit), stable.
 // 8-bit digits, one kernel per digit: a tile ranks its elements per digit value in shared memory,
 // publishes its 256 counts and looks back for those of the tiles before it, one thread per
-// digit value, and scatters. One kernel before them counts every digit over all keys. A sort of
-// one tile is a single kernel. Bound by the scattered 16-byte writes; against separate count, scan and
-// scatter kernels per digit it reads the keys once less per digit and a small sort of five digits
-// is 1 launch instead of 25 (the build of 15 points to dimension 5, seven sorts: 540 -> 330 us).
+// digit value, and scatters. One kernel before them counts every digit over all keys. Up to 8192 pairs
+// are sorted by one block, all digits in one kernel (k_radix_tiles). Bound by the scattered 16-byte
+// writes, by latency for short lists. With separate count, scan and scatter kernels per digit the
+// sorts of a 400-point cloud's edges and triangles took 0.75 ms; its edges take 55 us now. A block
+// of 8192 pairs takes as long as the kernels over the whole device (7140 pairs, 5 digits: 39 against
+// 43 us) but is one launch, and a batch's clouds sort side by side: the edges of 512 clouds of 80
+// points 290 -> 130 us.
 // ---------------------------------------------------------------------------------------------
 constexpr int kMaxDigits = 8;
 
@@ -193,6 +162,7 @@ __global__ void k_radix_count(const uint64_t* __restrict__ keys, int64_t n, int 
 // Ranks of a tile's elements: element i of a thread is the tile's element warp * 256 + 32 i + lane.
 // cnt[w][d] becomes the number of the tile's elements with digit d in warps before w; returns this
 // thread's digit value's (threadIdx.x) number in the tile.
+template <int NW>
 __device__ __forceinline__ unsigned tile_ranks(const unsigned (&digit)[kItems],
                                                unsigned (&rank)[kItems],
                                                unsigned (*cnt)[257]) {
@@ -210,8 +180,9 @@ __device__ __forceinline__ unsigned tile_ranks(const unsigned (&digit)[kItems],
   }
   __syncthreads();
   unsigned run = 0;
+  if (NW > kWarps && threadIdx.x >= 256) return run;
 #pragma unroll
-  for (int v = 0; v < kWarps; v++) {
+  for (int v = 0; v < NW; v++) {
     const unsigned c = cnt[v][threadIdx.x];
     cnt[v][threadIdx.x] = run;
     run += c;
@@ -241,17 +212,26 @@ __global__ void __launch_bounds__(kThreads) k_radix_pass(
     v[i] = in ? vin[i0 + 32 * i] : 0;
     digit[i] = in ? (unsigned)((k[i] >> shift) & 255u) : 256u;
   }
-  const unsigned mine = tile_ranks(digit, rank, cnt);
+  const unsigned mine = tile_ranks<kWarps>(digit, rank, cnt);
   int64_t tot;
   int64_t b = block_excl_sum<int64_t>((int64_t)hist[threadIdx.x], sh, tot);
   unsigned long long* st = state + t * 256 + threadIdx.x;
   atomicExch(st, (t == 0 ? kIncl : kAgg) | mine);
   if (t > 0) {
     int64_t prefix = 0;
-    for (const unsigned long long* p = st - 256;; p -= 256) {
-      const unsigned long long w = wait_state(p, fault);
-      prefix += (int64_t)(w & ~kFlags);
-      if ((w & kFlags) == kIncl) break;
+    bool done = false;
+    for (int64_t p = t - 1; !done; p -= 8) {  // eight states in flight
+      unsigned long long w[8];
+#pragma unroll
+      for (int q = 0; q < 8; q++)
+        w[q] = p >= q ? *(const volatile unsigned long long*)(st - (t - p + q) * 256) : kIncl;
+#pragma unroll
+      for (int q = 0; q < 8; q++) {
+        if (done) continue;
+        if (!(w[q] & kFlags)) w[q] = wait_state(st - (t - p + q) * 256, fault);
+        prefix += (int64_t)(w[q] & ~kFlags);
+        done = (w[q] & kFlags) == kIncl;
+      }
     }
     atomicExch(st, kIncl | (unsigned long long)(prefix + mine));
     b += prefix;
@@ -268,41 +248,55 @@ __global__ void __launch_bounds__(kThreads) k_radix_pass(
   }
 }
 
-// one tile, all digits: elements stay in registers and change places in shared memory
-__global__ void __launch_bounds__(kThreads) k_radix_tile(uint64_t* keys, uint64_t* vals, int n,
+// All digits of one tile per block: elements stay in registers and change places in shared memory.
+// Tile b: elements off[b] .. off[b + 1], or all n without off; at most NW * 256.
+template <int NW>
+__global__ void __launch_bounds__(NW * 32) k_radix_tiles(uint64_t* keys, uint64_t* vals,
+                                                         const int64_t* __restrict__ off, int64_t n,
                                                          int lo_bit, int digits) {
-  __shared__ unsigned cnt[kWarps][257];
-  __shared__ int64_t sh[kWarps + 1];
-  __shared__ unsigned base[256];
-  __shared__ uint64_t xk[kTile];
-  __shared__ uint64_t xv[kTile];
-  const int i0 = (threadIdx.x >> 5) * (32 * kItems) + (threadIdx.x & 31);
-  uint64_t k[kItems], v[kItems];
-  unsigned digit[kItems], rank[kItems];
+  extern __shared__ uint64_t sm[];
+  uint64_t* xk = sm;
+  uint64_t* xv = xk + NW * 256;
+  unsigned (*cnt)[257] = reinterpret_cast<unsigned (*)[257]>(xv + NW * 256);
+  __shared__ unsigned base[256], sums[8];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int64_t first = off ? off[blockIdx.x] : 0;
+  const int len = (int)(off ? off[blockIdx.x + 1] - first : n);
+  keys += first;
+  vals += first;
+  const int i0 = w * 256 + lane;
+  uint64_t k[8], v[8];
+  unsigned digit[8], rank[8];
 #pragma unroll
-  for (int i = 0; i < kItems; i++) {
-    k[i] = i0 + 32 * i < n ? keys[i0 + 32 * i] : 0;
-    v[i] = i0 + 32 * i < n ? vals[i0 + 32 * i] : 0;
+  for (int i = 0; i < 8; i++) {
+    k[i] = i0 + 32 * i < len ? keys[i0 + 32 * i] : 0;
+    v[i] = i0 + 32 * i < len ? vals[i0 + 32 * i] : 0;
   }
   for (int p = 0; p < digits; p++) {
 #pragma unroll
-    for (int i = 0; i < kItems; i++)
-      digit[i] = i0 + 32 * i < n ? (unsigned)((k[i] >> (lo_bit + 8 * p)) & 255u) : 256u;
-    const unsigned mine = tile_ranks(digit, rank, cnt);
-    int64_t tot;
-    base[threadIdx.x] = (unsigned)block_excl_sum<int64_t>((int64_t)mine, sh, tot);
+    for (int i = 0; i < 8; i++)
+      digit[i] = i0 + 32 * i < len ? (unsigned)((k[i] >> (lo_bit + 8 * p)) & 255u) : 256u;
+    const unsigned mine = tile_ranks<NW>(digit, rank, cnt);
+    unsigned inc = warp_incl_sum(mine);
+    if (threadIdx.x < 256 && lane == 31) sums[w] = inc;
+    // (also the barrier before the sums are read) one value for all: nothing moves
+    if (__syncthreads_or(threadIdx.x < 256 && (int)mine == len)) continue;
+    if (threadIdx.x < 256) {
+      for (int q = 0; q < w; q++) inc += sums[q];
+      base[threadIdx.x] = inc - mine;
+    }
     __syncthreads();
 #pragma unroll
-    for (int i = 0; i < kItems; i++) {
+    for (int i = 0; i < 8; i++) {
       if (digit[i] == 256u) continue;
-      const unsigned pos = base[digit[i]] + cnt[threadIdx.x >> 5][digit[i]] + rank[i];
+      const unsigned pos = base[digit[i]] + cnt[w][digit[i]] + rank[i];
       xk[pos] = k[i];
       xv[pos] = v[i];
     }
     __syncthreads();
 #pragma unroll
-    for (int i = 0; i < kItems; i++) {
-      if (i0 + 32 * i < n) {
+    for (int i = 0; i < 8; i++) {
+      if (i0 + 32 * i < len) {
         k[i] = xk[i0 + 32 * i];
         v[i] = xv[i0 + 32 * i];
       }
@@ -310,12 +304,34 @@ __global__ void __launch_bounds__(kThreads) k_radix_tile(uint64_t* keys, uint64_
     __syncthreads();
   }
 #pragma unroll
-  for (int i = 0; i < kItems; i++) {
-    if (i0 + 32 * i < n) {
+  for (int i = 0; i < 8; i++) {
+    if (i0 + 32 * i < len) {
       keys[i0 + 32 * i] = k[i];
       vals[i0 + 32 * i] = v[i];
     }
   }
+}
+
+template <int NW>
+static void launch_tiles(ph_ctx* ctx, uint64_t* keys, uint64_t* vals, const int64_t* off,
+                         int ntiles, int64_t n, int lo_bit, int digits) {
+  constexpr size_t bytes = NW * 256 * 16 + NW * 257 * sizeof(unsigned);
+  if (bytes > 48 * 1024)
+    PH_CUDA(cudaFuncSetAttribute(k_radix_tiles<NW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)bytes));
+  k_radix_tiles<NW><<<ntiles, NW * 32, bytes, ctx->stream>>>(keys, vals, off, n, lo_bit, digits);
+  PH_CHECK_LAUNCH();
+}
+
+// sorts each of ntiles ranges (off[t] .. off[t + 1], device) of at most longest <= kSortTile pairs
+// by itself, in one kernel; off null: one range of longest pairs
+void radix_sort_tiles(ph_ctx* ctx, uint64_t* keys, uint64_t* vals, const int64_t* off, int ntiles,
+                      int64_t longest, int lo_bit, int hi_bit) {
+  if (longest <= 1 || hi_bit <= lo_bit) return;
+  const int digits = (hi_bit - lo_bit + 7) / 8;
+  if (longest <= 2048) launch_tiles<8>(ctx, keys, vals, off, ntiles, longest, lo_bit, digits);
+  else if (longest <= 4096) launch_tiles<16>(ctx, keys, vals, off, ntiles, longest, lo_bit, digits);
+  else launch_tiles<32>(ctx, keys, vals, off, ntiles, longest, lo_bit, digits);
 }
 
 // fault: device word, set when a bounded wait ran out (the order is then incomplete)
@@ -324,9 +340,8 @@ void radix_sort_u64(ph_ctx* ctx, uint64_t* keys, uint64_t* vals, int64_t n, int 
   if (n <= 1 || hi_bit <= lo_bit) return;
   cudaStream_t st = ctx->stream;
   const int digits = (hi_bit - lo_bit + 7) / 8;
-  if (n <= kTile) {
-    k_radix_tile<<<1, kThreads, 0, st>>>(keys, vals, (int)n, lo_bit, digits);
-    PH_CHECK_LAUNCH();
+  if (n <= kSortTile) {
+    radix_sort_tiles(ctx, keys, vals, nullptr, 1, n, lo_bit, hi_bit);
     return;
   }
   const int64_t ntiles = (n + kTile - 1) / kTile;
