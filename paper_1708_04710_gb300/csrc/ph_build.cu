@@ -96,17 +96,10 @@ __device__ __forceinline__ int packed_vert(const CloudTabs& ct, uint64_t p, int 
 }
 
 // ------------------------------------------------------------------------------------------
-__global__ void k_check_coords(const int32_t* __restrict__ x, int64_t n, int32_t* bad) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    int32_t v = x[i];
-    if (v > (1 << 24) || v < -(1 << 24)) *bad = 1;
-  }
-}
-
-// squared distances of every ordered pair of each cloud; block row y = cloud
+// squared distances of every ordered pair of each cloud; block row y = cloud. The points are
+// checked with their own pair; one atomic per warp that raises the maximum
 __global__ void k_pairwise(const int32_t* __restrict__ x, int D, CloudTabs ct, int64_t* d2,
-                           unsigned long long* maxd2) {
+                           unsigned long long* maxd2, int32_t* bad) {
   int c = blockIdx.y;
   int64_t p0 = ct.pt_off[c];
   int n = (int)(ct.pt_off[c + 1] - p0);
@@ -114,13 +107,14 @@ __global__ void k_pairwise(const int32_t* __restrict__ x, int D, CloudTabs ct, i
   unsigned long long mx = 0;
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < nn;
        t += (int64_t)gridDim.x * blockDim.x) {
-    int a = (int)(t / n), b = (int)(t % n);
+    const unsigned a = (unsigned)t / (unsigned)n, b = (unsigned)t % (unsigned)n;  // n < 2^12
     const int32_t* xa = x + (p0 + a) * D;
     const int32_t* xb = x + (p0 + b) * D;
     int64_t s = 0;
     for (int k = 0; k < D; k++) {
       int64_t dd = (int64_t)xa[k] - (int64_t)xb[k];
       s += dd * dd;
+      if (a == b && (xa[k] > (1 << 24) || xa[k] < -(1 << 24))) *bad = 1;
     }
     d2[ct.mo[c] + t] = s;
     mx = s > (int64_t)mx ? (unsigned long long)s : mx;
@@ -129,7 +123,7 @@ __global__ void k_pairwise(const int32_t* __restrict__ x, int D, CloudTabs ct, i
     unsigned long long y = __shfl_down_sync(0xffffffffu, mx, o);
     mx = y > mx ? y : mx;
   }
-  if ((threadIdx.x & 31) == 0) atomicMax(maxd2, mx);
+  if ((threadIdx.x & 31) == 0 && mx > *(volatile unsigned long long*)maxd2) atomicMax(maxd2, mx);
 }
 
 // Index of the first scale r_i = i * step with d <= 2 r_i for a squared distance d2 (Sec. 2.2:
@@ -346,15 +340,17 @@ __global__ void k_high_finish(const uint64_t* __restrict__ keys, const uint64_t*
 // counts per edge, scanned, are the places, and the filtration indices and left(i) (Definition 3)
 // of edges follow from them. With sorted candidates (each unranked by binary searches, five
 // kernels per 8-bit digit, then an atomic per row for left and two searches per simplex for the
-// index) the build of a 400-point cloud took 2.1 ms and now takes 0.58 ms, that of 120 points in
-// 8-d to dimension 3 with a cut 1.24 -> 0.47 ms, of 512 clouds of 64 points 6.4 -> 2.5 ms. Each
-// kernel reads two rows of the edge table per edge (from L2) and writes a simplex's 32 to 40 bytes
-// once, neighbouring lanes to neighbouring addresses.
+// index) the build of a 400-point cloud took 2.1 ms and now takes 0.48 ms, that of 120 points in
+// 8-d to dimension 3 with a cut 1.24 -> 0.33 ms, of 512 clouds of 80 points 6.4 -> 2.1 ms. Bound
+// by instruction issue: an edge costs 225 warp instructions to count and 645 to list (80 points, 26
+// triangles an edge), of which the writes of a triangle's 40 bytes, neighbouring lanes to
+// neighbouring addresses, are a third of the time.
 // The direct listing is taken whenever it applies: it is faster at every size measured (40
-// points: 470 -> 158 us, the one-tile sort of the edges included). With ties, and in dimensions 4
+// points: 470 -> 150 us, the one-block sort of the edges included). With ties, and in dimensions 4
 // and 5, candidates are sorted.
 constexpr int kDirectPoints = 512;   // points per cloud with tetrahedra (a warp's list of L(ab))
 constexpr int kDirectWarps = 4;
+static_assert(kVertBits == 12, "packed simplices are written here");
 
 struct Direct {
   const uint64_t* edge;   // sorted edges (packed), E of them; edge e has id N + e
@@ -363,19 +359,11 @@ struct Direct {
   const int64_t* es;      // per cloud: first edge
   const int64_t* off2;    // [E + 1] triangles before each edge's
   const int64_t* off3;    // [E + 1] tetrahedra, null without them
-  const uint32_t* mask;   // [E][words] L(ab) as bits (with tetrahedra)
+  const uint32_t* mask;   // [E][words] L(ab) as bits
   int words;
   int32_t* left;          // per row id
   int64_t* gidx;
 };
-
-// the lane's vertex c = c0 + lane is in L(ab)
-__device__ __forceinline__ bool in_link(const int32_t* ra, const int32_t* rb, int n, int c,
-                                        int32_t e, int32_t& ac, int32_t& bc) {
-  ac = c < n ? ra[c] : -1;
-  bc = c < n ? rb[c] : -1;
-  return ac >= 0 && bc >= 0 && ac < e && bc < e;
-}
 
 __global__ void __launch_bounds__(32 * kDirectWarps) k_link_count(CloudTabs ct, Direct g,
                                                                   int32_t* cnt2, int32_t* cnt3,
@@ -390,15 +378,30 @@ __global__ void __launch_bounds__(32 * kDirectWarps) k_link_count(CloudTabs ct, 
     const int32_t* tab = g.eid + ct.mo[c];
     const int32_t id = (int32_t)(g.N + e);
     int n2 = 0;
-    for (int c0 = 0; c0 < n; c0 += 32) {
-      int32_t ac, bc;
-      const bool f = in_link(tab + (int64_t)a * n, tab + (int64_t)b * n, n, c0 + lane, id, ac, bc);
-      const unsigned m = __ballot_sync(0xffffffffu, f);
-      if (cnt3) {
-        if (f) s_list[w][n2 + __popc(m & ((1u << lane) - 1u))] = (uint16_t)(c0 + lane);
-        if (lane == 0) mask[e * g.words + (c0 >> 5)] = m;
+    const int32_t* ra = tab + (int64_t)a * n;
+    const int32_t* rb = tab + (int64_t)b * n;
+    uint32_t mine = 0;  // mask word lane of the current 32
+    for (int c0 = 0; c0 < n; c0 += 64) {
+      int32_t ac[2], bc[2];
+#pragma unroll
+      for (int q = 0; q < 2; q++) {
+        const int x = c0 + 32 * q + lane;
+        ac[q] = x < n ? ra[x] : -1;
+        bc[q] = x < n ? rb[x] : -1;
       }
-      n2 += __popc(m);
+#pragma unroll
+      for (int q = 0; q < 2; q++) {
+        const bool f = (uint32_t)ac[q] < (uint32_t)id && (uint32_t)bc[q] < (uint32_t)id;
+        const unsigned m = __ballot_sync(0xffffffffu, f);
+        if (lane == (((c0 >> 5) + q) & 31)) mine = m;
+        if (cnt3 && f) s_list[w][n2 + __popc(m & ((1u << lane) - 1u))] = (uint16_t)(c0 + 32 * q + lane);
+        n2 += __popc(m);
+      }
+      if ((c0 & 1023) == 960 || c0 + 64 >= n) {
+        const int word = ((c0 >> 5) & ~31) + lane;
+        if (word < g.words) mask[e * g.words + word] = mine;
+        mine = 0;
+      }
     }
     if (lane == 0) cnt2[e] = n2;
     if (!cnt3) continue;
@@ -429,57 +432,20 @@ __device__ __forceinline__ void lower_left(int32_t* left, int32_t row, int32_t c
   if (left[row] > col) atomicMin(&left[row], col);
 }
 
-__global__ void __launch_bounds__(32 * kDirectWarps) k_tri_emit(CloudTabs ct, Direct g, IdOut o,
-                                                                int64_t rowbase) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  for (int64_t e = (int64_t)blockIdx.x * kDirectWarps + w; e < g.E;
-       e += (int64_t)gridDim.x * kDirectWarps) {
-    const uint64_t p = g.edge[e];
-    const int c = (int)packed_cloud(p), a = packed_vert(ct, p, 0), b = packed_vert(ct, p, 1);
-    const int n = (int)(ct.pt_off[c + 1] - ct.pt_off[c]);
-    const int32_t* tab = g.eid + ct.mo[c];
-    const int32_t id = (int32_t)(g.N + e);
-    const int64_t es = g.es[c], t0 = g.off2[e], ts = g.off2[es];
-    const int64_t qs = g.off3 ? g.off3[e] - g.off3[es] : 0;
-    const int64_t first = g.N + g.E + t0;  // id of this edge's first triangle
-    const bool any = g.off2[e + 1] > t0;
-    if (lane == 0) {
-      g.gidx[id] = n + (e - es) + (t0 - ts) + qs;
-      const int64_t v0 = ct.pt_off[c];
-      lower_left(g.left, (int32_t)(v0 + a), id);
-      lower_left(g.left, (int32_t)(v0 + b), id);
-      // an edge's first column is its own first triangle: it is shorter than the longest edge of
-      // any other triangle that holds it
-      if (any) g.left[id] = (int32_t)first;
-    }
-    if (!any) continue;
-    const int64_t gi = n + (e - es) + 1 + (t0 - ts) + qs;
-    int run = 0;
-    for (int c0 = 0; c0 < n; c0 += 32) {
-      const int x = c0 + lane;
-      int32_t ac, bc;
-      const bool f = in_link(tab + (int64_t)a * n, tab + (int64_t)b * n, n, x, id, ac, bc);
-      const unsigned m = __ballot_sync(0xffffffffu, f);
-      if (f) {
-        const int k = run + __popc(m & ((1u << lane) - 1u));
-        const int64_t t = first + k;
-        const int v[3] = {min(a, x), x < a ? a : min(x, b), max(b, x)};
-        o.verts[t] = pack_simplex((uint32_t)c, 3, v, ct.vbits);
-        o.seg[t] = 2 * ct.nc + c;
-        o.key[t] = (int32_t)e;
-        o.low[t] = id;
-        int32_t* r = o.rows0 + rowbase + 3 * (t0 + k);
-        r[0] = min(ac, bc);
-        r[1] = max(ac, bc);
-        r[2] = id;
-        g.gidx[t] = gi + k;
-        // ... so only an edge without triangles of its own looks for its first column here
-        if (g.off2[ac - g.N] == g.off2[ac - g.N + 1]) lower_left(g.left, ac, (int32_t)t);
-        if (g.off2[bc - g.N] == g.off2[bc - g.N + 1]) lower_left(g.left, bc, (int32_t)t);
-      }
-      run += __popc(m);
-    }
+// lists the vertices of up to kListWords mask words from word q0 on (in order) by one warp
+constexpr int kListWords = kDirectPoints / 32;
+__device__ __forceinline__ int list_mask(const uint32_t* mask, int q0, int words, uint16_t* list) {
+  const int lane = threadIdx.x & 31;
+  const int nq = min(kListWords, words - q0);
+  const uint32_t mine = lane < nq ? mask[q0 + lane] : 0;
+  int n = 0;
+  for (int q = 0; q < nq; q++) {
+    const uint32_t m = __shfl_sync(0xffffffffu, mine, q);
+    if ((m >> lane) & 1u) list[n + __popc(m & ((1u << lane) - 1u))] = (uint16_t)((q0 + q) * 32 + lane);
+    n += __popc(m);
   }
+  __syncwarp();
+  return n;
 }
 
 // id of the triangle on three vertices of one cloud: its longest edge's place plus the number of
@@ -505,12 +471,95 @@ __device__ __forceinline__ int32_t triangle_id(const Direct& g, const int32_t* t
   return (int32_t)(g.N + g.E + g.off2[ei] + k);
 }
 
-__global__ void __launch_bounds__(32 * kDirectWarps) k_tet_emit(CloudTabs ct, Direct g, IdOut o,
-                                                                int64_t id0, int64_t rowbase) {
+__global__ void __launch_bounds__(32 * kDirectWarps) k_tri_emit(CloudTabs ct, Direct g, IdOut o,
+                                                                int64_t rowbase) {
   __shared__ uint16_t s_list[kDirectWarps][kDirectPoints];
+  __shared__ int32_t s_rows[kDirectWarps][96];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < g.N;
+       i += (int64_t)gridDim.x * blockDim.x)  // a vertex's index is its place in its cloud
+    g.gidx[i] = i - ct.pt_off[find_cloud(ct.pt_off, ct.nc, i)];
   for (int64_t e = (int64_t)blockIdx.x * kDirectWarps + w; e < g.E;
        e += (int64_t)gridDim.x * kDirectWarps) {
+    const uint64_t p = g.edge[e];
+    const int64_t t0 = g.off2[e], t1 = g.off2[e + 1];
+    const int c = (int)packed_cloud(p), a = packed_vert(ct, p, 0), b = packed_vert(ct, p, 1);
+    const int64_t v0 = ct.pt_off[c];
+    const int n = (int)(ct.pt_off[c + 1] - v0);
+    const int32_t id = (int32_t)(g.N + e);
+    const int64_t es = g.es[c], ts = g.off2[es];
+    const int64_t qs = g.off3 ? g.off3[e] - g.off3[es] : 0;
+    const int64_t first = g.N + g.E + t0;  // id of this edge's first triangle
+    const int64_t gi = n + (e - es) + (t0 - ts) + qs;
+    const int32_t* tab = g.eid + ct.mo[c];
+    const int32_t* ra = tab + (int64_t)a * n;
+    const int32_t* rb = tab + (int64_t)b * n;
+    if (lane < 2) lower_left(g.left, (int32_t)(v0 + (lane ? b : a)), id);
+    if (lane == 0) g.gidx[id] = gi;
+    // an edge's first column is its own first triangle: it is shorter than the longest edge of
+    // any other triangle that holds it. Without one (the edges of the relative neighbourhood graph)
+    // it is the triangle on it whose longest edge is least: no two share that edge
+    if (t1 == t0) {
+      uint32_t least = 0x7f7f7f7fu;
+      int third = -1;
+      for (int x = lane; x < n; x += 32) {
+        const int32_t ac = ra[x], bc = rb[x];
+        const uint32_t longest = ac < 0 || bc < 0 ? 0x7f7f7f7fu : (uint32_t)max(ac, bc);
+        if (longest < least) {
+          least = longest;
+          third = x;
+        }
+      }
+      const uint32_t all = __reduce_min_sync(0xffffffffu, least);
+      if (third >= 0 && least == all) g.left[id] = triangle_id(g, tab, n, a, b, third);
+      continue;
+    }
+    if (lane == 0) g.left[id] = (int32_t)first;
+    const uint64_t high = (uint64_t)c << 48 | ((1u << 12) - 1u);  // cloud, last slot empty
+    int64_t t = first;
+    const int words = (n + 31) >> 5;  // of this cloud
+    for (int q0 = 0; q0 < words; q0 += kListWords) {
+      const int n2 = list_mask(g.mask + e * g.words, q0, words, s_list[w]);
+      for (int k0 = 0; k0 < n2; k0 += 32) {
+        const int k = k0 + lane;
+        const int have = min(32, n2 - k0);
+        if (k < n2) {
+          const int x = s_list[w][k];
+          const int32_t ac = ra[x], bc = rb[x];
+          o.verts[t + k] = high | (uint64_t)min(a, x) << 36 |
+                           (uint64_t)(x < a ? a : min(x, b)) << 24 | (uint64_t)max(b, x) << 12;
+          o.seg[t + k] = 2 * ct.nc + c;
+          o.key[t + k] = (int32_t)e;
+          o.low[t + k] = id;
+          g.gidx[t + k] = gi + 1 + (t - first) + k;
+          s_rows[w][3 * lane] = min(ac, bc);
+          s_rows[w][3 * lane + 1] = max(ac, bc);
+          s_rows[w][3 * lane + 2] = id;
+        }
+        __syncwarp();
+        int32_t* r = o.rows0 + rowbase + 3 * (t + k0 - g.N - g.E);
+#pragma unroll
+        for (int q = 0; q < 3; q++)
+          if (q * 32 + lane < 3 * have) r[q * 32 + lane] = s_rows[w][q * 32 + lane];
+        __syncwarp();
+      }
+      t += n2;
+    }
+  }
+}
+
+// One block per edge: its rows of pairs are counted, then written, by all warps. The edges with the
+// longest lists bound it: with a warp per edge the 920,000 tetrahedra of 120 points took 198 us, with
+// eight warps 87 us.
+constexpr int kTetThreads = 256, kTetWarps = kTetThreads / 32;
+
+__global__ void __launch_bounds__(kTetThreads) k_tet_emit(CloudTabs ct, Direct g, IdOut o,
+                                                          int64_t id0, int64_t rowbase) {
+  __shared__ uint16_t s_list[kDirectPoints];
+  __shared__ int32_t s_row[kDirectPoints];
+  __shared__ int s_n2;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  for (int64_t e = blockIdx.x; e < g.E; e += gridDim.x) {
     const int64_t q0 = g.off3[e];
     if (g.off3[e + 1] == q0) continue;
     const uint64_t p = g.edge[e];
@@ -521,22 +570,41 @@ __global__ void __launch_bounds__(32 * kDirectWarps) k_tet_emit(CloudTabs ct, Di
     const int64_t es = g.es[c];
     const int64_t gi = n + (e - es) + 1 + (g.off2[e + 1] - g.off2[es]) + (q0 - g.off3[es]);
     const int32_t tri0 = (int32_t)(g.N + g.E + g.off2[e]);
-    __syncwarp();
-    int n2 = 0;
-    for (int c0 = 0; c0 < n; c0 += 32) {
-      const unsigned m = g.mask[e * g.words + (c0 >> 5)];
-      if ((m >> lane) & 1u)
-        s_list[w][n2 + __popc(m & ((1u << lane) - 1u))] = (uint16_t)(c0 + lane);
-      n2 += __popc(m);
+    __syncthreads();  // the lists of the edge before are done with
+    if (w == 0) {
+      const int k = list_mask(g.mask + e * g.words, 0, (n + 31) >> 5, s_list);
+      if (lane == 0) s_n2 = k;
     }
-    __syncwarp();
-    int run = 0;
-    for (int i = 0; i + 1 < n2; i++) {
-      const int x = s_list[w][i];
+    __syncthreads();
+    const int n2 = s_n2;
+    for (int i = w; i < n2; i += kTetWarps) {
+      const int32_t* rc = tab + (int64_t)s_list[i] * n;
+      int k = 0;
+      for (int j = i + 1 + lane; j < n2; j += 32) {
+        const int32_t cd = rc[s_list[j]];
+        k += cd >= 0 && cd < id ? 1 : 0;
+      }
+      k = (int)__reduce_add_sync(0xffffffffu, (unsigned)k);
+      if (lane == 0) s_row[i] = k;
+    }
+    __syncthreads();
+    if (w == 0) {
+      int run = 0;
+      for (int i = 0; i < n2; i += 32) {
+        const int k = i + lane < n2 ? s_row[i + lane] : 0;
+        const int inc = warp_incl_sum(k);
+        if (i + lane < n2) s_row[i + lane] = run + inc - k;
+        run += __shfl_sync(0xffffffffu, inc, 31);
+      }
+    }
+    __syncthreads();
+    for (int i = w; i < n2; i += kTetWarps) {
+      const int x = s_list[i];
       const int32_t* rc = tab + (int64_t)x * n;
+      int run = s_row[i];
       for (int j0 = i + 1; j0 < n2; j0 += 32) {
         const int j = j0 + lane;
-        const int y = j < n2 ? s_list[w][j] : 0;
+        const int y = j < n2 ? s_list[j] : 0;
         const int32_t cd = j < n2 ? rc[y] : -1;
         const bool f = cd >= 0 && cd < id;
         const unsigned m = __ballot_sync(0xffffffffu, f);
@@ -545,10 +613,12 @@ __global__ void __launch_bounds__(32 * kDirectWarps) k_tet_emit(CloudTabs ct, Di
           const int64_t t = id0 + q0 + k;
           int32_t v[4] = {a, b, x, y};
           sort_small(v, 4);
+          const uint64_t packed = (uint64_t)c << 48 | (uint64_t)v[0] << 36 | (uint64_t)v[1] << 24 |
+                                  (uint64_t)v[2] << 12 | (uint64_t)v[3];
           int32_t r[4] = {tri0 + i, tri0 + j, triangle_id(g, tab, n, a, x, y),
                           triangle_id(g, tab, n, b, x, y)};
           sort_small(r, 4);
-          o.verts[t] = pack_simplex((uint32_t)c, 4, v, ct.vbits);
+          o.verts[t] = packed;
           o.seg[t] = 3 * ct.nc + c;
           o.key[t] = (int32_t)e;
           o.low[t] = r[3];
@@ -563,13 +633,6 @@ __global__ void __launch_bounds__(32 * kDirectWarps) k_tet_emit(CloudTabs ct, Di
       }
     }
   }
-}
-
-// filtration index of a vertex: its place in its cloud
-__global__ void k_vertex_gidx(CloudTabs ct, int64_t N, int64_t* gidx) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N;
-       i += (int64_t)gridDim.x * blockDim.x)
-    gidx[i] = i - ct.pt_off[find_cloud(ct.pt_off, ct.nc, i)];
 }
 
 __global__ void k_vertex_init(CloudTabs ct, int64_t N, IdOut o) {
@@ -801,7 +864,7 @@ static void build_direct(ph_ctx* ctx, const CloudTabs& ct, Direct g, const IdOut
   int32_t* cnt3 = tets ? alloc_n<int32_t>(ctx, g.E) : nullptr;
   int64_t* off2 = alloc_n<int64_t>(ctx, g.E + 1);
   int64_t* off3 = tets ? alloc_n<int64_t>(ctx, g.E + 1) : nullptr;
-  uint32_t* mask = tets ? alloc_n<uint32_t>(ctx, g.E * words) : nullptr;
+  uint32_t* mask = alloc_n<uint32_t>(ctx, g.E * words);
   g.es = d_es;
   g.off2 = off2;
   g.off3 = off3;
@@ -834,12 +897,10 @@ static void build_direct(ph_ctx* ctx, const CloudTabs& ct, Direct g, const IdOut
   g.gidx = ctx->gidx;
   PH_CUDA(cudaMemsetAsync(left, 0x7f, rows * sizeof(int32_t), st));  // > every id
   PH_CUDA(cudaMemsetAsync(ctx->beta, 0xff, m * sizeof(int32_t), st));
-  k_vertex_gidx<<<grid_for(ctx, g.N, kThreads), kThreads, 0, st>>>(ct, g.N, g.gidx);
-  PH_CHECK_LAUNCH();
   k_tri_emit<<<grid, 32 * kDirectWarps, 0, st>>>(ct, g, o, 2 * g.E);
   PH_CHECK_LAUNCH();
   if (tets && cnts[3] > 0) {
-    k_tet_emit<<<grid, 32 * kDirectWarps, 0, st>>>(ct, g, o, id3, 2 * g.E + 3 * cnts[2]);
+    k_tet_emit<<<grid_for(ctx, g.E, 1, 16), kTetThreads, 0, st>>>(ct, g, o, id3, 2 * g.E + 3 * cnts[2]);
     PH_CHECK_LAUNCH();
   }
   k_beta<<<grid_for(ctx, rows, kThreads), kThreads, 0, st>>>(rows, m, left, ctx->beta);
@@ -908,9 +969,6 @@ void build_vr(ph_ctx* ctx, const int32_t* coords, const int64_t* cloud_offsets, 
   int64_t* d_misc = alloc_n<int64_t>(ctx, 2 + (int64_t)kMaxVrDim * nc);
   PH_CUDA(cudaMemsetAsync(d_misc, 0, (2 + (int64_t)kMaxVrDim * nc) * sizeof(int64_t), st));
   auto cnt_dim = [&](int d) { return d_misc + 2 + (int64_t)(d - 1) * nc; };  // d >= 1
-  k_check_coords<<<grid_for(ctx, n_points * D, kThreads), kThreads, 0, st>>>(
-      coords, n_points * D, (int32_t*)d_misc);
-  PH_CHECK_LAUNCH();
 
   int64_t nn = mo[nc];
   int64_t* d2 = alloc_n<int64_t>(ctx, nn);
@@ -923,7 +981,8 @@ void build_vr(ph_ctx* ctx, const int32_t* coords, const int64_t* cloud_offsets, 
   {
     dim3 g((unsigned)std::max<int64_t>(1, std::min<int64_t>((nmax * nmax + 255) / 256, 4096)),
            (unsigned)nc);
-    k_pairwise<<<g, kThreads, 0, st>>>(coords, D, ct, d2, (unsigned long long*)(d_misc + 1));
+    k_pairwise<<<g, kThreads, 0, st>>>(coords, D, ct, d2, (unsigned long long*)(d_misc + 1),
+                                     (int32_t*)d_misc);
     PH_CHECK_LAUNCH();
   }
   // page-locked scratch: status words and per-cloud counts come back through it
@@ -957,8 +1016,16 @@ void build_vr(ph_ctx* ctx, const int32_t* coords, const int64_t* cloud_offsets, 
     k_edge_cand<<<grid_for(ctx, cand[2][nc], kThreads), kThreads, 0, st>>>(
         ct, d_cand(2), cand[2][nc], d2, max_diam2, sent_e, kbuf, vbuf, cnt_dim(1));
     PH_CHECK_LAUNCH();
-    radix_sort_u64(ctx, kbuf, vbuf, cand[2][nc], 0, d2bits, ktmp, vtmp, d_fault);
-    if (nc > 1) {
+    // every cloud's edges in one block, if they fit; truncated ones of several clouds have to
+    // come after all clouds' edges
+    int64_t longest = 0;
+    for (int c = 0; c < nc; c++) longest = std::max(longest, cand[2][c + 1] - cand[2][c]);
+    const bool tiles = longest <= kSortTile && (nc == 1 || max_diam2 < 0);
+    if (tiles)
+      radix_sort_tiles(ctx, kbuf, vbuf, d_cand(2), nc, longest, 0, d2bits);
+    else
+      radix_sort_u64(ctx, kbuf, vbuf, cand[2][nc], 0, d2bits, ktmp, vtmp, d_fault);
+    if (nc > 1 && !tiles) {
       k_rekey_cloud<<<grid_for(ctx, cand[2][nc], kThreads), kThreads, 0, st>>>(
           vbuf, kbuf, cand[2][nc], sent_e, (uint64_t)nc);
       PH_CHECK_LAUNCH();

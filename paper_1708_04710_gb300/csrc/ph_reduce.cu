@@ -419,8 +419,12 @@ __global__ void k_tab(RArgs a) {
     for (int k = 0; k < kTI; k++) j[k] = i0 + k < v.n_act ? v.act[i0 + k] : -1;
 #pragma unroll
     for (int k = 0; k < kTI; k++) l[k] = j[k] >= 0 ? a.low[j[k]] : -1;
+    const int32_t before = i0 > 0 ? a.low[v.act[i0 - 1]] : -1;
 #pragma unroll
     for (int k = 0; k < kTI; k++) {
+      // in the first pass's list (every id in order) a run of columns with one low has its least
+      // column first
+      if (l[k] == (k > 0 ? l[k - 1] : before)) continue;
       if (l[k] >= 0 && PH_DCHECK(&a.ds->debug_fault, l[k] < a.rows_end, 1)) {
         const unsigned long long key = tab_key_of(a.ds->pass) | (unsigned)j[k];
         if (a.tab[l[k]] > key) atomicMin(&a.tab[l[k]], key);

@@ -74,3 +74,72 @@ def test_direct_listing_equals_sorted_listing(ph, orc, n, max_dim, cut):
     ca, cm, cb = _r0(alone, 0), _r0(mixed, 1), _r0(batch, 1)
     for i in (0, 1):
         assert np.array_equal(ca[i], cm[i]) and np.array_equal(ca[i], cb[i])
+
+
+# one block sorts up to 2048, 4096 or 8192 edges of a cloud (64, 91 and 128 points have 2016, 4095 and
+# 8128); above, and with several truncated clouds, all edges are sorted over the whole device
+@pytest.mark.parametrize("sizes", [[64], [65], [91], [92], [128], [129], [3, 1, 128, 2, 64],
+                                   [129, 1, 2]])
+@pytest.mark.parametrize("cut", [-1, 65536 ** 2])
+def test_edge_sort_sizes(ph, orc, sizes, cut):
+    clouds = [pc.lattice_cloud(n, 2, 700 + n, side=40) for n in sizes]  # with ties: stable
+    ctx = _build(ph.Context(), clouds, 1, cut)
+    for c, x in enumerate(clouds):
+        K, f = orc.vr_build(x, 1, cut), ctx.filtration(c)
+        assert np.array_equal(f["diam2"], K["diam2"]) and np.array_equal(f["verts"], K["verts"])
+
+
+# 1024 and 4096 ids are a writer's round and a scan's tile; 235 points have more than 2^21 ids (long
+# rounds); three hundred clouds put many segments, some empty, into one tile
+@pytest.mark.parametrize("sizes,max_dim,passes", [
+    ([1], 2, -1), ([2, 1, 1], 2, -1), ([18, 1], 2, -1), ([25], 3, -1), ([29, 30], 2, 1),
+    ([1 + i % 6 for i in range(300)], 2, -1), ([235], 2, 2),
+])
+def test_extraction_routes(ph, sizes, max_dim, passes):
+    import ctypes
+
+    import torch
+
+    clouds = [pc.random_cloud(n, 3, 900 + i) for i, n in enumerate(sizes)]
+    ctx = _build(ph.Context(), clouds, max_dim)
+    ctx.reduce(max_passes=passes)
+    pr, es = ctx.pairs(-1), ctx.essential(-1)  # written straight into the tensors
+    pr = {k: v.cpu().numpy() for k, v in pr.items()}
+    es = {k: v.cpu().numpy() for k, v in es.items()}
+    want_p = {k: [] for k in pr}
+    want_e = {k: [] for k in es}
+    for c in range(len(sizes)):
+        f = ctx.filtration(c)
+        order = np.argsort(f["dim"], kind="stable")  # (dimension, index)
+        death = order[f["low"][order] >= 0]
+        birth = f["low"][death]
+        is_low = np.zeros(len(order), bool)
+        is_low[birth] = True
+        e = order[(f["low"][order] < 0) & ~is_low[order]]
+        one = dict(birth=birth, death=death, dim=f["dim"][birth], birth_diam2=f["diam2"][birth],
+                   death_diam2=f["diam2"][death])
+        onee = dict(idx=e, dim=f["dim"][e], diam2=f["diam2"][e])
+        for w, o in ((want_p, one), (want_e, onee)):
+            for k, v in o.items():
+                w[k].append(v)
+        if c in (0, len(sizes) - 1):  # internal arrays and copies
+            for host in (False, True):
+                got = {**{"p" + k: v for k, v in ctx.pairs(c, not host).items()},
+                       **{"e" + k: v for k, v in ctx.essential(c, not host).items()}}
+                for k, v in [("p" + k, v) for k, v in one.items()] + [
+                        ("e" + k, v) for k, v in onee.items()]:
+                    assert np.array_equal(got[k].cpu().numpy(), v), k
+    for w, o in ((want_p, pr), (want_e, es)):
+        for k in o:
+            assert np.array_equal(o[k], np.concatenate(w[k])), k
+    # an array off its type's alignment, and one left out, in a fresh extraction
+    ctx2 = _build(ph.Context(), clouds, max_dim)
+    ctx2.reduce(max_passes=passes)
+    n = ctypes.c_int64(len(pr["death"]))
+    for shift in (0, 1):
+        raw = torch.zeros(2 * n.value + 1, dtype=torch.int32, device="cuda")
+        rc = ctx2.lib.ph_get_pairs(ctx2._h, -1, None, ctypes.c_void_p(raw.data_ptr() + 4 * shift),
+                                   None, None, None, n.value, ctypes.byref(n), 1)
+        assert rc == 0
+        got = raw[shift:2 * n.value + shift].cpu().numpy().view(np.int64)
+        assert np.array_equal(got, pr["death"])
