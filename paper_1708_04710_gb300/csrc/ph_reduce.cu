@@ -146,6 +146,7 @@ struct RArgs {
   int strict;
   int cor10;
   unsigned long long* tile_st;  // per Phase I tile: look-back state of its aggregate / prefix
+  unsigned long long* loop_tile_st;  // the same for the loop kernel's tiles
   unsigned long long* look;  // per Phase II chunk: look-back state of the survivor count
   int32_t* dlist;     // columns whose update (nxt_ptr, nxt_len) waits for k_commit
   int32_t* newpos;    // per active slot, in a pass that compacts: its place in the next list, -1
@@ -240,6 +241,12 @@ __device__ __forceinline__ void stat_add(int64_t* stats, int k, int64_t v) {
   if (lane_id() == 0 && s != 0) atomicAdd((unsigned long long*)&stats[k], (unsigned long long)s);
 }
 
+
+__device__ __forceinline__ int64_t warp_sum64(int64_t v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
 
 // Programmatic dependent launch. The kernels of a pass are launched so that each may start
 // while the one before it in the stream drains (its blocks fill the SMs that kernel frees): every
@@ -648,14 +655,26 @@ __device__ __forceinline__ int64_t look_back(const RArgs& a, int32_t pass, int64
 // the space this pass's Phase II can need (arena, pivot store) against what the host provided;
 // no column has changed yet, and the marks made depend only on the pass's starting state, so a
 // pass stopped here continues at Phase II once the host has grown the buffers
+struct Space {
+  unsigned long long arena_used, arena_cap, piv_used, piv_cap;
+};
+__device__ __forceinline__ Space space_of(const DevState* ds) {
+  return Space{*(const volatile unsigned long long*)&ds->arena_used,
+               (unsigned long long)*(const volatile int64_t*)&ds->arena_cap[ds->arena_cur],
+               *(const volatile unsigned long long*)&ds->piv_used,
+               (unsigned long long)*(const volatile int64_t*)&ds->piv_cap};
+}
+__device__ __forceinline__ int lacks_space(const DevState* ds, const Space& s) {
+  const unsigned long long words = *(const volatile unsigned long long*)&ds->bound_words;
+  const unsigned long long piv = *(const volatile unsigned long long*)&ds->bound_piv;
+  return (s.arena_used + words > s.arena_cap ? 1 : 0) | (piv + s.piv_used > s.piv_cap ? 2 : 0);
+}
+__device__ __forceinline__ void stop_for_space(DevState* ds, int reason) {
+  ds->host_reason = reason;
+  ds->status = ST_HOST;
+}
 __device__ __forceinline__ void check_capacity(DevState* ds) {
-  int reason = 0;
-  if (ds->arena_used + ds->bound_words > (unsigned long long)ds->arena_cap[ds->arena_cur]) reason |= 1;
-  if (ds->bound_piv + ds->piv_used > (unsigned long long)ds->piv_cap) reason |= 2;
-  if (reason) {
-    ds->host_reason = reason;
-    ds->status = ST_HOST;
-  }
+  if (const int reason = lacks_space(ds, space_of(ds))) stop_for_space(ds, reason);
 }
 
 // Phase I and the marks in one kernel, a single-pass scan over tiles of kFTile active slots
@@ -684,11 +703,10 @@ __device__ __forceinline__ SegMax tile_value(unsigned long long w) {
 
 // by warp 0: publishes tile t's aggregate, returns the Phase I value of every tile before it
 // (SegMax{-1, -1}, a left identity of segmax_combine, for none) and publishes t's inclusive state
-__device__ __forceinline__ SegMax tile_look_back(const RArgs& a, int32_t pass, int64_t t,
+__device__ __forceinline__ SegMax tile_look_back(unsigned long long* st, int32_t pass, int64_t t,
                                                  SegMax agg, bool& fault) {
   const int lane = lane_id();
   const unsigned long long tag = (unsigned long long)(pass & 0xff) << 56;
-  unsigned long long* st = a.tile_st;
   const SegMax none{-1, -1};
   if (t == 0) {
     if (lane == 0) atomicExch(st, tile_word(tag, kTIncl, agg));
@@ -741,7 +759,10 @@ __device__ __forceinline__ SegMax tile_look_back(const RArgs& a, int32_t pass, i
 // A pass that compacts also gives every slot whose column may survive its place in the next active
 // list (newpos), by a second look-back over the tiles: a column that left all the same (proven
 // by its P_j, or cleared) leaves a dead place there.
-template <bool kLookAhead>
+//
+// kLoop: in the loop kernel (every block resident) tiles of one slot per thread are dealt out in
+// order instead, to all `parts` blocks.
+template <bool kLookAhead, bool kLoop>
 __device__ __forceinline__ void phase1_pass(const RArgs& a, unsigned parts) {
   __shared__ SegMax sh[kWarps + 1];
   __shared__ int64_t shs[kWarps + 1];
@@ -749,7 +770,8 @@ __device__ __forceinline__ void phase1_pass(const RArgs& a, unsigned parts) {
   __shared__ SegMax s_pre;
   __shared__ int s_keep[kWarps + 1];
   __shared__ int64_t s_place;
-  constexpr int kFI = kFItems;
+  constexpr int kFI = kLoop ? 1 : kFItems;
+  constexpr int64_t kFTile = kThreads * kFI;
   if (blockIdx.x >= parts) return;
   DevState* ds = a.ds;
   const PV v = pass_view(ds);
@@ -763,10 +785,12 @@ __device__ __forceinline__ void phase1_pass(const RArgs& a, unsigned parts) {
   int64_t n_zero = 0, n_piv = 0, n_c10 = 0, n_pred = 0, n_empty = 0;
   bool want = false;  // a target whose addition may reach its dimension's bit-packing threshold
   bool fault = false;
-  for (;;) {  // (a tile is claimed only when its work begins: later tiles wait for its state)
-    if (threadIdx.x == 0) s_tile = atomicAdd(&ds->tile_queue, 1u);
-    __syncthreads();
-    const int64_t t = s_tile;
+  for (int64_t t = blockIdx.x;; t += parts) {
+    if constexpr (!kLoop) {  // a tile is claimed only when its work begins: later tiles wait for it
+      if (threadIdx.x == 0) s_tile = atomicAdd(&ds->tile_queue, 1u);
+      __syncthreads();
+      t = s_tile;
+    }
     if (t >= ntiles) break;
     const int64_t tile0 = t * kFTile;
     // bit-packing thresholds of the tile's columns (ascending ids, so dimensions too): exact in
@@ -830,7 +854,7 @@ __device__ __forceinline__ void phase1_pass(const RArgs& a, unsigned parts) {
     SegMax tot;
     const SegMax pre_t = block_scan_segmax(agg, SegMax{-1, -1}, sh, tot);  // within the tile
     if (threadIdx.x < 32) {
-      const SegMax P = tile_look_back(a, pass, t, tot, fault);
+      const SegMax P = tile_look_back(kLoop ? a.loop_tile_st : a.tile_st, pass, t, tot, fault);
       if (threadIdx.x == 0) s_pre = P;
     }
     // the marks: a new pivot proven by Thm 5 (left-most, low = beta) or by Phase I (left-most,
@@ -947,6 +971,14 @@ __device__ __forceinline__ void phase1_pass(const RArgs& a, unsigned parts) {
   }
   if (want && !v.dense_on) ds->dense_want = 1;  // bit-packed additions from the next pass
   if (__any_sync(0xffffffffu, fault) && lane_id() == 0) ds->fault = 1;
+  if constexpr (kLoop) {
+    const int64_t ww = warp_sum64(bw), wp = warp_sum64(bp);
+    if (lane_id() == 0 && (ww || wp)) {
+      atomicAdd(&ds->bound_words, (unsigned long long)ww);
+      atomicAdd(&ds->bound_piv, (unsigned long long)wp);
+    }
+    return;
+  }
   int64_t tw, tp;
   block_excl_sum<int64_t>(bw, shs, tw);
   block_excl_sum<int64_t>(bp, shs, tp);
@@ -971,7 +1003,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_phase1(RArgs a) {
   if (ds->status != ST_RUN) return;
   const unsigned parts = phase1_parts(ds, gridDim.x);
   if (blockIdx.x >= parts) return;
-  phase1_pass<kLookAhead>(a, parts);
+  phase1_pass<kLookAhead, false>(a, parts);
   // the last of the taking-part blocks checks the space this pass's Phase II needs
   if (last_block(&ds->blocks_done, parts)) {
     if (threadIdx.x == 0) {
@@ -1792,12 +1824,6 @@ __device__ __forceinline__ void next_tab(const RArgs& a, const PV& v, int32_t l,
 enum : int {
   kCntTargets, kCntActive, kCntCleared, kCntAdds, kCntXors, kCntCopied, kCntPacked, kNumCnt
 };
-
-__device__ __forceinline__ int64_t warp_sum64(int64_t v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
 
 // Merges by one warp: per lane the column A (rows, or a bit-packed column if dense_a) and the
 // source B (likewise, dense_b; null: the column moves) into the lane's slot of the arena (null: no
@@ -2770,13 +2796,40 @@ __global__ void k_commit(RArgs a, cudaGraphConditionalHandle cond, int mode) {
 // (every block resident, so they may wait for each other), the parts of a pass separated by
 // grid barriers.
 //
-// A grid barrier: true in every block once all have arrived and the last one to arrive has run
-// `tail`; what was written before it is visible after it. The wait is bounded: a block that gives
-// up records a fault, and returns false.
+// A grid barrier is one counter: every block adds one and waits until all of the pass's blocks have,
+// that many times the barriers so far (`target`). What was written before it is visible after it.
+// The last barrier of a pass (grid_last) runs `tail` in the block that arrives last, which then
+// clears the counter and lets the others go by a second word. The waits are bounded: a block that
+// gives up records a fault, and both return false.
+__device__ __forceinline__ bool poll_until(DevState* ds, const unsigned int* p, unsigned int value,
+                                           bool at_least) {
+  for (int it = 0; it < kBarrierLimit; it++) {
+    const unsigned int x = *(const volatile unsigned int*)p;
+    if (at_least ? x >= value : x != value) return true;
+  }
+  ds->fault = 1;
+  return false;
+}
+__device__ __forceinline__ bool grid_sync(DevState* ds, unsigned blocks, unsigned int& target) {
+  if (blocks == 1) {
+    __syncthreads();
+    return true;
+  }
+  target += blocks;
+  bool ok = true;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(&ds->bar_count, 1u);
+    ok = poll_until(ds, &ds->bar_count, target, true);
+    __threadfence();
+  }
+  return __syncthreads_and(ok);
+}
 template <typename F>
-__device__ __forceinline__ bool grid_sync(DevState* ds, unsigned blocks, F tail) {
-  __shared__ int s_last, s_ok;
-  __shared__ unsigned int s_gen;
+__device__ __forceinline__ bool grid_last(DevState* ds, unsigned blocks, unsigned int target,
+                                          unsigned int& gen, F tail) {
+  __shared__ int s_last;
   __syncthreads();
   if (blocks == 1) {
     tail();
@@ -2784,12 +2837,11 @@ __device__ __forceinline__ bool grid_sync(DevState* ds, unsigned blocks, F tail)
     return true;
   }
   if (threadIdx.x == 0) {
-    s_gen = *(volatile unsigned int*)&ds->bar_gen;
-    s_ok = 1;
     __threadfence();
-    s_last = atomicAdd(&ds->bar_count, 1u) == blocks - 1;
+    s_last = atomicAdd(&ds->bar_count, 1u) == target + blocks - 1;
   }
   __syncthreads();
+  bool ok = true;
   if (s_last) {
     __threadfence();
     tail();
@@ -2797,48 +2849,51 @@ __device__ __forceinline__ bool grid_sync(DevState* ds, unsigned blocks, F tail)
     if (threadIdx.x == 0) {
       ds->bar_count = 0;
       __threadfence();
-      atomicExch(&ds->bar_gen, s_gen + 1);
+      atomicExch(&ds->bar_gen, gen + 1);
     }
   } else if (threadIdx.x == 0) {
-    int it = 0;
-    while (*(volatile unsigned int*)&ds->bar_gen == s_gen) {
-      if (++it > kBarrierLimit) {
-        ds->fault = 1;
-        s_ok = 0;
-        break;
-      }
-      __nanosleep(20);
-    }
+    ok = poll_until(ds, &ds->bar_gen, gen, false);
+    __threadfence();
   }
-  if (threadIdx.x == 0) __threadfence();
-  __syncthreads();
-  return s_ok != 0;
+  gen++;
+  return __syncthreads_and(ok);
 }
 
+constexpr int64_t kLoopBelow = (int64_t)1 << 14;  // columns from which k_loop takes over
+constexpr int64_t kLoopSingle = 64;  // columns left to one block
 constexpr int kLoopBlocks = 2;  // per SM: registers for every part of a pass without spills
 __global__ void __launch_bounds__(kThreads, kLoopBlocks) k_loop(RArgs a, int64_t m) {
   extern __shared__ __align__(16) unsigned char add_smem[];
   WarpStage& S = reinterpret_cast<WarpStage*>(add_smem)[threadIdx.x >> 5];
   DevState* ds = a.ds;
-  const auto nothing = [] {};
+  // (no block can let the others go before this one has arrived)
+  unsigned int gen = *(volatile unsigned int*)&ds->bar_gen;
   // a shrinking list is left to fewer blocks, at last to one, whose barriers cost next to nothing
   for (;;) {
     const unsigned blocks = *(volatile unsigned int*)&ds->loop_blocks;
     if (blockIdx.x >= blocks || *(volatile int32_t*)&ds->status != ST_RUN) return;
-    phase1_pass<false>(a, phase1_parts(ds, blocks));
-    if (!grid_sync(ds, blocks, [&] {
-          if (threadIdx.x == 0) check_capacity(ds);
-        }))
+    unsigned int target = 0;
+    const int64_t n = *(volatile int64_t*)&ds->n_act;
+    // what every block needs to see for itself whether the pass's space suffices, as it stands
+    // before the additions take any
+    const Space space = space_of(ds);
+    phase1_pass<false, true>(a, blocks);
+    if (!grid_sync(ds, blocks, target)) return;
+    if (const int reason = lacks_space(ds, space)) {
+      if (blockIdx.x == 0 && threadIdx.x == 0) stop_for_space(ds, reason);
       return;
-    if (*(volatile int32_t*)&ds->status != ST_RUN) return;
+    }
     if (ds->stats) {
       ess_count(a, m, blocks);
-      if (!grid_sync(ds, blocks, nothing)) return;
+      if (!grid_sync(ds, blocks, target)) return;
     }
-    add_pass<true, 32, false, kThreads, true>(a, S, blocks);
-    if (!grid_sync(ds, blocks, nothing)) return;
+    // few columns: narrow chunks, so that every warp has some
+    if (n <= 4 * kWarps) add_pass<true, 4, false, kThreads, true>(a, S, blocks);
+    else if (n <= 8 * kWarps * (int64_t)blocks) add_pass<true, 8, false, kThreads, true>(a, S, blocks);
+    else add_pass<true, 32, false, kThreads, true>(a, S, blocks);
+    if (!grid_sync(ds, blocks, target)) return;
     commit_pass(a, blocks);
-    if (!grid_sync(ds, blocks, [&] { commit_last(a, 0, kInLoop, blocks); })) return;
+    if (!grid_last(ds, blocks, target, gen, [&] { commit_last(a, 0, kInLoop, blocks); })) return;
   }
 }
 
@@ -2851,10 +2906,12 @@ __device__ __forceinline__ unsigned long long global_ns() {
 
 __global__ void k_clock_start(DevState* ds) { ds->t_start = global_ns(); }
 
-// blocks of the loop kernel for an active list of n columns: one for a tile of Phase I, else one per
-// 256 columns
+// blocks of the loop kernel for an active list of n columns: a warp for 8 columns, up to
+// kLoopMost blocks
+constexpr int kLoopMost = 64;
 __host__ __device__ inline unsigned int loop_blocks_for(int64_t n) {
-  return n <= kFTile ? 1u : (unsigned int)std::min<int64_t>((n + kThreads - 1) / kThreads, 1 << 20);
+  return n <= kLoopSingle ? 1u
+                          : (unsigned int)std::min<int64_t>((n + 8 * kWarps - 1) / (8 * kWarps), kLoopMost);
 }
 
 // end of a pass: the next active list, convergence (no target left), the pass cap, the time
@@ -3020,6 +3077,7 @@ static RArgs make_args(ph_ctx* ctx) {
   a.strict = ctx->opts.strict_phase2;
   a.cor10 = ctx->opts.use_cor10;
   a.tile_st = static_cast<unsigned long long*>(rs.tiles);
+  a.loop_tile_st = a.tile_st + (ctx->m + kFTile - 1) / kFTile + 1;
   a.look = static_cast<unsigned long long*>(rs.look);
   a.dlist = static_cast<int32_t*>(rs.dlist);
   a.src_e = static_cast<int32_t*>(rs.src_e);
@@ -3217,11 +3275,14 @@ void reduce_init(ph_ctx* ctx) {
   rs.dirty = alloc_n<int32_t>(ctx, 3 * nseg);  // next_unp, dirty_on, dirty
   PH_CUDA(cudaMemsetAsync(rs.dirty, 0x7f, nseg * sizeof(int32_t), st));
   PH_CUDA(cudaMemsetAsync(rs.dirty + nseg, 0, nseg * sizeof(int32_t), st));
+  // Phase I's tile states; the loop kernel's tiles are of another size and have their own
   const int64_t ntiles = (m + kFTile - 1) / kFTile;
-  rs.tiles_bytes = (ntiles + 1) * sizeof(unsigned long long);
+  const int64_t loop_tiles = (std::min<int64_t>(m, kLoopBelow) + kThreads - 1) / kThreads;
+  rs.tiles_bytes = (ntiles + 1 + loop_tiles) * sizeof(unsigned long long);
   rs.tiles = ctx->dalloc(rs.tiles_bytes);
   PH_CUDA(cudaMemsetAsync(rs.tiles, 0, rs.tiles_bytes, st));  // no state published yet
-  const int64_t nchunks = (m + 7) / 8 + 1;  // chunks of any shape (8 slots or more), or tiles
+  // chunks of any shape (8 slots or more; 4 for a few columns), or tiles
+  const int64_t nchunks = (m + 7) / 8 + 1 + kWarps;
   rs.look = alloc_n<unsigned long long>(ctx, nchunks);
   PH_CUDA(cudaMemsetAsync(rs.look, 0, nchunks * sizeof(unsigned long long), st));
   rs.dlist = alloc_n<int32_t>(ctx, m);
@@ -3404,9 +3465,8 @@ static unsigned loop_grid(ph_ctx* ctx) {
     PH_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctx->loop_blocks_per_sm, k_loop, kThreads,
                                                           kLoopSmem));
   const int64_t most = (int64_t)ctx->num_sms * ctx->loop_blocks_per_sm;
-  return (unsigned)std::min<int64_t>(most, (ctx->m + kThreads - 1) / kThreads);
+  return (unsigned)std::min<int64_t>(most, kLoopMost);
 }
-constexpr int64_t kLoopBelow = (int64_t)1 << 14;
 
 // the pass loop as one graph: a conditional while node around one pass, with one of the
 // additions kernel variants (see launch_pass)
@@ -3533,6 +3593,7 @@ int reduce_run(ph_ctx* ctx, int32_t max_passes) {
     }
     PH_CUDA(cudaMemcpyAsync(&h, rs.dstate, sizeof(DevState), cudaMemcpyDeviceToHost, st));
     PH_CUDA(cudaStreamSynchronize(st));
+    h.bar_count = 0;  // k_loop leaves a pass without space half-way
     if (ran_graph) {  // kernels per executed pass of the graph's loop
       const int32_t last = (h.status == ST_DONE || h.status == ST_CAPPED) ? h.passes : h.pass;
       const int per_pass = (variant >= 10 ? 4 : 3) + (ctx->opts.collect_stats ? 1 : 0);
