@@ -2,6 +2,7 @@
 // simplices (Lemma 1, Eq. paired), and inspection of the filtration.
 #include <algorithm>
 #include <cstring>
+#include <functional>
 #include <new>
 
 #include "ph_internal.cuh"
@@ -36,11 +37,14 @@ void ph_ctx::drop_kept(int64_t before) {
 
 void* ph_ctx::dalloc(size_t bytes) {
   bytes = bytes <= 256 ? 256 : (bytes + 255) & ~size_t(255);
-  // the smallest kept block that fits without much waste
+  // the smallest kept block that fits without much waste, the first in memory of several: builds of
+  // one size then get the same blocks again, and find their pass graphs made (60 us each)
   size_t best = kept.size();
   for (size_t i = 0; i < kept.size(); i++) {
-    const size_t n = kept[i].b.bytes;
-    if (n >= bytes && n <= 2 * bytes + 65536 && (best == kept.size() || n < kept[best].b.bytes))
+    const Block& b = kept[i].b;
+    if (b.bytes < bytes || b.bytes > 2 * bytes + 65536) continue;
+    if (best == kept.size() || b.bytes < kept[best].b.bytes ||
+        (b.bytes == kept[best].b.bytes && std::less<void*>()(b.p, kept[best].b.p)))
       best = i;
   }
   if (best < kept.size()) {

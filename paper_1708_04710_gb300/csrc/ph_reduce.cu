@@ -2859,8 +2859,15 @@ __device__ __forceinline__ bool grid_last(DevState* ds, unsigned blocks, unsigne
   return __syncthreads_and(ok);
 }
 
-constexpr int64_t kLoopBelow = (int64_t)1 << 14;  // columns from which k_loop takes over
-constexpr int64_t kLoopSingle = 64;  // columns left to one block
+// A call that begins with up to kLoopStart columns runs in k_loop alone: it saves the graph's launch
+// and the return to the host (about 100 us: 121,575 columns 1256 -> 1061 us, 36,050 columns 678 ->
+// 557 us, 43,904 of a batch 614 -> 472 us), while its passes over long lists are slower than the
+// graph's (166,750 columns, 8 passes: 500 us there, 580 us here). A call that begins in the graph
+// goes over to it at kLoopBelow columns (16,384 to 65,536 measure alike, 131,072 costs 50 to 90 us).
+constexpr int64_t kLoopBelow = (int64_t)1 << 14;
+constexpr int64_t kLoopStart = (int64_t)1 << 17;
+// columns left to one block, whose barriers are __syncthreads (64 and 256 measure alike)
+constexpr int64_t kLoopSingle = 64;
 constexpr int kLoopBlocks = 2;  // per SM: registers for every part of a pass without spills
 __global__ void __launch_bounds__(kThreads, kLoopBlocks) k_loop(RArgs a, int64_t m) {
   extern __shared__ __align__(16) unsigned char add_smem[];
@@ -2887,8 +2894,10 @@ __global__ void __launch_bounds__(kThreads, kLoopBlocks) k_loop(RArgs a, int64_t
       ess_count(a, m, blocks);
       if (!grid_sync(ds, blocks, target)) return;
     }
-    // few columns: narrow chunks, so that every warp has some
-    if (n <= 4 * kWarps) add_pass<true, 4, false, kThreads, true>(a, S, blocks);
+    // few columns: narrow chunks, so that every warp has some (a merge round of a warp takes 1.1 us
+    // whatever its share: 25 columns of some hundred rows 13.5 us by one warp, 6.5 us by seven)
+    if (n <= kWarps) add_pass<true, 1, false, kThreads, true>(a, S, blocks);
+    else if (n <= 4 * kWarps) add_pass<true, 4, false, kThreads, true>(a, S, blocks);
     else if (n <= 8 * kWarps * (int64_t)blocks) add_pass<true, 8, false, kThreads, true>(a, S, blocks);
     else add_pass<true, 32, false, kThreads, true>(a, S, blocks);
     if (!grid_sync(ds, blocks, target)) return;
@@ -2906,12 +2915,12 @@ __device__ __forceinline__ unsigned long long global_ns() {
 
 __global__ void k_clock_start(DevState* ds) { ds->t_start = global_ns(); }
 
-// blocks of the loop kernel for an active list of n columns: a warp for 8 columns, up to
-// kLoopMost blocks
+// blocks of the loop kernel for an active list of n columns: a warp for 8 columns, up to kLoopMost
+// blocks (a barrier of 64 blocks takes 1.4 us), then a thread for each
 constexpr int kLoopMost = 64;
 __host__ __device__ inline unsigned int loop_blocks_for(int64_t n) {
-  return n <= kLoopSingle ? 1u
-                          : (unsigned int)std::min<int64_t>((n + 8 * kWarps - 1) / (8 * kWarps), kLoopMost);
+  const int64_t per8 = (n + 8 * kWarps - 1) / (8 * kWarps), per32 = (n + kThreads - 1) / kThreads;
+  return n <= kLoopSingle ? 1u : (unsigned int)(per8 < kLoopMost ? per8 : per32 > kLoopMost ? per32 : kLoopMost);
 }
 
 // end of a pass: the next active list, convergence (no target left), the pass cap, the time
@@ -3277,11 +3286,11 @@ void reduce_init(ph_ctx* ctx) {
   PH_CUDA(cudaMemsetAsync(rs.dirty + nseg, 0, nseg * sizeof(int32_t), st));
   // Phase I's tile states; the loop kernel's tiles are of another size and have their own
   const int64_t ntiles = (m + kFTile - 1) / kFTile;
-  const int64_t loop_tiles = (std::min<int64_t>(m, kLoopBelow) + kThreads - 1) / kThreads;
+  const int64_t loop_tiles = (std::min<int64_t>(m, kLoopStart) + kThreads - 1) / kThreads;
   rs.tiles_bytes = (ntiles + 1 + loop_tiles) * sizeof(unsigned long long);
   rs.tiles = ctx->dalloc(rs.tiles_bytes);
   PH_CUDA(cudaMemsetAsync(rs.tiles, 0, rs.tiles_bytes, st));  // no state published yet
-  // chunks of any shape (8 slots or more; 4 for a few columns), or tiles
+  // chunks of any shape (8 slots or more; 1 or 4 for a few columns), or tiles
   const int64_t nchunks = (m + 7) / 8 + 1 + kWarps;
   rs.look = alloc_n<unsigned long long>(ctx, nchunks);
   PH_CUDA(cudaMemsetAsync(rs.look, 0, nchunks * sizeof(unsigned long long), st));
@@ -3465,7 +3474,7 @@ static unsigned loop_grid(ph_ctx* ctx) {
     PH_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctx->loop_blocks_per_sm, k_loop, kThreads,
                                                           kLoopSmem));
   const int64_t most = (int64_t)ctx->num_sms * ctx->loop_blocks_per_sm;
-  return (unsigned)std::min<int64_t>(most, kLoopMost);
+  return (unsigned)most;
 }
 
 // the pass loop as one graph: a conditional while node around one pass, with one of the
@@ -3564,6 +3573,7 @@ int reduce_run(ph_ctx* ctx, int32_t max_passes) {
   PH_CHECK_LAUNCH();
   const RArgs a = make_args(ctx);
 
+  bool started = false;    // this call has launched passes
   bool rest_only = false;  // a pass stopped for space after its marks continues at Phase II
   for (;;) {
     const int32_t first_pass = h.pass;
@@ -3574,7 +3584,8 @@ int reduce_run(ph_ctx* ctx, int32_t max_passes) {
       rest_only = false;
       launch_pass_rest(ctx, a, 0, false, variant, time_add, st);
       if (time_add) rs.add_launches++;
-    } else if (use_graph && loop_blocks && h.ahead == 1 && h.n_act <= h.loop_below) {
+    } else if (use_graph && loop_blocks && h.ahead == 1 &&
+               h.n_act <= (started ? h.loop_below : kLoopStart)) {
       h.loop_blocks = std::min(loop_blocks, loop_blocks_for(h.n_act));
       PH_CUDA(cudaMemcpyAsync(&static_cast<DevState*>(rs.dstate)->loop_blocks, &h.loop_blocks,
                               sizeof(h.loop_blocks), cudaMemcpyHostToDevice, st));
@@ -3591,6 +3602,7 @@ int reduce_run(ph_ctx* ctx, int32_t max_passes) {
       launch_pass(ctx, a, 0, false, variant, time_add, st);
       if (time_add) rs.add_launches++;
     }
+    started = true;
     PH_CUDA(cudaMemcpyAsync(&h, rs.dstate, sizeof(DevState), cudaMemcpyDeviceToHost, st));
     PH_CUDA(cudaStreamSynchronize(st));
     h.bar_count = 0;  // k_loop leaves a pass without space half-way
