@@ -143,3 +143,37 @@ def test_extraction_routes(ph, sizes, max_dim, passes):
         assert rc == 0
         got = raw[shift:2 * n.value + shift].cpu().numpy().view(np.int64)
         assert np.array_equal(got, pr["death"])
+
+
+# pairs are listed 2048 columns at a time and taken 256 at a time: 65 points have 2080 edges, 30 points
+# 4060 triangles and 406 pairs; points on the grid, so the 64-bit lengths come from the pairs
+@pytest.mark.parametrize("sizes,dim", [([65], 0), ([2, 65, 3, 30], 0), ([30, 3, 5], 1), ([3], 1),
+                                       ([40, 12], 1)])
+def test_diagram_loss_rounds(ph, sizes, dim):
+    import torch
+
+    clouds = [pc.random_cloud(n, 3, 1300 + n) for n in sizes]
+    off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+    x = torch.from_numpy((np.concatenate(clouds) / 65536).astype(np.float32)).cuda()
+    ctx = ph.Context()
+    ctx.build_filtration_f32(x, off if len(sizes) > 1 else None, dim + 1)
+    ctx.reduce()
+    loss = ctx.diagram_loss(x, dim).cpu().numpy()
+    w = torch.arange(1, len(sizes) + 1, dtype=torch.float32, device="cuda")
+    grad = ctx.diagram_backward(x, w, dim).cpu().numpy()
+    n_pairs = 0
+    for c in range(len(sizes)):
+        pr = ctx.pairs(c, on_device=False)
+        sel = pr["dim"].numpy() == dim
+        b, d = (np.sqrt(pr[k].numpy()[sel].astype(np.float64)) / 65536
+                for k in ("birth_diam2", "death_diam2"))
+        n_pairs += len(d)
+        want = ((d - b) ** 2).sum()
+        # a length is off by 4 roundings at most, a sum of positive terms by one per addition
+        bound = 2 ** -24 * (8 * (np.abs(d - b) * (d + b)).sum() + (len(d) / 256 + 16) * want)
+        assert abs(loss[c] - want) <= bound
+        # the gradient moves points along edges: it sums to zero, up to one rounding per addition
+        g = grad[off[c]:off[c + 1]]
+        size = 4 * (c + 1) * np.abs(d - b).sum()
+        assert np.abs(g.sum(0)).max() <= 2 ** -24 * (len(d) + 8) * max(size, 1e-30)
+    assert ctx.last_pairs == n_pairs
