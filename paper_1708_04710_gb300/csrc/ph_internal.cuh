@@ -161,6 +161,8 @@ struct ph_ctx {
   ph_allocator alloc{};
   bool has_alloc = false;
   ph::ReduceState::Loop loops[ph::ReduceState::kAddVariants];
+  std::vector<ph::ReduceState::Loop> retired;  // replaced, not yet given back
+  cudaStream_t capture_stream = nullptr;       // private: graphs are captured on it
   int loop_blocks_per_sm = -1;  // resident blocks of the loop kernel (-1: not asked yet)
   std::string err;
   int64_t launches = 0;  // kernels launched by this context
