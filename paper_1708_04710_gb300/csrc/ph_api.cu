@@ -360,7 +360,7 @@ __global__ void __launch_bounds__(kThreads) k_write_out(
 static void drop_extraction(ph_ctx* ctx) {
   for (void* p : {(void*)ctx->p_birth, (void*)ctx->p_death, (void*)ctx->p_dim, (void*)ctx->p_bd2,
                   (void*)ctx->p_dd2, (void*)ctx->e_idx, (void*)ctx->e_dim, (void*)ctx->e_d2,
-                  (void*)ctx->is_low, (void*)ctx->out_before, (void*)ctx->out_delta})
+                  (void*)ctx->out_before, (void*)ctx->out_delta})
     ctx->dfree(p);
   ctx->p_birth = ctx->p_death = ctx->p_bd2 = ctx->p_dd2 = ctx->e_idx = ctx->e_d2 = nullptr;
   ctx->p_dim = ctx->e_dim = nullptr;
@@ -379,13 +379,13 @@ static void extract_places(ph_ctx* ctx) {
   const int64_t nout = (m + kOutTile - 1) / kOutTile;
   const int nc = ctx->n_clouds;
   const int nseg = (int)ctx->seg_start.size() - 1;
-  ctx->is_low = alloc_n<uint8_t>(ctx, m);
-  // counts before each tile, the writers' error word, the scan's ticket, fault word and tile states
-  ctx->out_before = alloc_n<unsigned long long>(ctx, nout + 3 + ntiles);
+  // counts before each tile, the writers' error word, the scan's ticket, fault word and tile states,
+  // the image of low
+  ctx->out_before = alloc_n<unsigned long long>(ctx, nout + 3 + ntiles + (m + 7) / 8);
   ctx->out_delta = alloc_n<int64_t>(ctx, 2 * (nseg + 1));
   unsigned long long* words = ctx->out_before + nout;
-  PH_CUDA(cudaMemsetAsync(ctx->is_low, 0, m, st));
-  PH_CUDA(cudaMemsetAsync(words, 0, (3 + ntiles) * sizeof(unsigned long long), st));
+  ctx->is_low = reinterpret_cast<uint8_t*>(words + 3 + ntiles);
+  PH_CUDA(cudaMemsetAsync(words, 0, (3 + ntiles) * sizeof(unsigned long long) + m, st));
   k_mark_image<<<grid_for(ctx, m, kThreads), kThreads, 0, st>>>(m, ctx->low, ctx->is_low);
   PH_CHECK_LAUNCH();
   k_out_scan<<<(unsigned)ntiles, kThreads, 0, st>>>(

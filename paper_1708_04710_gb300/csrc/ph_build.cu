@@ -150,10 +150,11 @@ __device__ __forceinline__ void count_kept(int64_t* count_per_cloud, int c, bool
     atomicAdd((unsigned long long*)&count_per_cloud[c], (unsigned long long)__popc(peers));
 }
 
-// edge candidates in (cloud, lex) order; truncated edges get key = sent
+// edge candidates in (cloud, lex) order; truncated edges get key = sent, or, if given, a key of one
+// bit more than *largest. Kept ones are counted if some may be truncated
 __global__ void k_edge_cand(CloudTabs ct, const int64_t* __restrict__ cand, int64_t ncand,
                             const int64_t* __restrict__ d2, int64_t max_d2, uint64_t sent,
-                            uint64_t* keys, uint64_t* vals, int64_t* count_per_cloud) {
+                            const unsigned long long* largest, uint64_t* keys, uint64_t* vals, int64_t* count_per_cloud) {
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < ncand;
        t += (int64_t)gridDim.x * blockDim.x) {
     int c = find_cloud(cand, ct.nc, t);
@@ -162,9 +163,10 @@ __global__ void k_edge_cand(CloudTabs ct, const int64_t* __restrict__ cand, int6
     lex_unrank(t - cand[c], n, 2, v);
     int64_t e = d2[ct.mo[c] + (int64_t)v[0] * n + v[1]];
     bool keep = max_d2 < 0 || e <= max_d2;
+    if (largest && !keep) sent = (2ull << (64 - __clzll((long long)*largest))) - 1ull;
     keys[t] = keep ? (uint64_t)e : sent;
     vals[t] = pack_simplex((uint32_t)c, 2, v, ct.vbits);
-    count_kept(count_per_cloud, c, keep);
+    if (max_d2 >= 0) count_kept(count_per_cloud, c, keep);
   }
 }
 
@@ -987,19 +989,32 @@ void build_vr(ph_ctx* ctx, const int32_t* coords, const int64_t* cloud_offsets, 
   }
   // page-locked scratch: status words and per-cloud counts come back through it
   int64_t* h_misc = static_cast<int64_t*>(ctx->pinned((3 + 3 * ((int64_t)nc + 1)) * sizeof(int64_t)));
-  PH_CUDA(cudaMemcpyAsync(h_misc, d_misc, 2 * sizeof(int64_t), cudaMemcpyDeviceToHost, st));
-  PH_CUDA(cudaStreamSynchronize(st));
-  PH_REQUIRE(h_misc[0] == 0, PH_ERR_INVALID, "coordinates must lie in [-2^24, 2^24] grid units");
-  int64_t maxkey = h_misc[1];
-  if (scale_step > 0) {  // filtration values on the grid of scales: d2 -> scale index
-    PH_REQUIRE(n_scales >= 1 && scale_step <= (int64_t)1 << 26, PH_ERR_INVALID,
-               "the scale grid needs n_scales >= 1 and a step of at most 2^26 grid units");
-    k_scale_index<<<grid_for(ctx, nn, kThreads), kThreads, 0, st>>>(d2, nn, scale_step);
-    PH_CHECK_LAUNCH();
-    maxkey = scale_index_of(h_misc[1], scale_step);
-    max_diam2 = n_scales;  // simplices above the largest scale are left out
+  static const char* const kBadCoords = "coordinates must lie in [-2^24, 2^24] grid units";
+  // Every cloud's edges are sorted by one block, if they fit (truncated ones of several clouds have
+  // to come after all clouds' edges). That sort finds the largest squared distance by itself;
+  // otherwise the host needs it, to choose the digits or to put it on the grid of scales
+  int64_t longest = 0;
+  for (int c = 0; c < nc; c++) longest = std::max(longest, cand[2][c + 1] - cand[2][c]);
+  const bool tiles = longest <= kSortTile && (nc == 1 || (max_diam2 < 0 && scale_step == 0));
+  const unsigned long long* largest = nullptr;
+  int d2bits = 0;
+  if (tiles && scale_step == 0) {
+    largest = (const unsigned long long*)(d_misc + 1);
+  } else {
+    PH_CUDA(cudaMemcpyAsync(h_misc, d_misc, 2 * sizeof(int64_t), cudaMemcpyDeviceToHost, st));
+    PH_CUDA(cudaStreamSynchronize(st));
+    PH_REQUIRE(h_misc[0] == 0, PH_ERR_INVALID, kBadCoords);
+    int64_t maxkey = h_misc[1];
+    if (scale_step > 0) {  // filtration values on the grid of scales: d2 -> scale index
+      PH_REQUIRE(n_scales >= 1 && scale_step <= (int64_t)1 << 26, PH_ERR_INVALID,
+                 "the scale grid needs n_scales >= 1 and a step of at most 2^26 grid units");
+      k_scale_index<<<grid_for(ctx, nn, kThreads), kThreads, 0, st>>>(d2, nn, scale_step);
+      PH_CHECK_LAUNCH();
+      maxkey = scale_index_of(h_misc[1], scale_step);
+      max_diam2 = n_scales;  // simplices above the largest scale are left out
+    }
+    d2bits = bitlen((uint64_t)maxkey) + 1;  // one extra bit for the sentinel
   }
-  const int d2bits = bitlen((uint64_t)maxkey) + 1;  // one extra bit for the sentinel
 
   // ---------------- edges ----------------
   const int64_t ncand2 = cand[2][nc];
@@ -1014,15 +1029,10 @@ void build_vr(ph_ctx* ctx, const int32_t* coords, const int64_t* cloud_offsets, 
   std::vector<int64_t> h_cnt((int64_t)kMaxVrDim * nc, 0);  // per (dimension >= 1, cloud)
   if (cand[2][nc] > 0) {
     k_edge_cand<<<grid_for(ctx, cand[2][nc], kThreads), kThreads, 0, st>>>(
-        ct, d_cand(2), cand[2][nc], d2, max_diam2, sent_e, kbuf, vbuf, cnt_dim(1));
+        ct, d_cand(2), cand[2][nc], d2, max_diam2, sent_e, largest, kbuf, vbuf, cnt_dim(1));
     PH_CHECK_LAUNCH();
-    // every cloud's edges in one block, if they fit; truncated ones of several clouds have to
-    // come after all clouds' edges
-    int64_t longest = 0;
-    for (int c = 0; c < nc; c++) longest = std::max(longest, cand[2][c + 1] - cand[2][c]);
-    const bool tiles = longest <= kSortTile && (nc == 1 || max_diam2 < 0);
     if (tiles)
-      radix_sort_tiles(ctx, kbuf, vbuf, d_cand(2), nc, longest, 0, d2bits);
+      radix_sort_tiles(ctx, kbuf, vbuf, d_cand(2), nc, longest, 0, d2bits, largest);
     else
       radix_sort_u64(ctx, kbuf, vbuf, cand[2][nc], 0, d2bits, ktmp, vtmp, d_fault);
     if (nc > 1 && !tiles) {
@@ -1062,6 +1072,11 @@ void build_vr(ph_ctx* ctx, const int32_t* coords, const int64_t* cloud_offsets, 
 
   ctx->d2tab = alloc_n<int64_t>(ctx, std::max<int64_t>(E, 1));
   int64_t n_d2 = 0;
+  if (E == 0 && largest) {
+    PH_CUDA(cudaMemcpyAsync(h_misc, d_misc, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
+    PH_CUDA(cudaStreamSynchronize(st));
+    PH_REQUIRE(*(int32_t*)h_misc == 0, PH_ERR_INVALID, kBadCoords);
+  }
   if (E > 0) {
     int32_t* flag = alloc_n<int32_t>(ctx, E);
     int64_t* excl = alloc_n<int64_t>(ctx, E + 1);
@@ -1075,6 +1090,7 @@ void build_vr(ph_ctx* ctx, const int32_t* coords, const int64_t* cloud_offsets, 
     PH_CUDA(cudaMemcpyAsync(h_misc, d_misc, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
     PH_CUDA(cudaMemcpyAsync(h_misc + 1, excl + E, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
     PH_CUDA(cudaStreamSynchronize(st));
+    PH_REQUIRE(*(int32_t*)h_misc == 0, PH_ERR_INVALID, kBadCoords);
     PH_REQUIRE(h_misc[0] == 0, PH_ERR_CUDA, kSortFault);
     n_d2 = h_misc[1];
     ctx->dfree(flag);
@@ -1165,8 +1181,6 @@ void build_vr(ph_ctx* ctx, const int32_t* coords, const int64_t* cloud_offsets, 
         ctx->m, nc, max_dim, ctx->seg, ctx->key, ctx->d_seg_start, d_tabs, ctx->gidx);
     PH_CHECK_LAUNCH();
   }
-  PH_CUDA(cudaStreamSynchronize(st));
-
   ctx->dfree(kbuf);
   ctx->dfree(vbuf);
   ctx->dfree(ktmp);

@@ -120,6 +120,7 @@ struct ReduceState {
   uint64_t* set_key = nullptr;   // [4][rows] priority sort keys, rows, and their scratch
   int64_t tiles_bytes = 0;
   void* dstate = nullptr;      // per-pass state in device memory
+  bool fresh = false;         // set up, not run yet
   void* hstate = nullptr;      // pinned host mirror of it
   int64_t* pass_stats = nullptr;  // device [stats_rows][PH_PS_N]
   int32_t stats_rows = 0;
@@ -426,7 +427,8 @@ void reduced_columns(ph_ctx* ctx, int32_t cloud, int64_t n, int64_t* colptr, int
 void excl_scan_i64(ph_ctx* ctx, const int64_t* in, int64_t* out, int64_t n, int64_t* total_dev);
 constexpr int kSortTile = 8192;  // pairs that one block sorts
 void radix_sort_tiles(ph_ctx* ctx, uint64_t* keys, uint64_t* vals, const int64_t* off, int ntiles,
-                      int64_t longest, int lo_bit, int hi_bit);
+                      int64_t longest, int lo_bit, int hi_bit,
+                      const unsigned long long* largest = nullptr);
 void radix_sort_u64(ph_ctx* ctx, uint64_t* keys, uint64_t* vals, int64_t n, int lo_bit,
                     int hi_bit, uint64_t* tmp_keys, uint64_t* tmp_vals, int32_t* fault);
 void scan_counts(ph_ctx* ctx, const int32_t* a, const int32_t* b, int64_t n, int64_t* oa,

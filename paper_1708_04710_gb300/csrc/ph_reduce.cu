@@ -373,8 +373,11 @@ __device__ __forceinline__ void next_unpaired_last(const RArgs& a, unsigned bloc
   }
 }
 
-// set-up: the first pass's row state
-__global__ void k_rows_first(RArgs a) {
+__device__ __forceinline__ void first_tab(const RArgs& a);
+
+// set-up: the first pass's table and row state (independent of each other)
+__global__ void k_first(RArgs a) {
+  first_tab(a);
   rows_of_pass<true>(a, gridDim.x);
   if (last_block(&a.ds->blocks_done, gridDim.x)) {
     rows_of_pass_last(a);
@@ -412,10 +415,7 @@ __device__ __forceinline__ int32_t predicted_low(const RArgs& a, int32_t b, int3
 // marked as seen for the essential estimate. kTI consecutive slots per thread and iteration,
 // their loads issued together.
 constexpr int kTabItems = 4;
-__global__ void k_tab(RArgs a) {
-  pdl_wait();
-  pdl_trigger();
-  if (a.ds->status != ST_RUN) return;
+__device__ __forceinline__ void first_tab(const RArgs& a) {
   const PV v = pass_view(a.ds);
   constexpr int kTI = kTabItems;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x * kTI;
@@ -3400,12 +3400,11 @@ void reduce_init(ph_ctx* ctx) {
   // the first pass's row state and table (the later ones come from the pass before)
   {
     const RArgs a0 = make_args(ctx);
-    launch_k(ctx, false, k_rows_first, (unsigned)grid_for(ctx, a0.rows_end, kThreads), kThreads,
+    launch_k(ctx, false, k_first, (unsigned)grid_for(ctx, std::max(m, a0.rows_end), kThreads), kThreads,
              0, st, a0);
-    launch_k(ctx, false, k_tab, (unsigned)grid_for(ctx, m, kThreads * kTabItems), kThreads, 0, st,
-             a0);
   }
   rs.passes = 0;
+  rs.fresh = true;
   rs.init = true;
   rs.done = false;
   rs.status = PH_OK;
@@ -3533,8 +3532,7 @@ static cudaGraphExec_t pass_graph(ph_ctx* ctx, const RArgs& a, int variant) {
     PH_CUDA(ce);
   }
   const cudaStream_t cs = ctx->capture_stream;
-  ce = cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0,
-                                                 cudaStreamCaptureModeThreadLocal);
+  ce = cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
   if (ce != cudaSuccess) {
     cudaGraphDestroy(g);
     PH_CUDA(ce);
@@ -3565,8 +3563,11 @@ int reduce_run(ph_ctx* ctx, int32_t max_passes) {
   const bool time_add = ctx->opts.time_kernels != 0 && !use_graph;
   DevState& h = *static_cast<DevState*>(rs.hstate);
   // a resumed reduction continues after the pass that hit the previous cap
-  PH_CUDA(cudaMemcpyAsync(&h, rs.dstate, sizeof(DevState), cudaMemcpyDeviceToHost, st));
-  PH_CUDA(cudaStreamSynchronize(st));
+  if (!rs.fresh) {  // (what set-up wrote is still in the host's copy)
+    PH_CUDA(cudaMemcpyAsync(&h, rs.dstate, sizeof(DevState), cudaMemcpyDeviceToHost, st));
+    PH_CUDA(cudaStreamSynchronize(st));
+  }
+  rs.fresh = false;
   if (h.status == ST_CAPPED) {  // every column is up to date there
     h.pass = h.passes + 1;
     h.status = ST_RUN;

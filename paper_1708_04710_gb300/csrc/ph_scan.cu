@@ -249,11 +249,13 @@ __global__ void __launch_bounds__(kThreads) k_radix_pass(
 }
 
 // All digits of one tile per block: elements stay in registers and change places in shared memory.
-// Tile b: elements off[b] .. off[b + 1], or all n without off; at most NW * 256.
+// Tile b: elements off[b] .. off[b + 1], or all n without off; at most NW * 256. largest (device):
+// the keys have one bit more than this value, instead of `digits`
 template <int NW>
 __global__ void __launch_bounds__(NW * 32) k_radix_tiles(uint64_t* keys, uint64_t* vals,
                                                          const int64_t* __restrict__ off, int64_t n,
-                                                         int lo_bit, int digits) {
+                                                         int lo_bit, int digits,
+                                                         const unsigned long long* largest) {
   extern __shared__ uint64_t sm[];
   uint64_t* xk = sm;
   uint64_t* xv = xk + NW * 256;
@@ -261,6 +263,7 @@ __global__ void __launch_bounds__(NW * 32) k_radix_tiles(uint64_t* keys, uint64_
   __shared__ unsigned base[256], sums[8];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int64_t first = off ? off[blockIdx.x] : 0;
+  if (largest) digits = (min(64, 65 - __clzll((long long)*largest)) + 7) / 8;
   const int len = (int)(off ? off[blockIdx.x + 1] - first : n);
   keys += first;
   vals += first;
@@ -314,24 +317,29 @@ __global__ void __launch_bounds__(NW * 32) k_radix_tiles(uint64_t* keys, uint64_
 
 template <int NW>
 static void launch_tiles(ph_ctx* ctx, uint64_t* keys, uint64_t* vals, const int64_t* off,
-                         int ntiles, int64_t n, int lo_bit, int digits) {
+                         int ntiles, int64_t n, int lo_bit, int digits,
+                         const unsigned long long* largest) {
   constexpr size_t bytes = NW * 256 * 16 + NW * 257 * sizeof(unsigned);
   if (bytes > 48 * 1024)
     PH_CUDA(cudaFuncSetAttribute(k_radix_tiles<NW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)bytes));
-  k_radix_tiles<NW><<<ntiles, NW * 32, bytes, ctx->stream>>>(keys, vals, off, n, lo_bit, digits);
+  k_radix_tiles<NW><<<ntiles, NW * 32, bytes, ctx->stream>>>(keys, vals, off, n, lo_bit, digits,
+                                                             largest);
   PH_CHECK_LAUNCH();
 }
 
 // sorts each of ntiles ranges (off[t] .. off[t + 1], device) of at most longest <= kSortTile pairs
-// by itself, in one kernel; off null: one range of longest pairs
+// by itself, in one kernel; off null: one range of longest pairs. largest: see k_radix_tiles
 void radix_sort_tiles(ph_ctx* ctx, uint64_t* keys, uint64_t* vals, const int64_t* off, int ntiles,
-                      int64_t longest, int lo_bit, int hi_bit) {
-  if (longest <= 1 || hi_bit <= lo_bit) return;
+                      int64_t longest, int lo_bit, int hi_bit, const unsigned long long* largest) {
+  if (longest <= 1 || (!largest && hi_bit <= lo_bit)) return;
   const int digits = (hi_bit - lo_bit + 7) / 8;
-  if (longest <= 2048) launch_tiles<8>(ctx, keys, vals, off, ntiles, longest, lo_bit, digits);
-  else if (longest <= 4096) launch_tiles<16>(ctx, keys, vals, off, ntiles, longest, lo_bit, digits);
-  else launch_tiles<32>(ctx, keys, vals, off, ntiles, longest, lo_bit, digits);
+  if (longest <= 2048) launch_tiles<8>(ctx, keys, vals, off, ntiles, longest, lo_bit, digits,
+                                        largest);
+  else if (longest <= 4096) launch_tiles<16>(ctx, keys, vals, off, ntiles, longest, lo_bit, digits,
+                                        largest);
+  else launch_tiles<32>(ctx, keys, vals, off, ntiles, longest, lo_bit, digits,
+                                        largest);
 }
 
 // fault: device word, set when a bounded wait ran out (the order is then incomplete)
