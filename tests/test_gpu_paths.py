@@ -177,3 +177,72 @@ def test_diagram_loss_rounds(ph, sizes, dim):
         size = 4 * (c + 1) * np.abs(d - b).sum()
         assert np.abs(g.sum(0)).max() <= 2 ** -24 * (len(d) + 8) * max(size, 1e-30)
     assert ctx.last_pairs == n_pairs
+
+
+def _state(ctx, cloud=0):
+    ptr, rows = ctx.columns(cloud)
+    return ctx.filtration(cloud)["low"], ptr, rows, ctx.essential_estimate(cloud)
+
+
+def _same_reduction(ph, build, opts, caps, cloud=0):
+    """A context with per-pass counters takes every pass of every column, in k_add."""
+    ref = ph.Context(**{**opts, "collect_stats": True, "use_graph": False})
+    got = ph.Context(**opts)
+    for ctx in (ref, got):
+        build(ctx)
+    for cap in caps:
+        st = []
+        for ctx in (ref, got):
+            ctx.reset_reduction()
+            st.append(ctx.reduce(max_passes=cap))
+        assert st[0]["passes"] == st[1]["passes"] and st[0]["converged"] == st[1]["converged"]
+        for r, g in zip(_state(ref, cloud), _state(got, cloud)):
+            assert np.array_equal(r, g), (opts, cap)
+    for ctx in (ref, got):  # in steps: a call resumes where the last one stopped
+        ctx.reset_reduction()
+        for cap in (2, 3, 9, 10):
+            ctx.reduce(max_passes=cap)
+        ctx.reduce()
+    for r, g in zip(_state(ref, cloud), _state(got, cloud)):
+        assert np.array_equal(r, g), opts
+
+
+# from 3,000,000 columns of at most three rows a visit runs up to eight passes of a column; a cap,
+# a horizon of eight passes, zeroing rules, bit-packed columns and space stops cut through that
+@pytest.mark.parametrize("opts", [
+    {}, {"strict_phase2": True}, {"use_cor10": False}, {"dense_threshold": 1}, {"arena_words": 1},
+    {"use_graph": False}, {"predict_pairs": True},
+], ids=str)
+def test_look_ahead_equals_pass_by_pass(ph, opts):
+    x = pc.to_grid(pc.sphere(270, np.random.Generator(np.random.PCG64(3)), noise=0.05))
+    _same_reduction(ph, lambda c: _build(c, [x], 2), opts, (1, 7, 8, 9, -1))
+
+
+def test_look_ahead_of_a_batch(ph):
+    clouds = [pc.random_cloud(60 + i % 17, 3, 1500 + i) for i in range(64)]
+    assert sum(len(c) * (len(c) - 1) * (len(c) - 2) // 6 for c in clouds) > 3_000_000
+    _same_reduction(ph, lambda c: _build(c, clouds, 2), {}, (4, -1), cloud=37)
+
+
+# the loop kernel: 1, 4, 8 or 32 columns per warp (8, 32, 64 columns, then 8 per warp of up to 64
+# blocks), one block up to 64 columns, several tiles per block above 77,824 (90 points), and 93 points
+# (134,230 columns) that begin in the pass graph; a lack of space stops it within a pass
+@pytest.mark.parametrize("n", [3, 4, 5, 7, 8, 12, 17, 40, 90, 93])
+@pytest.mark.parametrize("opts", [{}, {"arena_words": 1}, {"predict_pairs": True}], ids=str)
+def test_loop_kernel_equals_host_loop(ph, n, opts):
+    x = pc.random_cloud(n, 2, 1700 + n)
+    _same_reduction(ph, lambda c: _build(c, [x], 2), opts, (0, 1, 3, -1))
+
+
+def test_rebuilt_contexts(ph):
+    """Blocks, graphs and pinned memory that a context keeps hold nothing of an earlier build."""
+    ctx = ph.Context()
+    for i, (n, max_dim) in enumerate([(93, 2), (93, 2), (40, 2), (93, 2), (30, 3), (95, 2), (93, 2)]):
+        x = pc.random_cloud(n, 3, 1900 + i)
+        fresh = _build(ph.Context(), [x], max_dim)
+        _build(ctx, [x], max_dim)
+        assert ctx.reduce()["passes"] == fresh.reduce()["passes"]
+        for r, g in zip(_state(fresh), _state(ctx)):
+            assert np.array_equal(r, g)
+        for a, b in ((fresh.pairs(), ctx.pairs()), (fresh.essential(), ctx.essential())):
+            assert all(np.array_equal(a[k].cpu(), b[k].cpu()) for k in a)
