@@ -467,14 +467,15 @@ static bool writable(ph_ctx* ctx, const void* p, size_t align) {
          reinterpret_cast<uintptr_t>(p) % align == 0;
 }
 
-__global__ void k_inspect(int64_t lo, int64_t hi, const int32_t* __restrict__ seg, int nc,
+__global__ void k_inspect(CloudIds ids, const int32_t* __restrict__ seg, int nc,
                           const int64_t* __restrict__ gidx, const int32_t* __restrict__ key,
                           const int64_t* __restrict__ d2tab, const uint64_t* __restrict__ verts,
                           const int32_t* __restrict__ beta, const int32_t* __restrict__ low,
                           int32_t* o_dim, int64_t* o_d2, int32_t* o_v, int32_t* o_beta,
                           int32_t* o_low, int64_t n, int vbits, int32_t* bad) {
-  for (int64_t x = lo + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < hi;
-       x += (int64_t)gridDim.x * blockDim.x) {
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < ids.n;
+       t += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t x = ids.id(t);
     int64_t g = gidx[x];
     if (g < 0 || g >= n) {
       *bad = 1;
@@ -819,16 +820,13 @@ int ph_get_filtration(ph_ctx* ctx, int32_t cloud, int32_t* dim, int64_t* diam2, 
   int32_t* o_low = ph::alloc_n<int32_t>(ctx, n);
   int32_t* d_bad = ph::alloc_n<int32_t>(ctx, 1);
   PH_CUDA(cudaMemsetAsync(d_bad, 0, sizeof(int32_t), ctx->stream));
-  for (int d = 0; d <= ctx->max_dim; d++) {
-    int64_t lo = ctx->seg_start[d * nc + cloud], hi = ctx->seg_start[d * nc + cloud + 1];
-    if (hi <= lo) continue;
-    ph::k_inspect<<<ph::grid_for(ctx, hi - lo, ph::kThreads), ph::kThreads, 0, ctx->stream>>>(
-        lo, hi, ctx->seg, nc, ctx->gidx, ctx->key, ctx->d2tab, ctx->verts, ctx->beta, ctx->low,
-        o_dim, o_d2, o_v, o_beta, o_low, n, ctx->vbits, d_bad);
-    PH_CHECK_LAUNCH();
-  }
-  int32_t bad = 0;
-  PH_CUDA(cudaMemcpyAsync(&bad, d_bad, sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
+  const ph::CloudIds ids = ph::cloud_ids(ctx, cloud);
+  ph::k_inspect<<<ph::grid_for(ctx, ids.n, ph::kThreads), ph::kThreads, 0, ctx->stream>>>(
+      ids, ctx->seg, nc, ctx->gidx, ctx->key, ctx->d2tab, ctx->verts, ctx->beta, ctx->low, o_dim, o_d2,
+      o_v, o_beta, o_low, n, ctx->vbits, d_bad);
+  PH_CHECK_LAUNCH();
+  int32_t* bad = static_cast<int32_t*>(ctx->pinned(sizeof(int32_t)));
+  PH_CUDA(cudaMemcpyAsync(bad, d_bad, sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
   copy_out(ctx, dim, o_dim, n * 4, 0);
   copy_out(ctx, diam2, o_d2, n * 8, 0);
   copy_out(ctx, verts, o_v, n * 4 * ph::kVrSlots, 0);
@@ -838,7 +836,7 @@ int ph_get_filtration(ph_ctx* ctx, int32_t cloud, int32_t* dim, int64_t* diam2, 
   for (void* p : {(void*)o_dim, (void*)o_d2, (void*)o_v, (void*)o_beta, (void*)o_low,
                   (void*)d_bad})
     ctx->dfree(p);
-  PH_REQUIRE(bad == 0, PH_ERR_INVALID, "internal error: filtration index out of range");
+  PH_REQUIRE(*bad == 0, PH_ERR_INVALID, "internal error: filtration index out of range");
   return PH_OK;
   PH_API_END
 }

@@ -405,6 +405,19 @@ __device__ __forceinline__ int64_t tile_prefix(unsigned long long* st, int64_t t
 
 // host entry points shared between translation units
 namespace ph {
+// the ids of one cloud, dimension by dimension: one launch covers them all
+struct CloudIds {
+  int64_t n = 0;                     // simplices of the cloud
+  int64_t first[kMaxDim + 2] = {0};  // per dimension: those of lower dimensions
+  int64_t lo[kMaxDim + 1] = {0};     // ... and its first id
+  int nd = 0;
+  __device__ __forceinline__ int64_t id(int64_t t) const {
+    int d = 0;
+    while (d + 1 < nd && t >= first[d + 1]) d++;
+    return lo[d] + (t - first[d]);
+  }
+};
+CloudIds cloud_ids(const ph_ctx* ctx, int32_t cloud);
 // scale_step > 0: simplices enter at the first scale r_i = i * scale_step (grid units,
 // i = 0..n_scales) with diameter <= 2 r_i, and the filtration value is i
 void build_vr(ph_ctx* ctx, const int32_t* coords, const int64_t* cloud_offsets, int32_t n_clouds,
@@ -424,7 +437,6 @@ void predicted_lows(ph_ctx* ctx, int32_t cloud, int32_t* host_out, int64_t n);
 void reduced_columns(ph_ctx* ctx, int32_t cloud, int64_t n, int64_t* colptr, int32_t* rows,
                      int64_t capacity, int64_t* nnz_out);
 // generic device helpers (ph_scan.cu)
-void excl_scan_i64(ph_ctx* ctx, const int64_t* in, int64_t* out, int64_t n, int64_t* total_dev);
 constexpr int kSortTile = 8192;  // pairs that one block sorts
 void radix_sort_tiles(ph_ctx* ctx, uint64_t* keys, uint64_t* vals, const int64_t* off, int ntiles,
                       int64_t longest, int lo_bit, int hi_bit,

@@ -1,9 +1,7 @@
 // Device scans and the LSD radix sort used to order simplices by squared diameter.
 //
-// Both are tile based: a tile is kThreads * kItems consecutive elements handled by one block.
-// excl_scan_i64: (1) per-tile reduction, (2) one block scans the tile aggregates, (3) per-tile scan
-// with the tile's prefix. The others take one kernel, whose tiles wait for earlier ones (in order,
-// with a bound).
+// Both are tile based: a tile is kThreads * kItems consecutive elements handled by one block. Tiles
+// take their turns from a ticket and wait for earlier ones (with a bound).
 #include <utility>
 
 #include "ph_internal.cuh"
@@ -12,68 +10,6 @@ namespace ph {
 
 constexpr int kItems = 8;
 constexpr int kTile = kThreads * kItems;
-
-// ---------------------------------------------------------------------------------------------
-// exclusive scan of int64
-// ---------------------------------------------------------------------------------------------
-__global__ void k_tile_sum_i64(const int64_t* __restrict__ in, int64_t n, int64_t* tile_sums) {
-  __shared__ int64_t sh[kWarps + 1];
-  int64_t base = (int64_t)blockIdx.x * kTile;
-  int64_t s = 0;
-  for (int it = 0; it < kItems; it++) {
-    int64_t i = base + it * kThreads + threadIdx.x;
-    if (i < n) s += in[i];
-  }
-  int64_t total;
-  block_excl_sum<int64_t>(s, sh, total);
-  if (threadIdx.x == 0) tile_sums[blockIdx.x] = total;
-}
-
-// single block: exclusive scan of the tile sums in place; writes the grand total
-__global__ void k_scan_tiles_i64(int64_t* sums, int64_t ntiles, int64_t* total_out) {
-  __shared__ int64_t sh[kWarps + 1];
-  int64_t carry = 0;
-  for (int64_t base = 0; base < ntiles; base += kThreads) {
-    int64_t i = base + threadIdx.x;
-    int64_t v = i < ntiles ? sums[i] : 0;
-    int64_t tot;
-    int64_t ex = block_excl_sum<int64_t>(v, sh, tot);
-    if (i < ntiles) sums[i] = carry + ex;
-    carry += tot;
-  }
-  if (threadIdx.x == 0 && total_out) *total_out = carry;
-}
-
-__global__ void k_tile_scan_i64(const int64_t* __restrict__ in, int64_t* out, int64_t n,
-                                const int64_t* __restrict__ tile_prefix) {
-  __shared__ int64_t sh[kWarps + 1];
-  int64_t base = (int64_t)blockIdx.x * kTile;
-  int64_t carry = tile_prefix[blockIdx.x];
-  for (int it = 0; it < kItems; it++) {
-    int64_t i = base + it * kThreads + threadIdx.x;
-    int64_t v = i < n ? in[i] : 0;
-    int64_t tot;
-    int64_t ex = block_excl_sum<int64_t>(v, sh, tot);
-    if (i < n) out[i] = carry + ex;
-    carry += tot;
-  }
-}
-
-void excl_scan_i64(ph_ctx* ctx, const int64_t* in, int64_t* out, int64_t n, int64_t* total_dev) {
-  int64_t ntiles = (n + kTile - 1) / kTile;
-  if (ntiles == 0) {
-    if (total_dev) PH_CUDA(cudaMemsetAsync(total_dev, 0, sizeof(int64_t), ctx->stream));
-    return;
-  }
-  int64_t* sums = alloc_n<int64_t>(ctx, ntiles);
-  k_tile_sum_i64<<<(unsigned)ntiles, kThreads, 0, ctx->stream>>>(in, n, sums);
-  PH_CHECK_LAUNCH();
-  k_scan_tiles_i64<<<1, kThreads, 0, ctx->stream>>>(sums, ntiles, total_dev);
-  PH_CHECK_LAUNCH();
-  k_tile_scan_i64<<<(unsigned)ntiles, kThreads, 0, ctx->stream>>>(in, out, n, sums);
-  PH_CHECK_LAUNCH();
-  ctx->dfree(sums);
-}
 
 // ---------------------------------------------------------------------------------------------
 // exclusive scans of one or two int32 arrays into int64 (n + 1 values each, the total last), in one
