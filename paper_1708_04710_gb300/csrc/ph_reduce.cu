@@ -4,11 +4,12 @@
 // the state at its start, so the result of a pass does not depend on thread scheduling:
 //   (table)      tab[low(j)] = min j over the active columns and the pivots: the left-most
 //                column with each low, which defines the neighbour sets N(j) (Eq. neighbours).
-//                Two tables alternate between passes: the pass before resets one to the proven
-//                pivots (owner), and its new pivots (k_phase1) and its survivors with their new
-//                lows (k_add, atomicMin) fill it, so no kernel gathers the lows again; k_tab
-//                builds the first pass's at set-up. With it, the first row of each (cloud, dim)
-//                that is not known to be paired (for Corollary 10).
+//                One 64-bit word per row whose high half falls from pass to pass, so the entries
+//                of a pass beat those of earlier ones in an atomicMin and nothing is reset (a
+//                proven pivot's entry has high half 0 and stays); the survivors of a pass enter
+//                the next one's as their new lows appear, so no kernel gathers the lows
+//                again; k_first fills the first pass's at set-up. With it, the first row of each
+//                (cloud, dim) that is not known to be paired (for Corollary 10).
 //   k_phase1     Phase I (Algorithm 5) as a segmented exclusive prefix-max over the active
 //                columns of each (cloud, dim), P_j = largest low of an earlier colliding column,
 //                in one pass over tiles with a decoupled look-back; then the marks: j is proven
@@ -32,15 +33,23 @@
 //                pieces. Ten specialisations (row lists / bitmaps x block / 32-slot warp
 //                chunks x lane / piece merges, and 8-slot warp chunks with pieces); the loop
 //                switches between them at most four times per reduction.
+//   k_visit,     Phase II for long lists of columns of at most three rows (look-ahead): nineteen
+//   k_merge      of twenty additions have a proven pivot as their source, which will not change
+//                any more, so a visit runs up to eight passes of a column at once as long as its
+//                low meets proven pivots of few rows; the lows on the way are stored for the
+//                passes they belong to. What was added is kept beside the column's list (its
+//                delta) and merged into it every eighth pass. Lows, marks, pass counts and the
+//                reduced matrix are those of the pass-by-pass run.
 //   (p sets)     With Phase II limited to p neighbour sets (Sec. 3.4), k_set_* rank the sets
 //                between k_phase1 and k_add and hold back the other targets.
 //   k_commit     publishes the new locations of the columns other jobs may have been reading
-//                and prepares the next pass's row state; its last block ends the pass: the
-//                next active list, convergence (no collision left, Thm 8), the pass cap and
+//                and moves on the first unpaired row of the segments where it was paired; its last
+//                block ends the pass: the next active list, convergence (no collision left, Thm 8), the pass cap and
 //                time bound, and inside a CUDA graph the conditional that repeats the pass.
 // All per-pass state lives in device memory (DevState), so the same kernel sequence runs either
 // from a host loop or as the body of a graph's conditional while node. Each kernel may start
-// while its predecessor drains (programmatic dependent launch) and waits for it first.
+// while its predecessor drains (programmatic dependent launch) and waits for it first. Short lists
+// run in k_loop, one cooperative kernel for all their passes.
 #include <algorithm>
 #include <cstring>
 #include <utility>
@@ -53,7 +62,7 @@ namespace ph {
 enum : int32_t { ST_RUN = 0, ST_DONE = 1, ST_CAPPED = 2, ST_HOST = 3, ST_FAULT = 4,
                  ST_TIMEOUT = 5, ST_SWITCH = 6 };
 constexpr int kSpinLimit = 1 << 22;  // iterations of a look-back wait before it gives up
-constexpr int kBarrierLimit = 1 << 24;  // ... of a grid barrier's (a second or so)
+constexpr int kBarrierLimit = 1 << 24;  // ... of a grid barrier's (some seconds)
 
 struct DevState {
   int32_t* act;   // active ids, ascending
@@ -318,7 +327,8 @@ __device__ void rows_of_pass_last(const RArgs& a) {
 // the first pass, or when the row that held up a long run of paired ones is paired at last.
 // A few segments are searched by all blocks together, in strides that end once a lower row is
 // found, and next_unpaired_last, by the last block, takes over the result; many (of a batch, or
-// by a single block) by one block each.
+// by a single block) by one block each. (One block alone took 455 us over all passes of 120 points in
+// 8-d, whose next row is far.)
 constexpr unsigned kSearchTogether = 4;
 __device__ __forceinline__ void next_unpaired(const RArgs& a, unsigned blocks) {
   const unsigned nd = a.ds->n_dirty;
@@ -532,6 +542,13 @@ constexpr int kAheadMax = 8;  // passes per visit (a power of two: rows of store
 // dimensions, 120 points, 0.9 M simplices, 1.8 -> 2.8 ms.)
 constexpr int kSourceRows = 2;
 constexpr int kOld = 8;
+// Look-ahead is bound by instruction issue (some 230 warp instructions per pass of a visit) where
+// pass-by-pass additions are bound by memory traffic: every pass rewrites every column and reads its
+// source. Pass by pass -> look-ahead: 10.67 M columns (400 points on a torus) 48.8 -> 36.9 ms, 4.5 M
+// on a torus 29.2 -> 22.6 ms, on a sphere 12.8 -> 8.7 ms, 42.7 M in 512 clouds 45.5 -> 41.8 ms; on
+// 2.6 M columns 11.9 -> 11.8 ms, on 1.3 M 6.5 -> 6.2 ms, on 0.9 M 4.4 -> 4.3 ms: little to gain
+// below kAheadFrom, where a visit's two kernels and the larger tables also cost memory. Lists that
+// shrink under kAheadAbove go on pass by pass (half and twice as many measure alike).
 constexpr int64_t kAheadFrom = 3000000;   // columns from which look-ahead pays, and
 constexpr int64_t kAheadAbove = 500000;   // down to which it goes on
 constexpr int kLonger = 12;  // the longest source inside a visit: kRecRows + this many rows
@@ -2808,7 +2825,10 @@ __global__ void k_commit(RArgs a, cudaGraphConditionalHandle cond, int mode) {
 // On a short active list a pass's kernels take some microseconds each, whatever they do: launch,
 // first loads, last-block handshakes, drain. k_loop runs all passes in one cooperative grid
 // (every block resident, so they may wait for each other), the parts of a pass separated by
-// grid barriers.
+// grid barriers. Bound by latency: a pass is a chain of some forty loads and atomics that wait for
+// L2, and three barriers (10,700 columns: 3.5 us Phase I, 7 us additions, 2 us commit, 8 us barriers
+// and the end of the pass). As kernels of a graph 18 passes of 10,700 columns took 739 us, here 490;
+// 237 passes of a 96 x 80 image grid 6.6 ms, here 2.6 to 3.1.
 //
 // A grid barrier is one counter: every block adds one and waits until all of the pass's blocks have,
 // that many times the barriers so far (`target`). What was written before it is visible after it.
