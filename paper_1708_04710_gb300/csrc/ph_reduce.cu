@@ -553,12 +553,20 @@ constexpr int64_t kAheadFrom = 3000000;   // columns from which look-ahead pays,
 constexpr int64_t kAheadAbove = 500000;   // down to which it goes on
 constexpr int kLonger = 12;  // the longest source inside a visit: kRecRows + this many rows
 constexpr int kDeltaRows = kOld + kSourceRows * kAheadMax;
+// words per row of stored lows, and of due words: threads read eight slots in two 16-byte loads
+__host__ __device__ inline int64_t lows_stride_of(int64_t m) { return (m + 7) & ~int64_t(7); }
 
 // The rows of a row's proven pivot, one 16-byte record: x is its length (0: no pivot yet), y, z
 // and w its rows below the low, then INT32_MAX (length <= kRecRows), or y and z the address of its rows. A
 // bit-packed pivot's record holds kRecLong alone.
 constexpr int32_t kRecRows = 4;
 constexpr int32_t kRecLong = INT32_MAX;
+
+// The word of a slot that says when its column is visited next: the pass itself, ~pass for a column
+// without beta, which Corollary 10 may zero, kDeadDue for a slot whose column left. A pass before the
+// horizon needs no more of a column ahead of it than this word and the stored low.
+constexpr int32_t kDeadDue = INT32_MAX;
+__device__ __forceinline__ int32_t due_pass(int32_t d) { return d < 0 ? ~d : d; }
 
 __device__ __forceinline__ int32_t dead_slot(int32_t j) { return -2 - j; }
 __device__ __forceinline__ int32_t slot_id(int32_t a) { return a >= 0 ? a : -2 - a; }
@@ -718,6 +726,12 @@ __device__ __forceinline__ SegMax tile_value(unsigned long long w) {
   return SegMax{(int32_t)((w >> 31) & 0x7fffff), (int32_t)(w & 0x7fffffffu) - 1};
 }
 
+__device__ __forceinline__ void tile_publish(unsigned long long* st, int32_t pass, int64_t t,
+                                             SegMax agg) {
+  const unsigned long long tag = (unsigned long long)(pass & 0xff) << 56;
+  atomicExch(st + t, tile_word(tag, t == 0 ? kTIncl : kTAgg, agg));
+}
+
 // by warp 0: publishes tile t's aggregate, returns the Phase I value of every tile before it
 // (SegMax{-1, -1}, a left identity of segmax_combine, for none) and publishes t's inclusive state
 __device__ __forceinline__ SegMax tile_look_back(unsigned long long* st, int32_t pass, int64_t t,
@@ -725,11 +739,8 @@ __device__ __forceinline__ SegMax tile_look_back(unsigned long long* st, int32_t
   const int lane = lane_id();
   const unsigned long long tag = (unsigned long long)(pass & 0xff) << 56;
   const SegMax none{-1, -1};
-  if (t == 0) {
-    if (lane == 0) atomicExch(st, tile_word(tag, kTIncl, agg));
-    return none;
-  }
-  if (lane == 0) atomicExch(st + t, tile_word(tag, kTAgg, agg));
+  if (lane == 0) tile_publish(st, pass, t, agg);
+  if (t == 0) return none;
   SegMax acc = none;
   bool have = false;
   for (int64_t p = t - 1;; p -= 32) {
@@ -830,7 +841,7 @@ __device__ __forceinline__ void phase1_pass(const RArgs& a, unsigned parts) {
       j[i] = e0 + i < v.n_act ? v.act[e0 + i] : INT32_MIN;
       s[i] = l[i] = -1;
       if (ahead > 1 && e0 + i < v.n_act) {
-        if (a.due[e0 + i] > pass) s[i] = kAhead;
+        if (due_pass(a.due[e0 + i]) > pass) s[i] = kAhead;
         l[i] = lows[e0 + i];
       }
     }
@@ -870,8 +881,17 @@ __device__ __forceinline__ void phase1_pass(const RArgs& a, unsigned parts) {
     for (int i = 1; i < kFI; i++) agg = segmax_combine(agg, x[i]);
     SegMax tot;
     const SegMax pre_t = block_scan_segmax(agg, SegMax{-1, -1}, sh, tot);  // within the tile
-    if (threadIdx.x < 32) {
-      const SegMax P = tile_look_back(kLoop ? a.loop_tile_st : a.tile_st, pass, t, tot, fault);
+    // a tile without a mark that needs P_j only publishes its value (every 16th its prefix, so that
+    // walks stay short): 24 clouds, 2.28 M columns 3250 -> 3165 us, 10,700 columns 468 -> 448 us
+    bool needs = false;
+#pragma unroll
+    for (int i = 0; i < kFI; i++) needs |= l[i] >= 0 && s[i] == j[i] && l[i] != b[i];
+    unsigned long long* tile_st = kLoop ? a.loop_tile_st : a.tile_st;
+    needs = __syncthreads_or(needs) || (t & 15) == 0;
+    if (!needs) {
+      if (threadIdx.x == 0) tile_publish(tile_st, pass, t, tot);
+    } else if (threadIdx.x < 32) {
+      const SegMax P = tile_look_back(tile_st, pass, t, tot, fault);
       if (threadIdx.x == 0) s_pre = P;
     }
     // the marks: a new pivot proven by Thm 5 (left-most, low = beta) or by Phase I (left-most,
@@ -905,6 +925,7 @@ __device__ __forceinline__ void phase1_pass(const RArgs& a, unsigned parts) {
         a.meta[j[i]].len = 0;
         a.low[j[i]] = -1;
         v.act[e0 + i] = dead_slot(j[i]);
+        a.due[e0 + i] = kDeadDue;
       }
     };
     auto unproven = [&](int i) {  // true: zeroed
@@ -1005,6 +1026,195 @@ __device__ __forceinline__ void phase1_pass(const RArgs& a, unsigned parts) {
   }
 }
 
+// Phase I of a look-ahead pass before the horizon (no pair predictions). Nineteen of twenty columns
+// are ahead of it: their due word and stored low are all there is to read, eight slots per thread in
+// four loads, and what is left to do for one is the zero case of Corollary 10. The others' slots are
+// listed in shared memory and taken by one thread each. Bound by the chain of waits of each tile:
+// phase1_pass, which reads every slot's column, segment and beta, took 95 to 130 us for such a pass of
+// 10.67 M columns, this takes 50 to 100 us (the 85 MB of due words and lows would take 13 us). The
+// reduction of 10.67 M columns 36.0 -> 34.8 ms, of 42.7 M in 512 clouds 41.5 -> 39.7 ms.
+constexpr int kMidItems = 8, kMidTile = kThreads * kMidItems;
+__device__ __forceinline__ void mark_pivot(const RArgs& a, const int32_t* fu, int32_t j, int32_t l,
+                                           int32_t sg) {
+  auto dirty = [&](int32_t seg) {
+    if (atomicExch(&a.dirty_on[seg], 1) == 0) a.dirty[atomicAdd(&a.ds->n_dirty, 1u)] = seg;
+  };
+  const ColMeta mj = load_meta(a.meta + j);
+  a.prec[l] = rec_of(mj.ptr, mj.len);
+  a.meta[j].flags = F_PROVEN | F_NEWPIV;
+  a.owner[l] = j;
+  a.tab[l] = (unsigned)j;  // its row's left-most column from now on (as it is now)
+  if (l == fu[sg - a.nc]) dirty(sg - a.nc);
+  if (j == fu[sg]) dirty(sg);
+  a.meta[l].cleared = 1;  // clearing (Lemma 1)
+}
+
+__device__ __forceinline__ void phase1_mid(const RArgs& a) {
+  __shared__ SegMax sh[kWarps + 1];
+  __shared__ int64_t s_tile;
+  __shared__ SegMax s_pre;
+  __shared__ int s_n;
+  __shared__ uint16_t s_slot[kMidTile];
+  __shared__ int32_t s_val[kMidTile];   // of a listed slot: its Phase I value,
+  __shared__ int32_t s_wait[kMidTile];  // its column if the mark needs P_j, else -1
+  DevState* ds = a.ds;
+  const PV v = pass_view(ds);
+  const int32_t pass = ds->pass;
+  const int32_t* fu = a.first_unp;
+  const int32_t* lows = a.lows + (int64_t)(pass & a.ring) * a.lows_stride;
+  const int64_t ntiles = (v.n_act + kMidTile - 1) / kMidTile;
+  int64_t bw = 0, bp = 0;
+  bool want = false, fault = false;
+  for (;;) {
+    if (threadIdx.x == 0) {
+      s_tile = atomicAdd(&ds->tile_queue, 1u);
+      s_n = 0;
+    }
+    __syncthreads();
+    const int64_t t = s_tile;
+    if (t >= ntiles) break;
+    const int64_t tile0 = t * kMidTile, e0 = tile0 + (int64_t)threadIdx.x * kMidItems;
+    int32_t d[kMidItems], l[kMidItems];
+    {
+      const int64_t r0 = min(e0, a.lows_stride - kMidItems);  // (threads past the list read its end)
+      const int4 d0 = *reinterpret_cast<const int4*>(a.due + r0);
+      const int4 d1 = *reinterpret_cast<const int4*>(a.due + r0 + 4);
+      const int4 l0 = *reinterpret_cast<const int4*>(lows + r0);
+      const int4 l1 = *reinterpret_cast<const int4*>(lows + r0 + 4);
+      d[0] = d0.x, d[1] = d0.y, d[2] = d0.z, d[3] = d0.w;
+      d[4] = d1.x, d[5] = d1.y, d[6] = d1.z, d[7] = d1.w;
+      l[0] = l0.x, l[1] = l0.y, l[2] = l0.z, l[3] = l0.w;
+      l[4] = l1.x, l[5] = l1.y, l[6] = l1.z, l[7] = l1.w;
+    }
+    // one segment for the whole tile, as a rule (ids, and so segments, ascend)
+    const int32_t sg0 = seg_of(a, slot_id(v.act[tile0]));
+    const int32_t sg1 = seg_of(a, slot_id(v.act[min(tile0 + kMidTile, v.n_act) - 1]));
+    const bool one = sg0 == sg1;
+    int32_t sg[kMidItems];
+#pragma unroll
+    for (int i = 0; i < kMidItems; i++)
+      sg[i] = e0 + i >= v.n_act ? INT32_MAX : one ? sg0 : seg_of(a, slot_id(v.act[e0 + i]));
+    const int32_t fu0 = sg0 >= a.nc ? fu[sg0 - a.nc] : INT32_MIN;
+    unsigned listed = 0;
+#pragma unroll
+    for (int i = 0; i < kMidItems; i++) {
+      const int32_t dp = due_pass(d[i]);
+      const bool dead = e0 + i >= v.n_act || d[i] == kDeadDue;
+      if (dead) {
+        l[i] = -1;
+      } else if (dp <= pass) {
+        listed |= 1u << i;
+      } else if (l[i] < 0 || (d[i] < 0 && l[i] < (one ? fu0 : fu[sg[i] - a.nc]))) {
+        const int32_t j = v.act[e0 + i];  // zeroed: it leaves its slot at once
+        a.meta[j].flags = F_FINAL;
+        a.meta[j].len = 0;
+        a.low[j] = -1;
+        v.act[e0 + i] = dead_slot(j);
+        a.due[e0 + i] = kDeadDue;
+      }
+    }
+    if (listed) {
+      int p = atomicAdd(&s_n, __popc(listed));
+#pragma unroll
+      for (int i = 0; i < kMidItems; i++)
+        if ((listed >> i) & 1u) {
+          s_slot[p++] = (uint16_t)(threadIdx.x * kMidItems + i);
+          s_val[threadIdx.x * kMidItems + i] = l[i];
+        }
+    }
+    __syncthreads();
+    const int n_list = s_n;
+    if (n_list > 0) {
+      // bit-packing thresholds, as in phase1_pass
+      int32_t t_b = 0, t_hi = INT32_MAX, t_lo = INT32_MAX;
+      if (a.dense_floor != INT32_MAX) {
+        const int32_t j0 = slot_id(v.act[tile0]);
+        const int32_t j1 = slot_id(v.act[min(tile0 + kMidTile, v.n_act) - 1]);
+        t_b = dim_start_of(a, j1);
+        t_hi = dense_min_of(a, j1);
+        t_lo = dense_min_between(a, j0, t_b - 1);
+      }
+      for (int k = threadIdx.x; k < n_list; k += kThreads) {
+        const int x = s_slot[k];
+        const int64_t e = tile0 + x;
+        const int32_t lj = s_val[x];
+        const int32_t s = lj >= 0 ? (int32_t)(unsigned)a.tab[lj] : -1;
+        const int32_t j = v.act[e], nj = v.alen[e];
+        int32_t wait = -1, val = -1, src = -1;
+        if (PH_DCHECK(&ds->debug_fault, j >= 0 && lj < a.rows_end, 2)) {
+          const int32_t b = a.beta[j], sj = one ? sg0 : seg_of(a, j);
+          (void)PH_DCHECK(&ds->debug_fault, a.meta[j].flags == 0, 7);
+          bw += stored_words(nj);
+          if (lj < 0) {
+            a.meta[j].flags = F_FINAL;
+          } else if (s != j) {
+            const int32_t ns = stored_words(a.meta[s].len);
+            bw += max(ns, kDeltaRows);
+            want |= nj + ns > (j >= t_b ? t_hi : t_lo);
+            val = lj;
+            src = s;
+            if (a.cor10 && b < 0 && lj < fu[sj - a.nc]) a.meta[j].flags = F_FINAL;
+          } else {
+            bp += stored_words(nj);
+            if (lj == b) mark_pivot(a, fu, j, lj, sj);
+            else wait = j;
+          }
+          a.src_e[e] = src;
+        }
+        s_val[x] = val;
+        s_wait[x] = wait;
+      }
+      __syncthreads();
+    }
+    unsigned waits = 0;
+    SegMax agg{-1, -1};
+#pragma unroll
+    for (int i = 0; i < kMidItems; i++) {
+      if ((listed >> i) & 1u) {
+        const int x = threadIdx.x * kMidItems + i;
+        if (s_wait[x] >= 0) waits |= 1u << i;
+        else l[i] = s_val[x];
+      }
+      const SegMax xi{sg[i], (waits >> i) & 1u ? -1 : l[i]};
+      agg = i == 0 ? xi : segmax_combine(agg, xi);
+    }
+    SegMax tot;
+    const SegMax pre_t = block_scan_segmax(agg, SegMax{-1, -1}, sh, tot);  // within the tile
+    // a tile without such a mark only publishes its value (every 16th its prefix, so walks stay short)
+    if (!__syncthreads_or(waits) && (t & 15)) {
+      if (threadIdx.x == 0) tile_publish(a.tile_st, pass, t, tot);
+      continue;
+    }
+    if (threadIdx.x < 32) {
+      const SegMax P = tile_look_back(a.tile_st, pass, t, tot, fault);
+      if (threadIdx.x == 0) s_pre = P;
+    }
+    __syncthreads();
+    if (waits) {
+      SegMax run = threadIdx.x == 0 ? s_pre : segmax_combine(s_pre, pre_t);
+#pragma unroll
+      for (int i = 0; i < kMidItems; i++) {
+        const SegMax pre = run;
+        const bool w = (waits >> i) & 1u;
+        run = segmax_combine(run, SegMax{sg[i], w ? -1 : l[i]});
+        if (!w) continue;
+        const int32_t j = s_wait[threadIdx.x * kMidItems + i];
+        const int32_t P = pre.seg == sg[i] ? pre.val : -1;
+        if (l[i] > P) mark_pivot(a, fu, j, l[i], sg[i]);
+        else if (a.cor10 && a.beta[j] < 0 && l[i] < fu[sg[i] - a.nc]) a.meta[j].flags = F_FINAL;
+      }
+    }
+    __syncthreads();  // the lists are done with
+  }
+  if (want && !v.dense_on) ds->dense_want = 1;
+  if (__any_sync(0xffffffffu, fault) && lane_id() == 0) ds->fault = 1;
+  const int64_t ww = warp_sum64(bw), wp = warp_sum64(bp);
+  if (lane_id() == 0 && (ww || wp)) {
+    atomicAdd(&ds->bound_words, (unsigned long long)ww);
+    atomicAdd(&ds->bound_piv, (unsigned long long)wp);
+  }
+}
+
 // no more blocks take part in Phase I than there are tiles (the others leave at once: a short
 // pass's grid is mostly idle); block 0 always does
 __device__ __forceinline__ unsigned phase1_parts(const DevState* ds, unsigned blocks) {
@@ -1020,7 +1230,8 @@ __global__ void __launch_bounds__(kThreads, 4) k_phase1(RArgs a) {
   if (ds->status != ST_RUN) return;
   const unsigned parts = phase1_parts(ds, gridDim.x);
   if (blockIdx.x >= parts) return;
-  phase1_pass<kLookAhead, false>(a, parts);
+  if (kLookAhead && !ds->compact && !a.predict) phase1_mid(a);
+  else phase1_pass<kLookAhead, false>(a, parts);
   // the last of the taking-part blocks checks the space this pass's Phase II needs
   if (last_block(&ds->blocks_done, parts)) {
     if (threadIdx.x == 0) {
@@ -2371,6 +2582,7 @@ __device__ __forceinline__ void visit_round(const RArgs& a, const PV& v, int32_t
   w.due = pass + 1;
   const int na0 = w.na;
   const bool visit = add && !eager;
+  bool no_beta = false;  // Corollary 10 may zero it
   if (__any_sync(0xffffffffu, visit)) {
     int32_t* block = a.delta + (int64_t)max(j, 0) * kDeltaRows;
 #pragma unroll
@@ -2385,6 +2597,7 @@ __device__ __forceinline__ void visit_round(const RArgs& a, const PV& v, int32_t
 #pragma unroll
     for (int i = kOld; i < kDeltaRows; i++) w.d.c[i] = kEmpty;
     const bool c10 = visit && a.cor10 && a.beta[j] < 0;
+    no_beta = c10;
     const int32_t fu =
         c10 ? a.first_unp[seg_of(a, j) - a.nc] : INT32_MIN;
     if (look_ahead(a, v, pass, visit, fu, pos, w)) tidy<0>(w, visit && !w.gone);
@@ -2414,11 +2627,15 @@ __device__ __forceinline__ void visit_round(const RArgs& a, const PV& v, int32_t
   if (v.compact) {
     if (j >= 0 && pos >= 0 && PH_DCHECK(&a.ds->debug_fault, pos < v.n_act, 5)) {
       v.act2[pos] = surv ? j : dead_slot(j);
+      if (!surv) a.due[pos] = kDeadDue;
       v.alen2[pos] = w.na;
       a.kind[pos] = (uint8_t)kind;
     }
   } else {
-    if (j >= 0 && !surv) v.act[e] = dead_slot(j);
+    if (j >= 0 && !surv) {
+      v.act[e] = dead_slot(j);
+      a.due[e] = kDeadDue;
+    }
     if (visit) v.alen[e] = w.na;
     const unsigned km = __ballot_sync(0xffffffffu, kind != kNothing);
     if (km) {
@@ -2473,7 +2690,7 @@ __device__ __forceinline__ void visit_round(const RArgs& a, const PV& v, int32_t
   // ---- publish: the lows of the coming passes (k_merge knows those of its additions), a visited
   // column's shortened list and its delta, a zeroed column
   if (surv && PH_DCHECK(&a.ds->debug_fault, pos >= 0 && pos < v.n_act, 5)) {
-    a.due[pos] = w.due;
+    a.due[pos] = no_beta ? ~w.due : w.due;
     if (visit) {
       if (w.due == pass + 1) next_tab<true>(a, v, w.low, j);
     } else if (!eager) {  // its low stays
@@ -2525,31 +2742,34 @@ __device__ __forceinline__ void visit_pass(const RArgs& a, VisitStage& S, unsign
       }
     } else {
       for (; np < 32 && i0 < v.n_act; i0 += (int64_t)blocks * warps * kScan) {
-        int32_t js[kScan / 32], ds[kScan / 32];
+        // only columns below the top dimension can be cleared: those of the others are not read
+        const bool below = slot_id(v.act[i0]) < a.rows_end;
+        int32_t ds[kScan / 32];
 #pragma unroll
         for (int u = 0; u < kScan / 32; u++) {
           const int64_t x = i0 + 32 * u + lane;
-          js[u] = x < v.n_act ? v.act[x] : -1;
-          ds[u] = x < v.n_act ? a.due[x] : 0;
+          ds[u] = x < v.n_act ? a.due[x] : kDeadDue;
         }
 #pragma unroll
         for (int u = 0; u < kScan / 32; u++) {
           const int32_t x = (int32_t)(i0 + 32 * u + lane);
-          const int32_t j = js[u];
-          if (j >= 0 && ds[u] > pass) {
-            if (j < a.rows_end && a.meta[j].cleared) {
+          const int32_t d = due_pass(ds[u]);
+          if (d > pass && d != kDeadDue) {
+            const bool enters = d == pass + 1;
+            const int32_t j = below || enters ? v.act[x] : INT32_MAX;
+            if (below && j < a.rows_end && a.meta[j].cleared) {
               a.meta[j].flags |= F_FINAL;
               a.meta[j].len = 0;
               a.low[j] = -1;
               v.act[x] = dead_slot(j);
+              a.due[x] = kDeadDue;
             } else {
               n_tgt++;
-              if (ds[u] == pass + 1) next_tab<true>(a, v, lows_next[x], j);
+              if (enters) next_tab<true>(a, v, lows_next[x], j);
             }
           }
-          const bool due = j >= 0 && ds[u] <= pass;
-          const unsigned m = __ballot_sync(0xffffffffu, due);
-          if (due) S.pend[np + __popc(m & ((1u << lane) - 1u))] = x;
+          const unsigned m = __ballot_sync(0xffffffffu, d <= pass);
+          if (d <= pass) S.pend[np + __popc(m & ((1u << lane) - 1u))] = x;
           np += __popc(m);
         }
         __syncwarp();
@@ -3126,7 +3346,7 @@ static RArgs make_args(ph_ctx* ctx) {
   a.src_e = static_cast<int32_t*>(rs.src_e);
   a.lows = rs.lows;
   a.due = rs.due;
-  a.lows_stride = std::max<int64_t>(ctx->m, 1);
+  a.lows_stride = lows_stride_of(ctx->m);
   a.ring = kAheadMax - 1;
   a.prec = static_cast<int4*>(rs.prec);
   a.delta = rs.delta;
@@ -3338,8 +3558,8 @@ void reduce_init(ph_ctx* ctx) {
   rs.prec = alloc_n<int4>(ctx, ahead > 1 ? ctx->dimoff[ctx->max_dim] : 1);
   if (ahead > 1) {
     rs.lows_rows = kAheadMax;
-    rs.lows = alloc_n<int32_t>(ctx, rs.lows_rows * m);
-    rs.due = alloc_n<int32_t>(ctx, m);
+    rs.lows = alloc_n<int32_t>(ctx, rs.lows_rows * lows_stride_of(m));
+    rs.due = alloc_n<int32_t>(ctx, lows_stride_of(m));
     rs.delta = alloc_n<int32_t>(ctx, kDeltaRows * m + kColSlack);
     rs.kind = alloc_n<uint8_t>(ctx, m);
     rs.newpos = alloc_n<int32_t>(ctx, m);
