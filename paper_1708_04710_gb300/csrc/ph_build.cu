@@ -343,13 +343,12 @@ __global__ void k_high_finish(const uint64_t* __restrict__ keys, const uint64_t*
 // counts per edge, scanned, are the places, and the filtration indices and left(i) (Definition 3)
 // of edges follow from them. With sorted candidates (each unranked by binary searches, five
 // kernels per 8-bit digit, then an atomic per row for left and two searches per simplex for the
-// index) the build of a 400-point cloud took 2.1 ms and now takes 0.48 ms, that of 120 points in
-// 8-d to dimension 3 with a cut 1.24 -> 0.33 ms, of 512 clouds of 80 points 6.4 -> 2.1 ms. Bound
-// by instruction issue: an edge costs 225 warp instructions to count and 645 to list (80 points, 26
-// triangles an edge), of which the writes of a triangle's 40 bytes, neighbouring lanes to
-// neighbouring addresses, are a third of the time.
+// index) the build of a 400-point cloud took 2.1 ms and now takes 0.46 ms, that of 120 points in
+// 8-d to dimension 3 with a cut 1.24 -> 0.31 ms, of 512 clouds of 20 to 120 points 6.4 -> 1.43 ms.
+// Counting is bound by instruction issue (225 warp instructions an edge of 80 points), listing by
+// issue and by its writes of 40 bytes a triangle.
 // The direct listing is taken whenever it applies: it is faster at every size measured (40
-// points: 470 -> 150 us, the one-block sort of the edges included). With ties, and in dimensions 4
+// points: 470 -> 128 us, the one-block sort of the edges included). With ties, and in dimensions 4
 // and 5, candidates are sorted.
 constexpr int kDirectPoints = 512;   // points per cloud with tetrahedra (a warp's list of L(ab))
 constexpr int kDirectWarps = 4;
@@ -474,38 +473,55 @@ __device__ __forceinline__ int32_t triangle_id(const Direct& g, const int32_t* t
   return (int32_t)(g.N + g.E + g.off2[ei] + k);
 }
 
+// A warp takes `group` consecutive edges (a power of two, up to 32; as many as leave every warp of the
+// machine some): what an edge needs is loaded by one lane each, and their triangles are one run that
+// the lanes share, 32 at a time. A lane finds its edge by a search over the group's places and its
+// vertex by a search in the edge's mask. With a warp per edge 645 instructions went into an edge of 26
+// triangles: 10.7 M triangles in 256 clouds of 64 points took 384 us, now 139; 42 M in 512 clouds 1178,
+// now 569; 10.6 M of 400 points 176, now 161 (their writes alone take 62 us at the copy rate).
 __global__ void __launch_bounds__(32 * kDirectWarps) k_tri_emit(CloudTabs ct, Direct g, IdOut o,
-                                                                int64_t rowbase) {
-  __shared__ uint16_t s_list[kDirectWarps][kDirectPoints];
+                                                                int64_t rowbase, int group) {
   __shared__ int32_t s_rows[kDirectWarps][96];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < g.N;
        i += (int64_t)gridDim.x * blockDim.x)  // a vertex's index is its place in its cloud
     g.gidx[i] = i - ct.pt_off[find_cloud(ct.pt_off, ct.nc, i)];
-  for (int64_t e = (int64_t)blockIdx.x * kDirectWarps + w; e < g.E;
-       e += (int64_t)gridDim.x * kDirectWarps) {
-    const uint64_t p = g.edge[e];
-    const int64_t t0 = g.off2[e], t1 = g.off2[e + 1];
-    const int c = (int)packed_cloud(p), a = packed_vert(ct, p, 0), b = packed_vert(ct, p, 1);
-    const int64_t v0 = ct.pt_off[c];
-    const int n = (int)(ct.pt_off[c + 1] - v0);
-    const int32_t id = (int32_t)(g.N + e);
-    const int64_t es = g.es[c], ts = g.off2[es];
-    const int64_t qs = g.off3 ? g.off3[e] - g.off3[es] : 0;
-    const int64_t first = g.N + g.E + t0;  // id of this edge's first triangle
-    const int64_t gi = n + (e - es) + (t0 - ts) + qs;
-    const int32_t* tab = g.eid + ct.mo[c];
-    const int32_t* ra = tab + (int64_t)a * n;
-    const int32_t* rb = tab + (int64_t)b * n;
-    if (lane < 2) lower_left(g.left, (int32_t)(v0 + (lane ? b : a)), id);
-    if (lane == 0) g.gidx[id] = gi;
-    // an edge's first column is its own first triangle: it is shorter than the longest edge of
-    // any other triangle that holds it. Without one (the edges of the relative neighbourhood graph)
-    // it is the triangle on it whose longest edge is least: no two share that edge
-    if (t1 == t0) {
+  for (int64_t e0 = ((int64_t)blockIdx.x * kDirectWarps + w) * group; e0 < g.E;
+       e0 += (int64_t)gridDim.x * kDirectWarps * group) {
+    const int64_t e = e0 + lane;
+    const bool mine = lane < group && e < g.E;
+    int c = 0, a = 0, b = 0, n = 0;
+    int64_t t0 = 0, t1 = 0, gi = 0;
+    if (mine) {
+      const uint64_t p = g.edge[e];
+      t0 = g.off2[e];
+      t1 = g.off2[e + 1];
+      c = (int)packed_cloud(p);
+      a = packed_vert(ct, p, 0);
+      b = packed_vert(ct, p, 1);
+      const int64_t v0 = ct.pt_off[c], es = g.es[c];
+      n = (int)(ct.pt_off[c + 1] - v0);
+      const int32_t id = (int32_t)(g.N + e);
+      gi = n + (e - es) + (t0 - g.off2[es]) + (g.off3 ? g.off3[e] - g.off3[es] : 0);
+      g.gidx[id] = gi;
+      lower_left(g.left, (int32_t)(v0 + a), id);
+      lower_left(g.left, (int32_t)(v0 + b), id);
+      // an edge's first column is its own first triangle: it is shorter than the longest edge of
+      // any other triangle that holds it
+      if (t1 > t0) g.left[id] = (int32_t)(g.N + g.E + t0);
+    }
+    // Without one (the edges of the relative neighbourhood graph) it is the triangle on it whose
+    // longest edge is least: no two share that edge
+    for (unsigned none = __ballot_sync(0xffffffffu, mine && t1 == t0); none; none &= none - 1) {
+      const int src = __ffs(none) - 1;
+      const int ea = __shfl_sync(0xffffffffu, a, src), eb = __shfl_sync(0xffffffffu, b, src);
+      const int en = __shfl_sync(0xffffffffu, n, src);
+      const int32_t* tab = g.eid + ct.mo[__shfl_sync(0xffffffffu, c, src)];
+      const int32_t* ra = tab + (int64_t)ea * en;
+      const int32_t* rb = tab + (int64_t)eb * en;
       uint32_t least = 0x7f7f7f7fu;
       int third = -1;
-      for (int x = lane; x < n; x += 32) {
+      for (int x = lane; x < en; x += 32) {
         const int32_t ac = ra[x], bc = rb[x];
         const uint32_t longest = ac < 0 || bc < 0 ? 0x7f7f7f7fu : (uint32_t)max(ac, bc);
         if (longest < least) {
@@ -514,39 +530,66 @@ __global__ void __launch_bounds__(32 * kDirectWarps) k_tri_emit(CloudTabs ct, Di
         }
       }
       const uint32_t all = __reduce_min_sync(0xffffffffu, least);
-      if (third >= 0 && least == all) g.left[id] = triangle_id(g, tab, n, a, b, third);
-      continue;
+      if (third >= 0 && least == all)
+        g.left[g.N + e0 + src] = triangle_id(g, tab, en, ea, eb, third);
     }
-    if (lane == 0) g.left[id] = (int32_t)first;
-    const uint64_t high = (uint64_t)c << 48 | ((1u << 12) - 1u);  // cloud, last slot empty
-    int64_t t = first;
-    const int words = (n + 31) >> 5;  // of this cloud
-    for (int q0 = 0; q0 < words; q0 += kListWords) {
-      const int n2 = list_mask(g.mask + e * g.words, q0, words, s_list[w]);
-      for (int k0 = 0; k0 < n2; k0 += 32) {
-        const int k = k0 + lane;
-        const int have = min(32, n2 - k0);
-        if (k < n2) {
-          const int x = s_list[w][k];
-          const int32_t ac = ra[x], bc = rb[x];
-          o.verts[t + k] = high | (uint64_t)min(a, x) << 36 |
-                           (uint64_t)(x < a ? a : min(x, b)) << 24 | (uint64_t)max(b, x) << 12;
-          o.seg[t + k] = 2 * ct.nc + c;
-          o.key[t + k] = (int32_t)e;
-          o.low[t + k] = id;
-          g.gidx[t + k] = gi + 1 + (t - first) + k;
-          s_rows[w][3 * lane] = min(ac, bc);
-          s_rows[w][3 * lane + 1] = max(ac, bc);
-          s_rows[w][3 * lane + 2] = id;
+    // the group's triangles, as places from its first one's on
+    const int last = (int)min((int64_t)group, g.E - e0) - 1;
+    const int64_t first = __shfl_sync(0xffffffffu, t0, 0);
+    const int total = (int)(__shfl_sync(0xffffffffu, t1, last) - first);
+    const int place = mine ? (int)(t0 - first) : INT32_MAX;
+    const int ab = a | b << 16;
+    for (int r0 = 0; r0 < total; r0 += 32) {
+      const int r = r0 + lane;
+      int i = 0;  // the last edge of the group whose place is not above r
+      for (int step = group >> 1; step > 0; step >>= 1)
+        if (__shfl_sync(0xffffffffu, place, i + step) <= r) i += step;
+      int k = r - __shfl_sync(0xffffffffu, place, i);
+      const int eab = __shfl_sync(0xffffffffu, ab, i), ec = __shfl_sync(0xffffffffu, c, i);
+      const int en = __shfl_sync(0xffffffffu, n, i);
+      const int64_t index = __shfl_sync(0xffffffffu, gi, i) + 1 + k;
+      if (r < total) {
+        const int64_t ee = e0 + i, t = g.N + g.E + first + r;
+        const int ea = eab & 0xffff, eb = eab >> 16;
+        const int32_t id = (int32_t)(g.N + ee);
+        // vertex k of L(ab)
+        const uint32_t* m = g.mask + ee * g.words;
+        uint32_t bits = *m;
+        int x = 0;
+        for (int pc = __popc(bits); pc <= k; pc = __popc(bits)) {
+          k -= pc;
+          bits = *++m;
+          x += 32;
         }
-        __syncwarp();
-        int32_t* r = o.rows0 + rowbase + 3 * (t + k0 - g.N - g.E);
 #pragma unroll
-        for (int q = 0; q < 3; q++)
-          if (q * 32 + lane < 3 * have) r[q * 32 + lane] = s_rows[w][q * 32 + lane];
-        __syncwarp();
+        for (int half = 16; half > 0; half >>= 1) {
+          const uint32_t low = bits & ((1u << half) - 1u);
+          const int pc = __popc(low);
+          const bool up = k >= pc;
+          k -= up ? pc : 0;
+          x += up ? half : 0;
+          bits = up ? bits >> half : low;
+        }
+        const int32_t* tab = g.eid + ct.mo[ec];
+        const int32_t ac = tab[ea * en + x], bc = tab[eb * en + x];
+        o.verts[t] = (uint64_t)ec << 48 | (uint64_t)min(ea, x) << 36 |
+                     (uint64_t)(x < ea ? ea : min(x, eb)) << 24 | (uint64_t)max(eb, x) << 12 |
+                     ((1u << 12) - 1u);  // the last slot is empty
+        o.seg[t] = 2 * ct.nc + ec;
+        o.key[t] = (int32_t)ee;
+        o.low[t] = id;
+        g.gidx[t] = index;
+        s_rows[w][3 * lane] = min(ac, bc);
+        s_rows[w][3 * lane + 1] = max(ac, bc);
+        s_rows[w][3 * lane + 2] = id;
       }
-      t += n2;
+      __syncwarp();
+      const int have = 3 * min(32, total - r0);
+      int32_t* rows = o.rows0 + rowbase + 3 * (first + r0);
+#pragma unroll
+      for (int q = 0; q < 3; q++)
+        if (q * 32 + lane < have) rows[q * 32 + lane] = s_rows[w][q * 32 + lane];
+      __syncwarp();
     }
   }
 }
@@ -931,7 +974,10 @@ static void build_direct(ph_ctx* ctx, const CloudTabs& ct, Direct g, const IdOut
   g.gidx = ctx->gidx;
   PH_CUDA(cudaMemsetAsync(left, 0x7f, rows * sizeof(int32_t), st));  // > every id
   PH_CUDA(cudaMemsetAsync(ctx->beta, 0xff, m * sizeof(int32_t), st));
-  k_tri_emit<<<grid, 32 * kDirectWarps, 0, st>>>(ct, g, o, 2 * g.E);
+  int group = 1;
+  while (group < 32 && g.E / (2 * group) >= (int64_t)ctx->num_sms * 64) group *= 2;
+  k_tri_emit<<<grid_for(ctx, (g.E + group - 1) / group, kDirectWarps, 16), 32 * kDirectWarps, 0, st>>>(
+      ct, g, o, 2 * g.E, group);
   PH_CHECK_LAUNCH();
   if (tets && cnts[3] > 0) {
     k_tet_emit<<<grid_for(ctx, g.E, 1, 16), kTetThreads, 0, st>>>(ct, g, o, id3, 2 * g.E + 3 * cnts[2]);

@@ -51,10 +51,10 @@ TIED = np.array([[0, 0], [1, 0], [2, 0], [3, 0]], np.int32)  # equal edges: sort
 # clouds without two edges of one length list triangles and tetrahedra per edge, without a sort;
 # a batch with a tie in any cloud sorts all candidates. 64 and 65 points have 2016 and 2080 edges,
 # around one 2048-element sort and scan tile; 33 and 65 points take a second and third word of an
-# edge's vertex mask
+# edge's vertex mask; 200 points have 19900 edges, listed by warps of two
 @pytest.mark.parametrize("n,max_dim,cut", [
     (3, 2, -1), (4, 3, -1), (33, 2, -1), (64, 2, -1), (65, 2, -1), (65, 1, -1), (130, 2, 2.0),
-    (5, 3, -1), (32, 3, -1), (33, 3, -1), (65, 3, 1.5), (33, 3, 0.2),
+    (200, 2, -1), (5, 3, -1), (32, 3, -1), (33, 3, -1), (65, 3, 1.5), (33, 3, 0.2),
 ])
 def test_direct_listing_equals_sorted_listing(ph, orc, n, max_dim, cut):
     x = pc.random_cloud(n, 2, 500 + n)
