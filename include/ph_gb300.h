@@ -51,7 +51,9 @@ typedef struct ph_ctx ph_ctx;
  * `stream`, aligned to 256 bytes (as cudaMalloc's is), or NULL on failure; free releases it.
  * Both are called from the thread that calls the library. A misaligned block is given back and
  * the call fails with PH_ERR_ALLOC. With a NULL provider the library uses cudaMallocAsync /
- * cudaFreeAsync. */
+ * cudaFreeAsync. A context keeps freed blocks of up to 32 MB, 256 MB in all, for its next
+ * allocations; it gives back those that two builds have not used, all of them when an
+ * allocation fails, and at ph_destroy. */
 typedef struct {
   void* (*alloc)(size_t bytes, void* user, void* stream);
   void (*free)(void* ptr, size_t bytes, void* user, void* stream);
@@ -94,7 +96,9 @@ typedef struct {
    * (two 128-thread blocks each; 0 = library default, 4) */
   int32_t add_blocks_per_sm;
   /* wall-clock bound of one ph_reduce's pass loop in ms, checked on the device at the end of
-   * every pass (0 = library default, 60000); past it the call returns PH_ERR_TIMEOUT */
+   * every pass (0 = library default, 60000); past it the call returns PH_ERR_TIMEOUT, for a
+   * complex of 3,000,000 columns or more once the up to eight passes that its columns may be
+   * ahead by are done */
   int32_t timeout_ms;
   /* 1: every pass also applies the non-zero case of Corollary 10 (Lemma 9): an active column j
    * with beta_j >= 0 whose candidate set L_j (rows of K_{d-1} in [beta_j, low(j)] not known to
@@ -137,7 +141,8 @@ typedef struct {
   int32_t phase2_sets;
   int32_t phase2_priority;
   /* Initial capacity of each of the two survivor arenas, in int32 words (0, default: twice the
-   * boundary's nonzeros). A pass whose Phase I bound does not fit stops after its marks,
+   * boundary's nonzeros; from 3,000,000 columns of at most three rows on, the nonzeros and 24
+   * words per column). A pass whose Phase I bound does not fit stops after its marks,
    * before any column changes; the host grows the arena and the pass continues with its column
    * additions, so a small value trades memory for extra host round trips; results are the
    * same. */
@@ -254,7 +259,8 @@ int ph_load_boundary(ph_ctx* ctx, int64_t m, const int32_t* dims, const int64_t*
  * A later call continues a reduction that stopped at its pass cap (PH_NOT_CONVERGED), at the
  * time bound (PH_ERR_TIMEOUT) or on a failed allocation (PH_ERR_ALLOC, the state left as
  * before the pass that needed the memory); after a complete reduction it returns the result
- * again. The pass loop runs in a CUDA graph (use_graph) or from the host. Synchronises the
+ * again. The pass loop runs in a CUDA graph and, for short active lists, in one cooperative
+ * kernel (use_graph), or from the host. Synchronises the
  * stream. */
 int ph_reduce(ph_ctx* ctx, int32_t max_passes, ph_stats* out);
 

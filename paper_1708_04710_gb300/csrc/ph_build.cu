@@ -1259,6 +1259,8 @@ void build_vr(ph_ctx* ctx, const int32_t* coords, const int64_t* cloud_offsets, 
         ctx->m, nc, max_dim, ctx->seg, ctx->key, ctx->d_seg_start, d_tabs, ctx->gidx);
     PH_CHECK_LAUNCH();
   }
+  PH_CUDA(cudaStreamSynchronize(st));
+
   ctx->dfree(kbuf);
   ctx->dfree(vbuf);
   ctx->dfree(ktmp);

@@ -74,8 +74,8 @@ void scan_counts(ph_ctx* ctx, const int32_t* a, const int32_t* b, int64_t n, int
 // writes, by latency for short lists. With separate count, scan and scatter kernels per digit the
 // sorts of a 400-point cloud's edges and triangles took 0.75 ms; its edges take 55 us now. A block
 // of 8192 pairs takes as long as the kernels over the whole device (7140 pairs, 5 digits: 39 against
-// 43 us) but is one launch, and a batch's clouds sort side by side: the edges of 512 clouds of 80
-// points 290 -> 130 us.
+// 43 us) but is one launch, and a batch's clouds sort side by side: the edges of 512 clouds of 20 to
+// 120 points 290 -> 130 us.
 // ---------------------------------------------------------------------------------------------
 constexpr int kMaxDigits = 8;
 
