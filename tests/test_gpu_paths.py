@@ -57,13 +57,14 @@ TIED = np.array([[0, 0], [1, 0], [2, 0], [3, 0]], np.int32)  # equal edges: sort
     (200, 2, -1), (5, 3, -1), (32, 3, -1), (33, 3, -1), (65, 3, 1.5), (33, 3, 0.2),
 ])
 def test_direct_listing_equals_sorted_listing(ph, orc, n, max_dim, cut):
-    x = pc.random_cloud(n, 2, 500 + n)
+    x = pc.random_cloud(n, 2 if n < 200 else 3, 500 + n)  # (the 200 points tie in the plane)
     cut2 = -1 if cut < 0 else int((cut * 65536) ** 2)
     K = orc.vr_build(x, max_dim, cut2)
     edges = K["diam2"][K["dim"] == 1]
     assert len(np.unique(edges)) == len(edges)  # no tie: the direct path
     alone = _build(ph.Context(), [x], max_dim, cut2)
-    mixed = _build(ph.Context(), [TIED, x, x[: n // 2 + 1]], max_dim, cut2)  # sorted
+    tied = np.pad(TIED, ((0, 0), (0, x.shape[1] - 2)))
+    mixed = _build(ph.Context(), [tied, x, x[: n // 2 + 1]], max_dim, cut2)  # sorted
     batch = _build(ph.Context(), [x[: n // 2 + 1], x], max_dim, cut2)  # direct, several clouds
     fa, fm, fb = alone.filtration(0), mixed.filtration(1), batch.filtration(1)
     assert np.array_equal(fa["beta"], orc.beta(K))
