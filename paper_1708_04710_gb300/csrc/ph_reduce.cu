@@ -3602,6 +3602,49 @@ static void grow_store(ph_ctx* ctx, ColStore& s, int64_t need_words) {
   s.cap = cap;
 }
 
+static int64_t first_arena(const ph_ctx* ctx, bool look_ahead) {
+  return ctx->opts.arena_words > 0 ? ctx->opts.arena_words
+         : look_ahead              ? ctx->nnz + kDeltaRows * (ctx->m - ctx->dimoff[1]) + 1
+                                   : 2 * ctx->nnz + 1;
+}
+
+// Look-ahead's arrays and first arenas, about 360 bytes per column (pass by pass: 50). Without room for
+// them, or when they would take more than a quarter of the device's memory, the reduction runs
+// pass by pass: what fitted without look-ahead still does.
+static bool take_ahead(ph_ctx* ctx) {
+  ReduceState& rs = ctx->rs;
+  const int64_t m = ctx->m, rows = ctx->dimoff[ctx->max_dim];
+  size_t free_bytes = 0, total_bytes = 0;
+  PH_CUDA(cudaMemGetInfo(&free_bytes, &total_bytes));
+  const double bytes = 16.0 * rows + (4.0 * (kAheadMax + 1 + kDeltaRows + 2) + 1.0) * m +
+                       8.0 * first_arena(ctx, true);
+  if (bytes > total_bytes / 4.0) return false;
+  try {
+    rs.prec = alloc_n<int4>(ctx, rows);
+    rs.lows_rows = kAheadMax;
+    rs.lows = alloc_n<int32_t>(ctx, rs.lows_rows * lows_stride_of(m));
+    rs.due = alloc_n<int32_t>(ctx, lows_stride_of(m));
+    rs.delta = alloc_n<int32_t>(ctx, kDeltaRows * m + kColSlack);
+    rs.kind = alloc_n<uint8_t>(ctx, m);
+    rs.newpos = alloc_n<int32_t>(ctx, m);
+    rs.work = alloc_n<int32_t>(ctx, m);
+    grow_store(ctx, rs.arena[0], first_arena(ctx, true));
+    grow_store(ctx, rs.arena[1], first_arena(ctx, true));
+    return true;
+  } catch (const Fail&) {
+    ctx->err.clear();
+    for (void* p : {(void*)rs.prec, (void*)rs.lows, (void*)rs.due, (void*)rs.delta, (void*)rs.kind,
+                    (void*)rs.newpos, (void*)rs.work, (void*)rs.arena[0].p, (void*)rs.arena[1].p})
+      ctx->dfree(p);
+    rs.prec = nullptr;
+    rs.lows_rows = 0;
+    rs.lows = rs.due = rs.delta = rs.newpos = rs.work = nullptr;
+    rs.kind = nullptr;
+    rs.arena[0] = rs.arena[1] = ColStore{};
+    return false;
+  }
+}
+
 void reduce_init(ph_ctx* ctx) {
   free_reduce_state(ctx);  // whatever an earlier, failed initialisation left
   // Phase I's tile states carry a (cloud, dimension) segment in 23 bits
@@ -3639,20 +3682,10 @@ void reduce_init(ph_ctx* ctx) {
   rs.dlist = alloc_n<int32_t>(ctx, m);
   // look-ahead for long lists (per-pass counters, and sets chosen pass by pass, need every pass to
   // take every column)
-  const int32_t ahead =
-      ctx->opts.collect_stats || ctx->opts.phase2_sets > 0 || !ctx->three_rows() || m < kAheadFrom
-          ? 1
-          : kAheadMax;
-  rs.prec = alloc_n<int4>(ctx, ahead > 1 ? ctx->dimoff[ctx->max_dim] : 1);
-  if (ahead > 1) {
-    rs.lows_rows = kAheadMax;
-    rs.lows = alloc_n<int32_t>(ctx, rs.lows_rows * lows_stride_of(m));
-    rs.due = alloc_n<int32_t>(ctx, lows_stride_of(m));
-    rs.delta = alloc_n<int32_t>(ctx, kDeltaRows * m + kColSlack);
-    rs.kind = alloc_n<uint8_t>(ctx, m);
-    rs.newpos = alloc_n<int32_t>(ctx, m);
-    rs.work = alloc_n<int32_t>(ctx, m);
-  }
+  const bool look_ahead = !ctx->opts.collect_stats && ctx->opts.phase2_sets <= 0 &&
+                          ctx->three_rows() && m >= kAheadFrom && take_ahead(ctx);
+  const int32_t ahead = look_ahead ? kAheadMax : 1;
+  if (!look_ahead) rs.prec = alloc_n<int4>(ctx, 1);
   rs.src_e = alloc_n<int32_t>(ctx, m);
   if (ctx->opts.predict_pairs) {
     const int64_t rows = ctx->dimoff[ctx->max_dim];
@@ -3686,10 +3719,7 @@ void reduce_init(ph_ctx* ctx) {
   PH_CHECK_LAUNCH();
   // first arenas: pass 0 needs at most the boundary matrix twice over, or once and a visit's
   // rows per column; later passes need less (they grow on demand otherwise)
-  const int64_t n_cols = m - ctx->dimoff[1];
-  const int64_t arena0 = ctx->opts.arena_words > 0 ? ctx->opts.arena_words
-                         : ahead > 1               ? ctx->nnz + kDeltaRows * n_cols + 1
-                                                   : 2 * ctx->nnz + 1;
+  const int64_t arena0 = first_arena(ctx, look_ahead);
   grow_store(ctx, rs.arena[0], arena0);
   grow_store(ctx, rs.arena[1], arena0);
   ColStore c{};
@@ -3924,7 +3954,7 @@ int reduce_run(ph_ctx* ctx, int32_t max_passes) {
   h.max_passes = max_passes < 0 ? (int32_t)std::min<int64_t>(ctx->m + 1, INT32_MAX) : max_passes;
   h.blocks_done = 0;
   h.bar_count = h.bar_gen = 0;
-  const unsigned loop_blocks = use_graph ? loop_grid(ctx) : 0;
+  unsigned loop_blocks = use_graph ? loop_grid(ctx) : 0;
   h.loop_below = loop_blocks ? kLoopBelow : -1;
   h.drain = 0;
   const int64_t limit_ms = ctx->opts.timeout_ms > 0 ? ctx->opts.timeout_ms : 60000;
@@ -3953,8 +3983,17 @@ int reduce_run(ph_ctx* ctx, int32_t max_passes) {
       RArgs args = a;
       int64_t m = ctx->m;
       void* params[] = {&args, &m};
-      PH_CUDA(cudaLaunchCooperativeKernel((const void*)k_loop, dim3(h.loop_blocks), dim3(kThreads),
-                                          params, kLoopSmem, st));
+      const cudaError_t ce = cudaLaunchCooperativeKernel(
+          (const void*)k_loop, dim3(h.loop_blocks), dim3(kThreads), params, kLoopSmem, st);
+      if (ce == cudaErrorCooperativeLaunchTooLarge || ce == cudaErrorNotSupported) {
+        cudaGetLastError();  // a share of the device without room for it: the graph throughout
+        loop_blocks = 0;
+        h.loop_below = -1;
+        PH_CUDA(cudaMemcpyAsync(rs.dstate, &h, sizeof(DevState), cudaMemcpyHostToDevice, st));
+        PH_CUDA(cudaStreamSynchronize(st));
+        continue;
+      }
+      PH_CUDA(ce);
       PH_CHECK_LAUNCH();
     } else if (use_graph) {
       ran_graph = true;

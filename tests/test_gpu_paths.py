@@ -247,3 +247,26 @@ def test_rebuilt_contexts(ph):
             assert np.array_equal(r, g)
         for a, b in ((fresh.pairs(), ctx.pairs()), (fresh.essential(), ctx.essential())):
             assert all(np.array_equal(a[k].cpu(), b[k].cpu()) for k in a)
+
+
+def test_look_ahead_without_room_runs_pass_by_pass(ph):
+    """Its arrays take 360 bytes per column: a refused one (96 bytes per column) leaves the rest."""
+    import torch
+
+    refused = []
+
+    def alloc(nbytes, stream):
+        if nbytes > 250 << 20:
+            refused.append(nbytes)
+            return 0
+        return torch.cuda.caching_allocator_alloc(nbytes, stream=stream)
+
+    x = pc.to_grid(pc.sphere(270, np.random.Generator(np.random.PCG64(3)), noise=0.05))
+    ref = _build(ph.Context(), [x], 2)
+    got = _build(ph.Context(device_alloc=alloc, device_free=torch.cuda.caching_allocator_delete),
+                 [x], 2)
+    assert not refused
+    assert got.reduce(max_passes=5)["passes"] == ref.reduce(max_passes=5)["passes"] == 5
+    assert refused
+    for r, g in zip(_state(ref), _state(got)):
+        assert np.array_equal(r, g)
