@@ -585,9 +585,10 @@ constexpr int kOld = 8;
 // on a torus 29.2 -> 22.6 ms, on a sphere 12.8 -> 8.7 ms, 42.7 M in 512 clouds 45.5 -> 41.8 ms; on
 // 2.6 M columns 11.9 -> 11.8 ms, on 1.3 M 6.5 -> 6.2 ms, on 0.9 M 4.4 -> 4.3 ms: little to gain
 // below kAheadFrom, where a visit's two kernels and the larger tables also cost memory. Lists that
-// shrink under kAheadAbove go on pass by pass (half and twice as many measure alike).
+// shrink under kAheadAbove go on pass by pass (10.67 M columns: 34.3 ms with twice as many, 33.7 with
+// 100,000; 3.7 M in 48 clouds: 5.85 and 5.95 ms; here 34.1 and 5.85).
 constexpr int64_t kAheadFrom = 3000000;   // columns from which look-ahead pays, and
-constexpr int64_t kAheadAbove = 500000;   // down to which it goes on
+constexpr int64_t kAheadAbove = 250000;   // down to which it goes on
 constexpr int kLonger = 12;  // the longest source inside a visit: kRecRows + this many rows
 constexpr int kDeltaRows = kOld + kSourceRows * kAheadMax;
 // words per row of stored lows, and of due words: threads read eight slots in two 16-byte loads
