@@ -180,7 +180,9 @@ __global__ void k_rekey_cloud(const uint64_t* __restrict__ vals, uint64_t* keys,
 
 // first element of each distinct (cloud, squared diameter) among the sorted edges
 __global__ void k_edge_newflag(const uint64_t* __restrict__ vals, int64_t E, CloudTabs ct,
-                               const int64_t* __restrict__ d2, int32_t* flag, int64_t* ed2) {
+                               const int64_t* __restrict__ d2, int32_t* flag, int64_t* ed2,
+                               const int32_t* fault) {
+  if (*fault) return;  // (a wait of the sort ran out)
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < E;
        i += (int64_t)gridDim.x * blockDim.x) {
     uint64_t p = vals[i];
@@ -212,7 +214,9 @@ struct IdOut {
 __global__ void k_edge_finish(const uint64_t* __restrict__ vals, int64_t E, CloudTabs ct,
                               const int32_t* __restrict__ flag, const int64_t* __restrict__ excl,
                               const int64_t* __restrict__ ed2, int64_t id0, int32_t* eid,
-                              int32_t* erank, int64_t* d2tab, IdOut o, int64_t rowbase) {
+                              int32_t* erank, int64_t* d2tab, IdOut o, int64_t rowbase,
+                              const int32_t* fault) {
+  if (*fault) return;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < E;
        i += (int64_t)gridDim.x * blockDim.x) {
     uint64_t p = vals[i];
@@ -274,10 +278,30 @@ __device__ __forceinline__ void sort_small(int32_t* r, int k) {
   }
 }
 
+// Where a dimension's simplices go: known on the device before the host reads the counts
+struct DimPlace {
+  int64_t n, id0, rowbase;
+};
+// by one block: the place of a dimension (k vertices) of count[0..nc) simplices after the one before
+// (nothing is written after a sort whose wait ran out)
+__global__ void k_dim_place(const int64_t* __restrict__ count, int nc, int k, DimPlace* place,
+                            const int32_t* fault) {
+  __shared__ int64_t sh[kWarps + 1];
+  int64_t n = 0;
+  for (int c = threadIdx.x; c < nc; c += kThreads) n += count[c];
+  int64_t total;
+  block_excl_sum<int64_t>(n, sh, total);
+  if (threadIdx.x == 0) {
+    const DimPlace before = place[-1];
+    *place = DimPlace{*fault ? 0 : total, before.id0 + before.n, before.rowbase + (k - 1) * before.n};
+  }
+}
+
 __global__ void k_tri_finish(const uint64_t* __restrict__ keys, const uint64_t* __restrict__ vals,
-                             int64_t T, CloudTabs ct, const int32_t* __restrict__ eid, int64_t id0,
-                             IdOut o, int64_t rowbase, int32_t* tid_tab,
+                             const DimPlace* __restrict__ place, CloudTabs ct,
+                             const int32_t* __restrict__ eid, IdOut o, int32_t* tid_tab,
                              const int64_t* __restrict__ tri_lex_off) {
+  const int64_t T = place->n, id0 = place->id0, rowbase = place->rowbase;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < T;
        i += (int64_t)gridDim.x * blockDim.x) {
     uint64_t p = vals[i];
@@ -302,10 +326,11 @@ __global__ void k_tri_finish(const uint64_t* __restrict__ keys, const uint64_t* 
 // lexicographic rank in the table the previous dimension filled; this dimension fills its own
 // table when a higher one follows
 __global__ void k_high_finish(const uint64_t* __restrict__ keys, const uint64_t* __restrict__ vals,
-                              int64_t Q, int k, CloudTabs ct, const int32_t* __restrict__ face_tab,
+                              const DimPlace* __restrict__ place, int k, CloudTabs ct,
+                              const int32_t* __restrict__ face_tab,
                               const int64_t* __restrict__ face_lex_off, int32_t* self_tab,
-                              const int64_t* __restrict__ self_lex_off, int64_t id0, IdOut o,
-                              int64_t rowbase) {
+                              const int64_t* __restrict__ self_lex_off, IdOut o) {
+  const int64_t Q = place->n, id0 = place->id0, rowbase = place->rowbase;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < Q;
        i += (int64_t)gridDim.x * blockDim.x) {
     uint64_t p = vals[i];
@@ -1066,7 +1091,8 @@ void build_vr(ph_ctx* ctx, const int32_t* coords, const int64_t* cloud_offsets, 
     PH_CHECK_LAUNCH();
   }
   // page-locked scratch: status words and per-cloud counts come back through it
-  int64_t* h_misc = static_cast<int64_t*>(ctx->pinned((3 + 3 * ((int64_t)nc + 1)) * sizeof(int64_t)));
+  int64_t* h_misc = static_cast<int64_t*>(ctx->pinned(
+      (3 + kMaxVrDim * ((int64_t)nc + 1)) * sizeof(int64_t)));
   static const char* const kBadCoords = "coordinates must lie in [-2^24, 2^24] grid units";
   // Every cloud's edges are sorted by one block, if they fit (truncated ones of several clouds have
   // to come after all clouds' edges). That sort finds the largest squared distance by itself;
@@ -1159,11 +1185,11 @@ void build_vr(ph_ctx* ctx, const int32_t* coords, const int64_t* cloud_offsets, 
     int32_t* flag = alloc_n<int32_t>(ctx, E);
     int64_t* excl = alloc_n<int64_t>(ctx, E + 1);
     int64_t* ed2 = alloc_n<int64_t>(ctx, E);
-    k_edge_newflag<<<grid_for(ctx, E, kThreads), kThreads, 0, st>>>(vbuf, E, ct, d2, flag, ed2);
+    k_edge_newflag<<<grid_for(ctx, E, kThreads), kThreads, 0, st>>>(vbuf, E, ct, d2, flag, ed2, d_fault);
     PH_CHECK_LAUNCH();
     scan_counts(ctx, flag, nullptr, E, excl, nullptr, d_fault);
     k_edge_finish<<<grid_for(ctx, E, kThreads), kThreads, 0, st>>>(
-        vbuf, E, ct, flag, excl, ed2, N, eid, erank, ctx->d2tab, o, 0);
+        vbuf, E, ct, flag, excl, ed2, N, eid, erank, ctx->d2tab, o, 0, d_fault);
     PH_CHECK_LAUNCH();
     PH_CUDA(cudaMemcpyAsync(h_misc, d_misc, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
     PH_CUDA(cudaMemcpyAsync(h_misc + 1, excl + E, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
@@ -1182,7 +1208,6 @@ void build_vr(ph_ctx* ctx, const int32_t* coords, const int64_t* cloud_offsets, 
   // id of each simplex by the lexicographic rank of its vertex set, for the next dimension's
   // faces (edges use the n x n table eid instead)
   std::vector<int32_t*> lex_tab(kVrSlots + 1, nullptr);
-  int64_t id0 = N + E, rowbase = 2 * E;
   // no two edges of a cloud of one length: triangles and tetrahedra need no sort
   const bool direct = (max_dim == 2 || (max_dim == 3 && nmax <= kDirectPoints)) && E > 0 && n_d2 == E;
   if (direct) {
@@ -1197,40 +1222,46 @@ void build_vr(ph_ctx* ctx, const int32_t* coords, const int64_t* cloud_offsets, 
       *b = alloc_n<uint64_t>(ctx, most);
     }
   }
-  for (int k = 3; k <= K && !direct; k++) {
-    const int d = k - 1;
-    if (k < K) {  // the next dimension looks its faces up here
-      lex_tab[k] = alloc_n<int32_t>(ctx, std::max<int64_t>(cand[k][nc], 1));
-      PH_CUDA(cudaMemsetAsync(lex_tab[k], 0xff,
-                              std::max<int64_t>(cand[k][nc], 1) * sizeof(int32_t), st));
-    }
-    int64_t Q = 0;
-    if (cand[k][nc] > 0) {
-      k_simplex_cand<<<grid_for(ctx, cand[k][nc], kThreads), kThreads, 0, st>>>(
-          ct, d_cand(k), cand[k][nc], k, erank, (uint64_t)n_d2, kbuf, vbuf, cnt_dim(d));
-      PH_CHECK_LAUNCH();
-      radix_sort_u64(ctx, kbuf, vbuf, cand[k][nc], 0, rbits, ktmp, vtmp, d_fault);
-      PH_CUDA(cudaMemcpyAsync(h_misc, d_misc, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
-      PH_CUDA(cudaMemcpyAsync(h_misc + 1, cnt_dim(d), nc * sizeof(int64_t),
-                              cudaMemcpyDeviceToHost, st));
-      PH_CUDA(cudaStreamSynchronize(st));
-      PH_REQUIRE(h_misc[0] == 0, PH_ERR_CUDA, kSortFault);
-      for (int c = 0; c < nc; c++) Q += h_cnt[(int64_t)(d - 1) * nc + c] = h_misc[1 + c];
-    }
-    if (Q > 0) {
-      if (k == 3) {
-        k_tri_finish<<<grid_for(ctx, Q, kThreads), kThreads, 0, st>>>(
-            kbuf, vbuf, Q, ct, eid, id0, o, rowbase, lex_tab[3], d_cand(3));
-      } else {
-        k_high_finish<<<grid_for(ctx, Q, kThreads), kThreads, 0, st>>>(
-            kbuf, vbuf, Q, k, ct, lex_tab[k - 1], d_cand(k - 1), lex_tab[k], d_cand(k), id0, o,
-            rowbase);
+  if (!direct && max_dim >= 2) {
+    // every dimension is sorted and written before the host reads a count
+    DimPlace* place = alloc_n<DimPlace>(ctx, K);  // per dimension
+    DimPlace* h_place = reinterpret_cast<DimPlace*>(h_misc);
+    *h_place = DimPlace{E, N, 0};
+    PH_CUDA(cudaMemcpyAsync(place + 1, h_place, sizeof(DimPlace), cudaMemcpyHostToDevice, st));
+    for (int k = 3; k <= K; k++) {
+      const int d = k - 1;
+      const int64_t n_cand = cand[k][nc];
+      if (k < K) {  // the next dimension looks its faces up here
+        lex_tab[k] = alloc_n<int32_t>(ctx, std::max<int64_t>(n_cand, 1));
+        PH_CUDA(cudaMemsetAsync(lex_tab[k], 0xff, std::max<int64_t>(n_cand, 1) * sizeof(int32_t), st));
       }
+      if (n_cand > 0) {
+        k_simplex_cand<<<grid_for(ctx, n_cand, kThreads), kThreads, 0, st>>>(
+            ct, d_cand(k), n_cand, k, erank, (uint64_t)n_d2, kbuf, vbuf, cnt_dim(d));
+        PH_CHECK_LAUNCH();
+        radix_sort_u64(ctx, kbuf, vbuf, n_cand, 0, rbits, ktmp, vtmp, d_fault);
+      }
+      k_dim_place<<<1, kThreads, 0, st>>>(cnt_dim(d), nc, k, place + d, d_fault);
       PH_CHECK_LAUNCH();
+      if (n_cand > 0) {
+        const unsigned grid = grid_for(ctx, n_cand, kThreads);
+        if (k == 3)
+          k_tri_finish<<<grid, kThreads, 0, st>>>(kbuf, vbuf, place + d, ct, eid, o, lex_tab[3],
+                                                  d_cand(3));
+        else
+          k_high_finish<<<grid, kThreads, 0, st>>>(kbuf, vbuf, place + d, k, ct, lex_tab[k - 1],
+                                                   d_cand(k - 1), lex_tab[k], d_cand(k), o);
+        PH_CHECK_LAUNCH();
+      }
     }
-    cnts[d] = Q;
-    id0 += Q;
-    rowbase += (int64_t)k * Q;
+    PH_CUDA(cudaMemcpyAsync(h_misc, d_misc, (2 + (int64_t)max_dim * nc) * sizeof(int64_t),
+                            cudaMemcpyDeviceToHost, st));
+    PH_CUDA(cudaStreamSynchronize(st));
+    PH_REQUIRE(h_misc[0] == 0, PH_ERR_CUDA, kSortFault);
+    for (int d = 2; d <= max_dim; d++)
+      for (int c = 0; c < nc; c++)
+        cnts[d] += h_cnt[(int64_t)(d - 1) * nc + c] = h_misc[2 + (int64_t)(d - 1) * nc + c];
+    ctx->dfree(place);
   }
 
   // ---------------- layout ----------------
