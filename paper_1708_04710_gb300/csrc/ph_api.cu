@@ -456,16 +456,20 @@ static void renew(ph_ctx* ctx, T*& p, int64_t n) {
 
 // whether a kernel of this context may write the array (a copy takes more: another device's
 // memory, any alignment)
-static bool writable(ph_ctx* ctx, const void* p, size_t align) {
+static bool writable(ph_ctx* ctx, const void* p, size_t align, bool on_device) {
   if (!p) return true;
   cudaPointerAttributes at;
   if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
-  return at.type == cudaMemoryTypeDevice && at.device == ctx->device &&
-         reinterpret_cast<uintptr_t>(p) % align == 0;
+  const bool there = on_device ? at.type == cudaMemoryTypeDevice && at.device == ctx->device
+                               : at.type == cudaMemoryTypeHost && at.devicePointer == p;
+  return there && reinterpret_cast<uintptr_t>(p) % align == 0;
 }
+// A few results go straight into page-locked host arrays too, without internal arrays and copies: 780
+// pairs 84 -> 78 us, 9140 essentials 35 -> 31 us; from 18,000 on both ways measure alike.
+constexpr int64_t kHostDirect = 16384;
 
 __global__ void k_inspect(CloudIds ids, const int32_t* __restrict__ seg, int nc,
                           const int64_t* __restrict__ gidx, const int32_t* __restrict__ key,
@@ -697,9 +701,10 @@ int ph_get_pairs(ph_ctx* ctx, int32_t cloud, int64_t* birth, int64_t* death, int
   if (count) *count = n;
   if (!birth && !death && !dim && !birth_diam2 && !death_diam2) return PH_OK;
   PH_REQUIRE(capacity >= n, PH_ERR_CAPACITY, "output capacity too small");
-  if (on_device && n == ctx->n_pairs && !ctx->p_birth && ph::writable(ctx, birth, 8) &&
-      ph::writable(ctx, death, 8) && ph::writable(ctx, dim, 4) &&
-      ph::writable(ctx, birth_diam2, 8) && ph::writable(ctx, death_diam2, 8)) {
+  if (n == ctx->n_pairs && !ctx->p_birth && (on_device || n <= ph::kHostDirect) &&
+      ph::writable(ctx, birth, 8, on_device) && ph::writable(ctx, death, 8, on_device) &&
+      ph::writable(ctx, dim, 4, on_device) && ph::writable(ctx, birth_diam2, 8, on_device) &&
+      ph::writable(ctx, death_diam2, 8, on_device)) {
     ph::write_out<false>(ctx, ph::OutArrays{birth, death, birth_diam2, death_diam2, dim});
     ph::finish_out(ctx);
     return PH_OK;
@@ -735,8 +740,9 @@ int ph_get_essential(ph_ctx* ctx, int32_t cloud, int64_t* idx, int32_t* dim, int
   if (count) *count = n;
   if (!idx && !dim && !diam2) return PH_OK;
   PH_REQUIRE(capacity >= n, PH_ERR_CAPACITY, "output capacity too small");
-  if (on_device && n == ctx->n_ess && !ctx->e_idx && ph::writable(ctx, idx, 8) &&
-      ph::writable(ctx, dim, 4) && ph::writable(ctx, diam2, 8)) {
+  if (n == ctx->n_ess && !ctx->e_idx && (on_device || n <= ph::kHostDirect) &&
+      ph::writable(ctx, idx, 8, on_device) && ph::writable(ctx, dim, 4, on_device) &&
+      ph::writable(ctx, diam2, 8, on_device)) {
     ph::write_out<true>(ctx, ph::OutArrays{nullptr, idx, nullptr, diam2, dim});
     ph::finish_out(ctx);
     return PH_OK;
