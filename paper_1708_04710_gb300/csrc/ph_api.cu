@@ -379,26 +379,25 @@ static void extract_places(ph_ctx* ctx) {
   const int64_t nout = (m + kOutTile - 1) / kOutTile;
   const int nc = ctx->n_clouds;
   const int nseg = (int)ctx->seg_start.size() - 1;
-  // counts before each tile, the writers' error word, the scan's ticket, fault word and tile states,
-  // the image of low
-  ctx->out_before = alloc_n<unsigned long long>(ctx, nout + 3 + ntiles + (m + 7) / 8);
-  ctx->out_delta = alloc_n<int64_t>(ctx, 2 * (nseg + 1));
+  // counts before each tile, the scan's ticket and tile states, the image of low
+  ctx->out_before = alloc_n<unsigned long long>(ctx, nout + 1 + ntiles + (m + 7) / 8);
+  ctx->out_delta = alloc_n<int64_t>(ctx, 2 * nseg);
   unsigned long long* words = ctx->out_before + nout;
-  ctx->is_low = reinterpret_cast<uint8_t*>(words + 3 + ntiles);
-  PH_CUDA(cudaMemsetAsync(words, 0, (3 + ntiles) * sizeof(unsigned long long) + m, st));
+  ctx->is_low = reinterpret_cast<uint8_t*>(words + 1 + ntiles);
+  PH_CUDA(cudaMemsetAsync(words, 0, (1 + ntiles) * sizeof(unsigned long long) + m, st));
+  // the segments' counts and the fault word: written by the scan into page-locked memory (a copy back
+  // would be two more operations to wait for)
+  int64_t* sg = static_cast<int64_t*>(ctx->pinned((2 * (nseg + 1) + 1) * sizeof(int64_t)));
+  int32_t* fault = reinterpret_cast<int32_t*>(sg + 2 * (nseg + 1));
+  *fault = 0;
   k_mark_image<<<grid_for(ctx, m, kThreads), kThreads, 0, st>>>(m, ctx->low, ctx->is_low);
   PH_CHECK_LAUNCH();
   k_out_scan<<<(unsigned)ntiles, kThreads, 0, st>>>(
-      m, nseg, ctx->low, ctx->is_low, ctx->d_seg_start, words + 3, ntiles, ctx->out_before,
-      ctx->out_delta, (unsigned int*)(words + 1), (int32_t*)(words + 2));
+      m, nseg, ctx->low, ctx->is_low, ctx->d_seg_start, words + 1, ntiles, ctx->out_before, sg,
+      (unsigned int*)words, fault);
   PH_CHECK_LAUNCH();
-  int64_t* sg = static_cast<int64_t*>(ctx->pinned((2 * (nseg + 1) + 1) * sizeof(int64_t)));
-  PH_CUDA(cudaMemcpyAsync(sg, ctx->out_delta, 2 * (nseg + 1) * sizeof(int64_t),
-                          cudaMemcpyDeviceToHost, st));
-  PH_CUDA(cudaMemcpyAsync(sg + 2 * (nseg + 1), words + 2, sizeof(int64_t), cudaMemcpyDeviceToHost,
-                          st));
   PH_CUDA(cudaStreamSynchronize(st));
-  PH_REQUIRE(sg[2 * (nseg + 1)] == 0, PH_ERR_CUDA, "a bounded wait of the extraction ran out");
+  PH_REQUIRE(*fault == 0, PH_ERR_CUDA, "a bounded wait of the extraction ran out");
   // output bases: clouds in order, inside a cloud dimensions in order
   const int ndim = ctx->max_dim + 1;
   std::vector<int64_t> delta(2 * nseg);
@@ -425,8 +424,11 @@ static void extract_places(ph_ctx* ctx) {
   ctx->extracted = true;
 }
 
+// the writers' error word is page-locked memory as well (finish_out reads it)
 template <bool kEss>
 static void write_out(ph_ctx* ctx, const OutArrays& o) {
+  int32_t* bad = static_cast<int32_t*>(ctx->pinned(sizeof(int32_t)));
+  *bad = 0;
   const int64_t nout = (ctx->m + kOutTile - 1) / kOutTile;
   const bool lng = ctx->m >= kLongOut;
   const unsigned grid = grid_for(ctx, lng ? (ctx->m + kScanTile - 1) / kScanTile : nout, 1);
@@ -434,17 +436,16 @@ static void write_out(ph_ctx* ctx, const OutArrays& o) {
                                                                        ctx->stream>>>(
       ctx->m, ctx->n_clouds, ctx->seg, ctx->low, ctx->is_low, ctx->gidx, ctx->key, ctx->d2tab,
       ctx->out_before, ctx->out_delta, o, kEss ? ctx->n_ess : ctx->n_pairs,
-      (int32_t*)(ctx->out_before + nout));
+      bad);
   PH_CHECK_LAUNCH();
 }
 
 // after the results were written (and copied): waits, and checks the writers' error word
-static void finish_out(ph_ctx* ctx) {
-  int32_t* bad = static_cast<int32_t*>(ctx->pinned(sizeof(int32_t)));
-  PH_CUDA(cudaMemcpyAsync(bad, ctx->out_before + (ctx->m + kOutTile - 1) / kOutTile,
-                          sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
+static void finish_out(ph_ctx* ctx, bool written) {
   PH_CUDA(cudaStreamSynchronize(ctx->stream));
-  PH_REQUIRE(*bad == 0, PH_ERR_INVALID, "internal error: extraction index out of range");
+  const int32_t bad = written ? *static_cast<int32_t*>(ctx->pinned(sizeof(int32_t))) : 0;
+  if (bad) ctx->extracted = false;
+  PH_REQUIRE(bad == 0, PH_ERR_INVALID, "internal error: extraction index out of range");
 }
 
 template <typename T>
@@ -706,10 +707,11 @@ int ph_get_pairs(ph_ctx* ctx, int32_t cloud, int64_t* birth, int64_t* death, int
       ph::writable(ctx, dim, 4, on_device) && ph::writable(ctx, birth_diam2, 8, on_device) &&
       ph::writable(ctx, death_diam2, 8, on_device)) {
     ph::write_out<false>(ctx, ph::OutArrays{birth, death, birth_diam2, death_diam2, dim});
-    ph::finish_out(ctx);
+    ph::finish_out(ctx, true);
     return PH_OK;
   }
-  if (!ctx->p_birth) {
+  const bool written = !ctx->p_birth;
+  if (written) {
     const int64_t all = ctx->n_pairs;
     ph::renew(ctx, ctx->p_death, all);
     ph::renew(ctx, ctx->p_dim, all);
@@ -724,7 +726,7 @@ int ph_get_pairs(ph_ctx* ctx, int32_t cloud, int64_t* birth, int64_t* death, int
   copy_out(ctx, dim, ctx->p_dim + a, n * 4, on_device);
   copy_out(ctx, birth_diam2, ctx->p_bd2 + a, n * 8, on_device);
   copy_out(ctx, death_diam2, ctx->p_dd2 + a, n * 8, on_device);
-  ph::finish_out(ctx);
+  ph::finish_out(ctx, written);
   return PH_OK;
   PH_API_END
 }
@@ -744,10 +746,11 @@ int ph_get_essential(ph_ctx* ctx, int32_t cloud, int64_t* idx, int32_t* dim, int
       ph::writable(ctx, idx, 8, on_device) && ph::writable(ctx, dim, 4, on_device) &&
       ph::writable(ctx, diam2, 8, on_device)) {
     ph::write_out<true>(ctx, ph::OutArrays{nullptr, idx, nullptr, diam2, dim});
-    ph::finish_out(ctx);
+    ph::finish_out(ctx, true);
     return PH_OK;
   }
-  if (!ctx->e_idx) {
+  const bool written = !ctx->e_idx;
+  if (written) {
     const int64_t all = ctx->n_ess;
     ph::renew(ctx, ctx->e_dim, all);
     ph::renew(ctx, ctx->e_d2, all);
@@ -757,7 +760,7 @@ int ph_get_essential(ph_ctx* ctx, int32_t cloud, int64_t* idx, int32_t* dim, int
   copy_out(ctx, idx, ctx->e_idx + a, n * 8, on_device);
   copy_out(ctx, dim, ctx->e_dim + a, n * 4, on_device);
   copy_out(ctx, diam2, ctx->e_d2 + a, n * 8, on_device);
-  ph::finish_out(ctx);
+  ph::finish_out(ctx, written);
   return PH_OK;
   PH_API_END
 }
