@@ -215,8 +215,12 @@ __global__ void k_edge_finish(const uint64_t* __restrict__ vals, int64_t E, Clou
                               const int32_t* __restrict__ flag, const int64_t* __restrict__ excl,
                               const int64_t* __restrict__ ed2, int64_t id0, int32_t* eid,
                               int32_t* erank, int64_t* d2tab, IdOut o, int64_t rowbase,
-                              const int32_t* fault) {
-  if (*fault) return;
+                              const int64_t* __restrict__ status, int64_t* host) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) {  // for the host, in page-locked memory
+    host[0] = *status;  // bad coordinates (low half), a wait of the sort that ran out (high half)
+    host[1] = excl[E];  // distinct lengths
+  }
+  if (*status >> 32) return;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < E;
        i += (int64_t)gridDim.x * blockDim.x) {
     uint64_t p = vals[i];
@@ -447,8 +451,10 @@ __global__ void __launch_bounds__(32 * kDirectWarps) k_link_count(CloudTabs ct, 
   }
 }
 
-// per cloud (and the end): triangles and tetrahedra before its first edge
-__global__ void k_cloud_bounds(Direct g, int nc, int64_t* out) {
+// per cloud (and the end): triangles and tetrahedra before its first edge, then whether a wait ran out;
+// into page-locked memory
+__global__ void k_cloud_bounds(Direct g, int nc, int64_t* out, const int32_t* fault) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) out[2 * (nc + 1)] = *fault;
   for (int c = blockIdx.x * blockDim.x + threadIdx.x; c <= nc; c += gridDim.x * blockDim.x) {
     out[c] = g.off2[g.es[c]];
     out[nc + 1 + c] = g.off3 ? g.off3[g.es[c]] : 0;
@@ -957,8 +963,7 @@ static void build_direct(ph_ctx* ctx, const CloudTabs& ct, Direct g, const IdOut
   const int nc = ct.nc;
   const bool tets = ctx->max_dim == 3;
   // per cloud: first edge; then, from the device, triangles and tetrahedra before it
-  int64_t* d_es = alloc_n<int64_t>(ctx, 3 * (nc + 1));
-  int64_t* d_bounds = d_es + nc + 1;
+  int64_t* d_es = alloc_n<int64_t>(ctx, nc + 1);
   scratch[0] = 0;
   for (int c = 0; c < nc; c++) scratch[c + 1] = scratch[c] + h_cnt[c];
   PH_CUDA(cudaMemcpyAsync(d_es, scratch, (nc + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, st));
@@ -976,15 +981,11 @@ static void build_direct(ph_ctx* ctx, const CloudTabs& ct, Direct g, const IdOut
   k_link_count<<<grid, 32 * kDirectWarps, 0, st>>>(ct, g, cnt2, cnt3, mask);
   PH_CHECK_LAUNCH();
   scan_counts(ctx, cnt2, cnt3, g.E, off2, off3, d_fault);
-  k_cloud_bounds<<<grid_for(ctx, nc + 1, kThreads), kThreads, 0, st>>>(g, nc, d_bounds);
-  PH_CHECK_LAUNCH();
   int64_t* h_bounds = scratch + nc + 1;
-  int32_t* h_fault = reinterpret_cast<int32_t*>(scratch + 3 * (nc + 1));
-  PH_CUDA(cudaMemcpyAsync(h_bounds, d_bounds, 2 * (nc + 1) * sizeof(int64_t),
-                          cudaMemcpyDeviceToHost, st));
-  PH_CUDA(cudaMemcpyAsync(h_fault, d_fault, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+  k_cloud_bounds<<<grid_for(ctx, nc + 1, kThreads), kThreads, 0, st>>>(g, nc, h_bounds, d_fault);
+  PH_CHECK_LAUNCH();
   PH_CUDA(cudaStreamSynchronize(st));
-  PH_REQUIRE(*h_fault == 0, PH_ERR_CUDA, kSortFault);
+  PH_REQUIRE(h_bounds[2 * (nc + 1)] == 0, PH_ERR_CUDA, kSortFault);
   for (int d = 2; d <= ctx->max_dim; d++) {
     const int64_t* b = h_bounds + (d - 2) * (nc + 1);
     for (int c = 0; c < nc; c++) h_cnt[(int64_t)(d - 1) * nc + c] = b[c + 1] - b[c];
@@ -1189,10 +1190,8 @@ void build_vr(ph_ctx* ctx, const int32_t* coords, const int64_t* cloud_offsets, 
     PH_CHECK_LAUNCH();
     scan_counts(ctx, flag, nullptr, E, excl, nullptr, d_fault);
     k_edge_finish<<<grid_for(ctx, E, kThreads), kThreads, 0, st>>>(
-        vbuf, E, ct, flag, excl, ed2, N, eid, erank, ctx->d2tab, o, 0, d_fault);
+        vbuf, E, ct, flag, excl, ed2, N, eid, erank, ctx->d2tab, o, 0, d_misc, h_misc);
     PH_CHECK_LAUNCH();
-    PH_CUDA(cudaMemcpyAsync(h_misc, d_misc, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
-    PH_CUDA(cudaMemcpyAsync(h_misc + 1, excl + E, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
     PH_CUDA(cudaStreamSynchronize(st));
     PH_REQUIRE(*(int32_t*)h_misc == 0, PH_ERR_INVALID, kBadCoords);
     PH_REQUIRE(h_misc[0] == 0, PH_ERR_CUDA, kSortFault);
