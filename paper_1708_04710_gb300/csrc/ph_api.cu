@@ -165,7 +165,7 @@ __global__ void k_mark_image(int64_t m, const int32_t* __restrict__ low, uint8_t
 // gathered birth each), by the two waits of a request for short ones. With two flag arrays, six scan
 // kernels and a copy of every result the pairs and essentials of 512 clouds of 20 to 120 points (42.7 M
 // simplices) took 1.51 + 0.29 ms, now 0.38 + 0.39 ms; of 400 points 0.49 + 0.12 ms, now 0.16 + 0.14;
-// of 40 points 183 + 37 us, now 96 + 46 us.
+// of 40 points 183 + 37 us, now 67 + 28 us.
 constexpr int kScanTile = 4096, kOutTile = 1024;  // ids per block of the scan; per counted place
 // a writer's round takes kScanTile ids of a long complex (a round of 1024 held 39 pairs of a 512-cloud
 // batch's and waited on each in turn: 256 us), kOutTile of a short one, whose rounds run side by side

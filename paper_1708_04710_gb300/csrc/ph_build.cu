@@ -155,7 +155,8 @@ __device__ __forceinline__ void count_kept(int64_t* count_per_cloud, int c, bool
 // bit more than *largest. Kept ones are counted if some may be truncated
 __global__ void k_edge_cand(CloudTabs ct, const int64_t* __restrict__ cand, int64_t ncand,
                             const int64_t* __restrict__ d2, int64_t max_d2, uint64_t sent,
-                            const unsigned long long* largest, uint64_t* keys, uint64_t* vals, int64_t* count_per_cloud) {
+                            const unsigned long long* largest, uint64_t* keys, uint64_t* vals,
+                            int64_t* count_per_cloud) {
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < ncand;
        t += (int64_t)gridDim.x * blockDim.x) {
     int c = find_cloud(cand, ct.nc, t);
@@ -878,7 +879,7 @@ void load_boundary(ph_ctx* ctx, int64_t m, const int32_t* dims, const int64_t* c
   }
   // One host buffer, copied at once: the filtration index and the column's end per id, the columns'
   // rows as ids; then, not copied, the id per index. Kept page-locked memory up to a size (fresh pages
-  // and seven copies were a fifth of the 374 us of a 96 x 80 image grid's 30,369 simplices; 304 us now).
+  // and seven copies were a fifth of the 374 us of a 96 x 80 image grid's 30,369 simplices; 300 us now).
   constexpr int64_t kLoadPinned = 16 << 20;
   const int64_t copied = (2 * m + 1) * 8 + (nnz + (nnz & 1)) * 4, bytes = copied + 4 * m;
   std::unique_ptr<char[]> pageable;
@@ -1186,7 +1187,8 @@ void build_vr(ph_ctx* ctx, const int32_t* coords, const int64_t* cloud_offsets, 
     int32_t* flag = alloc_n<int32_t>(ctx, E);
     int64_t* excl = alloc_n<int64_t>(ctx, E + 1);
     int64_t* ed2 = alloc_n<int64_t>(ctx, E);
-    k_edge_newflag<<<grid_for(ctx, E, kThreads), kThreads, 0, st>>>(vbuf, E, ct, d2, flag, ed2, d_fault);
+    k_edge_newflag<<<grid_for(ctx, E, kThreads), kThreads, 0, st>>>(vbuf, E, ct, d2, flag, ed2,
+                                                                  d_fault);
     PH_CHECK_LAUNCH();
     scan_counts(ctx, flag, nullptr, E, excl, nullptr, d_fault);
     k_edge_finish<<<grid_for(ctx, E, kThreads), kThreads, 0, st>>>(

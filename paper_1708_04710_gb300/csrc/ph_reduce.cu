@@ -44,8 +44,8 @@
 //                between k_phase1 and k_add and hold back the other targets.
 //   k_commit     publishes the new locations of the columns other jobs may have been reading
 //                and moves on the first unpaired row of the segments where it was paired; its last
-//                block ends the pass: the next active list, convergence (no collision left, Thm 8), the pass cap and
-//                time bound, and inside a CUDA graph the conditional that repeats the pass.
+//                block ends the pass: the next active list, convergence (no collision left,
+//                Thm 8), the pass cap and time bound, and inside a CUDA graph the conditional that repeats the pass.
 // All per-pass state lives in device memory (DevState), so the same kernel sequence runs either
 // from a host loop or as the body of a graph's conditional while node. Each kernel may start
 // while its predecessor drains (programmatic dependent launch) and waits for it first. Short lists
@@ -595,8 +595,8 @@ constexpr int kDeltaRows = kOld + kSourceRows * kAheadMax;
 __host__ __device__ inline int64_t lows_stride_of(int64_t m) { return (m + 7) & ~int64_t(7); }
 
 // The rows of a row's proven pivot, one 16-byte record: x is its length (0: no pivot yet), y, z
-// and w its rows below the low, then INT32_MAX (length <= kRecRows), or y and z the address of its rows. A
-// bit-packed pivot's record holds kRecLong alone.
+// and w its rows below the low, then INT32_MAX (length <= kRecRows), or y and z the address of its
+// rows. A bit-packed pivot's record holds kRecLong alone.
 constexpr int32_t kRecRows = 4;
 constexpr int32_t kRecLong = INT32_MAX;
 
@@ -2590,11 +2590,11 @@ enum : uint8_t {
   kMoveLate,  // ... but others may be reading it in this pass: published by k_commit
 };
 
-// Phase II with look-ahead, first half: every column that is due gets its source for this pass. A source of few
-// rows starts a visit (look_ahead), which leaves the column's list as it is, only shortened, and
-// its delta beside it; the columns whose list has to be rewritten, or whose source is too long
-// for a visit, are left to k_merge. In a pass that compacts that is every survivor: it gets its
-// place in the next active list from a decoupled look-back over the chunks. New pivots are
+// Phase II with look-ahead, first half: every column that is due gets its source for this pass. A
+// source of few rows starts a visit (look_ahead), which leaves the column's list as it is, only
+// shortened, and its delta beside it; the columns whose list has to be rewritten, or whose source is
+// too long for a visit, are left to k_merge. In a pass that compacts that is every survivor: its
+// place in the next active list comes from Phase I (newpos). New pivots are
 // copied to the pivot store. Targets and zeroed columns are updated in place (no other job reads
 // them this pass); new pivots and left-most survivors, which other jobs may be reading as
 // sources, are updated by k_commit.
@@ -3263,7 +3263,8 @@ __global__ void k_clock_start(DevState* ds) { ds->t_start = global_ns(); }
 constexpr int kLoopMost = 64;
 __host__ __device__ inline unsigned int loop_blocks_for(int64_t n) {
   const int64_t per8 = (n + 8 * kWarps - 1) / (8 * kWarps), per32 = (n + kThreads - 1) / kThreads;
-  return n <= kLoopSingle ? 1u : (unsigned int)(per8 < kLoopMost ? per8 : per32 > kLoopMost ? per32 : kLoopMost);
+  const int64_t many = per32 > kLoopMost ? per32 : kLoopMost;
+  return n <= kLoopSingle ? 1u : (unsigned int)(per8 < kLoopMost ? per8 : many);
 }
 
 // end of a pass: the next active list, convergence (no target left), the pass cap, the time
