@@ -3203,12 +3203,13 @@ __device__ __forceinline__ bool grid_last(DevState* ds, unsigned blocks, unsigne
 }
 
 // A call that begins with up to kLoopStart columns runs in k_loop alone: it saves the graph's launch
-// and the return to the host (about 100 us: 121,575 columns 1256 -> 1061 us, 36,050 columns 678 ->
-// 557 us, 43,904 of a batch 614 -> 472 us), while its passes over long lists are slower than the
-// graph's (166,750 columns, 8 passes: 500 us there, 580 us here). A call that begins in the graph
-// goes over to it at kLoopBelow columns (16,384 to 65,536 measure alike, 131,072 costs 50 to 90 us).
+// and the return to the host, while its passes over long lists are slower than the graph's. Graph ->
+// k_loop: 85,400 columns 881 -> 853 and 733 -> 715 us, 65,856 of a batch 402 -> 361; 102,425 columns
+// 875 -> 799, but 495 -> 527 where lists stay long; 121,575 columns 1078 -> 1052, but 366 -> 443; 166,750
+// columns, 8 passes, 336 -> 431. A call that begins in the graph goes over to it at kLoopBelow columns
+// (16,384 to 65,536 measure alike, 131,072 costs 50 to 90 us).
 constexpr int64_t kLoopBelow = (int64_t)1 << 14;
-constexpr int64_t kLoopStart = (int64_t)1 << 17;
+constexpr int64_t kLoopStart = 110000;
 // columns left to one block, whose barriers are __syncthreads (64 and 256 measure alike)
 constexpr int64_t kLoopSingle = 64;
 constexpr int kLoopBlocks = 2;  // per SM: registers for every part of a pass without spills
@@ -3937,6 +3938,7 @@ int reduce_run(ph_ctx* ctx, int32_t max_passes) {
   const bool time_add = ctx->opts.time_kernels != 0 && !use_graph;
   DevState& h = *static_cast<DevState*>(rs.hstate);
   // a resumed reduction continues after the pass that hit the previous cap
+  bool loop_states_clear = rs.fresh;  // k_loop's tile states: nothing of an earlier pass in them
   if (!rs.fresh) {  // (what set-up wrote is still in the host's copy)
     PH_CUDA(cudaMemcpyAsync(&h, rs.dstate, sizeof(DevState), cudaMemcpyDeviceToHost, st));
     PH_CUDA(cudaStreamSynchronize(st));
@@ -3967,6 +3969,7 @@ int reduce_run(ph_ctx* ctx, int32_t max_passes) {
   const RArgs a = make_args(ctx);
 
   bool started = false;    // this call has launched passes
+  bool in_loop = false;    // the last of them by k_loop
   bool rest_only = false;  // a pass stopped for space after its marks continues at Phase II
   for (;;) {
     const int32_t first_pass = h.pass;
@@ -3978,7 +3981,14 @@ int reduce_run(ph_ctx* ctx, int32_t max_passes) {
       launch_pass_rest(ctx, a, 0, false, variant, time_add, st);
       if (time_add) rs.add_launches++;
     } else if (use_graph && loop_blocks && h.ahead == 1 &&
-               h.n_act <= (started ? h.loop_below : kLoopStart)) {
+               h.n_act <= (started && !in_loop ? h.loop_below : kLoopStart)) {
+      // a state's tag has eight bits: one left by an earlier stay in k_loop could pass for this one's
+      if (!in_loop && !loop_states_clear) {
+        const int64_t tiles = (std::min<int64_t>(ctx->m, kLoopStart) + kThreads - 1) / kThreads;
+        PH_CUDA(cudaMemsetAsync(a.loop_tile_st, 0, tiles * sizeof(unsigned long long), st));
+      }
+      loop_states_clear = false;
+      in_loop = true;
       h.loop_blocks = std::min(loop_blocks, loop_blocks_for(h.n_act));
       PH_CUDA(cudaMemcpyAsync(&static_cast<DevState*>(rs.dstate)->loop_blocks, &h.loop_blocks,
                               sizeof(h.loop_blocks), cudaMemcpyHostToDevice, st));
@@ -3990,6 +4000,7 @@ int reduce_run(ph_ctx* ctx, int32_t max_passes) {
       if (ce == cudaErrorCooperativeLaunchTooLarge || ce == cudaErrorNotSupported) {
         cudaGetLastError();  // a share of the device without room for it: the graph throughout
         loop_blocks = 0;
+        in_loop = false;
         h.loop_below = -1;
         PH_CUDA(cudaMemcpyAsync(rs.dstate, &h, sizeof(DevState), cudaMemcpyHostToDevice, st));
         PH_CUDA(cudaStreamSynchronize(st));
@@ -3999,6 +4010,7 @@ int reduce_run(ph_ctx* ctx, int32_t max_passes) {
       PH_CHECK_LAUNCH();
     } else if (use_graph) {
       ran_graph = true;
+      in_loop = false;
       PH_CUDA(cudaGraphLaunch(pass_graph(ctx, a, variant), st));
     } else {
       launch_pass(ctx, a, 0, false, variant, time_add, st);

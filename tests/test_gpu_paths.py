@@ -226,9 +226,9 @@ def test_look_ahead_of_a_batch(ph):
 
 
 # the loop kernel: 1, 4, 8 or 32 columns per warp (8, 32, 64 columns, then 8 per warp of up to 64
-# blocks), one block up to 64 columns, several tiles per block above 77,824 (90 points), and 93 points
-# (134,230 columns) that begin in the pass graph; a lack of space stops it within a pass
-@pytest.mark.parametrize("n", [3, 4, 5, 7, 8, 12, 17, 40, 90, 93])
+# blocks), one block up to 64 columns, several tiles per block above 77,824 (86 points, 106,081), and 93
+# points (134,230 columns) that begin in the pass graph; a lack of space stops it within a pass
+@pytest.mark.parametrize("n", [3, 4, 5, 7, 8, 12, 17, 40, 86, 93])
 @pytest.mark.parametrize("opts", [{}, {"arena_words": 1}, {"predict_pairs": True}], ids=str)
 def test_loop_kernel_equals_host_loop(ph, n, opts):
     x = pc.random_cloud(n, 2, 1700 + n)
