@@ -289,18 +289,23 @@ void radix_sort_u64(ph_ctx* ctx, uint64_t* keys, uint64_t* vals, int64_t n, int 
     return;
   }
   const int64_t ntiles = (n + kTile - 1) / kTile;
-  // per digit: its counts, its tiles' states, its ticket
-  const int64_t words = 256 * digits + 256 * ntiles * digits + digits;
+  // per digit: its counts, its ticket, its tiles' states (long sorts: one digit's, cleared in between)
+  constexpr int64_t kManyStates = 4 << 20;
+  const int64_t states = 256 * ntiles;
+  const bool again = states * digits > kManyStates;
+  const int64_t words = 257 * digits + states * (again ? 1 : digits);
   unsigned long long* buf = alloc_n<unsigned long long>(ctx, words);
-  unsigned long long* state = buf + 256 * digits;
-  unsigned long long* ticket = state + 256 * ntiles * digits;
+  unsigned long long* ticket = buf + 256 * digits;
+  unsigned long long* state = ticket + digits;
   PH_CUDA(cudaMemsetAsync(buf, 0, words * sizeof(unsigned long long), st));
   k_radix_count<<<grid_for(ctx, n, kThreads * 4), kThreads, 0, st>>>(keys, n, lo_bit, digits, buf);
   PH_CHECK_LAUNCH();
   uint64_t *ka = keys, *va = vals, *kb = tmp_keys, *vb = tmp_vals;
   for (int p = 0; p < digits; p++) {
+    if (again && p > 0)
+      PH_CUDA(cudaMemsetAsync(state, 0, states * sizeof(unsigned long long), st));
     k_radix_pass<<<(unsigned)ntiles, kThreads, 0, st>>>(
-        ka, va, kb, vb, n, lo_bit + 8 * p, buf + 256 * p, state + 256 * ntiles * p,
+        ka, va, kb, vb, n, lo_bit + 8 * p, buf + 256 * p, state + (again ? 0 : states * p),
         (unsigned int*)(ticket + p), fault);
     PH_CHECK_LAUNCH();
     std::swap(ka, kb);

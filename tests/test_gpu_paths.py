@@ -90,6 +90,23 @@ def test_edge_sort_sizes(ph, orc, sizes, cut):
         assert np.array_equal(f["diam2"], K["diam2"]) and np.array_equal(f["verts"], K["verts"])
 
 
+def test_long_sort_clears_its_states(ph):
+    """12,259,940 triangles by three digits: one digit's tile states at a time."""
+    n = 420
+    x = pc.random_cloud(n, 3, 77).astype(np.int64)
+    x[1] = 2 * x[0] - x[2]  # x0 halfway between x1 and x2: a tie, so candidates are sorted
+    ctx = _build(ph.Context(), [x], 2)
+    f = ctx.filtration(0)
+    tri = f["dim"] == 2
+    d2 = ((x[:, None] - x[None]) ** 2).sum(-1)
+    i, j, k = f["verts"][tri, :3].T.astype(np.int64)
+    want = np.maximum(np.maximum(d2[i, j], d2[i, k]), d2[j, k])
+    assert len(want) == 12_259_940 and (i < j).all() and (j < k).all()
+    assert np.array_equal(f["diam2"][tri], want) and (np.diff(want) >= 0).all()
+    code = (i * n + j) * n + k  # ties in lexicographic order, so no triangle twice
+    assert (np.diff(code)[np.diff(want) == 0] > 0).all()
+
+
 # 1024 and 4096 ids are a writer's round and a scan's tile; 235 points have more than 2^21 ids (long
 # rounds); three hundred clouds put many segments, some empty, into one tile
 @pytest.mark.parametrize("sizes,max_dim,passes", [
