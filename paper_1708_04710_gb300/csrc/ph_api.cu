@@ -137,6 +137,7 @@ void ph_ctx::free_all() {
   gidx = nullptr;
   verts = nullptr;
   d2tab = nullptr;
+  d_pt_off = nullptr;
   d_seg_start = nullptr;
   m = nnz = 0;
   D = 0;

@@ -1070,6 +1070,7 @@ void build_vr(ph_ctx* ctx, const int32_t* coords, const int64_t* cloud_offsets, 
   PH_CUDA(cudaMemcpyAsync(d_tabs, h_tabs.data(), h_tabs.size() * sizeof(int64_t),
                           cudaMemcpyHostToDevice, st));
   CloudTabs ct{d_tabs, d_tabs + (nc + 1), nc, vbits};
+  ctx->d_pt_off = d_tabs;
   auto d_cand = [&](int k) -> const int64_t* { return d_tabs + (int64_t)k * (nc + 1); };
 
   // scratch: status words [0] bad coords, [1] max d2, then per-cloud counts of every dimension
@@ -1303,7 +1304,7 @@ void build_vr(ph_ctx* ctx, const int32_t* coords, const int64_t* cloud_offsets, 
   for (int32_t* t : lex_tab)
     if (t) ctx->dfree(t);
   ctx->dfree(d_misc);
-  // d_tabs holds pt_off, needed by extraction: keep it alive as ctx->... (freed with ctx)
+  // (d_tabs stays: the diagram losses read pt_off)
 }
 
 }  // namespace ph

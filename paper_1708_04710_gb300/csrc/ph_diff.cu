@@ -256,15 +256,13 @@ int ph_build_filtration_f32(ph_ctx* ctx, const float* coords, const int64_t* clo
   const int64_t n = n_points * D;
   // the rounded copy lives with the filtration (freed with it)
   int32_t* g = ph::alloc_n<int32_t>(ctx, n);
-  int32_t* bad = ph::alloc_n<int32_t>(ctx, 1);
-  PH_CUDA(cudaMemsetAsync(bad, 0, sizeof(int32_t), ctx->stream));
+  int32_t* bad = static_cast<int32_t*>(ctx->pinned(sizeof(int32_t)));  // written by the kernel
+  *bad = 0;
   ph::k_to_grid<<<ph::grid_for(ctx, n, ph::kThreads), ph::kThreads, 0, ctx->stream>>>(coords, n,
                                                                                      g, bad);
   PH_CHECK_LAUNCH();
-  int32_t h_bad = 0;
-  PH_CUDA(cudaMemcpyAsync(&h_bad, bad, sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
   PH_CUDA(cudaStreamSynchronize(ctx->stream));
-  PH_REQUIRE(h_bad == 0, PH_ERR_INVALID, "coordinates must be finite with |x| <= 256");
+  PH_REQUIRE(*bad == 0, PH_ERR_INVALID, "coordinates must be finite with |x| <= 256");
   ph::build_vr(ctx, g, cloud_offsets, n_clouds, n_points, D, max_dim, max_diam2);
   ctx->built = true;
   ctx->is_vr = true;
@@ -286,21 +284,18 @@ int ph_diagram_loss(ph_ctx* ctx, const float* coords, int32_t D, int32_t dim, fl
              "D must equal the D of the build (" + std::to_string(ctx->D) + ")");
   const ph::DiagLayout L = ph::layout_of(ctx);
   unsigned long long* cnt = ph::alloc_n<unsigned long long>(ctx, 1);
-  int64_t* d_pt = ph::alloc_n<int64_t>(ctx, ctx->n_clouds + 1);
-  PH_CUDA(cudaMemcpyAsync(d_pt, ctx->pt_off.data(), (ctx->n_clouds + 1) * sizeof(int64_t),
-                          cudaMemcpyHostToDevice, ctx->stream));
+  const int64_t* d_pt = ctx->d_pt_off;
   PH_CUDA(cudaMemsetAsync(cnt, 0, sizeof(unsigned long long), ctx->stream));
   ph::k_diag_loss<<<ctx->n_clouds, ph::kThreads, 0, ctx->stream>>>(
       L, dim + 1, ctx->d_seg_start, ctx->low, ctx->rows0, ctx->verts, d_pt, coords, D, loss, cnt);
   PH_CHECK_LAUNCH();
   ph::k_diag_total<<<1, 32, 0, ctx->stream>>>(loss, ctx->n_clouds, loss + ctx->n_clouds);
   PH_CHECK_LAUNCH();
-  unsigned long long h = 0;
-  PH_CUDA(cudaMemcpyAsync(&h, cnt, sizeof(h), cudaMemcpyDeviceToHost, ctx->stream));
+  auto* h = static_cast<unsigned long long*>(ctx->pinned(sizeof(*cnt)));
+  PH_CUDA(cudaMemcpyAsync(h, cnt, sizeof(*cnt), cudaMemcpyDeviceToHost, ctx->stream));
   PH_CUDA(cudaStreamSynchronize(ctx->stream));
   ctx->dfree(cnt);
-  ctx->dfree(d_pt);
-  if (n_pairs) *n_pairs = (int64_t)h;
+  if (n_pairs) *n_pairs = (int64_t)*h;
   return PH_OK;
   PH_API_END
 }
@@ -316,15 +311,12 @@ int ph_diagram_backward(ph_ctx* ctx, const float* coords, int32_t D, int32_t dim
   PH_REQUIRE(D == ctx->D, PH_ERR_INVALID,
              "D must equal the D of the build (" + std::to_string(ctx->D) + ")");
   const ph::DiagLayout L = ph::layout_of(ctx);
-  int64_t* d_pt = ph::alloc_n<int64_t>(ctx, ctx->n_clouds + 1);
-  PH_CUDA(cudaMemcpyAsync(d_pt, ctx->pt_off.data(), (ctx->n_clouds + 1) * sizeof(int64_t),
-                          cudaMemcpyHostToDevice, ctx->stream));
+  const int64_t* d_pt = ctx->d_pt_off;
   const int64_t lo = ctx->dimoff[dim + 1], hi = ctx->dimoff[dim + 2];
   ph::k_diag_bwd<<<ph::grid_for(ctx, hi - lo, ph::kPairRound), ph::kThreads, 0, ctx->stream>>>(
       L, dim + 1, lo, hi, ctx->seg, ctx->low, ctx->rows0, ctx->verts, d_pt, coords, D, grad_loss,
       grad_coords);
   PH_CHECK_LAUNCH();
-  ctx->dfree(d_pt);
   return PH_OK;
   PH_API_END
 }

@@ -204,6 +204,7 @@ struct ph_ctx {
   uint64_t* verts = nullptr;  // per id: packed (cloud, vertex slots of vbits bits)
   int vbits = ph::kVertBits;  // bits per packed vertex of this build
   int64_t* d2tab = nullptr;   // dense rank -> squared diameter
+  const int64_t* d_pt_off = nullptr;  // VR builds: per cloud, its first point (device, nc + 1)
   int64_t n_d2 = 0;
   int32_t* rows0 = nullptr;   // initial column storage (boundary matrix, CSC by id)
   // loaded matrices: per id, the offset of its column in rows0 ([m + 1]); VR builds store
