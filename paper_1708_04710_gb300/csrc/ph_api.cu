@@ -627,10 +627,12 @@ int ph_load_boundary(ph_ctx* ctx, int64_t m, const int32_t* dims, const int64_t*
 int ph_reduce(ph_ctx* ctx, int32_t max_passes, ph_stats* out) {
   PH_API_BEGIN
   PH_REQUIRE(ctx->built, PH_ERR_INVALID, "no filtration: call ph_build_filtration first");
+  // the places of the results belong to the lows as they are: they go before any pass changes these,
+  // since the call may also end part-way (time bound, refused allocation)
+  ctx->extracted = false;
   if (!ctx->rs.init) ph::reduce_init(ctx);
   int rc = ctx->rs.status;
   if (!(ctx->rs.done && ctx->rs.status == PH_OK)) rc = ph::reduce_run(ctx, max_passes);
-  ctx->extracted = false;
   ctx->reduced = true;
   if (out) {
     std::memset(out, 0, sizeof(*out));

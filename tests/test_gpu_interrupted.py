@@ -1,0 +1,111 @@
+"""What a caller reads after a reduction that stopped part-way: at the time bound or for want of memory.
+
+Every such stop leaves the reduction after some whole number of passes, so the reads are compared with
+a pass-by-pass run (a context with per-pass counters) capped there, and with each other. From 3,000,000
+columns on columns run ahead of the pass; 270 points have 3,280,455, 200 points 1,333,500.
+"""
+import numpy as np
+import pytest
+
+import pointclouds as pc
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ph():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_1708_04710_gb300 import build
+
+    build.build()
+    import paper_1708_04710_gb300 as ph
+
+    return ph
+
+
+def _cloud(n):
+    return pc.to_grid(pc.sphere(n, np.random.Generator(np.random.PCG64(3)), noise=0.05))
+
+
+def _built(ph, n, **opts):
+    import torch
+
+    ctx = ph.Context(**opts)
+    ctx.build_filtration(torch.from_numpy(_cloud(n)).cuda(), None, 2)
+    return ctx
+
+
+class PassByPass:
+    """The states of a reduction first capped at pass `first` (a cap takes the pass's marks, and the
+    next call goes on behind them) and then at pass k, for any k."""
+
+    def __init__(self, ph, n, first):
+        self.ctx, self.first, self.lows = _built(ph, n, collect_stats=True), first, {}
+        self.passes = self.state(-1)["passes"]
+
+    def state(self, k):
+        self.ctx.reset_reduction()
+        st = self.ctx.reduce(max_passes=self.first)
+        return st if k == self.first else self.ctx.reduce(max_passes=k)
+
+    def low(self, k):
+        if k not in self.lows:
+            self.state(k)
+            self.lows[k] = self.ctx.filtration(0)["low"]
+        return self.lows[k]
+
+
+_refs = {}
+
+
+def _ref(ph, n, first):
+    if (n, first) not in _refs:
+        _refs[n, first] = PassByPass(ph, n, first)
+    return _refs[n, first]
+
+
+def _check_pairs(ctx):
+    """pairs() and essential() are those of the lows."""
+    f = ctx.filtration(0)
+    order = np.argsort(f["dim"], kind="stable")  # (dimension, index)
+    death = order[f["low"][order] >= 0]
+    birth = f["low"][death]
+    is_low = np.zeros(len(order), bool)
+    is_low[birth] = True
+    ess = order[(f["low"][order] < 0) & ~is_low[order]]
+    for cloud in (-1, 0):
+        pr, es = ctx.pairs(cloud, on_device=cloud < 0), ctx.essential(cloud)
+        assert np.array_equal(pr["death"].cpu().numpy(), death)
+        assert np.array_equal(pr["birth"].cpu().numpy(), birth)
+        assert np.array_equal(pr["birth_diam2"].cpu().numpy(), f["diam2"][birth])
+        assert np.array_equal(es["idx"].cpu().numpy(), ess)
+
+
+def _finish(ctx, ref):
+    st = ctx.reduce()
+    assert st["converged"] and st["passes"] == ref.passes
+    assert np.array_equal(ctx.filtration(0)["low"], ref.low(ref.passes))
+    _check_pairs(ctx)
+
+
+def _until_done(ph, ctx, each):
+    """Calls reduce until it ends, `each` after every call that the time bound stopped."""
+    for stops in range(200):
+        try:
+            ctx.reduce()
+            return stops
+        except ph.PHError as err:
+            assert err.code == -5
+            each()
+    pytest.fail("the reduction did not finish")
+
+
+@pytest.mark.parametrize("n,use_graph", [(200, True), (270, True), (270, False)])
+def test_pairs_after_the_time_bound(ph, n, use_graph):
+    ctx = _built(ph, n, use_graph=use_graph, timeout_ms=1)
+    ctx.reduce(max_passes=0)
+    _check_pairs(ctx)
+    assert _until_done(ph, ctx, lambda: _check_pairs(ctx)) >= 1
+    _finish(ctx, _ref(ph, n, 0))
