@@ -136,7 +136,7 @@ struct DevState {
   int32_t horizon;
   int32_t compact;    // this pass compacts the active list (its columns are all up to date)
   int32_t arena_cur;  // the arena this pass writes into
-  int32_t drain;      // past the time bound: no more look-ahead, stop at the horizon
+  int32_t drain;      // past the time bound: no more look-ahead, stop after the horizon's pass
   int32_t leave;      // the last pass of look-ahead
 };
 
@@ -214,6 +214,7 @@ struct PV {
   int32_t limit;      // the last pass a column visited now may run ahead to
   int32_t ahead;      // passes a visit may run ahead; 1: every pass visits every column
   int32_t whole;      // ... and the lists must be whole there (the pass cap, or the time bound)
+  int32_t drain;      // past the time bound
 };
 
 // The left-most-column table holds, per row, a column below the pass it was entered for, counted
@@ -243,7 +244,8 @@ __device__ __forceinline__ PV pass_view(const DevState* ds) {
   v.ahead = ds->ahead;
   v.limit = ds->drain || ds->leave ? ds->pass + 1
                       : min(min(ds->pass + ds->ahead, ds->horizon), ds->max_passes);
-  v.whole = ds->drain || v.limit == ds->max_passes;
+  v.drain = ds->drain;
+  v.whole = v.drain || v.limit == ds->max_passes;
   return v;
 }
 
@@ -2667,8 +2669,8 @@ __device__ __forceinline__ void visit_round(const RArgs& a, const PV& v, int32_t
     for (int i = kOld; i < kDeltaRows; i++) w.d.c[i] = kEmpty;
     const bool c10 = visit && a.cor10 && a.beta[j] < 0;
     no_beta = c10;
-    const int32_t fu =
-        c10 ? a.first_unp[seg_of(a, j) - a.nc] : INT32_MIN;
+    // (at the time bound the loop may stop before the pass that zeroes the column: it keeps its rows)
+    const int32_t fu = c10 && !v.drain ? a.first_unp[seg_of(a, j) - a.nc] : INT32_MIN;
     if (look_ahead(a, v, pass, visit, fu, pos, w)) tidy<0>(w, visit && !w.gone);
     else tidy<kOld>(w, visit && !w.gone);
     if (visit) {
@@ -3342,11 +3344,13 @@ __device__ void end_of_pass(const RArgs& a, cudaGraphConditionalHandle cond, int
       const bool to_narrow = compact && (warp_on || to_warp) && ahead == 1 &&
                              (!lane_on || to_pieces) && !narrow_on && n_surv < narrow_below;
       if (to_narrow) ds->narrow_on = 1;
-      // the pass is complete, so a later call can resume from the next one
-      // (with columns ahead of the pass, it first runs on to where all are up to date)
+      // past the time bound a later call resumes from the next pass, and what the caller reads until
+      // then is this pass's result: with columns ahead of the pass it first runs on without look-ahead
+      // to the horizon, whose pass visits every column, makes its list whole and runs it no further
       const bool late = drain || global_ns() - t_start > t_limit;
+      const bool whole = was_ahead == 1 || (compact && drain);
       if (late) ds->drain = 1;
-      if (late && next_compact) status = ST_TIMEOUT;
+      if (late && whole) status = ST_TIMEOUT;
       else if (mode != kInLoop && (to_dense || to_warp || to_pieces || to_narrow || to_add))
         status = ST_SWITCH;
       else if (in_graph && ahead == 1 && n_surv <= loop_below) status = ST_SWITCH;

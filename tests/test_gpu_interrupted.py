@@ -56,6 +56,18 @@ class PassByPass:
             self.lows[k] = self.ctx.filtration(0)["low"]
         return self.lows[k]
 
+    def columns(self, k):
+        self.state(k)
+        return self.ctx.columns(0)
+
+    def passes_of(self, low):
+        """At which cap the lows are these (those that its marks zero may still be there)."""
+        for k in range(self.first, self.passes + 1):
+            r = self.low(k)
+            if np.all((low == r) | (r < 0)):
+                return k
+        pytest.fail("the lows are those of no pass")
+
 
 _refs = {}
 
@@ -81,6 +93,22 @@ def _check_pairs(ctx):
         assert np.array_equal(pr["birth"].cpu().numpy(), birth)
         assert np.array_equal(pr["birth_diam2"].cpu().numpy(), f["diam2"][birth])
         assert np.array_equal(es["idx"].cpu().numpy(), ess)
+
+
+def _check_columns(ctx, ref):
+    """columns() and the lows are those after some pass; returns its number."""
+    low = ctx.filtration(0)["low"]
+    ptr, rows = ctx.columns(0)
+    last = np.full(len(low), -1, np.int64)
+    some = np.diff(ptr) > 0
+    last[some] = rows[ptr[1:][some] - 1]
+    assert np.array_equal(last, low)
+    k = ref.passes_of(low)
+    rptr, rrows = ref.columns(k)
+    kept = ref.low(k) >= 0  # (the others' columns are empty there already)
+    assert np.array_equal(np.diff(ptr)[kept], np.diff(rptr)[kept])
+    assert np.array_equal(rows[np.repeat(kept, np.diff(ptr))], rrows)
+    return k
 
 
 def _finish(ctx, ref):
@@ -109,3 +137,14 @@ def test_pairs_after_the_time_bound(ph, n, use_graph):
     _check_pairs(ctx)
     assert _until_done(ph, ctx, lambda: _check_pairs(ctx)) >= 1
     _finish(ctx, _ref(ph, n, 0))
+
+
+@pytest.mark.parametrize("n,use_graph", [(200, True), (270, True), (270, False)])
+def test_columns_after_the_time_bound(ph, n, use_graph):
+    ref = _ref(ph, n, 0)
+    ctx = _built(ph, n, use_graph=use_graph, timeout_ms=1)
+    ctx.reduce(max_passes=0)
+    seen = []
+    _until_done(ph, ctx, lambda: seen.append(_check_columns(ctx, ref)))
+    assert seen and seen == sorted(set(seen))  # every call runs at least one more pass
+    _finish(ctx, ref)
