@@ -90,7 +90,6 @@ struct ReduceState {
   int32_t* act2 = nullptr;
   int32_t* alen = nullptr;     // per slot: the column's stored length (both lists)
   int32_t* alen2 = nullptr;
-  int64_t act_cap = 0;
   void* meta = nullptr;        // per id: ColMeta (rows, length, flags, clearing mark)
   int32_t** nxt_ptr = nullptr; // per active slot: new location
   int32_t* nxt_len = nullptr;
@@ -102,8 +101,8 @@ struct ReduceState {
   void* look = nullptr;        // look-back states of the survivor scan
   void* dlist = nullptr;       // deferred column updates
   void* src_e = nullptr;       // per active slot: source candidate of Phase II
-  int32_t* lows = nullptr;     // [lows_rows][m] per pass (ring) and slot: the low at its start
-  int32_t lows_rows = 0;
+  // look-ahead (lows is null without it)
+  int32_t* lows = nullptr;     // [kAheadMax][m] per pass (ring) and slot: the low at its start
   int32_t* due = nullptr;      // per slot: the pass whose additions visit its column next
   void* prec = nullptr;        // per row: its proven pivot's rows (int4)
   int32_t* delta = nullptr;    // per id: rows added to the column that are not in its list yet
@@ -131,6 +130,7 @@ struct ReduceState {
   };
   std::vector<Retired> retired;  // arena buffers outgrown between two compacting passes
   std::vector<ColStore> pivots;  // chunks holding proven columns
+  std::vector<ColStore> spare;   // ... and chunks for the next ones, left by a restart
   // the pass loop: one pass as the body of a conditional while node, per variant of its additions
   // (add_variant), with the arguments it was made with; a graph outlives the reduction and runs
   // again while another one's arguments are the same (a context that builds complexes of one
@@ -142,6 +142,8 @@ struct ReduceState {
     std::vector<unsigned char> args;
   };
   int32_t passes = 0;
+  std::vector<int32_t> caps;  // the passes at which calls were capped, and
+  size_t caps_met = 0;        // how many of them a restarted reduction has come by
   bool init = false;
   bool done = false;
   int status = PH_OK;
@@ -165,6 +167,7 @@ struct ph_ctx {
   std::vector<ph::ReduceState::Loop> retired;  // replaced, not yet given back
   cudaStream_t capture_stream = nullptr;       // private: graphs are captured on it
   int loop_blocks_per_sm = -1;  // resident blocks of the loop kernel (-1: not asked yet)
+  size_t device_bytes = 0;      // memory of the device (0: not asked yet)
   std::string err;
   int64_t launches = 0;  // kernels launched by this context
 

@@ -3412,6 +3412,9 @@ __global__ void k_reduce_init(int64_t m, InitLayout L, int32_t* rows0,
   }
 }
 
+// look-back states: chunks of any shape (8 slots or more; 1 or 4 for a few columns), or tiles
+static int64_t look_words(int64_t m) { return (m + 7) / 8 + 1 + kWarps; }
+
 static RArgs make_args(ph_ctx* ctx) {
   ReduceState& rs = ctx->rs;
   RArgs a;
@@ -3615,103 +3618,75 @@ static int64_t first_arena(const ph_ctx* ctx, bool look_ahead) {
                                    : 2 * ctx->nnz + 1;
 }
 
-// Look-ahead's arrays and first arenas, about 360 bytes per column (pass by pass: 50). Without room for
-// them, or when they would take more than a quarter of the device's memory, the reduction runs
-// pass by pass: what fitted without look-ahead still does.
+// the first arenas and the pivot store's first chunk: pass 0 needs at most the boundary matrix twice
+// over, or once and a visit's rows per column; later passes need less (they grow on demand otherwise)
+static void take_stores(ph_ctx* ctx, bool look_ahead) {
+  ReduceState& rs = ctx->rs;
+  for (ColStore& s : rs.arena) grow_store(ctx, s, first_arena(ctx, look_ahead));
+  ColStore c{};
+  grow_store(ctx, c, ctx->nnz / 4 + 1);
+  rs.pivots.push_back(c);
+}
+
+static void free_ahead(ph_ctx* ctx) {
+  ReduceState& rs = ctx->rs;
+  for (void* p : {(void*)rs.prec, (void*)rs.lows, (void*)rs.due, (void*)rs.delta, (void*)rs.kind,
+                  (void*)rs.newpos, (void*)rs.work})
+    ctx->dfree(p);
+  rs.prec = nullptr;
+  rs.lows = rs.due = rs.delta = rs.newpos = rs.work = nullptr;
+  rs.kind = nullptr;
+}
+
+// Look-ahead's arrays and stores: some 580 bytes per column, where pass by pass the stores take 100.
+// They come last at set-up: without room for them, or when they would take more than two fifths of the
+// device's memory, the reduction runs pass by pass. When a later allocation fails it starts again pass
+// by pass (restart_pass_by_pass).
 static bool take_ahead(ph_ctx* ctx) {
   ReduceState& rs = ctx->rs;
   const int64_t m = ctx->m, rows = ctx->dimoff[ctx->max_dim];
-  size_t free_bytes = 0, total_bytes = 0;
-  PH_CUDA(cudaMemGetInfo(&free_bytes, &total_bytes));
+  if (ctx->device_bytes == 0) {  // (how much of it is free tells little: allocators hold blocks back)
+    size_t free_bytes = 0;
+    PH_CUDA(cudaMemGetInfo(&free_bytes, &ctx->device_bytes));
+  }
   const double bytes = 16.0 * rows + (4.0 * (kAheadMax + 1 + kDeltaRows + 2) + 1.0) * m +
-                       8.0 * first_arena(ctx, true);
-  if (bytes > total_bytes / 4.0) return false;
+                       16.0 * first_arena(ctx, true);  // (two arenas of twice that many words)
+  if (bytes > 0.4 * ctx->device_bytes) return false;
   try {
     rs.prec = alloc_n<int4>(ctx, rows);
-    rs.lows_rows = kAheadMax;
-    rs.lows = alloc_n<int32_t>(ctx, rs.lows_rows * lows_stride_of(m));
+    rs.lows = alloc_n<int32_t>(ctx, kAheadMax * lows_stride_of(m));
     rs.due = alloc_n<int32_t>(ctx, lows_stride_of(m));
     rs.delta = alloc_n<int32_t>(ctx, kDeltaRows * m + kColSlack);
     rs.kind = alloc_n<uint8_t>(ctx, m);
     rs.newpos = alloc_n<int32_t>(ctx, m);
     rs.work = alloc_n<int32_t>(ctx, m);
-    grow_store(ctx, rs.arena[0], first_arena(ctx, true));
-    grow_store(ctx, rs.arena[1], first_arena(ctx, true));
+    take_stores(ctx, true);
     return true;
   } catch (const Fail&) {
     ctx->err.clear();
-    for (void* p : {(void*)rs.prec, (void*)rs.lows, (void*)rs.due, (void*)rs.delta, (void*)rs.kind,
-                    (void*)rs.newpos, (void*)rs.work, (void*)rs.arena[0].p, (void*)rs.arena[1].p})
-      ctx->dfree(p);
-    rs.prec = nullptr;
-    rs.lows_rows = 0;
-    rs.lows = rs.due = rs.delta = rs.newpos = rs.work = nullptr;
-    rs.kind = nullptr;
-    rs.arena[0] = rs.arena[1] = ColStore{};
+    free_ahead(ctx);
+    for (ColStore& s : rs.arena) {
+      ctx->dfree(s.p);
+      s = ColStore{};
+    }
     return false;
   }
 }
 
-void reduce_init(ph_ctx* ctx) {
-  free_reduce_state(ctx);  // whatever an earlier, failed initialisation left
-  // Phase I's tile states carry a (cloud, dimension) segment in 23 bits
-  PH_REQUIRE((int64_t)ctx->seg_start.size() - 1 < (1 << 23), PH_ERR_CAPACITY,
-             "at most 8,388,607 (cloud, dimension) segments per reduction");
+// the unreduced state of a reduction whose memory is there, with or without look-ahead
+static void set_up(ph_ctx* ctx) {
   ReduceState& rs = ctx->rs;
   cudaStream_t st = ctx->stream;
   const int64_t m = ctx->m;
-  rs.act = alloc_n<int32_t>(ctx, m);
-  rs.act2 = alloc_n<int32_t>(ctx, m);
-  rs.alen = alloc_n<int32_t>(ctx, m);
-  rs.alen2 = alloc_n<int32_t>(ctx, m);
-  rs.act_cap = m;
-  rs.meta = alloc_n<ColMeta>(ctx, m);
-  rs.nxt_ptr = alloc_n<int32_t*>(ctx, m);
-  rs.nxt_len = alloc_n<int32_t>(ctx, m);
-  rs.owner = alloc_n<int32_t>(ctx, m);
-  rs.tab = alloc_n<unsigned long long>(ctx, ctx->dimoff[ctx->max_dim]);
-  int nseg = (int)ctx->seg_start.size() - 1;
-  rs.first_unp = alloc_n<int32_t>(ctx, nseg);
+  const int nseg = (int)ctx->seg_start.size() - 1;
   PH_CUDA(cudaMemsetAsync(rs.first_unp, 0x7f, nseg * sizeof(int32_t), st));  // above every id
-  rs.dirty = alloc_n<int32_t>(ctx, 3 * nseg);  // next_unp, dirty_on, dirty
   PH_CUDA(cudaMemsetAsync(rs.dirty, 0x7f, nseg * sizeof(int32_t), st));
   PH_CUDA(cudaMemsetAsync(rs.dirty + nseg, 0, nseg * sizeof(int32_t), st));
-  // Phase I's tile states; the loop kernel's tiles are of another size and have their own
-  const int64_t ntiles = (m + kFTile - 1) / kFTile;
-  const int64_t loop_tiles = (std::min<int64_t>(m, kLoopStart) + kThreads - 1) / kThreads;
-  rs.tiles_bytes = (ntiles + 1 + loop_tiles) * sizeof(unsigned long long);
-  rs.tiles = ctx->dalloc(rs.tiles_bytes);
   PH_CUDA(cudaMemsetAsync(rs.tiles, 0, rs.tiles_bytes, st));  // no state published yet
-  // chunks of any shape (8 slots or more; 1 or 4 for a few columns), or tiles
-  const int64_t nchunks = (m + 7) / 8 + 1 + kWarps;
-  rs.look = alloc_n<unsigned long long>(ctx, nchunks);
-  PH_CUDA(cudaMemsetAsync(rs.look, 0, nchunks * sizeof(unsigned long long), st));
-  rs.dlist = alloc_n<int32_t>(ctx, m);
-  // look-ahead for long lists (per-pass counters, and sets chosen pass by pass, need every pass to
-  // take every column)
-  const bool look_ahead = !ctx->opts.collect_stats && ctx->opts.phase2_sets <= 0 &&
-                          ctx->three_rows() && m >= kAheadFrom && take_ahead(ctx);
-  const int32_t ahead = look_ahead ? kAheadMax : 1;
-  if (!look_ahead) rs.prec = alloc_n<int4>(ctx, 1);
-  rs.src_e = alloc_n<int32_t>(ctx, m);
-  if (ctx->opts.predict_pairs) {
-    const int64_t rows = ctx->dimoff[ctx->max_dim];
-    const int64_t nwords = (rows + 31) / 32;
-    rs.unp_bits = alloc_n<uint32_t>(ctx, nwords + 1);
-    rs.unp_words = alloc_n<int32_t>(ctx, nwords + 1);
-    rs.pred = alloc_n<int32_t>(ctx, m);
-    PH_CUDA(cudaMemsetAsync(rs.pred, 0xff, (size_t)m * sizeof(int32_t), st));
-  }
-  if (ctx->opts.phase2_sets > 0) {
-    const int64_t rows = std::max<int64_t>(ctx->dimoff[ctx->max_dim], 1);
-    rs.set_n = alloc_n<int32_t>(ctx, rows);
-    rs.set_neg = alloc_n<int32_t>(ctx, rows);
-    rs.set_on = alloc_n<uint8_t>(ctx, rows);
-    rs.set_key = alloc_n<uint64_t>(ctx, 4 * rows);
-  }
-  rs.dstate = ctx->dalloc(sizeof(DevState));
-  if (!rs.hstate) PH_CUDA(cudaMallocHost(&rs.hstate, sizeof(DevState)));  // kept by the context
-  rs.h_stats.clear();
+  PH_CUDA(cudaMemsetAsync(rs.look, 0, look_words(m) * sizeof(unsigned long long), st));
+  if (rs.pred) PH_CUDA(cudaMemsetAsync(rs.pred, 0xff, (size_t)m * sizeof(int32_t), st));
+  if (rs.pass_stats)
+    PH_CUDA(cudaMemsetAsync(rs.pass_stats, 0, (size_t)rs.stats_rows * PH_PS_N * 8, st));
   InitLayout L{};
   L.maxd = ctx->max_dim;
   for (int d = 0; d <= ctx->max_dim + 1; d++) L.dimoff[d] = ctx->dimoff[d];
@@ -3724,19 +3699,7 @@ void reduce_init(ph_ctx* ctx) {
       m, L, ctx->rows0, ctx->col_off, static_cast<ColMeta*>(rs.meta), ctx->low, rs.act,
       rs.alen, rs.owner, rs.tab, rs.lows, rs.due, static_cast<int4*>(rs.prec));
   PH_CHECK_LAUNCH();
-  // first arenas: pass 0 needs at most the boundary matrix twice over, or once and a visit's
-  // rows per column; later passes need less (they grow on demand otherwise)
-  const int64_t arena0 = first_arena(ctx, look_ahead);
-  grow_store(ctx, rs.arena[0], arena0);
-  grow_store(ctx, rs.arena[1], arena0);
-  ColStore c{};
-  grow_store(ctx, c, ctx->nnz / 4 + 1);
-  rs.pivots.push_back(c);
-  if (ctx->opts.collect_stats) {
-    rs.stats_rows = 256;
-    rs.pass_stats = alloc_n<int64_t>(ctx, (int64_t)rs.stats_rows * PH_PS_N);
-    PH_CUDA(cudaMemsetAsync(rs.pass_stats, 0, (size_t)rs.stats_rows * PH_PS_N * 8, st));
-  }
+  const int32_t ahead = rs.lows ? kAheadMax : 1;
   DevState& h = *static_cast<DevState*>(rs.hstate);
   h = DevState{};
   h.act = rs.act;
@@ -3748,8 +3711,8 @@ void reduce_init(ph_ctx* ctx) {
     h.arena[i] = rs.arena[i].p;
     h.arena_cap[i] = rs.arena[i].cap;
   }
-  h.piv_base = c.p;
-  h.piv_cap = c.cap;
+  h.piv_base = rs.pivots.back().p;
+  h.piv_cap = rs.pivots.back().cap;
   h.piv_used = 0;
   h.stats = rs.pass_stats;
   h.stats_rows = rs.stats_rows;
@@ -3782,11 +3745,104 @@ void reduce_init(ph_ctx* ctx) {
     launch_k(ctx, false, k_first, (unsigned)grid_for(ctx, std::max(m, a0.rows_end), kThreads), kThreads,
              0, st, a0);
   }
-  rs.passes = 0;
   rs.fresh = true;
+}
+
+void reduce_init(ph_ctx* ctx) {
+  free_reduce_state(ctx);  // whatever an earlier, failed initialisation left
+  // Phase I's tile states carry a (cloud, dimension) segment in 23 bits
+  PH_REQUIRE((int64_t)ctx->seg_start.size() - 1 < (1 << 23), PH_ERR_CAPACITY,
+             "at most 8,388,607 (cloud, dimension) segments per reduction");
+  ReduceState& rs = ctx->rs;
+  const int64_t m = ctx->m;
+  rs.act = alloc_n<int32_t>(ctx, m);
+  rs.act2 = alloc_n<int32_t>(ctx, m);
+  rs.alen = alloc_n<int32_t>(ctx, m);
+  rs.alen2 = alloc_n<int32_t>(ctx, m);
+  rs.meta = alloc_n<ColMeta>(ctx, m);
+  rs.nxt_ptr = alloc_n<int32_t*>(ctx, m);
+  rs.nxt_len = alloc_n<int32_t>(ctx, m);
+  rs.owner = alloc_n<int32_t>(ctx, m);
+  rs.tab = alloc_n<unsigned long long>(ctx, ctx->dimoff[ctx->max_dim]);
+  int nseg = (int)ctx->seg_start.size() - 1;
+  rs.first_unp = alloc_n<int32_t>(ctx, nseg);
+  rs.dirty = alloc_n<int32_t>(ctx, 3 * nseg);  // next_unp, dirty_on, dirty
+  // Phase I's tile states; the loop kernel's tiles are of another size and have their own
+  const int64_t ntiles = (m + kFTile - 1) / kFTile;
+  const int64_t loop_tiles = (std::min<int64_t>(m, kLoopStart) + kThreads - 1) / kThreads;
+  rs.tiles_bytes = (ntiles + 1 + loop_tiles) * sizeof(unsigned long long);
+  rs.tiles = ctx->dalloc(rs.tiles_bytes);
+  rs.look = alloc_n<unsigned long long>(ctx, look_words(m));
+  rs.dlist = alloc_n<int32_t>(ctx, m);
+  rs.src_e = alloc_n<int32_t>(ctx, m);
+  if (ctx->opts.predict_pairs) {
+    const int64_t rows = ctx->dimoff[ctx->max_dim];
+    const int64_t nwords = (rows + 31) / 32;
+    rs.unp_bits = alloc_n<uint32_t>(ctx, nwords + 1);
+    rs.unp_words = alloc_n<int32_t>(ctx, nwords + 1);
+    rs.pred = alloc_n<int32_t>(ctx, m);
+  }
+  if (ctx->opts.phase2_sets > 0) {
+    const int64_t rows = std::max<int64_t>(ctx->dimoff[ctx->max_dim], 1);
+    rs.set_n = alloc_n<int32_t>(ctx, rows);
+    rs.set_neg = alloc_n<int32_t>(ctx, rows);
+    rs.set_on = alloc_n<uint8_t>(ctx, rows);
+    rs.set_key = alloc_n<uint64_t>(ctx, 4 * rows);
+  }
+  if (ctx->opts.collect_stats) {
+    rs.stats_rows = 256;
+    rs.pass_stats = alloc_n<int64_t>(ctx, (int64_t)rs.stats_rows * PH_PS_N);
+  }
+  rs.dstate = ctx->dalloc(sizeof(DevState));
+  if (!rs.hstate) PH_CUDA(cudaMallocHost(&rs.hstate, sizeof(DevState)));  // kept by the context
+  rs.h_stats.clear();
+  // look-ahead for long lists (per-pass counters, and sets chosen pass by pass, need every pass to
+  // take every column)
+  const bool look_ahead = !ctx->opts.collect_stats && ctx->opts.phase2_sets <= 0 &&
+                          ctx->three_rows() && m >= kAheadFrom && take_ahead(ctx);
+  if (!look_ahead) take_stores(ctx, false);
+  set_up(ctx);
+  rs.passes = 0;
   rs.init = true;
   rs.done = false;
   rs.status = PH_OK;
+}
+
+// A reduction with look-ahead that found no memory starts again pass by pass. Between two horizons
+// columns are ahead of the pass, which is no state to leave behind; a pass-by-pass run decides the
+// same (reduce_run takes the caps of earlier calls again on the way) and stops for want of memory
+// before the pass that needs it, with all columns up to date. It keeps all memory it has, so that it comes as far as the run before if the allocator gives nothing more;
+// look-ahead's larger arenas are exchanged for its own if it gives these.
+static void restart_pass_by_pass(ph_ctx* ctx) {
+  ReduceState& rs = ctx->rs;
+  free_ahead(ctx);
+  for (auto& r : rs.retired) ctx->dfree(r.p);
+  rs.retired.clear();
+  const int64_t first = first_arena(ctx, false);
+  for (ColStore& s : rs.arena) {
+    if (ctx->opts.arena_words > 0 || s.cap <= 2 * first) continue;
+    ColStore c{};
+    try {
+      grow_store(ctx, c, first);
+    } catch (const Fail&) {
+      ctx->err.clear();
+      continue;
+    }
+    ctx->dfree(s.p);
+    s = c;
+  }
+  // the chunks of the pivot store: the largest one first
+  std::sort(rs.pivots.begin(), rs.pivots.end(),
+            [](const ColStore& x, const ColStore& y) { return x.cap < y.cap; });
+  rs.spare.insert(rs.spare.end(), rs.pivots.begin(), rs.pivots.end() - 1);
+  rs.pivots.erase(rs.pivots.begin(), rs.pivots.end() - 1);
+  for (auto e : rs.ev) cudaEventDestroy(e);
+  rs.ev.clear();
+  rs.add_launches = 0;
+  rs.ms_add = 0;
+  rs.add_ms.clear();
+  rs.caps_met = 0;
+  set_up(ctx);
 }
 
 // grows whatever the stopped pass asked for, in the host mirror h
@@ -3820,7 +3876,12 @@ static void serve_host_request(ph_ctx* ctx, DevState& h) {
   }
   if (h.host_reason & 2) {  // a new pivot chunk; the old ones stay (their columns live there)
     ColStore c{};
-    grow_store(ctx, c, std::max<int64_t>(2 * (int64_t)h.bound_piv, ctx->nnz / 4 + 1));
+    if (!rs.spare.empty() && rs.spare.back().cap >= (int64_t)h.bound_piv) {  // a restart left it
+      c = rs.spare.back();
+      rs.spare.pop_back();
+    } else {
+      grow_store(ctx, c, std::max<int64_t>(2 * (int64_t)h.bound_piv, ctx->nnz / 4 + 1));
+    }
     rs.pivots.push_back(c);
     h.piv_base = c.p;
     h.piv_cap = c.cap;
@@ -3959,18 +4020,23 @@ int reduce_run(ph_ctx* ctx, int32_t max_passes) {
     serve_host_request(ctx, h);
   }
   // every pass proves or zeroes at least one column, so m + 1 passes always suffice
-  h.max_passes = max_passes < 0 ? (int32_t)std::min<int64_t>(ctx->m + 1, INT32_MAX) : max_passes;
-  h.blocks_done = 0;
-  h.bar_count = h.bar_gen = 0;
+  int32_t cap = max_passes < 0 ? (int32_t)std::min<int64_t>(ctx->m + 1, INT32_MAX) : max_passes;
   unsigned loop_blocks = use_graph ? loop_grid(ctx) : 0;
-  h.loop_below = loop_blocks ? kLoopBelow : -1;
-  h.drain = 0;
   const int64_t limit_ms = ctx->opts.timeout_ms > 0 ? ctx->opts.timeout_ms : 60000;
-  h.t_limit = (unsigned long long)limit_ms * 1000000ull;
-  PH_CUDA(cudaMemcpyAsync(rs.dstate, &h, sizeof(DevState), cudaMemcpyHostToDevice, st));
-  k_clock_start<<<1, 1, 0, st>>>(static_cast<DevState*>(rs.dstate));
-  PH_CHECK_LAUNCH();
-  const RArgs a = make_args(ctx);
+  auto next_cap = [&] { return rs.caps_met < rs.caps.size() ? rs.caps[rs.caps_met] : cap; };
+  auto begin = [&] {
+    h.max_passes = next_cap();
+    h.blocks_done = 0;
+    h.bar_count = h.bar_gen = 0;
+    h.loop_below = loop_blocks ? kLoopBelow : -1;
+    h.drain = 0;
+    h.t_limit = (unsigned long long)limit_ms * 1000000ull;
+    PH_CUDA(cudaMemcpyAsync(rs.dstate, &h, sizeof(DevState), cudaMemcpyHostToDevice, st));
+    k_clock_start<<<1, 1, 0, st>>>(static_cast<DevState*>(rs.dstate));
+    PH_CHECK_LAUNCH();
+  };
+  begin();
+  RArgs a = make_args(ctx);
 
   bool started = false;    // this call has launched passes
   bool in_loop = false;    // the last of them by k_loop
@@ -4036,6 +4102,14 @@ int reduce_run(ph_ctx* ctx, int32_t max_passes) {
       PH_CUDA(cudaMemcpyAsync(rs.dstate, &h, sizeof(DevState), cudaMemcpyHostToDevice, st));
       continue;
     }
+    if (h.status == ST_CAPPED && rs.caps_met < rs.caps.size()) {  // after a restart
+      rs.caps_met++;
+      h.max_passes = next_cap();
+      h.pass = h.passes + 1;
+      h.status = ST_RUN;
+      PH_CUDA(cudaMemcpyAsync(rs.dstate, &h, sizeof(DevState), cudaMemcpyHostToDevice, st));
+      continue;
+    }
     if (h.status == ST_HOST) {
       if (time_add && rs.ev.size() >= 2) {  // the stopped pass's k_add did no work
         cudaEventDestroy(rs.ev.back());
@@ -4047,7 +4121,25 @@ int reduce_run(ph_ctx* ctx, int32_t max_passes) {
       // space for Phase II (reasons 1, 2): the pass continues there, its marks made; counter
       // rows (reason 4): asked for between two passes, the next pass runs whole
       rest_only = (h.host_reason & 3) != 0;
-      serve_host_request(ctx, h);
+      try {
+        serve_host_request(ctx, h);
+      } catch (const Fail& f) {
+        if (f.code != PH_ERR_ALLOC || !rs.lows) throw;
+        ctx->err.clear();
+        if (h.ahead > 1) {  // (as far as it had come, if the call's cap lies below)
+          cap = std::max(cap, h.pass);
+          restart_pass_by_pass(ctx);
+          rs.fresh = false;
+          rest_only = started = in_loop = false;
+          loop_states_clear = true;
+          begin();
+          a = make_args(ctx);
+          continue;
+        }
+        free_ahead(ctx);  // (look-ahead is over)
+        a = make_args(ctx);
+        serve_host_request(ctx, h);
+      }
       if (rest_only) {
         const DevState marked = h;  // what the marks left for the rest of the pass stays
         reset_counters(&h);
@@ -4069,6 +4161,8 @@ int reduce_run(ph_ctx* ctx, int32_t max_passes) {
   PH_REQUIRE(h.status != ST_TIMEOUT, PH_ERR_TIMEOUT,
              "the pass loop ran past the time bound (ph_opts.timeout_ms)");
   rs.passes = h.passes;
+  if (h.status == ST_CAPPED) rs.caps.push_back(h.passes);
+  rs.caps_met = rs.caps.size();
   rs.status = h.status == ST_DONE ? PH_OK : PH_NOT_CONVERGED;
   if (ctx->opts.collect_stats) {
     rs.h_stats.assign((size_t)(rs.passes + 1) * PH_PS_N, 0);
@@ -4261,6 +4355,7 @@ void free_reduce_state(ph_ctx* ctx) {
   for (auto& a : rs.arena) ctx->dfree(a.p);
   for (auto& r : rs.retired) ctx->dfree(r.p);
   for (auto& c : rs.pivots) ctx->dfree(c.p);
+  for (auto& c : rs.spare) ctx->dfree(c.p);
   for (auto e : rs.ev) cudaEventDestroy(e);
   void* hstate = rs.hstate;  // (page-locked: kept by the context)
   rs = ReduceState{};

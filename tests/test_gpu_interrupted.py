@@ -148,3 +148,56 @@ def test_columns_after_the_time_bound(ph, n, use_graph):
     _until_done(ph, ctx, lambda: seen.append(_check_columns(ctx, ref)))
     assert seen and seen == sorted(set(seen))  # every call runs at least one more pass
     _finish(ctx, ref)
+
+
+class Allocator:
+    """torch's allocator with a number of blocks left to give (None: any)."""
+
+    def __init__(self, blocks=None):
+        self.blocks, self.used, self.size = blocks, 0, {}
+
+    def alloc(self, nbytes, stream):
+        import torch
+
+        if self.blocks is not None:
+            if self.blocks == 0:
+                return 0
+            self.blocks -= 1
+        p = torch.cuda.caching_allocator_alloc(nbytes, stream=stream)
+        self.size[p] = nbytes
+        self.used += nbytes
+        return p
+
+    def free(self, p):
+        import torch
+
+        self.used -= self.size.pop(p)
+        torch.cuda.caching_allocator_delete(p)
+
+    def opts(self):
+        return dict(device_alloc=self.alloc, device_free=self.free)
+
+
+# one-word arenas, which the passes grow as they need: the call fails at the first to the eighth block
+@pytest.mark.parametrize("n,use_graph", [(200, True), (270, True), (270, False)])
+def test_reads_after_a_refused_allocation(ph, n, use_graph):
+    ref = _ref(ph, n, 1)
+    failed = []
+    for blocks in range(8):
+        mem = Allocator()
+        ctx = _built(ph, n, use_graph=use_graph, arena_words=1, **mem.opts())
+        ctx.reduce(max_passes=1)
+        _check_pairs(ctx)
+        mem.blocks = blocks
+        try:
+            ctx.reduce()
+        except ph.PHError as err:
+            assert err.code == -2
+            mem.blocks = None
+            _check_pairs(ctx)
+            failed.append(_check_columns(ctx, ref))
+        mem.blocks = None
+        _finish(ctx, ref)
+        ctx.close()
+        assert mem.used == 0
+    assert failed
