@@ -259,12 +259,13 @@ int ph_load_boundary(ph_ctx* ctx, int64_t m, const int32_t* dims, const int64_t*
  * A later call continues a reduction that stopped at its pass cap (PH_NOT_CONVERGED), at the
  * time bound (PH_ERR_TIMEOUT) or on a failed allocation (PH_ERR_ALLOC, the state left as
  * before the pass that needed the memory); after a complete reduction it returns the result
- * again. From 3,000,000 columns on a reduction takes more memory (some 640 bytes per column where it
- * takes 160) and runs faster. When it gets no more, the call starts again from the unreduced matrix
- * with the smaller need, its time bound anew, and goes by the passes it had done; if memory is
- * refused on that way too, the state left is that of the pass it came to. The pass loop runs in a CUDA graph and, for short active lists, in one cooperative
- * kernel (use_graph), or from the host. Synchronises the
- * stream. */
+ * again. From 3,000,000 columns on a reduction takes more memory (some 640 bytes per column where
+ * it takes 160; 140 go back when it is complete, or between two calls when an allocation of
+ * the context needs them) and runs faster. When it gets no more, the call starts again from the
+ * unreduced matrix with the smaller need, its time bound anew, and goes by the passes it had done;
+ * if memory is refused on that way too, the state left is that of the pass it came to. The
+ * pass loop runs in a CUDA graph and, for short active lists, in one cooperative kernel
+ * (use_graph), or from the host. Synchronises the stream. */
 int ph_reduce(ph_ctx* ctx, int32_t max_passes, ph_stats* out);
 
 /* Discards the reduction state (and extracted outputs) of the context; the next ph_reduce

@@ -56,9 +56,10 @@ void* ph_ctx::dalloc(size_t bytes) {
     return b.p;
   }
   void* p = nullptr;
-  for (int attempt = 0; attempt < 2 && !p; attempt++) {
-    if (attempt > 0) {  // make room
-      if (kept.empty()) break;
+  for (int attempt = 0; attempt < 3 && !p; attempt++) {
+    if (attempt > 0) {  // make room: the kept blocks, then those a reduction can do without
+      if (attempt > 1 && !ph::give_up_ahead(this)) break;
+      if (attempt == 1 && kept.empty()) continue;
       drop_kept(INT64_MAX);
     }
     if (has_alloc) {

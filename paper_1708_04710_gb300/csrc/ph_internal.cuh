@@ -120,6 +120,7 @@ struct ReduceState {
   int64_t tiles_bytes = 0;
   void* dstate = nullptr;      // per-pass state in device memory
   bool fresh = false;         // set up, not run yet
+  bool resting = false;       // between two calls, after a whole number of passes
   void* hstate = nullptr;      // pinned host mirror of it
   int64_t* pass_stats = nullptr;  // device [stats_rows][PH_PS_N]
   int32_t stats_rows = 0;
@@ -434,6 +435,8 @@ void reduce_init(ph_ctx* ctx);
 int reduce_run(ph_ctx* ctx, int32_t max_passes);
 void free_reduce_state(ph_ctx* ctx);
 void free_graphs(ph_ctx* ctx);
+// whether there was memory to give back
+bool give_up_ahead(ph_ctx* ctx);
 // E^l of one cloud, one byte per simplex in filtration order, into host memory (n bytes)
 void essential_estimate(ph_ctx* ctx, int32_t cloud, uint8_t* host_out, int64_t n);
 // predicted lowstar per simplex of one cloud (filtration indices, -1), into host memory

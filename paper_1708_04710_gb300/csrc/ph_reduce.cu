@@ -3641,7 +3641,8 @@ static void free_ahead(ph_ctx* ctx) {
 // Look-ahead's arrays and stores: some 580 bytes per column, where pass by pass the stores take 100.
 // They come last at set-up: without room for them, or when they would take more than two fifths of the
 // device's memory, the reduction runs pass by pass. When a later allocation fails it starts again pass
-// by pass (restart_pass_by_pass).
+// by pass (restart_pass_by_pass), and one that waits between two calls gives them back
+// (give_up_ahead). So what fits without look-ahead fits.
 static bool take_ahead(ph_ctx* ctx) {
   ReduceState& rs = ctx->rs;
   const int64_t m = ctx->m, rows = ctx->dimoff[ctx->max_dim];
@@ -3845,6 +3846,28 @@ static void restart_pass_by_pass(ph_ctx* ctx) {
   set_up(ctx);
 }
 
+// A reduction with look-ahead that rests between two calls (capped, or stopped at the time bound: all
+// columns up to date, all lists whole) goes on pass by pass, and gives look-ahead's arrays back. Its
+// next pass compacts into the other arena.
+bool give_up_ahead(ph_ctx* ctx) {
+  ReduceState& rs = ctx->rs;
+  if (!rs.resting || !rs.lows) return false;
+  DevState& h = *static_cast<DevState*>(rs.hstate);
+  if (h.ahead > 1) {
+    if (!h.compact) {
+      h.compact = 1;
+      h.arena_cur ^= 1;
+      h.arena_used = 0;
+    }
+    h.ahead = 1;
+    h.leave = 0;
+    h.horizon = (h.status == ST_CAPPED ? h.passes + 1 : h.pass) + 1;
+    PH_CUDA(cudaMemcpyAsync(rs.dstate, &h, sizeof(DevState), cudaMemcpyHostToDevice, ctx->stream));
+  }
+  free_ahead(ctx);
+  return true;
+}
+
 // grows whatever the stopped pass asked for, in the host mirror h
 static void serve_host_request(ph_ctx* ctx, DevState& h) {
   ReduceState& rs = ctx->rs;
@@ -4002,6 +4025,7 @@ int reduce_run(ph_ctx* ctx, int32_t max_passes) {
   const bool use_graph = ctx->opts.use_graph != 0 && ctx->opts.phase2_sets <= 0;
   const bool time_add = ctx->opts.time_kernels != 0 && !use_graph;
   DevState& h = *static_cast<DevState*>(rs.hstate);
+  rs.resting = false;
   // a resumed reduction continues after the pass that hit the previous cap
   bool loop_states_clear = rs.fresh;  // k_loop's tile states: nothing of an earlier pass in them
   if (!rs.fresh) {  // (what set-up wrote is still in the host's copy)
@@ -4158,6 +4182,7 @@ int reduce_run(ph_ctx* ctx, int32_t max_passes) {
              "device bounds check " + std::to_string(h.debug_fault) + " failed (debug build)");
   PH_REQUIRE(h.status != ST_FAULT, PH_ERR_CUDA,
              "a bounded wait in the addition kernel ran out (look-back did not complete)");
+  rs.resting = true;
   PH_REQUIRE(h.status != ST_TIMEOUT, PH_ERR_TIMEOUT,
              "the pass loop ran past the time bound (ph_opts.timeout_ms)");
   rs.passes = h.passes;
@@ -4180,6 +4205,7 @@ int reduce_run(ph_ctx* ctx, int32_t max_passes) {
   }
   rs.ev.clear();
   rs.done = true;
+  if (rs.status == PH_OK) free_ahead(ctx);
   return rs.status;
 }
 

@@ -151,10 +151,11 @@ def test_columns_after_the_time_bound(ph, n, use_graph):
 
 
 class Allocator:
-    """torch's allocator with a number of blocks left to give (None: any)."""
+    """torch's allocator with a number of blocks left to give, or a number of bytes in all."""
 
-    def __init__(self, blocks=None):
-        self.blocks, self.used, self.size = blocks, 0, {}
+    def __init__(self, blocks=None, budget=None):
+        self.blocks, self.budget = blocks, budget
+        self.size, self.used, self.peak, self.log = {}, 0, 0, []
 
     def alloc(self, nbytes, stream):
         import torch
@@ -163,9 +164,13 @@ class Allocator:
             if self.blocks == 0:
                 return 0
             self.blocks -= 1
+        if self.budget is not None and self.used + nbytes > self.budget:
+            return 0
         p = torch.cuda.caching_allocator_alloc(nbytes, stream=stream)
         self.size[p] = nbytes
         self.used += nbytes
+        self.peak = max(self.peak, self.used)
+        self.log.append(self.used)
         return p
 
     def free(self, p):
@@ -201,3 +206,31 @@ def test_reads_after_a_refused_allocation(ph, n, use_graph):
         ctx.close()
         assert mem.used == 0
     assert failed
+
+
+# budgets from the pass-by-pass run's need to look-ahead's, at every block that its call takes
+def test_what_fits_pass_by_pass_fits(ph):
+    n = 270
+    ref = _ref(ph, n, 5)
+
+    def run(mem, passes, **opts):
+        ctx = _built(ph, n, **mem.opts(), **opts)
+        built = len(mem.log)
+        ctx.reduce(max_passes=5)
+        _check_pairs(ctx)
+        assert _check_columns(ctx, ref) == 5
+        if passes < 0:
+            _finish(ctx, ref)
+        used = mem.log[built:]
+        ctx.close()
+        assert mem.used == 0
+        return used
+
+    for passes in (5, -1):
+        least, most = Allocator(), Allocator()
+        run(least, passes, collect_stats=True)
+        used = run(most, passes)
+        assert most.peak > least.peak
+        for budget in sorted({least.peak, (least.peak + most.peak) // 2}
+                             | {u for u in used if u > least.peak}):
+            run(Allocator(budget=budget), passes)
