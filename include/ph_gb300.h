@@ -96,9 +96,9 @@ typedef struct {
    * (two 128-thread blocks each; 0 = library default, 4) */
   int32_t add_blocks_per_sm;
   /* wall-clock bound of one ph_reduce's pass loop in ms, checked on the device at the end of
-   * every pass (0 = library default, 60000); past it the call returns PH_ERR_TIMEOUT, for a
-   * complex of 3,000,000 columns or more once the up to eight passes that its columns may be
-   * ahead by are done */
+   * every pass (0 = library default, 60000); past it the call returns PH_ERR_TIMEOUT, for
+   * 3,000,000 triangles or more without larger simplices once the up to eight passes that
+   * their columns may be ahead by are done */
   int32_t timeout_ms;
   /* 1: every pass also applies the non-zero case of Corollary 10 (Lemma 9): an active column j
    * with beta_j >= 0 whose candidate set L_j (rows of K_{d-1} in [beta_j, low(j)] not known to
@@ -140,9 +140,9 @@ typedef struct {
    * priority other than 0 or 1 (PH_ERR_INVALID). */
   int32_t phase2_sets;
   int32_t phase2_priority;
-  /* Initial capacity of each of the two survivor arenas, in int32 words (0, default: twice the
-   * boundary's nonzeros; from 3,000,000 columns of at most three rows on, the nonzeros and 24
-   * words per column). A pass whose Phase I bound does not fit stops after its marks,
+  /* What each of the two survivor arenas has to hold at first, in int32 words; it gets twice that,
+   * 2^20 words at least (0, default: twice the boundary's nonzeros; for 3,000,000 triangles or
+   * more without larger simplices the nonzeros and 24 words per column). A pass whose Phase I bound does not fit stops after its marks,
    * before any column changes; the host grows the arena and the pass continues with its column
    * additions, so a small value trades memory for extra host round trips; results are the
    * same. */
@@ -259,13 +259,13 @@ int ph_load_boundary(ph_ctx* ctx, int64_t m, const int32_t* dims, const int64_t*
  * A later call continues a reduction that stopped at its pass cap (PH_NOT_CONVERGED), at the
  * time bound (PH_ERR_TIMEOUT) or on a failed allocation (PH_ERR_ALLOC, the state left as
  * before the pass that needed the memory); after a complete reduction it returns the result
- * again. From 3,000,000 columns on a reduction takes more memory (some 640 bytes per column where
- * it takes 160; 140 go back when it is complete, or between two calls when an allocation of
- * the context needs them) and runs faster. When it gets no more, the call starts again from the
- * unreduced matrix with the smaller need, its time bound anew, and goes by the passes it had done;
- * if memory is refused on that way too, the state left is that of the pass it came to. The
- * pass loop runs in a CUDA graph and, for short active lists, in one cooperative kernel
- * (use_graph), or from the host. Synchronises the stream. */
+ * again. From 3,000,000 triangles on, without larger simplices, a reduction takes more memory (some
+ * 640 bytes per column where it takes 160; 140 go back when it is complete, or between two
+ * calls when an allocation of the context needs them) and runs faster. When it gets no more, the
+ * call starts again from the unreduced matrix with the smaller need, its time bound anew, and
+ * goes by the passes it had done; if memory is refused on that way too, the state left is that of
+ * the pass it came to. The pass loop runs in a CUDA graph and, for short active lists, in one
+ * cooperative kernel (use_graph), or from the host. Synchronises the stream. */
 int ph_reduce(ph_ctx* ctx, int32_t max_passes, ph_stats* out);
 
 /* Discards the reduction state (and extracted outputs) of the context; the next ph_reduce

@@ -231,8 +231,10 @@ struct ph_ctx {
   int64_t *e_idx = nullptr, *e_d2 = nullptr;
   int32_t* e_dim = nullptr;
 
-  // a column of the boundary matrix has at most three rows
-  bool three_rows() const { return col_off == nullptr && max_dim <= 2; }
+  // the triangles of a complex without larger simplices
+  int64_t three_row_columns() const {
+    return col_off == nullptr && max_dim == 2 ? dimoff[3] - dimoff[2] : 0;
+  }
 
   void* dalloc(size_t bytes);
   void dfree(void* p);

@@ -577,8 +577,9 @@ constexpr int kAheadMax = 8;  // passes per visit (a power of two: rows of store
 // What visits add to a column gathers in a block of its own (its delta) until it is merged into
 // the column's list: up to kOld rows are kept from visit to visit, and a visit adds up to R rows
 // per pass: R = 2, the rows of a triangle's boundary beside its low. (Look-ahead is for complexes
-// whose columns have at most three rows; with R = 3, for tetrahedra, it lost: 8 Gaussian
-// dimensions, 120 points, 0.9 M simplices, 1.8 -> 2.8 ms.)
+// whose top columns are triangles' three rows; with R = 3, for tetrahedra, it lost: 8 Gaussian
+// dimensions, 120 points, 0.9 M simplices, 1.8 -> 2.8 ms. So it did on the two rows of edges:
+// 4.5 M of 3000 points without triangles 3.9 -> 7.5 ms, 8 M of 4000 points 6.4 -> 13.6 ms.)
 constexpr int kSourceRows = 2;
 constexpr int kOld = 8;
 // Look-ahead is bound by instruction issue (some 230 warp instructions per pass of a visit) where
@@ -589,7 +590,7 @@ constexpr int kOld = 8;
 // below kAheadFrom, where a visit's two kernels and the larger tables also cost memory. Lists that
 // shrink under kAheadAbove go on pass by pass (10.67 M columns: 34.3 ms with twice as many, 33.7 with
 // 100,000; 3.7 M in 48 clouds: 5.85 and 5.95 ms; here 34.1 and 5.85).
-constexpr int64_t kAheadFrom = 3000000;   // columns from which look-ahead pays, and
+constexpr int64_t kAheadFrom = 3000000;   // triangles from which look-ahead pays, and columns
 constexpr int64_t kAheadAbove = 250000;   // down to which it goes on
 constexpr int kLonger = 12;  // the longest source inside a visit: kRecRows + this many rows
 constexpr int kDeltaRows = kOld + kSourceRows * kAheadMax;
@@ -3800,7 +3801,7 @@ void reduce_init(ph_ctx* ctx) {
   // look-ahead for long lists (per-pass counters, and sets chosen pass by pass, need every pass to
   // take every column)
   const bool look_ahead = !ctx->opts.collect_stats && ctx->opts.phase2_sets <= 0 &&
-                          ctx->three_rows() && m >= kAheadFrom && take_ahead(ctx);
+                          ctx->three_row_columns() >= kAheadFrom && take_ahead(ctx);
   if (!look_ahead) take_stores(ctx, false);
   set_up(ctx);
   rs.passes = 0;

@@ -234,3 +234,22 @@ def test_what_fits_pass_by_pass_fits(ph):
         for budget in sorted({least.peak, (least.peak + most.peak) // 2}
                              | {u for u in used if u > least.peak}):
             run(Allocator(budget=budget), passes)
+
+
+# 3,126,250 edges of 2500 points: look-ahead is for triangles, edges keep to the memory (and the two to
+# three times shorter time) of a pass-by-pass run
+def test_edges_alone_take_no_look_ahead(ph):
+    import torch
+
+    x = torch.from_numpy(pc.random_cloud(2500, 3, 41)).cuda()
+    out = []
+    for opts in ({"collect_stats": True}, {}):
+        mem = Allocator()
+        ctx = ph.Context(**mem.opts(), **opts)
+        ctx.build_filtration(x, None, 1)
+        built = len(mem.log)
+        assert ctx.reduce()["converged"]
+        out.append((max(mem.log[built:]), ctx.filtration(0)["low"]))
+        ctx.close()
+    assert abs(out[0][0] - out[1][0]) < 1 << 20  # (the counters)
+    assert np.array_equal(out[0][1], out[1][1])
