@@ -287,3 +287,27 @@ def test_look_ahead_without_room_runs_pass_by_pass(ph):
     assert refused
     for r, g in zip(_state(ref), _state(got)):
         assert np.array_equal(r, g)
+
+
+# read-out of columns: up to eight rows by a lane, longer ones and bitmaps by the warp, 32 columns at a time
+@pytest.mark.parametrize("n", [1, 31, 32, 33, 97])
+def test_columns_of_all_lengths(ph, n):
+    rng = np.random.default_rng(n)
+    rows0 = 400
+    length = rng.choice([0, 1, 7, 8, 9, 31, 32, 33, 64, 200], n)
+    cols = [np.sort(rng.choice(rows0, k, replace=False)) for k in length]
+    dims = np.repeat(np.array([0, 1], np.int32), [rows0, n])
+    colptr = np.concatenate([np.zeros(rows0, np.int64), [0], np.cumsum(length)])
+    rows = np.concatenate(cols + [[]]).astype(np.int32)
+    ctx = ph.Context(use_cor10=False)
+    ctx.load_boundary(dims, colptr, rows)
+    ctx.reduce(max_passes=0)  # no addition: the columns as they were loaded
+    ptr, got = ctx.columns(0)
+    assert np.array_equal(ptr, colptr) and np.array_equal(got, rows)
+    full = []
+    for threshold in (-1, 1):  # reduced, as rows and as bitmaps
+        c = ph.Context(dense_threshold=threshold)
+        c.load_boundary(dims, colptr, rows)
+        c.reduce()
+        full.append(c.columns(0))
+    assert all(np.array_equal(a, b) for a, b in zip(*full))
