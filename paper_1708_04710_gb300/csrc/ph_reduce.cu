@@ -3817,22 +3817,28 @@ void reduce_init(ph_ctx* ctx) {
 // look-ahead's larger arenas are exchanged for its own if it gives these.
 static void restart_pass_by_pass(ph_ctx* ctx) {
   ReduceState& rs = ctx->rs;
+  ColStore block{rs.delta, kDeltaRows * ctx->m};
+  rs.delta = nullptr;
   free_ahead(ctx);
   for (auto& r : rs.retired) ctx->dfree(r.p);
   rs.retired.clear();
   const int64_t first = first_arena(ctx, false);
   for (ColStore& s : rs.arena) {
-    if (ctx->opts.arena_words > 0 || s.cap <= 2 * first) continue;
     ColStore c{};
-    try {
-      grow_store(ctx, c, first);
-    } catch (const Fail&) {
-      ctx->err.clear();
-      continue;
+    if (s.cap < block.cap / 2) {  // one that look-ahead had no use for yet: the deltas' block will do
+      std::swap(c, block);
+    } else if (ctx->opts.arena_words <= 0 && s.cap > 2 * first) {
+      try {
+        grow_store(ctx, c, first);
+      } catch (const Fail&) {
+        ctx->err.clear();
+      }
     }
+    if (!c.p) continue;
     ctx->dfree(s.p);
     s = c;
   }
+  ctx->dfree(block.p);
   // the chunks of the pivot store: the largest one first
   std::sort(rs.pivots.begin(), rs.pivots.end(),
             [](const ColStore& x, const ColStore& y) { return x.cap < y.cap; });
