@@ -631,7 +631,7 @@ int ph_reduce(ph_ctx* ctx, int32_t max_passes, ph_stats* out) {
   // the places of the results belong to the lows as they are: they go before any pass changes these,
   // since the call may also end part-way (time bound, refused allocation)
   ctx->extracted = false;
-  if (!ctx->rs.init) ph::reduce_init(ctx);
+  if (!ctx->rs.init) ph::reduce_init(ctx, max_passes);
   int rc = ctx->rs.status;
   if (!(ctx->rs.done && ctx->rs.status == PH_OK)) rc = ph::reduce_run(ctx, max_passes);
   ctx->reduced = true;

@@ -121,6 +121,7 @@ struct ReduceState {
   void* dstate = nullptr;      // per-pass state in device memory
   bool fresh = false;         // set up, not run yet
   bool resting = false;       // between two calls, after a whole number of passes
+  int ahead_later = 0;        // look-ahead begins with the next call that is long enough, the n-th at last
   void* hstate = nullptr;      // pinned host mirror of it
   int64_t* pass_stats = nullptr;  // device [stats_rows][PH_PS_N]
   int32_t stats_rows = 0;
@@ -433,7 +434,7 @@ void build_vr(ph_ctx* ctx, const int32_t* coords, const int64_t* cloud_offsets, 
 void load_boundary(ph_ctx* ctx, int64_t m, const int32_t* dims, const int64_t* colptr,
                    const int32_t* rows);
 void compute_beta(ph_ctx* ctx);
-void reduce_init(ph_ctx* ctx);
+void reduce_init(ph_ctx* ctx, int32_t max_passes);
 int reduce_run(ph_ctx* ctx, int32_t max_passes);
 void free_reduce_state(ph_ctx* ctx);
 void free_graphs(ph_ctx* ctx);

@@ -254,3 +254,31 @@ def test_edges_alone_take_no_look_ahead(ph):
         ctx.close()
     assert abs(out[0][0] - out[1][0]) < 1 << 20  # (the counters)
     assert np.array_equal(out[0][1], out[1][1])
+
+
+# a first and a second call of up to two passes take no look-ahead (and its memory), a longer one or the
+# third begins it; every state on the way is that of a pass-by-pass run with the same caps
+@pytest.mark.parametrize("caps,ahead", [((0,), False), ((2,), False), ((3,), True), ((1, 3), False),
+                                        ((0, 1), False), ((0, 4), True), ((1, 2, 3), True),
+                                        ((2, -1), True)], ids=str)
+@pytest.mark.parametrize("opts", [{}, {"use_graph": False}, {"dense_threshold": 1},
+                                  {"predict_pairs": True}], ids=str)
+def test_look_ahead_begins_with_a_long_call(ph, caps, ahead, opts):
+    n, mem = 270, Allocator()
+    got = _built(ph, n, **mem.opts(), **opts)
+    ref = _built(ph, n, **{**opts, "collect_stats": True, "use_graph": False})
+    built = len(mem.log)
+    for i, cap in enumerate(caps):
+        st = got.reduce(max_passes=cap)
+        want = ref.reduce(max_passes=cap)
+        assert st["passes"] == want["passes"] and st["converged"] == want["converged"]
+        assert (max(mem.log[built:]) > 400 * got.m) == (ahead and i == len(caps) - 1)
+        assert np.array_equal(got.filtration(0)["low"], ref.filtration(0)["low"])
+        for a, b in zip(got.columns(0), ref.columns(0)):
+            assert np.array_equal(a, b)
+        assert np.array_equal(got.essential_estimate(0), ref.essential_estimate(0))
+    _check_pairs(got)
+    assert got.reduce()["passes"] == ref.reduce()["passes"]
+    assert np.array_equal(got.filtration(0)["low"], ref.filtration(0)["low"])
+    if "predict_pairs" in opts:
+        assert np.array_equal(got.predicted_lows(0), ref.predicted_lows(0))
