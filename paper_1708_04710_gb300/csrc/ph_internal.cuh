@@ -120,6 +120,7 @@ struct ReduceState {
   int64_t tiles_bytes = 0;
   void* dstate = nullptr;      // per-pass state in device memory
   bool fresh = false;         // set up, not run yet
+  bool loop_ran = false;      // passes ran in k_loop, which leaves the other kernels' tile states alone
   bool resting = false;       // between two calls, after a whole number of passes
   int ahead_later = 0;        // look-ahead begins with the next call that is long enough, the n-th at last
   void* hstate = nullptr;      // pinned host mirror of it

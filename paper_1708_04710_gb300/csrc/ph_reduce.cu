@@ -755,8 +755,10 @@ __device__ __forceinline__ void check_capacity(DevState* ds) {
 constexpr int kFItems = 4;
 constexpr int kFTile = kThreads * kFItems;
 // tile state word: pass tag (8 bits) | flags (2) | segment (23) | val + 1 (31). Eight bits of
-// tag tell this pass from the previous ones: the active list never grows within a reduction, so
-// a tile in use in pass p was in use, and published, in pass p - 1, and set-up clears every state
+// tag tell this pass from the previous ones: the active list never grows within a reduction, so a
+// tile in use in pass p was published in pass p - 1, or, by look-ahead's larger tiles between horizons,
+// eight passes before at most. Set-up clears every state, and a pass after k_loop, which has states of
+// its own, those that it left alone
 constexpr unsigned long long kTAgg = 1ull << 54, kTIncl = 2ull << 54, kTFlags = 3ull << 54;
 __device__ __forceinline__ unsigned long long tile_word(unsigned long long tag, unsigned long long flag,
                                                        SegMax x) {
@@ -3752,6 +3754,7 @@ static void set_up(ph_ctx* ctx) {
              0, st, a0);
   }
   rs.fresh = true;
+  rs.loop_ran = false;
 }
 
 // the stored lows of the active columns, which are all up to date, and the records of the pivots
@@ -4163,13 +4166,21 @@ int reduce_run(ph_ctx* ctx, int32_t max_passes) {
       }
       PH_CUDA(ce);
       PH_CHECK_LAUNCH();
-    } else if (use_graph) {
-      ran_graph = true;
-      in_loop = false;
-      PH_CUDA(cudaGraphLaunch(pass_graph(ctx, a, variant), st));
+      rs.loop_ran = true;
     } else {
-      launch_pass(ctx, a, 0, false, variant, time_add, st);
-      if (time_add) rs.add_launches++;
+      if (rs.loop_ran) {  // (a later call on a share of the device without room for k_loop)
+        PH_CUDA(cudaMemsetAsync(a.tile_st, 0, (a.loop_tile_st - a.tile_st) * sizeof(unsigned long long),
+                                st));
+        rs.loop_ran = false;
+      }
+      in_loop = false;
+      if (use_graph) {
+        ran_graph = true;
+        PH_CUDA(cudaGraphLaunch(pass_graph(ctx, a, variant), st));
+      } else {
+        launch_pass(ctx, a, 0, false, variant, time_add, st);
+        if (time_add) rs.add_launches++;
+      }
     }
     started = true;
     PH_CUDA(cudaMemcpyAsync(&h, rs.dstate, sizeof(DevState), cudaMemcpyDeviceToHost, st));
