@@ -282,3 +282,16 @@ def test_look_ahead_begins_with_a_long_call(ph, caps, ahead, opts):
     assert np.array_equal(got.filtration(0)["low"], ref.filtration(0)["low"])
     if "predict_pairs" in opts:
         assert np.array_equal(got.predicted_lows(0), ref.predicted_lows(0))
+
+
+# the pairs that Corollary 10 predicts, of columns ahead of the pass and in the loop kernel
+@pytest.mark.parametrize("n", [17, 40, 86, 270])
+def test_predictions_equal_pass_by_pass(ph, n):
+    ref = _built(ph, n, collect_stats=True, predict_pairs=True, use_graph=False)
+    got = _built(ph, n, predict_pairs=True)
+    for caps in ((0,), (1,), (4,), (8,), (9,), (-1,), (2, 3, 9, 10, -1)):
+        for ctx in (ref, got):
+            ctx.reset_reduction()
+            for cap in caps:
+                ctx.reduce(max_passes=cap)
+        assert np.array_equal(ref.predicted_lows(0), got.predicted_lows(0)), caps
