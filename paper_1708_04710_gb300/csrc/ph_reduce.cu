@@ -124,7 +124,9 @@ struct DevState {
   // ... and once merge pieces are on and fewer than narrow_below columns are active, rounds of
   // 8 columns per warp, so that the short late passes spread over more warps (ST_SWITCH, once)
   unsigned int loop_blocks;  // blocks of the loop kernel still at work
-  int64_t loop_below;  // the loop kernel takes over from the graph at this many columns (-1: never)
+  int64_t loop_below;  // the loop kernel takes over from the graph at this many columns (-1: never),
+  int64_t loop_words;  // and hands back to it after a pass of more arena words than this
+  int64_t pass_words;  // arena words of the last pass
   int32_t narrow_on;
   int64_t narrow_below;
   int32_t chunk_slots;  // slots per chunk of this pass's k_add (8, 32, 64 or 128)
@@ -3215,6 +3217,13 @@ __device__ __forceinline__ bool grid_last(DevState* ds, unsigned blocks, unsigne
 // (16,384 to 65,536 measure alike, 131,072 costs 50 to 90 us).
 constexpr int64_t kLoopBelow = (int64_t)1 << 14;
 constexpr int64_t kLoopStart = 110000;
+// Long columns, or bitmaps, want the whole machine: after a pass of more than kLoopWords arena words k_loop
+// hands back to the graph, which hands over again below half of that. Random columns of three rows,
+// k_loop alone -> with this rule: 14,000 on 8000 rows 98.4 -> 71.2 ms, 40,000 on 20,000 rows 565 -> 314
+// ms; 24,600 random triangles on 80 points 31.7 -> 28.4 ms. With half as many words 6000 columns on 4000
+// rows, whose passes k_loop does faster, take 22.9 ms instead of 19.0; with twice as many the triangles
+// take 29.3, with four times the 14,000 columns stay at 98.5.
+constexpr int64_t kLoopWords = (int64_t)1 << 20;
 // columns left to one block, whose barriers are __syncthreads (64 and 256 measure alike)
 constexpr int64_t kLoopSingle = 64;
 constexpr int kLoopBlocks = 2;  // per SM: registers for every part of a pass without spills
@@ -3288,6 +3297,7 @@ __device__ void end_of_pass(const RArgs& a, cudaGraphConditionalHandle cond, int
   const int64_t n_act = ds->n_act, warp_below = ds->warp_below, warp_words = ds->warp_words;
   const int64_t lane_words = ds->lane_words, narrow_below = ds->narrow_below;
   const int64_t ahead_above = ds->ahead_above, loop_below = ds->loop_below;
+  const int64_t loop_words = ds->loop_words;
   const unsigned long long used = ds->arena_used, targets = ds->totals[1];
   const unsigned long long t_start = ds->t_start, t_limit = ds->t_limit;
   int32_t* const act = ds->act;
@@ -3304,6 +3314,7 @@ __device__ void end_of_pass(const RArgs& a, cudaGraphConditionalHandle cond, int
   if (to_dense) ds->dense_on = 1;
   if (status == ST_RUN) {
     ds->n_act = n_surv;
+    ds->pass_words = (int64_t)used;
     if (compact) {
       ds->act = act2;
       ds->act2 = act;
@@ -3356,7 +3367,10 @@ __device__ void end_of_pass(const RArgs& a, cudaGraphConditionalHandle cond, int
       if (late && whole) status = ST_TIMEOUT;
       else if (mode != kInLoop && (to_dense || to_warp || to_pieces || to_narrow || to_add))
         status = ST_SWITCH;
-      else if (in_graph && ahead == 1 && n_surv <= loop_below) status = ST_SWITCH;
+      else if (mode == kInLoop ? (int64_t)used > loop_words
+                               : in_graph && ahead == 1 && n_surv <= loop_below &&
+                                     2 * (int64_t)used <= loop_words)
+        status = ST_SWITCH;
       // counter rows for the next pass: its first kernel writes them before any capacity check
       if (status != ST_TIMEOUT && stats && p + 1 >= stats_rows) {
         ds->host_reason = 4;
@@ -4117,6 +4131,7 @@ int reduce_run(ph_ctx* ctx, int32_t max_passes) {
     h.blocks_done = 0;
     h.bar_count = h.bar_gen = 0;
     h.loop_below = loop_blocks ? kLoopBelow : -1;
+    h.loop_words = kLoopWords;
     h.drain = 0;
     h.t_limit = (unsigned long long)limit_ms * 1000000ull;
     PH_CUDA(cudaMemcpyAsync(rs.dstate, &h, sizeof(DevState), cudaMemcpyHostToDevice, st));
@@ -4138,7 +4153,7 @@ int reduce_run(ph_ctx* ctx, int32_t max_passes) {
       rest_only = false;
       launch_pass_rest(ctx, a, 0, false, variant, time_add, st);
       if (time_add) rs.add_launches++;
-    } else if (use_graph && loop_blocks && h.ahead == 1 &&
+    } else if (use_graph && loop_blocks && h.ahead == 1 && h.pass_words <= h.loop_words &&
                h.n_act <= (started && !in_loop ? h.loop_below : kLoopStart)) {
       // a state's tag has eight bits: one left by an earlier stay in k_loop could pass for this one's
       if (!in_loop && !loop_states_clear) {

@@ -311,3 +311,25 @@ def test_columns_of_all_lengths(ph, n):
         c.reduce()
         full.append(c.columns(0))
     assert all(np.array_equal(a, b) for a, b in zip(*full))
+
+
+# a pass of more than 2^20 arena words goes back to the pass graph, one of half as many on to the loop kernel:
+# random columns of three rows fill in, and thin out at the end
+@pytest.mark.parametrize("opts", [{}, {"dense_threshold": -1}, {"arena_words": 1}], ids=str)
+def test_loop_kernel_hands_long_columns_back(ph, opts):
+    rows0, n = 6000, 10000
+    rng = np.random.default_rng(5)
+    cols = np.sort(rng.integers(0, rows0, (n, 3)), axis=1)
+    cols = cols[(np.diff(cols, axis=1) > 0).all(1)]
+    dims = np.repeat(np.array([0, 1], np.int32), [rows0, len(cols)])
+    colptr = np.concatenate([np.zeros(rows0, np.int64), 3 * np.arange(len(cols) + 1)])
+
+    def load(ctx):
+        ctx.load_boundary(dims, colptr, cols.reshape(-1).astype(np.int32))
+
+    _same_reduction(ph, load, opts, (200, -1))
+    ctx = ph.Context(**opts)
+    load(ctx)
+    before = ctx.kernel_launches()
+    ctx.reduce()
+    assert ctx.kernel_launches() - before > 300  # three kernels for each of the graph's passes
