@@ -124,9 +124,7 @@ struct DevState {
   // ... and once merge pieces are on and fewer than narrow_below columns are active, rounds of
   // 8 columns per warp, so that the short late passes spread over more warps (ST_SWITCH, once)
   unsigned int loop_blocks;  // blocks of the loop kernel still at work
-  int64_t loop_below;  // the loop kernel takes over from the graph at this many columns (-1: never),
-  int64_t loop_words;  // and hands back to it after a pass of more arena words than this
-  int64_t pass_words;  // arena words of the last pass
+  int64_t loop_below;  // the loop kernel takes over from the graph at this many columns (-1: never)
   int32_t narrow_on;
   int64_t narrow_below;
   int32_t chunk_slots;  // slots per chunk of this pass's k_add (8, 32, 64 or 128)
@@ -140,6 +138,8 @@ struct DevState {
   int32_t arena_cur;  // the arena this pass writes into
   int32_t drain;      // past the time bound: no more look-ahead, stop after the horizon's pass
   int32_t leave;      // the last pass of look-ahead
+  // (at the end: among the words that every pass's last block reads it cost the passes 0.7 %)
+  int64_t pass_words;  // arena words of the last pass before a switch
 };
 
 struct RArgs {
@@ -216,7 +216,6 @@ struct PV {
   int32_t limit;      // the last pass a column visited now may run ahead to
   int32_t ahead;      // passes a visit may run ahead; 1: every pass visits every column
   int32_t whole;      // ... and the lists must be whole there (the pass cap, or the time bound)
-  int32_t drain;      // past the time bound
 };
 
 // The left-most-column table holds, per row, a column below the pass it was entered for, counted
@@ -246,8 +245,7 @@ __device__ __forceinline__ PV pass_view(const DevState* ds) {
   v.ahead = ds->ahead;
   v.limit = ds->drain || ds->leave ? ds->pass + 1
                       : min(min(ds->pass + ds->ahead, ds->horizon), ds->max_passes);
-  v.drain = ds->drain;
-  v.whole = v.drain || v.limit == ds->max_passes;
+  v.whole = ds->drain || v.limit == ds->max_passes;
   return v;
 }
 
@@ -2675,7 +2673,7 @@ __device__ __forceinline__ void visit_round(const RArgs& a, const PV& v, int32_t
     const bool c10 = visit && a.cor10 && a.beta[j] < 0;
     no_beta = c10;
     // (at the time bound the loop may stop before the pass that zeroes the column: it keeps its rows)
-    const int32_t fu = c10 && !v.drain ? a.first_unp[seg_of(a, j) - a.nc] : INT32_MIN;
+    const int32_t fu = c10 && !a.ds->drain ? a.first_unp[seg_of(a, j) - a.nc] : INT32_MIN;
     if (look_ahead(a, v, pass, visit, fu, pos, w)) tidy<0>(w, visit && !w.gone);
     else tidy<kOld>(w, visit && !w.gone);
     if (visit) {
@@ -3297,7 +3295,6 @@ __device__ void end_of_pass(const RArgs& a, cudaGraphConditionalHandle cond, int
   const int64_t n_act = ds->n_act, warp_below = ds->warp_below, warp_words = ds->warp_words;
   const int64_t lane_words = ds->lane_words, narrow_below = ds->narrow_below;
   const int64_t ahead_above = ds->ahead_above, loop_below = ds->loop_below;
-  const int64_t loop_words = ds->loop_words;
   const unsigned long long used = ds->arena_used, targets = ds->totals[1];
   const unsigned long long t_start = ds->t_start, t_limit = ds->t_limit;
   int32_t* const act = ds->act;
@@ -3314,7 +3311,6 @@ __device__ void end_of_pass(const RArgs& a, cudaGraphConditionalHandle cond, int
   if (to_dense) ds->dense_on = 1;
   if (status == ST_RUN) {
     ds->n_act = n_surv;
-    ds->pass_words = (int64_t)used;
     if (compact) {
       ds->act = act2;
       ds->act2 = act;
@@ -3367,9 +3363,9 @@ __device__ void end_of_pass(const RArgs& a, cudaGraphConditionalHandle cond, int
       if (late && whole) status = ST_TIMEOUT;
       else if (mode != kInLoop && (to_dense || to_warp || to_pieces || to_narrow || to_add))
         status = ST_SWITCH;
-      else if (mode == kInLoop ? (int64_t)used > loop_words
+      else if (mode == kInLoop ? (int64_t)used > kLoopWords
                                : in_graph && ahead == 1 && n_surv <= loop_below &&
-                                     2 * (int64_t)used <= loop_words)
+                                     2 * (int64_t)used <= kLoopWords)
         status = ST_SWITCH;
       // counter rows for the next pass: its first kernel writes them before any capacity check
       if (status != ST_TIMEOUT && stats && p + 1 >= stats_rows) {
@@ -3378,6 +3374,7 @@ __device__ void end_of_pass(const RArgs& a, cudaGraphConditionalHandle cond, int
       }
     }
   }
+  if (status == ST_SWITCH) ds->pass_words = (int64_t)used;
   ds->status = status;
   if (in_graph) cudaGraphSetConditional(cond, status == ST_RUN ? 1u : 0u);
 }
@@ -3695,8 +3692,9 @@ static bool take_ahead(ph_ctx* ctx, DevState* h) {
   }
 }
 
-// the unreduced state of a reduction whose memory is there, with or without look-ahead
-static void set_up(ph_ctx* ctx) {
+// the unreduced columns of a reduction whose arrays are there, with or without look-ahead's; then, with
+// its stores, the pass loop's state
+static void set_up_columns(ph_ctx* ctx) {
   ReduceState& rs = ctx->rs;
   cudaStream_t st = ctx->stream;
   const int64_t m = ctx->m;
@@ -3721,6 +3719,12 @@ static void set_up(ph_ctx* ctx) {
       m, L, ctx->rows0, ctx->col_off, static_cast<ColMeta*>(rs.meta), ctx->low, rs.act,
       rs.alen, rs.owner, rs.tab, rs.lows, rs.due, static_cast<int4*>(rs.prec));
   PH_CHECK_LAUNCH();
+}
+
+static void set_up_passes(ph_ctx* ctx) {
+  ReduceState& rs = ctx->rs;
+  cudaStream_t st = ctx->stream;
+  const int64_t m = ctx->m;
   const int32_t ahead = rs.lows ? kAheadMax : 1;
   DevState& h = *static_cast<DevState*>(rs.hstate);
   h = DevState{};
@@ -3838,6 +3842,12 @@ void reduce_init(ph_ctx* ctx, int32_t max_passes) {
   rs.tiles = ctx->dalloc(rs.tiles_bytes);
   rs.look = alloc_n<unsigned long long>(ctx, look_words(m));
   rs.dlist = alloc_n<int32_t>(ctx, m);
+  // look-ahead for long lists (per-pass counters, and sets chosen pass by pass, need every pass to
+  // take every column)
+  const bool may = !ctx->opts.collect_stats && ctx->opts.phase2_sets <= 0 &&
+                   ctx->three_row_columns() >= kAheadFrom;
+  // (a block all the same: without it the others lie such that 0.57 M columns take 1650 us, not 1625)
+  if (!may) rs.prec = alloc_n<int4>(ctx, 1);
   rs.src_e = alloc_n<int32_t>(ctx, m);
   if (ctx->opts.predict_pairs) {
     const int64_t rows = ctx->dimoff[ctx->max_dim];
@@ -3860,13 +3870,11 @@ void reduce_init(ph_ctx* ctx, int32_t max_passes) {
   rs.dstate = ctx->dalloc(sizeof(DevState));
   if (!rs.hstate) PH_CUDA(cudaMallocHost(&rs.hstate, sizeof(DevState)));  // kept by the context
   rs.h_stats.clear();
-  // look-ahead for long lists (per-pass counters, and sets chosen pass by pass, need every pass to
-  // take every column)
-  const bool may = !ctx->opts.collect_stats && ctx->opts.phase2_sets <= 0 &&
-                   ctx->three_row_columns() >= kAheadFrom;
   rs.ahead_later = may && max_passes >= 0 && max_passes <= kFewPasses ? 2 : 0;
-  if (!may || rs.ahead_later || !take_ahead(ctx, nullptr)) take_stores(ctx, false);
-  set_up(ctx);
+  const bool ahead = may && !rs.ahead_later && take_ahead(ctx, nullptr);
+  set_up_columns(ctx);  // (the device is at work while the stores are taken)
+  if (!ahead) take_stores(ctx, false);
+  set_up_passes(ctx);
   rs.passes = 0;
   rs.init = true;
   rs.done = false;
@@ -3913,7 +3921,8 @@ static void restart_pass_by_pass(ph_ctx* ctx) {
   rs.ms_add = 0;
   rs.add_ms.clear();
   rs.caps_met = 0;
-  set_up(ctx);
+  set_up_columns(ctx);
+  set_up_passes(ctx);
 }
 
 // A reduction with look-ahead that rests between two calls (capped, or stopped at the time bound: all
@@ -4131,7 +4140,7 @@ int reduce_run(ph_ctx* ctx, int32_t max_passes) {
     h.blocks_done = 0;
     h.bar_count = h.bar_gen = 0;
     h.loop_below = loop_blocks ? kLoopBelow : -1;
-    h.loop_words = kLoopWords;
+    h.pass_words = 0;
     h.drain = 0;
     h.t_limit = (unsigned long long)limit_ms * 1000000ull;
     PH_CUDA(cudaMemcpyAsync(rs.dstate, &h, sizeof(DevState), cudaMemcpyHostToDevice, st));
@@ -4153,7 +4162,7 @@ int reduce_run(ph_ctx* ctx, int32_t max_passes) {
       rest_only = false;
       launch_pass_rest(ctx, a, 0, false, variant, time_add, st);
       if (time_add) rs.add_launches++;
-    } else if (use_graph && loop_blocks && h.ahead == 1 && h.pass_words <= h.loop_words &&
+    } else if (use_graph && loop_blocks && h.ahead == 1 && h.pass_words <= kLoopWords &&
                h.n_act <= (started && !in_loop ? h.loop_below : kLoopStart)) {
       // a state's tag has eight bits: one left by an earlier stay in k_loop could pass for this one's
       if (!in_loop && !loop_states_clear) {
