@@ -33,23 +33,24 @@
 //                pieces. Ten specialisations (row lists / bitmaps x block / 32-slot warp
 //                chunks x lane / piece merges, and 8-slot warp chunks with pieces); the loop
 //                switches between them at most four times per reduction.
-//   k_visit,     Phase II for long lists of columns of at most three rows (look-ahead): nineteen
-//   k_merge      of twenty additions have a proven pivot as their source, which will not change
-//                any more, so a visit runs up to eight passes of a column at once as long as its
-//                low meets proven pivots of few rows; the lows on the way are stored for the
-//                passes they belong to. What was added is kept beside the column's list (its
-//                delta) and merged into it every eighth pass. Lows, marks, pass counts and the
-//                reduced matrix are those of the pass-by-pass run.
+//   k_visit,     Phase II for long lists of triangles (look-ahead): nineteen of twenty additions
+//   k_merge      have a proven pivot as their source, which will not change any more, so a visit
+//                runs up to eight passes of a column at once as long as its low meets proven
+//                pivots of few rows; the lows on the way are stored for the passes they belong
+//                to. What was added is kept beside the column's list (its delta) and merged into
+//                it every eighth pass. Lows, marks, pass counts and the reduced matrix are those
+//                of the pass-by-pass run.
 //   (p sets)     With Phase II limited to p neighbour sets (Sec. 3.4), k_set_* rank the sets
 //                between k_phase1 and k_add and hold back the other targets.
 //   k_commit     publishes the new locations of the columns other jobs may have been reading
 //                and moves on the first unpaired row of the segments where it was paired; its last
 //                block ends the pass: the next active list, convergence (no collision left,
-//                Thm 8), the pass cap and time bound, and inside a CUDA graph the conditional that repeats the pass.
+//                Thm 8), the pass cap and time bound, and inside a CUDA graph the conditional
+//                that repeats the pass.
 // All per-pass state lives in device memory (DevState), so the same kernel sequence runs either
 // from a host loop or as the body of a graph's conditional while node. Each kernel may start
-// while its predecessor drains (programmatic dependent launch) and waits for it first. Short lists
-// run in k_loop, one cooperative kernel for all their passes.
+// while its predecessor drains (programmatic dependent launch) and waits for it first. Short lists of
+// short columns run in k_loop, one cooperative kernel for all their passes.
 #include <algorithm>
 #include <cstring>
 #include <utility>
@@ -87,7 +88,7 @@ struct DevState {
   unsigned int blocks_done;       // blocks of the current grid that have finished (last-block)
   unsigned long long t_start;     // global timer (ns) when this ph_reduce's loop began
   unsigned long long t_limit;     // ns the loop may run before it stops with ST_TIMEOUT
-  alignas(128) unsigned long long totals[2];  // [1]: targets of the current pass ([0] unused)
+  alignas(128) unsigned long long targets;  // of the current pass
   unsigned long long bound_words, bound_piv;
   alignas(128) unsigned long long arena_used;  // words taken in the arena of the current pass
   alignas(128) unsigned int queue;             // next chunk for k_add
@@ -121,10 +122,10 @@ struct DevState {
   // switches once per reduction (ST_SWITCH)
   int32_t lane_on;
   int64_t lane_words;
-  // ... and once merge pieces are on and fewer than narrow_below columns are active, rounds of
-  // 8 columns per warp, so that the short late passes spread over more warps (ST_SWITCH, once)
   unsigned int loop_blocks;  // blocks of the loop kernel still at work
   int64_t loop_below;  // the loop kernel takes over from the graph at this many columns (-1: never)
+  // ... and once merge pieces are on and fewer than narrow_below columns are active, rounds of
+  // 8 columns per warp, so that the short late passes spread over more warps (ST_SWITCH, once)
   int32_t narrow_on;
   int64_t narrow_below;
   int32_t chunk_slots;  // slots per chunk of this pass's k_add (8, 32, 64 or 128)
@@ -1281,7 +1282,7 @@ __device__ __forceinline__ void phase1_mid(const RArgs& a) {
     atomicAdd(&ds->bound_words, (unsigned long long)ww);
     atomicAdd(&ds->bound_piv, (unsigned long long)wp);
   }
-  if (lane_id() == 0 && wa) atomicAdd(&ds->totals[1], (unsigned long long)wa);  // still targets
+  if (lane_id() == 0 && wa) atomicAdd(&ds->targets, (unsigned long long)wa);  // still targets
 }
 
 // no more blocks take part in Phase I than there are tiles (the others leave at once: a short
@@ -2327,7 +2328,7 @@ __device__ __forceinline__ int merge_rows(const RArgs& a, const PV& v, WarpStage
 // by thread 0, after the block's rounds: its counters into the pass's
 __device__ __forceinline__ void flush_counters(const RArgs& a, const PV& v,
                                                const unsigned long long* s_cnt) {
-  if (s_cnt[kCntTargets]) atomicAdd(&a.ds->totals[1], s_cnt[kCntTargets]);
+  if (s_cnt[kCntTargets]) atomicAdd(&a.ds->targets, s_cnt[kCntTargets]);
   if (v.stats) {
     const int idx[kNumCnt] = {PH_PS_TARGETS, PH_PS_ACTIVE, PH_PS_CLEARED,
                               PH_PS_ADDS,    PH_PS_XORS,   PH_PS_COPIED, PH_PS_PACKED};
@@ -2983,9 +2984,8 @@ __device__ __forceinline__ void merge_round(const RArgs& a, const PV& v, int32_t
 }
 
 // kDense: the pass may meet bit-packed columns or convert some; the row-list variant carries none
-// of it. kSlots: columns per warp and round (32 or 8). kLane: each staged job merged by its own
-// lane (short columns), else merge pieces spread over the lanes. The host picks the variant from
-// DevState::dense_on, narrow_on and lane_on (a separate graph for each).
+// of it. kLane: each staged job merged by its own lane (short columns), else merge pieces spread over the
+// lanes. The host picks the variant from DevState::dense_on and lane_on (a separate graph for each).
 template <bool kDense, bool kLane>
 __device__ __forceinline__ void merge_pass(const RArgs& a, WarpStage& S, unsigned blocks) {
   __shared__ PV s_v;  // per-pass values from shared memory rather than held in registers
@@ -3039,7 +3039,6 @@ __global__ void k_ess_count(RArgs a, int64_t m) {
   ess_count(a, m, gridDim.x);
 }
 
-// E^l of the ids [lo, hi) (one dimension of one cloud), as bytes at their filtration index
 CloudIds cloud_ids(const ph_ctx* ctx, int32_t cloud) {
   CloudIds c;
   c.nd = ctx->max_dim + 1;
@@ -3053,6 +3052,7 @@ CloudIds cloud_ids(const ph_ctx* ctx, int32_t cloud) {
   return c;
 }
 
+// E^l of a cloud's ids, as bytes at their filtration index
 __global__ void k_ess_flags(CloudIds ids, const ColMeta* __restrict__ meta,
                             const int32_t* __restrict__ beta, const int32_t* __restrict__ owner,
                             const int64_t* __restrict__ gidx, int64_t n, uint8_t* out,
@@ -3072,7 +3072,6 @@ __global__ void k_ess_flags(CloudIds ids, const ColMeta* __restrict__ meta,
 // where a pass runs: host-driven, in the graph's loop (which stops when another variant of the
 // additions, or the loop kernel, suits the next passes better), in the loop kernel
 enum : int { kHostLoop = 0, kInGraph = 1, kInLoop = 2 };
-// the deferred column updates: new pivots (now in the pivot store) and left-most survivors
 __device__ void end_of_pass(const RArgs& a, cudaGraphConditionalHandle cond, int mode);
 
 // the counters a pass accumulates, cleared for the next one
@@ -3085,7 +3084,7 @@ __host__ __device__ inline void reset_counters(DevState* ds) {
   ds->n_work = 0;
   ds->n_dirty = 0;
   ds->n_due = ds->n_enter = ds->scan_end = 0;
-  ds->totals[0] = ds->totals[1] = 0;
+  ds->targets = 0;
 }
 
 // the deferred column updates and the next pass's row state, then (last block) the end of the
@@ -3295,7 +3294,7 @@ __device__ void end_of_pass(const RArgs& a, cudaGraphConditionalHandle cond, int
   const int64_t n_act = ds->n_act, warp_below = ds->warp_below, warp_words = ds->warp_words;
   const int64_t lane_words = ds->lane_words, narrow_below = ds->narrow_below;
   const int64_t ahead_above = ds->ahead_above, loop_below = ds->loop_below;
-  const unsigned long long used = ds->arena_used, targets = ds->totals[1];
+  const unsigned long long used = ds->arena_used, targets = ds->targets;
   const unsigned long long t_start = ds->t_start, t_limit = ds->t_limit;
   int32_t* const act = ds->act;
   int32_t* const act2 = ds->act2;
@@ -4267,7 +4266,7 @@ int reduce_run(ph_ctx* ctx, int32_t max_passes) {
         h.n_due = marked.n_due;
         h.n_enter = marked.n_enter;
         h.scan_end = marked.scan_end;
-        h.totals[1] = marked.totals[1];
+        h.targets = marked.targets;
       }
       PH_CUDA(cudaMemcpyAsync(rs.dstate, &h, sizeof(DevState), cudaMemcpyHostToDevice, st));
       continue;
