@@ -583,9 +583,10 @@ constexpr int kAheadMax = 8;  // passes per visit (a power of two: rows of store
 // 4.5 M of 3000 points without triangles 3.9 -> 7.5 ms, 8 M of 4000 points 6.4 -> 13.6 ms.)
 constexpr int kSourceRows = 2;
 constexpr int kOld = 8;
-// Look-ahead is bound by instruction issue (some 230 warp instructions per pass of a visit) where
-// pass-by-pass additions are bound by memory traffic: every pass rewrites every column and reads its
-// source. Pass by pass -> look-ahead: 10.67 M columns (400 points on a torus) 48.8 -> 36.9 ms, 4.5 M
+// Look-ahead spends instructions (4,360 warp instructions per round of 32 columns in a pass of 2.2 M, some
+// 230 of them per pass that a visit runs ahead; issue active 56 %, DRAM 13 %) where pass-by-pass
+// additions are bound by memory traffic: every pass rewrites every column and reads its source.
+// Pass by pass -> look-ahead: 10.67 M columns (400 points on a torus) 48.8 -> 36.9 ms, 4.5 M
 // on a torus 29.2 -> 22.6 ms, on a sphere 12.8 -> 8.7 ms, 42.7 M in 512 clouds 45.5 -> 41.8 ms; on
 // 2.6 M columns 11.9 -> 11.8 ms, on 1.3 M 6.5 -> 6.2 ms, on 0.9 M 4.4 -> 4.3 ms: little to gain
 // below kAheadFrom, where a visit's two kernels and the larger tables also cost memory. Lists that
