@@ -3884,8 +3884,9 @@ void reduce_init(ph_ctx* ctx, int32_t max_passes) {
 // A reduction with look-ahead that found no memory starts again pass by pass. Between two horizons
 // columns are ahead of the pass, which is no state to leave behind; a pass-by-pass run decides the
 // same (reduce_run takes the caps of earlier calls again on the way) and stops for want of memory
-// before the pass that needs it, with all columns up to date. It keeps all memory it has, so that it comes as far as the run before if the allocator gives nothing more;
-// look-ahead's larger arenas are exchanged for its own if it gives these.
+// before the pass that needs it, with all columns up to date. It keeps all memory it has, so that it
+// comes as far as the run before if the allocator gives nothing more; look-ahead's larger arenas are
+// exchanged for its own if it gives these.
 static void restart_pass_by_pass(ph_ctx* ctx) {
   ReduceState& rs = ctx->rs;
   ColStore block{rs.delta, kDeltaRows * ctx->m};
