@@ -142,10 +142,10 @@ typedef struct {
   int32_t phase2_priority;
   /* What each of the two survivor arenas has to hold at first, in int32 words; it gets twice that,
    * 2^20 words at least (0, default: twice the boundary's nonzeros; for 3,000,000 triangles or
-   * more without larger simplices the nonzeros and 24 words per column). A pass whose Phase I bound does not fit stops after its marks,
-   * before any column changes; the host grows the arena and the pass continues with its column
-   * additions, so a small value trades memory for extra host round trips; results are the
-   * same. */
+   * more without larger simplices the nonzeros and 24 words per column). A pass whose Phase I
+   * bound does not fit stops after its marks, before any column changes; the host grows the arena
+   * and the pass continues with its column additions, so a small value trades memory for extra
+   * host round trips; results are the same. */
   int64_t arena_words;
 } ph_opts;
 
